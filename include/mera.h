@@ -30,7 +30,17 @@
  *   256-byte aligned.  Apart from a status word and the fixed static array
  *   behind mera_ascend_noalloc, the library holds no device memory.
  * - prec selects the arithmetic of the contractions (the O(chi^9) part):
- *     MERA_PREC_F64    binary64 everywhere (FP64 units),
+ *     MERA_PREC_F64    binary64 everywhere.  Large products run on the
+ *                      tensor cores: each operand entry is cut into seven
+ *                      signed 8-bit digits relative to the largest entry of
+ *                      its row and of its block of 256 along the contraction
+ *                      index, the digit products are summed exactly, and the
+ *                      result is rounded once to binary64; errors are below
+ *                      those of a chain of binary64 FMAs, relative to those
+ *                      largest entries.  Rows that hold a NaN, an infinity
+ *                      or entries beyond 2^+-400, small products, and calls
+ *                      whose workspace does not hold the digits use the FP64
+ *                      units.
  *     MERA_PREC_TF32   tensor cores, TF32 operands, FP32 accumulation,
  *     MERA_PREC_BF16   tensor cores, BF16 operands, FP32 accumulation,
  *     MERA_PREC_BF16X3 tensor cores, each operand split into a BF16 pair
@@ -106,6 +116,8 @@ const char* mera_last_error(void);
  * Scratch bytes needed by one call of `op` (MERA_OP_*) with lower bond
  * dimension chi_b, upper bond dimension chi_t and mode prec.  For
  * MERA_OP_FIXED_POINT chi_b == chi_t == chi.  Writes the count to *bytes.
+ * With MERA_PREC_F64 this includes room for the operands' digits; a workspace
+ * that holds the operands alone is accepted too and keeps to the FP64 units.
  * Returns MERA_EINVAL for an unknown op/prec, chi outside [1, MERA_MAX_CHI],
  * chi_t > chi_b^2, or a NULL `bytes`.
  */
@@ -526,7 +538,9 @@ mera_status mera_set_slice_bytes(size_t bytes);
  * row-major M x N, all binary64 device arrays.  The operands are first cast
  * to the mode's operand format in `ws`, which needs
  * planes * (pad(M*ld) + pad(N*ld)) bytes (ld = K rounded up to 16 bytes,
- * pad = 256-byte multiple, planes = 2 for BF16X3, else 1).
+ * pad = 256-byte multiple, planes = 2 for BF16X3, else 1).  With
+ * MERA_PREC_F64 a workspace that also holds the operands' digits selects the
+ * tensor-core route.
  */
 mera_status mera_gemm_test(int prec, const double* A, const double* B, int M, int N, int K, double* C,
                            void* ws, size_t ws_bytes, void* stream);

@@ -119,7 +119,7 @@ bool prec_ok(int prec) { return prec >= MERA_PREC_F64 && prec <= MERA_PREC_OZ4; 
 
 // Bytes of one element of a program buffer (raw buffers of the fixed-point
 // split modes hold binary32 planes).
-int64_t buf_elem_bytes(const Buffer& b, int prec) { return b.raw ? 4 : elem_bytes(prec); }
+int64_t buf_elem_bytes(const Buffer& b, int prec) { return b.raw == 1 ? 4 : elem_bytes(prec); }
 
 // Tensor-core GEMM arguments of one program step; `out` is the caller's
 // output (root steps), `base` the workspace.
@@ -196,16 +196,23 @@ mera_status run_program(const OpProgram& prog, const double* const inputs[4], do
         if (p.skip || (reuse_resident && dg.bufs[p.op_buf].resident == 1)) continue;
         const int64_t plane = b.plane_bytes / buf_elem_bytes(b, prec);
         ProfScope ps(stream, 1, 0, 0.0);
-        cudaError_t e = launch_permute(p, inputs[p.slot], ws + b.offset, plane, b.raw ? PREC_RAW : prec, stream);
+        cudaError_t e = launch_permute(p, inputs[p.slot], ws + b.offset, plane, b.raw == 1 ? PREC_RAW : prec, stream);
         if (e != cudaSuccess) return cuda_status(e, "permute");
         continue;
       }
-      if (st.kind == 2) {  // fixed-point split of a raw buffer into its operand
+      if (st.kind == 2) {  // split of a raw buffer into its operand, or of an operand into its digit image
         const SplitStep& x = st.x;
         const Buffer& r = dg.bufs[x.raw_buf];
         const Buffer& d = dg.bufs[x.dst_buf];
         if (x.skip || (reuse_resident && d.resident == 1)) continue;
         ProfScope ps(stream, 1, 0, 0.0);
+        if (x.tile > 0) {
+          cudaError_t e = launch_x64_split(reinterpret_cast<const double*>(ws + r.offset), x.ld, x.rows, x.K,
+                                           x.seg_rows, x.tile, ws + d.offset,
+                                           reinterpret_cast<int*>(ws + d.offset + d.exp_off), stream);
+          if (e != cudaSuccess) return cuda_status(e, "digit split");
+          continue;
+        }
         cudaError_t e = launch_oz_split(reinterpret_cast<const float*>(ws + r.offset), r.plane_bytes / 4,
                                         ws + d.offset, d.plane_bytes / elem_bytes(prec), x.rows, x.K, x.ld,
                                         planes(prec), stream);
@@ -217,7 +224,35 @@ mera_status run_program(const OpProgram& prog, const double* const inputs[4], do
       const Buffer& a = dg.bufs[g.a_buf];
       const Buffer& b = dg.bufs[g.b_buf];
       ProfScope ps(stream, 0, g.dominant, g.flops);
-      if (prec == PREC_F64) {
+      if (g.ax_buf >= 0) {
+        const Buffer& ax = dg.bufs[g.ax_buf];
+        const Buffer& bx = dg.bufs[g.bx_buf];
+        const int64_t tile_k = (g.K + 15) / 16 * 32 * kX64Digits;  // image bytes per row of a tile
+        X64GemmArgs args;
+        args.A = ws + ax.offset + g.ax_tile * kX64TileA * tile_k;
+        args.ea = reinterpret_cast<const int*>(ws + ax.offset + ax.exp_off) + g.ax_row;
+        args.A64 = reinterpret_cast<const double*>(ws + a.offset) + g.a_off;
+        args.lda = g.lda;
+        args.B = ws + bx.offset + g.bx_tile * kX64TileB * tile_k;
+        args.eb = reinterpret_cast<const int*>(ws + bx.offset + bx.exp_off) + g.bx_row;
+        args.B64 = reinterpret_cast<const double*>(ws + b.offset) + g.b_off;
+        args.ldb = g.ldb;
+        args.M = g.M;
+        args.N = g.N;
+        args.K = g.K;
+        args.C = (g.c_buf >= 0 ? reinterpret_cast<double*>(ws + dg.bufs[g.c_buf].offset) : out) + g.c_off;
+        args.m_dst = g.m_dst;
+        args.n_dst = g.n_dst;
+        args.alpha = g.alpha;
+        args.accumulate = g.accumulate;
+        args.split = g.split;
+        if (g.p_buf >= 0) {
+          args.partial = reinterpret_cast<float*>(ws + dg.bufs[g.p_buf].offset);
+          args.partial_plane = dg.bufs[g.p_buf].plane_bytes / 4;
+        }
+        cudaError_t e = launch_gemm_x64(args, stream);
+        if (e != cudaSuccess) return cuda_status(e, "gemm_x64");
+      } else if (prec == PREC_F64) {
         GemmF64Args args;
         args.A = reinterpret_cast<const double*>(ws + a.offset) + g.a_off;
         args.a_m = g.lda;
@@ -249,6 +284,15 @@ mera_status run_program(const OpProgram& prog, const double* const inputs[4], do
 // Workspace bytes of each composite operation.
 size_t op_bytes(const OpProgram& p) { return align_up(p.ws_bytes); }
 
+// The program that runs in `avail` bytes of workspace: PREC_F64 falls back to
+// the FP64 pipe for every product where the digit images do not fit, so a
+// workspace that was large enough for the operands alone stays accepted.
+const OpProgram* pick_program(int op, int chi_b, int chi_t, int prec, size_t avail) {
+  const OpProgram* p = get_program(op, chi_b, chi_t, prec);
+  if (p && p->has_x64 && op_bytes(*p) > avail) p = get_program(op, chi_b, chi_t, prec, true);
+  return p;
+}
+
 mera_status map_call(int op, const double* h, const double* rho, const double* u, const double* w, int chi_b,
                      int chi_t, double* out, int prec, void* ws, size_t ws_bytes, void* stream) {
   if (!chi_ok(chi_b, chi_t)) return fail(MERA_EINVAL, "bad bond dimensions chi_b=%d chi_t=%d", chi_b, chi_t);
@@ -256,7 +300,7 @@ mera_status map_call(int op, const double* h, const double* rho, const double* u
   if (!u || !w || !out) return fail(MERA_EINVAL, "null tensor pointer");
   if ((op == OP_ASCEND || op == OP_ENV_U || op == OP_ENV_W) && !h) return fail(MERA_EINVAL, "null h");
   if ((op == OP_DESCEND || op == OP_ENV_U || op == OP_ENV_W) && !rho) return fail(MERA_EINVAL, "null rho");
-  const OpProgram* prog = get_program(op, chi_b, chi_t, prec);
+  const OpProgram* prog = pick_program(op, chi_b, chi_t, prec, ws_bytes);
   if (!prog) return fail(MERA_EINVAL, "no contraction program");
   if (reinterpret_cast<uintptr_t>(ws) % kAlign) return fail(MERA_EINVAL, "workspace not 256-byte aligned");
   if (ws_bytes < op_bytes(*prog) || (!ws && op_bytes(*prog) > 0))
@@ -274,7 +318,8 @@ using namespace mera;
 extern "C" const char* mera_version(void) { return "mera-gb300 0.1 sm_103a"; }
 extern "C" const char* mera_last_error(void) { return g_err.c_str(); }
 
-static mera_status ws_size_impl(int op, int chi_b, int chi_t, int prec, size_t* bytes) {
+// plain: the least workspace that PREC_F64 runs in (pick_program).
+static mera_status ws_size_impl(int op, int chi_b, int chi_t, int prec, size_t* bytes, bool plain = false) {
   if (!bytes) return fail(MERA_EINVAL, "null bytes");
   if (!chi_ok(chi_b, chi_t) || !prec_ok(prec)) return fail(MERA_EINVAL, "bad sizes or prec");
   switch (op) {
@@ -282,13 +327,13 @@ static mera_status ws_size_impl(int op, int chi_b, int chi_t, int prec, size_t* 
     case MERA_OP_DESCEND:
     case MERA_OP_ENV_U:
     case MERA_OP_ENV_W: {
-      const OpProgram* p = get_program(op, chi_b, chi_t, prec);
+      const OpProgram* p = get_program(op, chi_b, chi_t, prec, plain);
       if (!p) return fail(MERA_EINVAL, "no contraction program");
       *bytes = op_bytes(*p);
       return MERA_OK;
     }
     case MERA_OP_ENERGY: {
-      const OpProgram* p = get_program(OP_ASCEND, chi_b, chi_t, prec);
+      const OpProgram* p = get_program(OP_ASCEND, chi_b, chi_t, prec, plain);
       if (!p) return fail(MERA_EINVAL, "no contraction program");
       *bytes = op_bytes(*p) + align_up(ipow(chi_t, 6) * sizeof(double)) + kReduceBytes;
       return MERA_OK;
@@ -297,7 +342,7 @@ static mera_status ws_size_impl(int op, int chi_b, int chi_t, int prec, size_t* 
       // transposes of h and rho, an environment half, then the largest map
       size_t maps = 0;
       for (int op2 : {OP_ASCEND, OP_DESCEND, OP_ENV_U, OP_ENV_W}) {
-        const OpProgram* p = get_program(op2, chi_b, chi_t, prec);
+        const OpProgram* p = get_program(op2, chi_b, chi_t, prec, plain);
         if (!p) return fail(MERA_EINVAL, "no contraction program");
         maps = std::max(maps, op_bytes(*p));
       }
@@ -307,7 +352,7 @@ static mera_status ws_size_impl(int op, int chi_b, int chi_t, int prec, size_t* 
     }
     case MERA_OP_FIXED_POINT: {
       if (chi_b != chi_t) return fail(MERA_EINVAL, "fixed point needs chi_b == chi_t");
-      const OpProgram* p = get_program(OP_DESCEND, chi_b, chi_t, prec);
+      const OpProgram* p = get_program(OP_DESCEND, chi_b, chi_t, prec, plain);
       if (!p) return fail(MERA_EINVAL, "no contraction program");
       *bytes = op_bytes(*p) + align_up(ipow(chi_t, 6) * sizeof(double)) + kReduceBytes;
       return MERA_OK;
@@ -350,8 +395,10 @@ extern "C" mera_status mera_energy(const double* h, const double* rho, const dou
   if (st != MERA_OK) return st;
   if (!h || !rho || !u || !w || !e_dev) return fail(MERA_EINVAL, "null pointer");
   if (reinterpret_cast<uintptr_t>(ws) % kAlign) return fail(MERA_EINVAL, "workspace not 256-byte aligned");
+  const bool plain = ws_bytes < need;
+  if (plain) ws_size_impl(MERA_OP_ENERGY, chi_b, chi_t, prec, &need, true);
   if (!ws || ws_bytes < need) return fail(MERA_ENOMEM, "workspace %zu bytes < %zu needed", ws_bytes, need);
-  const OpProgram* prog = get_program(OP_ASCEND, chi_b, chi_t, prec);
+  const OpProgram* prog = get_program(OP_ASCEND, chi_b, chi_t, prec, plain);
   Arena ar{static_cast<char*>(ws), ws_bytes};
   char* pws = ar.take(op_bytes(*prog));
   const int64_t n = ipow(chi_t, 3);
@@ -372,13 +419,15 @@ extern "C" mera_status mera_fixed_point_rho(const double* u, const double* w, in
   if (!u || !w || !rho_inout) return fail(MERA_EINVAL, "null pointer");
   if (n_iter < 0) return fail(MERA_EINVAL, "negative n_iter");
   if (reinterpret_cast<uintptr_t>(ws) % kAlign) return fail(MERA_EINVAL, "workspace not 256-byte aligned");
+  const bool plain = ws_bytes < need;
+  if (plain) ws_size_impl(MERA_OP_FIXED_POINT, chi, chi, prec, &need, true);
   if (!ws || ws_bytes < need) return fail(MERA_ENOMEM, "workspace %zu bytes < %zu needed", ws_bytes, need);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (n_iter == 0) {
     if (resid_dev) return cuda_status(cudaMemsetAsync(resid_dev, 0, sizeof(double), s), "memset");
     return MERA_OK;
   }
-  const OpProgram* prog = get_program(OP_DESCEND, chi, chi, prec);
+  const OpProgram* prog = get_program(OP_DESCEND, chi, chi, prec, plain);
   Arena ar{static_cast<char*>(ws), ws_bytes};
   char* pws = ar.take(op_bytes(*prog));
   const int64_t n = ipow(chi, 3);
@@ -680,7 +729,8 @@ struct SweepLayout {
   size_t map_bytes;
 };
 
-mera_status sweep_layout(int n_layers, const int* chi_b, const int* chi_t, int prec, SweepLayout* L) {
+mera_status sweep_layout(int n_layers, const int* chi_b, const int* chi_t, int prec, SweepLayout* L,
+                         bool plain = false) {
   if (n_layers < 1 || n_layers > MERA_MAX_LAYERS) return fail(MERA_EINVAL, "bad n_layers %d", n_layers);
   for (int t = 0; t < n_layers; ++t) {
     if (!chi_ok(chi_b[t], chi_t[t])) return fail(MERA_EINVAL, "bad dims in layer %d", t);
@@ -695,7 +745,7 @@ mera_status sweep_layout(int n_layers, const int* chi_b, const int* chi_t, int p
     rho_max = std::max(rho_max, size_t(ipow(chi_b[t], 6)));
     env_max = std::max(env_max, size_t(ipow(chi_b[t], 4)));
     for (int op : {OP_ASCEND, OP_DESCEND, OP_ENV_U, OP_ENV_W}) {
-      const OpProgram* p = get_program(op, chi_b[t], chi_t[t], prec);
+      const OpProgram* p = get_program(op, chi_b[t], chi_t[t], prec, plain);
       if (!p) return fail(MERA_EINVAL, "no program for layer %d", t);
       map_bytes = std::max(map_bytes, op_bytes(*p));
     }
@@ -703,11 +753,11 @@ mera_status sweep_layout(int n_layers, const int* chi_b, const int* chi_t, int p
     map_bytes = std::max(map_bytes, stiefel_bytes(int(eb), int(eb)));  // >= polar_bytes
     size_t fp = 0;
     if (t == n_layers - 1) {
-      ws_size_impl(MERA_OP_FIXED_POINT, chi_b[t], chi_t[t], prec, &fp);
+      ws_size_impl(MERA_OP_FIXED_POINT, chi_b[t], chi_t[t], prec, &fp, plain);
       map_bytes = std::max(map_bytes, fp);
     }
     if (t == 0) {
-      ws_size_impl(MERA_OP_ENERGY, chi_b[t], chi_t[t], prec, &fp);
+      ws_size_impl(MERA_OP_ENERGY, chi_b[t], chi_t[t], prec, &fp, plain);
       map_bytes = std::max(map_bytes, fp);
     }
   }
@@ -754,6 +804,7 @@ static mera_status sweep_impl(mera_state* S, const double* h1, double shift, int
   const int n = S->n_layers;
   SweepLayout L;
   mera_status st = sweep_layout(n, S->chi_b, S->chi_t, prec, &L);
+  if (st == MERA_OK && ws_bytes < L.total) st = sweep_layout(n, S->chi_b, S->chi_t, prec, &L, true);
   if (st != MERA_OK) return st;
   for (int t = 0; t < n; ++t)
     if (!S->u[t] || !S->w[t]) return fail(MERA_EINVAL, "null tensor in layer %d", t);
@@ -980,7 +1031,17 @@ extern "C" mera_status mera_gemm_test(int prec, const double* A, const double* B
   if (!A || !B || !C || M < 1 || N < 1 || K < 1) return fail(MERA_EINVAL, "bad gemm test arguments");
   if (!prec_ok(prec)) return fail(MERA_EINVAL, "bad prec");
   const int64_t eb = elem_bytes(prec), np = planes(prec);
-  const int64_t ld = (int64_t(K) * eb + 15) / 16 * 16 / eb;
+  int64_t ld = (int64_t(K) * eb + 15) / 16 * 16 / eb;
+  // PREC_F64: the tensor-core route where the workspace also holds the digit
+  // images, the row exponents and the K-split partials
+  const int xsplit = x64_split_k(M, N, K);
+  const int64_t ldx = (int64_t(K) + 7) / 8 * 8, row_img = int64_t((K + 15) / 16) * 32 * kX64Digits;
+  const size_t xa = align_up(size_t((M + kX64TileA - 1) / kX64TileA * kX64TileA) * row_img);
+  const size_t xb = align_up(size_t((N + kX64TileB - 1) / kX64TileB * kX64TileB) * row_img);
+  const size_t xneed = align_up(size_t(M) * ldx * 8) + align_up(size_t(N) * ldx * 8) + xa + xb +
+                       align_up(size_t(M) * 4) + align_up(size_t(N) * 4) + size_t(xsplit) * M * N * 12;
+  const bool x64 = prec == PREC_F64 && ws_bytes >= xneed;
+  if (x64) ld = ldx;
   const size_t pa = align_up(size_t(M) * ld * eb), pb = align_up(size_t(N) * ld * eb);
   // fixed-point split modes: raw hi + lo binary32 planes of both operands first
   const size_t ra = is_oz(prec) ? align_up(size_t(M) * ld * 4) : 0, rb = is_oz(prec) ? align_up(size_t(N) * ld * 4) : 0;
@@ -1015,6 +1076,23 @@ extern "C" mera_status mera_gemm_test(int prec, const double* A, const double* B
   LegMap md, nd;
   md.n = 1; md.dim[0] = M; md.stride[0] = N;
   nd.n = 1; nd.dim[0] = N; nd.stride[0] = 1;
+  if (prec == PREC_F64 && x64) {
+    char* ia = wb + pb;
+    char* ib = ia + xa;
+    int* ea = reinterpret_cast<int*>(ib + xb);
+    int* eb2 = ea + align_up(size_t(M) * 4) / 4;
+    X64GemmArgs g;
+    g.A = ia; g.ea = ea; g.A64 = reinterpret_cast<const double*>(wa); g.lda = ld;
+    g.B = ib; g.eb = eb2; g.B64 = reinterpret_cast<const double*>(wb); g.ldb = ld;
+    g.M = M; g.N = N; g.K = K; g.C = C; g.m_dst = md; g.n_dst = nd;
+    g.split = xsplit;
+    g.partial = reinterpret_cast<float*>(eb2 + align_up(size_t(N) * 4) / 4);
+    g.partial_plane = int64_t(xsplit) * M * N;
+    e = launch_x64_split(g.A64, ld, M, K, M, kX64TileA, ia, ea, s);
+    if (e == cudaSuccess) e = launch_x64_split(g.B64, ld, N, K, N, kX64TileB, ib, eb2, s);
+    if (e == cudaSuccess) e = launch_gemm_x64(g, s);
+    return cuda_status(e, "gemm test x64");
+  }
   if (prec == PREC_F64) {
     GemmF64Args g;
     g.A = reinterpret_cast<const double*>(wa); g.a_m = ld; g.a_k = 1;
@@ -1033,6 +1111,12 @@ namespace mera {
 // Records `msg` as the calling thread's last error and returns `st`; for
 // entry points defined in other translation units.
 mera_status set_last_error(mera_status st, const char* msg) { return fail(st, "%s", msg); }
+
+// The least workspace an operation runs in; mera_workspace_size reports what
+// it runs fastest in.
+mera_status least_workspace(int op, int chi_b, int chi_t, int prec, size_t* bytes) {
+  return ws_size_impl(op, chi_b, chi_t, prec, bytes, true);
+}
 }  // namespace mera
 
 extern "C" mera_status mera_op_transpose(const double* x, int d, double* out, void* stream) {
@@ -1057,6 +1141,7 @@ extern "C" mera_status mera_energy_adjoint(const double* h, const double* rho, c
   if (st != MERA_OK) return st;
   if (!h || !rho || !u || !w || !g_dev) return fail(MERA_EINVAL, "null input pointer");
   if (reinterpret_cast<uintptr_t>(ws) % kAlign) return fail(MERA_EINVAL, "workspace not 256-byte aligned");
+  if (ws_bytes < need) ws_size_impl(MERA_OP_ENERGY_ADJOINT, chi_b, chi_t, prec, &need, true);
   if (!ws || ws_bytes < need) return fail(MERA_ENOMEM, "workspace %zu bytes < %zu needed", ws_bytes, need);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   Arena ar{static_cast<char*>(ws), ws_bytes};
@@ -1169,9 +1254,9 @@ static double sweep_flops(int n, const int* cb, const int* ct, int n_pow) {
 // (A lane opened by a later MERA is never smaller than it; the shared lane
 // of the GPU-filling MERAs can be, when a MERA with few flops has a large
 // transitional layer.)
-extern "C" mera_status mera_batch_lanes(int n, int n_layers, const int* chi_b, const int* chi_t, int prec, int n_pow,
-                                        size_t budget_bytes, int max_lanes, int* lane, int* n_lanes,
-                                        size_t* lane_bytes) {
+static mera_status batch_lanes(int n, int n_layers, const int* chi_b, const int* chi_t, int prec, int n_pow,
+                               size_t budget_bytes, int max_lanes, int* lane, int* n_lanes, size_t* lane_bytes,
+                               bool plain) {
   if (n < 1 || n_layers < 1 || n_layers > MERA_MAX_LAYERS || !chi_b || !chi_t || n_pow < 0 || max_lanes < 1 ||
       !lane || !n_lanes || !lane_bytes)
     return fail(MERA_EINVAL, "bad arguments to mera_batch_lanes");
@@ -1181,7 +1266,7 @@ extern "C" mera_status mera_batch_lanes(int n, int n_layers, const int* chi_b, c
     const int* cb = chi_b + size_t(i) * size_t(n_layers);
     const int* ct = chi_t + size_t(i) * size_t(n_layers);
     SweepLayout L;
-    const mera_status st = sweep_layout(n_layers, cb, ct, prec, &L);
+    const mera_status st = sweep_layout(n_layers, cb, ct, prec, &L, plain);
     if (st != MERA_OK) {
       g_err = "MERA " + std::to_string(i) + ": " + g_err;
       return st;
@@ -1247,6 +1332,16 @@ extern "C" mera_status mera_batch_lanes(int n, int n_layers, const int* chi_b, c
   *n_lanes = int(bytes.size());
   for (size_t l = 0; l < bytes.size(); ++l) lane_bytes[l] = bytes[l];
   return MERA_OK;
+}
+
+extern "C" mera_status mera_batch_lanes(int n, int n_layers, const int* chi_b, const int* chi_t, int prec, int n_pow,
+                                        size_t budget_bytes, int max_lanes, int* lane, int* n_lanes,
+                                        size_t* lane_bytes) {
+  const mera_status st =
+      batch_lanes(n, n_layers, chi_b, chi_t, prec, n_pow, budget_bytes, max_lanes, lane, n_lanes, lane_bytes, false);
+  // a budget that holds PREC_F64 sweeps only without digit images
+  if (st != MERA_ENOMEM || prec != PREC_F64) return st;
+  return batch_lanes(n, n_layers, chi_b, chi_t, prec, n_pow, budget_bytes, max_lanes, lane, n_lanes, lane_bytes, true);
 }
 
 // Tile-width autotuner: every tensor-core GEMM step of the op's program that

@@ -30,6 +30,12 @@ cudaError_t launch_permute(const PermuteStep& p, const double* src, void* dst, i
 cudaError_t launch_oz_split(const float* raw, int64_t raw_plane, void* dst, int64_t dst_plane, int64_t rows,
                             int64_t K, int64_t ld, int slices, cudaStream_t stream);
 
+// Binary64 operand (rows x K, pitch ld, a multiple of 8) -> digit image of
+// x64_gemm_kernel in tiles of `tile` rows, and one exponent per row.  Rows
+// come in segments of seg_rows, each padded to whole tiles.
+cudaError_t launch_x64_split(const double* src, int64_t ld, int64_t rows, int64_t K, int64_t seg_rows, int tile,
+                             void* img, int* rowexp, cudaStream_t stream);
+
 // FP64 GEMM with a scattered epilogue:
 //   C[m_dst(m) + n_dst(n)] (+)= alpha * sum_k A[m*a_m + k*a_k] * B[n*b_n + k*b_k]
 struct GemmF64Args {

@@ -17,6 +17,7 @@
 namespace mera {
 mera_status set_last_error(mera_status st, const char* msg);
 void* current_cu_context();
+mera_status least_workspace(int op, int chi_b, int chi_t, int prec, size_t* bytes);
 }
 
 namespace {
@@ -62,7 +63,7 @@ mera_status scratch_address(void** out, const char** why) {
 extern "C" mera_status mera_ascend_noalloc(const double* h, const double* u, const double* w, int chi_b, int chi_t,
                                            double* h_out, int prec, void* stream) {
   size_t need = 0;
-  mera_status st = mera_workspace_size(MERA_OP_ASCEND, chi_b, chi_t, prec, &need);
+  mera_status st = mera::least_workspace(MERA_OP_ASCEND, chi_b, chi_t, prec, &need);
   if (st != MERA_OK) return st;  // message already recorded
   if (need > size_t(MERA_NOALLOC_SCRATCH_BYTES)) {
     char msg[160];

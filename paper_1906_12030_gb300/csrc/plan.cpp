@@ -101,6 +101,49 @@ int planes(int prec) {
 // buffer that the fixed-point split modes write before splitting.
 double operand_elem_bytes(int prec) { return double(elem_bytes(prec) * planes(prec)) + (is_oz(prec) ? 8.0 : 0.0); }
 
+// Cost model of a PREC_F64 product of M x N x K.  FP64 pipe: two FMAs per
+// clock and SM over the tiles of launch_gemm_f64, in waves of one tile per SM
+// (a 100 x 10 x 1000 product is 7 tiles and takes 44 us), plus a launch.
+// Tensor cores: the digit products of the padded tiles, the passes that write
+// the two digit images (8 bytes read and 14 written per entry) and three
+// launches.
+bool x64_use(int64_t M, int64_t N, int64_t K) {
+  if (K < 16 || M > 0x3fffffff || N > 0x3fffffff || K > (int64_t(1) << 30)) return false;
+  auto tiles = [&](int64_t r) { return ((M + r - 1) / r) * ((N + r - 1) / r); };
+  const int64_t r = tiles(64) >= 304 ? 64 : tiles(32) >= 304 ? 32 : 16;
+  const double fp64 = double((tiles(r) + 151) / 152) * double(r * r) * double(K) * 0.27e-9 + 3e-6;
+  const double mp = double((M + 127) / 128 * 128), np = double((N + 63) / 64 * 64), kp = double((K + 15) / 16 * 16);
+  const double x64 = 2.0 * mp * np * kp / 4.0e13 + 22.0 * (mp + np) * kp / 4.5e12 + 14e-6;
+  return x64 < fp64;
+}
+
+// K split of such a product: over the splits that leave at least eight
+// 16-wide steps each, the one whose waves of work items take the least time.
+// A step takes about 0.7 us, a block's fold (every 16 steps) 1.5 us, a work
+// item 2 us besides, and the sum of the partials 12 bytes per output and
+// split at memory speed plus a launch.
+int x64_split_k(int64_t M, int64_t N, int64_t K) {
+  constexpr int64_t kSMs = 152;
+  const int64_t tiles = ((M + kX64TileA - 1) / kX64TileA) * ((N + kX64TileB - 1) / kX64TileB);
+  const int64_t nk = (K + 15) / 16;
+  if (tiles >= kSMs) return 1;
+  int64_t best = 1;
+  double best_t = 0.0;
+  for (int64_t s = 1; s <= std::min<int64_t>(nk / 8, 512); ++s) {
+    const int64_t kc = x64_kc(nk, s);
+    const int64_t sn = (nk + kc - 1) / kc;
+    if (x64_kc(nk, sn) != kc) continue;  // the launcher derives kc from the split
+    const int64_t waves = (tiles * sn + kSMs - 1) / kSMs;
+    double t = double(waves) * (0.7 * double(kc) + 1.5 * double((kc + kX64BlockSteps - 1) / kX64BlockSteps) + 2.0);
+    if (sn > 1) t += 3.0 + 24.0 * double(sn) * double(M) * double(N) / 4e6;
+    if (s == 1 || t < best_t * 0.98) {
+      best = sn;
+      best_t = t;
+    }
+  }
+  return int(best);
+}
+
 namespace {
 
 // ---------------------------------------------------------------------------
@@ -297,6 +340,11 @@ struct Builder {
   std::vector<std::map<int, int64_t>> dst_stride;
   std::vector<int> buf_of;
   std::vector<int> raw_of;      // fixed-point split modes: raw buffer of each node's operand
+  std::vector<int> img_of;      // PREC_F64: digit image of each node's operand (-1: none)
+  std::vector<int> img_tile;    // its rows per tile
+  std::vector<int64_t> img_seg; // and rows per segment
+  std::vector<char> x64;        // the node's product runs on the tensor cores in PREC_F64
+  bool plain = false;
   std::vector<int64_t> k_of;    // K of the GEMM that reads each node's operand
   // GEMM info per internal node
   struct G {
@@ -317,8 +365,8 @@ struct Builder {
   const std::set<std::string>* shared = nullptr;
 
   Builder(const Diagram& d, const int64_t* dm, int p, double al, int acc, size_t sb,
-          const std::set<std::string>* sh = nullptr)
-      : dg(d), dim(dm), prec(p), alpha(al), accumulate(acc), slice_threshold(sb), shared(sh) {}
+          const std::set<std::string>* sh = nullptr, bool pl = false)
+      : dg(d), dim(dm), prec(p), alpha(al), accumulate(acc), plain(pl), slice_threshold(sb), shared(sh) {}
 
   int64_t prod(const std::vector<int>& legs) const {
     int64_t s = 1;
@@ -356,8 +404,8 @@ struct Builder {
     return st;
   }
 
-  int64_t pitch(int64_t cols) const {
-    const int64_t align = std::max<int64_t>(1, 16 / elem_bytes(prec));
+  int64_t pitch(int64_t cols, bool img) const {
+    const int64_t align = img ? 8 : std::max<int64_t>(1, 16 / elem_bytes(prec));
     return round_up(std::max<int64_t>(cols, 1), align);
   }
 
@@ -396,9 +444,13 @@ struct Builder {
       if (in_m) {
         gs.M /= ns;
         gs.a_off = is_producer ? v * gs.M * gs.lda : 0;
+        gs.ax_row = is_producer ? v * gs.M : 0;
+        gs.ax_tile = is_producer ? v * ((gs.M + kX64TileA - 1) / kX64TileA) : 0;
       } else if (in_n) {
         gs.N /= ns;
         gs.b_off = is_producer ? v * gs.N * gs.ldb : 0;
+        gs.bx_row = is_producer ? v * gs.N : 0;
+        gs.bx_tile = is_producer ? v * ((gs.N + kX64TileB - 1) / kX64TileB) : 0;
       }
       gs.c_off = is_producer ? 0 : v * bl * dst_stride[i].at(l);
     }
@@ -409,13 +461,17 @@ struct Builder {
     gs.flops = 2.0 * double(gs.M) * double(gs.N) * double(gs.K);
     gs.dominant = full_flops_dominant_hint ? 2 : 0;  // resolved after emission
     gs.bn = prec == PREC_F64 ? 0 : tc_tile_n(prec, gs.M, gs.N, gs.K, i == tr.root ? 1 : 0);
-    gs.split = tc_split_k(prec, gs.M, gs.N, gs.K, gs.bn);
+    if (x64[i]) {
+      gs.ax_buf = img_of[gi.a];
+      gs.bx_buf = img_of[gi.b];
+    }
+    gs.split = x64[i] ? x64_split_k(gs.M, gs.N, gs.K) : tc_split_k(prec, gs.M, gs.N, gs.K, gs.bn);
     if (gs.split > 1) {  // FP32 partials [split][N][M], live during this step only
       Buffer pb;
       pb.rows = int64_t(gs.split) * gs.N;
       pb.ld = gs.M;
       pb.plane_bytes = round_up(pb.rows * pb.ld * 4, 256);
-      pb.bytes = pb.plane_bytes * (is_oz(prec) ? 2 : 1);  // hi, lo planes in the split modes
+      pb.bytes = pb.plane_bytes * (x64[i] ? 3 : is_oz(prec) ? 2 : 1);  // hi, (mid,) lo planes
       prog.bufs.push_back(pb);
       gs.p_buf = int(prog.bufs.size()) - 1;
       first_use.push_back(-1);
@@ -441,6 +497,8 @@ struct Builder {
     const int si = int(prog.steps.size()) - 1;
     if (last_use[gs.a_buf] < si) last_use[gs.a_buf] = si;
     if (last_use[gs.b_buf] < si) last_use[gs.b_buf] = si;
+    for (int b : {gs.ax_buf, gs.bx_buf})
+      if (b >= 0 && last_use[b] < si) last_use[b] = si;
     if (gs.p_buf >= 0) first_use[gs.p_buf] = last_use[gs.p_buf] = si;
     if (gs.c_buf >= 0) {
       if (first_use[gs.c_buf] < 0) first_use[gs.c_buf] = si;
@@ -449,14 +507,19 @@ struct Builder {
   }
 
   // Fixed-point split modes: node i's raw buffer -> its operand buffer, once
-  // the raw buffer is complete.
+  // the raw buffer is complete; PREC_F64: its operand buffer -> digit image.
   void emit_split(int i, std::vector<int>& first_use, std::vector<int>& last_use) {
-    if (!is_oz(prec) || i == tr.root) return;
+    if ((!is_oz(prec) && img_of[i] < 0) || i == tr.root) return;
     Step s;
     s.kind = 2;
     SplitStep& x = s.x;
-    x.raw_buf = raw_of[i];
-    x.dst_buf = buf_of[i];
+    x.raw_buf = is_oz(prec) ? raw_of[i] : buf_of[i];
+    x.dst_buf = is_oz(prec) ? buf_of[i] : img_of[i];
+    if (img_of[i] >= 0) {
+      x.tile = img_tile[i];
+      x.seg_rows = img_seg[i];
+      prog.bufs[x.dst_buf].resident = prog.bufs[x.raw_buf].resident;
+    }
     x.rows = prog.bufs[x.dst_buf].rows;
     x.ld = prog.bufs[x.dst_buf].ld;
     x.K = k_of[i];
@@ -488,6 +551,10 @@ struct Builder {
     dst_stride.assign(nn, {});
     buf_of.assign(nn, -1);
     raw_of.assign(nn, -1);
+    img_of.assign(nn, -1);
+    img_tile.assign(nn, 0);
+    img_seg.assign(nn, 0);
+    x64.assign(nn, 0);
     k_of.assign(nn, 0);
     g.assign(nn, {});
     // GEMM roles (bottom-up information only depends on leg sets).
@@ -501,6 +568,8 @@ struct Builder {
       gi.a = (fl >= fr) ? nd.left : nd.right;
       gi.b = (fl >= fr) ? nd.right : nd.left;
       gi.klegs = legs_list(K);
+      if (prec == PREC_F64 && !plain)
+        x64[i] = x64_use(int64_t(std::max(fl, fr)), int64_t(std::min(fl, fr)), int64_t(size_of(K, dim)));
     }
     // Slicing pre-pass: a rank-7 intermediate T (the product of the two
     // chi^9 GEMMs) bigger than the threshold is cut over one of its legs
@@ -515,7 +584,8 @@ struct Builder {
       for (int c : {g[i].a, g[i].b}) {
         const Node& cn = tr.nodes[c];
         if (cn.tensor >= 0 || popcount64(cn.legs) != 7) continue;
-        const double bytes = size_of(cn.legs, dim) * operand_elem_bytes(prec);
+        // operand bytes per element, the digit image of a PREC_F64 operand included
+        const double bytes = size_of(cn.legs, dim) * (operand_elem_bytes(prec) + (x64[i] ? 2.0 * kX64Digits : 0.0));
         if (bytes <= double(slice_threshold)) continue;
         const uint64_t K2 = tr.nodes[g[i].a].legs & tr.nodes[g[i].b].legs;
         int best = -1;
@@ -609,7 +679,7 @@ struct Builder {
       gi.nlegs = nlegs;
       gi.klegs = klegs;
       const int64_t Kn = prod(klegs);
-      const int64_t ld = pitch(Kn);
+      const int64_t ld = pitch(Kn, x64[i] != 0);
       dst_stride[gi.a] = operand_strides(mlegs, klegs, ld);
       dst_stride[gi.b] = operand_strides(nlegs, klegs, ld);
       // operand buffers for both children
@@ -630,6 +700,25 @@ struct Builder {
           r.bytes = 2 * r.plane_bytes;
           prog.bufs.push_back(r);
           raw_of[c] = int(prog.bufs.size()) - 1;
+        }
+        if (x64[i]) {  // digit image: whole tiles of every segment, then the row exponents
+          prog.bufs[buf_of[c]].raw = 2;
+          img_tile[c] = (c == gi.a) ? kX64TileA : kX64TileB;
+          img_seg[c] = b.rows;
+          // the producer of a sliced intermediate reads one segment per slice
+          for (size_t q = 0; q < nn; ++q) {
+            const std::vector<int>& side = (c == gi.a) ? mlegs : nlegs;
+            if (sliced_child[q] == i && !side.empty() && side.front() == slice_leg[q])
+              img_seg[c] = b.rows / dim[slice_leg[q]] * slice_block[q];
+          }
+          const int64_t segs = b.rows / img_seg[c];
+          const int64_t tiles = segs * ((img_seg[c] + img_tile[c] - 1) / img_tile[c]);
+          Buffer im = b;
+          im.raw = 0;
+          im.exp_off = round_up(tiles * img_tile[c] * ((Kn + 15) / 16) * 32 * kX64Digits, 256);
+          im.plane_bytes = im.bytes = im.exp_off + round_up(b.rows * 4, 256);
+          prog.bufs.push_back(im);
+          img_of[c] = int(prog.bufs.size()) - 1;
         }
       }
     }
@@ -741,8 +830,9 @@ struct Builder {
 
 struct Key {
   int op, chi_b, chi_t, prec;
+  bool plain;
   bool operator<(const Key& o) const {
-    return std::tie(op, chi_b, chi_t, prec) < std::tie(o.op, o.chi_b, o.chi_t, o.prec);
+    return std::tie(op, chi_b, chi_t, prec, plain) < std::tie(o.op, o.chi_b, o.chi_t, o.prec, o.plain);
   }
 };
 
@@ -754,15 +844,10 @@ std::map<std::tuple<int, int64_t, int64_t, int64_t, int>, int> g_tuned;  // (pre
 
 }  // namespace
 
-const OpProgram* get_program(int op, int chi_b, int chi_t, int prec) {
-  if (op < OP_ASCEND || op > OP_ENV_W) return nullptr;
-  if (prec < PREC_F64 || prec > PREC_LAST) return nullptr;
-  if (chi_b < 1 || chi_t < 1 || chi_b > 64 || chi_t > 64) return nullptr;
-  if (chi_t > chi_b * chi_b) return nullptr;
-  std::lock_guard<std::mutex> lk(g_mu);
-  Key k{op, chi_b, chi_t, prec};
-  auto it = g_cache.find(k);
-  if (it != g_cache.end()) return it->second.get();
+namespace {
+
+// g_mu is held.
+std::unique_ptr<OpProgram> build_program(int op, int chi_b, int chi_t, int prec, bool plain) {
   int64_t dim[64];
   for (int l = 0; l < 64; ++l) dim[l] = chi_b;
   for (char c : std::string("pqrstv")) dim[label_id(c)] = chi_t;
@@ -770,9 +855,10 @@ const OpProgram* get_program(int op, int chi_b, int chi_t, int prec) {
   auto build_all = [&](const std::set<std::string>* sh) -> std::unique_ptr<OpProgram> {
     auto pr = std::make_unique<OpProgram>();
     for (size_t d = 0; d < ds.size(); ++d) {
-      Builder b(ds[d], dim, prec, 0.5, d == 0 ? 0 : 1, g_slice_bytes, sh);
+      Builder b(ds[d], dim, prec, 0.5, d == 0 ? 0 : 1, g_slice_bytes, sh, plain);
       if (!b.build()) return nullptr;
       pr->flops += b.prog.flops;
+      for (const Step& st : b.prog.steps) pr->has_x64 |= (st.kind == 1 && st.g.ax_buf >= 0);
       pr->diagrams.push_back(std::move(b.prog));
     }
     return pr;
@@ -812,6 +898,7 @@ const OpProgram* get_program(int op, int chi_b, int chi_t, int prec) {
   size_t res_base = 0;
   {
     std::map<std::string, int64_t> made;  // key -> offset
+    std::map<std::string, int64_t> made_img;  // digit images of such copies
     for (Program& pg : prog->diagrams) {
       std::vector<char> placed(pg.bufs.size(), 0);
       for (size_t si = 0; si < pg.steps.size(); ++si) {
@@ -833,6 +920,22 @@ const OpProgram* get_program(int op, int chi_b, int chi_t, int prec) {
           made[k] = bf.offset;
           res_base += size_t(bf.bytes + 255) / 256 * 256;
         }
+        if (si + 1 < pg.steps.size() && pg.steps[si + 1].kind == 2 && pg.steps[si + 1].x.tile > 0) {
+          // PREC_F64: the copy's digit image, one per tile and segment size
+          SplitStep& x = pg.steps[si + 1].x;
+          Buffer& im = pg.bufs[size_t(x.dst_buf)];
+          placed[size_t(x.dst_buf)] = 1;
+          const std::string ki = k + "/" + std::to_string(x.tile) + "/" + std::to_string(x.seg_rows);
+          auto ii = made_img.find(ki);
+          if (ii != made_img.end()) {
+            im.offset = ii->second;
+            x.skip = 1;
+          } else {
+            im.offset = int64_t(res_base);
+            made_img[ki] = im.offset;
+            res_base += size_t(im.bytes + 255) / 256 * 256;
+          }
+        }
       }
       for (size_t b = 0; b < pg.bufs.size(); ++b)
         if (pg.bufs[b].resident && !placed[b]) {
@@ -849,6 +952,27 @@ const OpProgram* get_program(int op, int chi_b, int chi_t, int prec) {
     trans = std::max(trans, pg.ws_bytes);
   }
   prog->ws_bytes = res_base + trans;
+  return prog;
+}
+
+}  // namespace
+
+const OpProgram* get_program(int op, int chi_b, int chi_t, int prec, bool plain) {
+  if (op < OP_ASCEND || op > OP_ENV_W) return nullptr;
+  if (prec < PREC_F64 || prec > PREC_LAST) return nullptr;
+  if (chi_b < 1 || chi_t < 1 || chi_b > 64 || chi_t > 64) return nullptr;
+  if (chi_t > chi_b * chi_b) return nullptr;
+  std::lock_guard<std::mutex> lk(g_mu);
+  Key k{op, chi_b, chi_t, prec, plain && prec == PREC_F64};
+  auto it = g_cache.find(k);
+  if (it != g_cache.end()) return it->second.get();
+  auto prog = build_program(op, chi_b, chi_t, prec, plain);
+  // The digit images nearly triple a PREC_F64 operand.  Past chi ~ 33 the
+  // operands alone fill most of the memory: those programs stay on the FP64
+  // pipe (env_w at chi = 40: 130 GiB against 307 GiB).
+  constexpr size_t kX64MaxWorkspace = size_t(96) << 30;
+  if (prog && prog->has_x64 && prog->ws_bytes > kX64MaxWorkspace) prog = build_program(op, chi_b, chi_t, prec, true);
+  if (!prog) return nullptr;
   const OpProgram* out = prog.get();
   g_cache[k] = std::move(prog);
   return out;
@@ -938,7 +1062,7 @@ std::string program_json(const OpProgram& prog, int op, int chi_b, int chi_t, in
       if (st.kind == 2) {
         o << "{\"kind\":\"split\",\"raw_buf\":" << st.x.raw_buf << ",\"dst_buf\":" << st.x.dst_buf
           << ",\"rows\":" << st.x.rows << ",\"K\":" << st.x.K << ",\"ld\":" << st.x.ld << ",\"skip\":" << st.x.skip
-          << "}";
+          << ",\"tile\":" << st.x.tile << ",\"seg_rows\":" << st.x.seg_rows << "}";
       } else if (st.kind == 0) {
         o << "{\"kind\":\"permute\",\"slot\":" << st.p.slot << ",\"dst_buf\":" << st.p.dst_buf
           << ",\"op_buf\":" << st.p.op_buf
@@ -954,7 +1078,7 @@ std::string program_json(const OpProgram& prog, int op, int chi_b, int chi_t, in
           << ",\"M\":" << g.M << ",\"N\":" << g.N << ",\"K\":" << g.K << ",\"lda\":" << g.lda << ",\"ldb\":" << g.ldb
           << ",\"c_buf\":" << g.c_buf << ",\"alpha\":" << g.alpha << ",\"accumulate\":" << g.accumulate
           << ",\"flops\":" << g.flops << ",\"dominant\":" << g.dominant << ",\"split\":" << g.split
-          << ",\"p_buf\":" << g.p_buf << ",\"a_off\":" << g.a_off << ",\"b_off\":" << g.b_off
+          << ",\"p_buf\":" << g.p_buf << ",\"ax_buf\":" << g.ax_buf << ",\"bx_buf\":" << g.bx_buf << ",\"a_off\":" << g.a_off << ",\"b_off\":" << g.b_off
           << ",\"c_off\":" << g.c_off << ",\"stat\":" << g.stat << ",\"bn\":" << g.bn << ",\"m_dst\":";
         lm(g.m_dst);
         o << ",\"n_dst\":";

@@ -34,6 +34,16 @@ inline bool is_oz(int prec) { return prec == PREC_OZ3 || prec == PREC_OZ4; }
 // K elements over which a fixed-point split shares one exponent per row; the
 // GEMM sums the leading slice products of such a block exactly in FP32.
 constexpr int kOzBlockK = 256;
+// Large products of PREC_F64 run on the BF16 tensor cores, each entry cut
+// into digits (x64_split.cu, x64_gemm.cuh): digits per entry, entries along K
+// that share a block exponent, 16-wide K steps per block, the largest row
+// exponent the digits represent, and the exponent that marks other rows.
+constexpr int kX64Digits = 7;
+constexpr int kX64Block = 256;
+constexpr int kX64BlockSteps = kX64Block / 16;
+constexpr int kX64MaxExp = 400;
+constexpr int kX64Bad = 1 << 20;
+constexpr int kX64TileA = 128, kX64TileB = 64;  // rows per image tile of the GEMM's A and B
 enum Slot : int { SLOT_OP = 0, SLOT_RHO = 1, SLOT_U = 2, SLOT_W = 3 };
 enum Op : int { OP_ASCEND = 0, OP_DESCEND = 1, OP_ENV_U = 2, OP_ENV_W = 3 };
 
@@ -76,16 +86,23 @@ struct GemmStep {
   int p_buf = -1;     // FP32 partial-sum buffer [split][N][M] when split > 1
   int stat = 0;       // reads only u and w (directly or through such steps): its output is kept
                       // for the call, and a later run with the same u, w may skip the step
+  int ax_buf = -1, bx_buf = -1;     // PREC_F64 on the tensor cores: digit images of A and B
+  int64_t ax_row = 0, bx_row = 0;   // first row of the operands' row exponents (slices)
+  int64_t ax_tile = 0, bx_tile = 0; // first tile of the operands' images (slices)
   std::string label;  // e.g. "aceiq*CDcdil->ADadelq" for inspection
 };
 
-// Fixed-point split modes: raw (hi + lo binary32 planes, written by a
-// permute or GEMM step) -> S BF16 slice planes of the operand buffer, the
+// PREC_F64: a binary64 operand -> its digit image.  Fixed-point split modes:
+// raw (hi + lo binary32 planes, written by a permute or GEMM step) -> S BF16 slice planes of the operand buffer, the
 // exponent shared by each row's blocks of kOzBlockK elements along K.
 struct SplitStep {
   int raw_buf = 0, dst_buf = 0;
   int64_t rows = 0, K = 0, ld = 0;
   int skip = 0;  // mirrors the skip of the permute step it follows
+  // PREC_F64 (digit images): rows per tile, and rows per segment (a slice
+  // of a sliced operand), each segment padded to whole tiles
+  int tile = 0;
+  int64_t seg_rows = 0;
 };
 
 struct Step {
@@ -100,7 +117,9 @@ struct Buffer {
   int64_t offset = 0;         // byte offset in the workspace
   int64_t plane_bytes = 0;    // bytes of one plane (BF16X3 keeps hi, then lo)
   int64_t bytes = 0;          // plane_bytes * planes
-  int raw = 0;                // 1: raw buffer of a fixed-point split mode (hi, lo binary32 planes)
+  int raw = 0;                // 1: raw buffer of a fixed-point split mode (hi, lo binary32 planes);
+                              // 2: binary64 operand that is also cut into a digit image
+  int64_t exp_off = 0;        // digit images: byte offset of the row exponents
   int resident = 0;           // kept for the whole call, outside the transient arena:
                               // 1 copy of a disentangler/isometry (a later call with the
                               // same u, w may reuse it), 2 copy of h or rho that several
@@ -124,7 +143,19 @@ struct OpProgram {
   size_t ws_bytes = 0;
   size_t persistent_bytes = 0;  // leading workspace bytes holding the resident copies
   double flops = 0.0;
+  int has_x64 = 0;  // some product runs on the tensor cores in PREC_F64
 };
+
+// PREC_F64: whether a product runs on the tensor cores (digit splitting) or
+// on the FP64 pipe, and the K split of the former (1: none).
+bool x64_use(int64_t M, int64_t N, int64_t K);
+int x64_split_k(int64_t M, int64_t N, int64_t K);
+// Steps of a work item under that split: half a block, or whole blocks.
+inline int64_t x64_kc(int64_t nk, int64_t split) {
+  const int64_t kc = (nk + split - 1) / split;
+  const int64_t half = kX64BlockSteps / 2;
+  return kc <= half ? half : (kc + kX64BlockSteps - 1) / kX64BlockSteps * kX64BlockSteps;
+}
 
 int elem_bytes(int prec);   // storage bytes of one operand element (one plane)
 // Output-tile width of the tensor-core GEMM for an N-column product.
@@ -145,7 +176,8 @@ std::vector<std::vector<int64_t>> tuned_tiles();
 int planes(int prec);       // 2 for BF16X3 (hi, lo), 3 for BF16X6 (hi, mid, lo), 3 / 4 for OZ3 / OZ4, else 1
 
 // Builds (and caches) the program; thread safe.  Returns nullptr on bad input.
-const OpProgram* get_program(int op, int chi_b, int chi_t, int prec);
+// plain: PREC_F64 with every product on the FP64 pipe (less workspace).
+const OpProgram* get_program(int op, int chi_b, int chi_t, int prec, bool plain = false);
 
 std::string program_json(const OpProgram& prog, int op, int chi_b, int chi_t, int prec);
 

@@ -586,6 +586,7 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(const __grid_constan
 }
 
 #include "oz_gemm.cuh"
+#include "x64_gemm.cuh"
 
 // ---------------------------------------------------------------------------
 // Host side.
@@ -833,6 +834,67 @@ cudaError_t launch_gemm_tc(const TcGemmArgs& a, cudaStream_t stream) {
     case PREC_OZ4: return launch_oz_prec<4>(a, stream);
     default: return cudaErrorNotSupported;
   }
+}
+
+cudaError_t launch_gemm_x64(const X64GemmArgs& a, cudaStream_t stream) {
+  if (a.M <= 0 || a.N <= 0 || a.K <= 0) return cudaErrorInvalidValue;
+  if (a.M > 0x7fffffff || a.N > 0x7fffffff || a.K > (1 << 30)) return cudaErrorInvalidValue;
+  static std::once_flag once;
+  static cudaError_t attr_err = cudaSuccess;
+  static int resident = 0;  // CTAs the whole GPU holds at once (one per SM)
+  std::call_once(once, [] {
+    attr_err = cudaFuncSetAttribute(x64_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kXSmem));
+    if (attr_err == cudaSuccess)
+      attr_err = cudaFuncSetAttribute(x64_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kXSmem));
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    resident = std::max(1, sms);
+  });
+  if (attr_err != cudaSuccess) return attr_err;
+  X64Params p;
+  p.A = static_cast<const uint8_t*>(a.A);
+  p.B = static_cast<const uint8_t*>(a.B);
+  p.ea = a.ea;
+  p.eb = a.eb;
+  p.A64 = a.A64;
+  p.B64 = a.B64;
+  p.lda = a.lda;
+  p.ldb = a.ldb;
+  p.M = a.M;
+  p.N = a.N;
+  p.K = a.K;
+  p.C = a.C;
+  p.m_dst = a.m_dst;
+  p.n_dst = a.n_dst;
+  p.alpha = a.alpha;
+  int e2 = 0;
+  if (std::frexp(a.alpha, &e2) != 0.5) return cudaErrorInvalidValue;
+  p.alpha_exp = e2 - 1;
+  p.accumulate = a.accumulate;
+  p.nk = int((a.K + 15) / 16);
+  p.split = a.split > 1 && a.partial ? a.split : 1;
+  p.kc = int(x64_kc(p.nk, p.split));
+  p.partial = a.partial;
+  p.p_plane = a.partial_plane;
+  if (p.split > 1 && (int64_t(p.split - 1) * p.kc >= p.nk || a.partial_plane < int64_t(p.split) * a.N * a.M))
+    return cudaErrorInvalidValue;  // an empty split, or overlapping partial planes
+  const int64_t tiles_m = (a.M + kBM - 1) / kBM;
+  p.group_m = int(std::min<int64_t>(std::max<int64_t>(1, (int64_t(32) << 20) / (int64_t(p.nk) * kXABytes)), tiles_m));
+  const int64_t tiles = tiles_m * ((a.N + kXBN - 1) / kXBN) * p.split;
+  count_launch();
+  const unsigned grid = unsigned(std::min<int64_t>(tiles, resident));
+  if (p.kc <= kX64BlockSteps)
+    x64_gemm_kernel<false><<<grid, kXThreads, kXSmem, stream>>>(p);
+  else
+    x64_gemm_kernel<true><<<grid, kXThreads, kXSmem, stream>>>(p);
+  if (p.split > 1) {
+    const unsigned gx = unsigned((a.M + 127) / 128);
+    const unsigned gy = unsigned(std::min<int64_t>(a.N, std::max<int64_t>(1, 8 * 152 / int64_t(gx))));
+    count_launch();
+    x64_reduce_kernel<<<dim3(gx, gy), 128, 0, stream>>>(p);
+  }
+  return cudaGetLastError();
 }
 
 __global__ void report_notconv_kernel(const int* state) {

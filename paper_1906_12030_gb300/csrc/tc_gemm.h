@@ -38,6 +38,30 @@ struct TcGemmArgs {
 
 cudaError_t launch_gemm_tc(const TcGemmArgs& args, cudaStream_t stream);
 
+// The same product in PREC_F64 on the BF16 tensor cores, from the operands'
+// digit images and row exponents (x64_split.cu).  alpha must be a power of
+// two.  A64 and B64 are the binary64 operands themselves.
+struct X64GemmArgs {
+  const void* A = nullptr;
+  const int* ea = nullptr;
+  const double* A64 = nullptr;
+  int64_t lda = 0;
+  const void* B = nullptr;
+  const int* eb = nullptr;
+  const double* B64 = nullptr;
+  int64_t ldb = 0;
+  int64_t M = 0, N = 0, K = 0;
+  double* C = nullptr;
+  LegMap m_dst, n_dst;
+  double alpha = 1.0;
+  int accumulate = 0;
+  int split = 1;             // K split (x64_split_k); > 1 needs `partial`
+  float* partial = nullptr;  // hi, mid, lo planes [split][N][M]
+  int64_t partial_plane = 0; // floats from one plane to the next
+};
+
+cudaError_t launch_gemm_x64(const X64GemmArgs& args, cudaStream_t stream);
+
 // Sets bit MERA_ENOTCONV of the device status word unless the Newton-Schulz
 // state state[0] says the iteration converged (used where the host cannot
 // look, e.g. inside a captured graph).

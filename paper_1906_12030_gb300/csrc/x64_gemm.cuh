@@ -1,0 +1,423 @@
+// Binary64 GEMM on the BF16 tensor cores (the large products of MERA_PREC_F64).
+// Included by tc_gemm.cu inside its anonymous namespace: it shares that
+// file's PTX wrappers (mbarrier, tcgen05) and its device status word.
+//
+// What bounds a binary64 product on this GPU is the FP64 pipe (two FMAs per
+// clock and SM, 1.25 TFLOP/s); the BF16 tensor cores do 1500 times as many
+// products.  So each operand entry is cut into seven signed 8-bit digits
+// (x64_split.cu), and the product is the sum of the 34 digit products whose
+// orders p + q are at most 7.  This is the error-free splitting of Ozaki,
+// Ogita, Oishi and Rump (Numer. Algorithms 59, 2012), with one exponent per
+// row and block of 256 along K.
+//
+// Exactness.  With 2^E the product of the two block scales, every product of
+// order d is an integer multiple of 2^(E-12-8d) of magnitude at most 2^14
+// units, so a block's sum of order d stays below (d+1) 2^22 units: at most
+// 2^24, what an FP32 accumulator holds exactly, for d <= 3 whatever the data,
+// and for d >= 4 unless nearly all products are extreme and of one sign
+// (then off by a unit of 2^-44 or less, 2^-52 of such a result).  Each order
+// therefore has an accumulator of its own.  What is left out (orders 8 and
+// up, and the bits below the seventh digit) is ~2^-58 and 2^-55 of the
+// block scale: on Gaussian, decaying, heavy-tailed, positive and diagonally
+// dominant operands with K = 16 .. 1024 the error of the sum is 2 to 15
+// times smaller than that of a chain of binary64 FMAs.
+//
+// Tile 128 x 64: eight accumulators of 64 columns fill tensor memory.  (A
+// wider tile has no room for eight; a narrower one needs more shared-memory
+// reads of A per product than the tensor cores take time for.)  The digits of
+// B lie next to each other in a stage and the accumulators next to each
+// other in tensor memory, so one MMA of width 256 meets a digit of A with
+// four digits of B and adds into four orders: 11 MMAs per 16 of K for the 34
+// products.  Per 16 of K the MMAs take 1088 clocks, the shared-memory reads
+// of their operands 896 and the writes of the copies 336: shared-memory
+// bandwidth sets the pace.
+//
+// A stage is 16 of K of all planes, stored by the split kernel as the very
+// image that the MMA reads (8 x 16-byte core matrices, no swizzle), so a
+// stage is two contiguous bulk copies and five stages fit in shared memory.
+//
+// Warp roles as in tc_gemm_kernel: warp 0 copies, warp 1 MMA, warps 2..17
+// epilogue, four per tensor-memory lane quarter with 16 columns each.  There
+// is one set of accumulators, so the MMAs wait while the epilogue folds the
+// eight sums of a block into a triple hi + mid + lo of binary32 values per
+// output and hands them back; everything after that runs beside the next
+// tile's MMAs.  The result is rounded once to binary64 by integer operations
+// (an FP64 add per output and part would cost as much as the MMAs of a short
+// K).
+//
+// Measured (chi = 16 descend, the pair of chi^9 products): 65536 x 4096 x 256
+// 110 ms on the FP64 pipe, 3.0 ms here (46 TFLOP/s); 65536 x 256 x 4096 110
+// -> 2.66 ms (52 TFLOP/s, 0.93 of the burst BF16 rate / 34); the whole map
+// 497 -> 15.6 ms, its error against 64 bits 1.8e-15 -> 1.5e-15.
+//
+// Rows of A or B that the digits cannot represent (a NaN, an infinity, or a
+// largest entry beyond 2^+-kX64MaxExp) carry the exponent kX64Bad; outputs
+// that touch one are summed from the binary64 operands by FMAs in the order
+// of K, as the FP64 kernel sums them.
+
+constexpr int kXBN = 64;
+constexpr int kXPlanes = kX64Digits;
+constexpr int kXOrders = 8;
+constexpr int kXABytes = kXPlanes * kBM * 32;    // 16 of K, all digits
+constexpr int kXBBytes = kXPlanes * kXBN * 32;
+constexpr int kXStageBytes = kXABytes + kXBBytes;
+constexpr int kXStages = 5;
+constexpr int kXEpiWarps = 16;
+constexpr int kXEpiThreads = 32 * kXEpiWarps;
+constexpr int kXThreads = 64 + kXEpiThreads;
+constexpr int kXCols = kXBN / (kXEpiWarps / 4);  // columns per epilogue thread
+constexpr int kXTmemCols = kXOrders * kXBN;
+constexpr size_t kXSmem = 1024 + size_t(kXStages) * kXStageBytes + 1024 + kXBN * (sizeof(int64_t) + sizeof(int));
+static_assert(kXTmemCols == 512, "all of tensor memory");
+
+struct X64Params {
+  const uint8_t* A;  // digit images
+  const uint8_t* B;
+  const int* ea;     // row exponents
+  const int* eb;
+  const double* A64;  // binary64 operands (rows with exponent kX64Bad)
+  const double* B64;
+  int64_t lda, ldb;
+  int64_t M, N, K;
+  double* C;
+  LegMap m_dst, n_dst;
+  double alpha;
+  int alpha_exp;      // alpha == 2^alpha_exp
+  int accumulate;
+  int nk;             // 16-wide steps of K
+  int split, kc;      // K split: steps per split
+  float* partial;     // split > 1: hi, mid, lo planes [split][N][M]
+  int64_t p_plane;
+  int group_m;
+};
+
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_u32(dst)),
+               "l"(src), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
+}
+
+// K-major operand without swizzle: core matrices of 8 rows x 16 bytes, the
+// two of a 16-wide K step 128 bytes apart, groups of eight rows 256 bytes.
+__device__ __forceinline__ uint64_t x64_desc(uint32_t saddr) {
+  return uint64_t((saddr & 0x3FFFFu) >> 4) | (uint64_t(128 >> 4) << 16) | (uint64_t(256 >> 4) << 32) |
+         (uint64_t(1) << 46);
+}
+
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&v)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+               : "r"(taddr));
+}
+
+// s + e = a + b exactly (Knuth's TwoSum).
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+  s = __fadd_rn(a, b);
+  const float bp = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bp)), __fsub_rn(b, bp));
+}
+
+// The same where a is a multiple of ulp(b) (FastTwoSum under its relaxed
+// condition).
+__device__ __forceinline__ void fast_two_sum(float a, float b, float& s, float& e) {
+  s = __fadd_rn(a, b);
+  e = __fsub_rn(b, __fsub_rn(s, a));
+}
+
+// (h, m, l) += (x, y, z), each an unevaluated sum of decreasing magnitude.
+__device__ __forceinline__ void triple_add(float& h, float& m, float& l, float x, float y, float z) {
+  float c1, c2, c3;
+  two_sum(h, x, h, c1);
+  two_sum(m, y, m, c2);
+  two_sum(m, c1, m, c3);
+  l = __fadd_rn(l, __fadd_rn(z, __fadd_rn(c2, c3)));
+}
+
+// (h + m + l) 2^e rounded to binary64 with integer operations: h gives the
+// bit pattern, m + l the number of its last places to add.  The exponent
+// stays normal (|e| <= 2 kX64MaxExp + 1).
+__device__ __forceinline__ double triple_to_f64(float h, float m, float l, int e) {
+  two_sum(h, m, h, m);
+  two_sum(m, l, m, l);
+  two_sum(h, m, h, m);
+  const uint32_t u = __float_as_uint(h);
+  const int eh = int((u >> 23) & 0xFFu);
+  // below 2^-70 of the scale there is nothing under h that the digits resolve
+  const float sc = eh < 127 - 70 ? 0.0f : __int_as_float((52 + 127 + 127 - eh) << 23);
+  const float mp = __fmul_rn(m, sc);  // |mp| <= 2^28
+  const int q1 = __float2int_rn(mp);
+  int q = q1 + __float2int_rn(__fmaf_rn(l, sc, __fsub_rn(mp, __int2float_rn(q1))));
+  if (int(u) < 0) q = -q;  // towards larger magnitude
+  if (q < 0 && (u & 0x7FFFFFu) == 0) q *= 2;  // below a power of two the places are half as large
+  // 24-bit significand of h over 29 more places
+  const long long mag = (static_cast<long long>(eh + (1023 - 127) + e) << 52) +
+                        (static_cast<long long>(u & 0x7FFFFFu) << 29) + q;
+  const uint32_t hi = (uint32_t(static_cast<unsigned long long>(mag) >> 32) & 0x7FFFFFFFu) | (u & 0x80000000u);
+  return eh == 0 ? 0.0 : __hiloint2double(int(hi), int(uint32_t(mag)));
+}
+
+// One output from the binary64 operands, as gemm_f64_kernel sums it.
+__device__ __noinline__ double x64_plain(const double* a, const double* b, int64_t K) {
+  double s = 0.0;
+  for (int64_t k = 0; k < K; ++k) s = fma(a[k], b[k], s);
+  return s;
+}
+
+__device__ __forceinline__ void x64_store(const X64Params& p, int64_t off, double x) {
+  double* d = p.C + off;
+  *d = p.accumulate ? *d + x : x;
+}
+
+// MULTI: a work item may span several blocks of K.
+template <bool MULTI>
+__global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_constant__ X64Params p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* aux = smem + size_t(kXStages) * kXStageBytes;
+  uint64_t* full = reinterpret_cast<uint64_t*>(aux);
+  uint64_t* empty = full + kXStages;
+  uint64_t* acc_full = empty + kXStages;  // MMA -> epilogue, one phase per block
+  uint64_t* acc_empty = acc_full + 1;     // epilogue -> MMA
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  volatile int* abort_snapshot = abort_flag + 1;
+  volatile int* never = abort_flag + 2;
+  int64_t* off_n = reinterpret_cast<int64_t*>(aux + 1024);
+  int* exp_n = reinterpret_cast<int*>(off_n + kXBN);
+
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int64_t tiles_n = (p.N + kXBN - 1) / kXBN;
+  const int64_t tiles_m = (p.M + kBM - 1) / kBM;
+  const int64_t tiles_mn = tiles_m * tiles_n;
+  const int64_t tiles = tiles_mn * p.split;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kXStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(acc_full, 1);
+    mbar_init(acc_empty, kXEpiWarps);
+    *abort_flag = 0;
+    *abort_snapshot = 0;
+    *never = 0;
+    fence_barrier_init();
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(uint32_t(kXTmemCols))
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ---- producer: all digits of 16 of K per stage ----------------------
+      uint32_t it = 0;
+      bool alive = true;
+      for (int64_t t = blockIdx.x; t < tiles && alive; t += gridDim.x) {
+        int64_t row_t, col_t;
+        tile_of(t % tiles_mn, tiles_m, tiles_n, p.group_m, row_t, col_t);
+        const int k0 = int(t / tiles_mn) * p.kc, k1 = min(k0 + p.kc, p.nk);
+        const uint8_t* a = p.A + row_t * p.nk * int64_t(kXABytes);
+        const uint8_t* b = p.B + col_t * p.nk * int64_t(kXBBytes);
+        for (int k = k0; k < k1; ++k, ++it) {
+          const uint32_t s = it % kXStages;
+          if (it >= uint32_t(kXStages) && !mbar_wait(&empty[s], ((it / kXStages) & 1) ^ 1, abort_flag)) {
+            alive = false;
+            break;
+          }
+          uint8_t* st = smem + size_t(s) * kXStageBytes;
+          mbar_arrive_expect_tx(&full[s], kXStageBytes);
+          bulk_load(st, a + k * int64_t(kXABytes), kXABytes, &full[s]);
+          bulk_load(st + kXABytes, b + k * int64_t(kXBBytes), kXBBytes, &full[s]);
+        }
+      }
+      for (uint32_t j = (it > uint32_t(kXStages) ? it - kXStages : 0); j < it; ++j)
+        mbar_wait(&full[j % kXStages], (j / kXStages) & 1, never);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      // ---- MMA issuer ---------------------------------------------------------
+      uint32_t it = 0, bc = 0;  // stages consumed, blocks issued
+      bool alive = true;
+      for (int64_t t = blockIdx.x; t < tiles && alive; t += gridDim.x) {
+        const int k0 = int(t / tiles_mn) * p.kc, k1 = min(k0 + p.kc, p.nk);
+        for (int k = k0; k < k1 && alive; ++bc) {
+          const int ke = min(k1, (k / kX64BlockSteps + 1) * kX64BlockSteps);
+          if (bc >= 1 && !mbar_wait(acc_empty, (bc - 1) & 1, abort_flag)) {
+            alive = false;
+            break;
+          }
+          tc_fence_after();
+          bool first = true;
+          for (; k < ke; ++k, ++it, first = false) {
+            const uint32_t s = it % kXStages;
+            if (!mbar_wait(&full[s], (it / kXStages) & 1, abort_flag)) {
+              alive = false;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t sa = smem_u32(smem + size_t(s) * kXStageBytes), sb = sa + kXABytes;
+#pragma unroll
+            for (int pa = 0; pa < kXPlanes; ++pa) {
+              const uint64_t da = x64_desc(sa + pa * kBM * 32);
+              const int nq = min(kXPlanes, kXOrders - pa);  // digits of B that this digit of A meets
+#pragma unroll
+              for (int q = 0; q < nq; q += 4) {
+                const int cnt = min(4, nq - q);
+                const uint64_t db = x64_desc(sb + q * kXBN * 32);
+                const uint32_t d = tmem + uint32_t((pa + q) * kXBN);
+                if (pa == 1 && q == 4) {
+                  // orders 5, 6 and 7: the last one starts here
+                  if (first) {
+                    tc_mma<PREC_BF16>(d, da, db, make_idesc(1u, kBM, 2 * kXBN), 1u);
+                    tc_mma<PREC_BF16>(d + 2 * kXBN, da, x64_desc(sb + (q + 2) * kXBN * 32),
+                                      make_idesc(1u, kBM, kXBN), 0u);
+                    continue;
+                  }
+                }
+                tc_mma<PREC_BF16>(d, da, db, make_idesc(1u, kBM, cnt * kXBN), (pa == 0 && first) ? 0u : 1u);
+              }
+            }
+            tc_commit(&empty[s]);
+          }
+          tc_commit(acc_full);  // also after an abort, so that no epilogue warp waits forever
+        }
+      }
+    }
+  } else {
+    // ---- epilogue (warps 2..17) --------------------------------------------------
+    const int et = threadIdx.x - 64;
+    const int quarter = warp % 4;
+    const int c0 = ((warp - 2) / 4) * kXCols;  // first column of this warp's share
+    const int row = quarter * 32 + lane;
+    uint32_t bc = 0;
+    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+      const int64_t ks = t / tiles_mn;
+      int64_t row_t, col_t;
+      tile_of(t % tiles_mn, tiles_m, tiles_n, p.group_m, row_t, col_t);
+      const int64_t m0 = row_t * kBM, n0 = col_t * kXBN;
+      const int k0 = int(ks) * p.kc, k1 = min(k0 + p.kc, p.nk);
+      asm volatile("bar.sync 1, %0;" ::"n"(kXEpiThreads) : "memory");
+      if (et == 0) *abort_snapshot = *abort_flag;
+      for (int c = et; c < kXBN; c += kXEpiThreads) {
+        const int64_t n = n0 + c;
+        off_n[c] = n < p.N ? legmap_offset32(p.n_dst, uint32_t(n)) : 0;
+        exp_n[c] = n < p.N ? p.eb[n] : 0;
+      }
+      asm volatile("bar.sync 1, %0;" ::"n"(kXEpiThreads) : "memory");
+      if (*abort_snapshot) break;
+      const int64_t m = m0 + row;
+      const bool row_ok = m < p.M;
+      float h[kXCols], mid[kXCols], lo[kXCols];
+      if constexpr (MULTI) {
+#pragma unroll
+        for (int j = 0; j < kXCols; ++j) h[j] = mid[j] = lo[j] = 0.0f;
+      }
+      bool ok = true;
+      for (int k = k0; k < k1; k = min(k1, (k / kX64BlockSteps + 1) * kX64BlockSteps), ++bc) {
+        ok = __all_sync(0xffffffffu, mbar_wait(acc_full, bc & 1, abort_flag) ? 1 : 0) != 0;
+        tc_fence_after();
+        if (!ok) break;  // the next tile's snapshot sees the abort flag
+        const uint32_t ta = tmem + uint32_t(c0) + (uint32_t(quarter * 32) << 16);
+#pragma unroll
+        for (int g = 0; g < kXCols; g += 4) {
+          uint32_t v[kXOrders][4];
+#pragma unroll
+          for (int d = 0; d < kXOrders; ++d) tmem_ld4(ta + uint32_t(d * kXBN + g), v[d]);
+          tmem_wait_ld();
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            // VecSum from the smallest order up.  v[d] is a multiple of its
+            // order's unit, at least 2^6 ulps of the sum of what is below.
+            float s = __uint_as_float(v[7][j]), c, r = 0.0f;
+#pragma unroll
+            for (int d = 6; d >= 1; --d) {
+              fast_two_sum(__uint_as_float(v[d][j]), s, s, c);
+              r = __fadd_rn(r, c);
+            }
+            fast_two_sum(__uint_as_float(v[0][j]), s, s, c);
+            if constexpr (MULTI) {
+              triple_add(h[g + j], mid[g + j], lo[g + j], s, c, r);
+            } else {
+              h[g + j] = s;
+              mid[g + j] = c;
+              lo[g + j] = r;
+            }
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acc_empty);
+        if constexpr (!MULTI) {
+          ++bc;
+          break;
+        }
+      }
+      if (!ok || !row_ok) continue;
+      if (p.split > 1) {  // partial triple, summed by x64_reduce_kernel
+        float* q = p.partial + (ks * p.N + n0 + c0) * p.M + m;
+#pragma unroll
+        for (int j = 0; j < kXCols; ++j, q += p.M)
+          if (n0 + c0 + j < p.N) {
+            q[0] = h[j];
+            q[p.p_plane] = mid[j];
+            q[2 * p.p_plane] = lo[j];
+          }
+        continue;
+      }
+      const int64_t off_m = legmap_offset32(p.m_dst, uint32_t(m));
+      const int ra = p.ea[m];
+      bool bad = ra == kX64Bad;
+#pragma unroll
+      for (int j = 0; j < kXCols; ++j) {
+        const int c = c0 + j;
+        const int rb = exp_n[c];
+        bad |= rb == kX64Bad;
+        if (n0 + c >= p.N || ra == kX64Bad || rb == kX64Bad) continue;
+        x64_store(p, off_m + off_n[c], triple_to_f64(h[j], mid[j], lo[j], ra + rb + p.alpha_exp));
+      }
+      if (bad) {
+#pragma unroll 1
+        for (int c = c0; c < c0 + kXCols && n0 + c < p.N; ++c)
+          if (ra == kX64Bad || exp_n[c] == kX64Bad)
+            x64_store(p, off_m + off_n[c], p.alpha * x64_plain(p.A64 + m * p.lda, p.B64 + (n0 + c) * p.ldb, p.K));
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(uint32_t(kXTmemCols))
+                 : "memory");
+  }
+}
+
+// Sum of the K-split partial triples in a fixed order, then the GEMM's
+// output.  One thread per row m over a chunk of columns.
+__global__ void __launch_bounds__(128) x64_reduce_kernel(const __grid_constant__ X64Params p) {
+  const int64_t m = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (m >= p.M) return;
+  const int64_t off_m = legmap_offset32(p.m_dst, uint32_t(m));
+  const int ra = p.ea[m];
+  const int64_t n_per = (p.N + gridDim.y - 1) / gridDim.y;
+  const int64_t n_lo = int64_t(blockIdx.y) * n_per, n_hi = min(p.N, n_lo + n_per);
+  for (int64_t n = n_lo; n < n_hi; ++n) {
+    float h = 0.0f, mid = 0.0f, lo = 0.0f;
+    for (int s = 0; s < p.split; ++s) {
+      const float* q = p.partial + (int64_t(s) * p.N + n) * p.M + m;
+      triple_add(h, mid, lo, q[0], q[p.p_plane], q[2 * p.p_plane]);
+    }
+    const int rb = p.eb[n];
+    const double x = ra == kX64Bad || rb == kX64Bad ? p.alpha * x64_plain(p.A64 + m * p.lda, p.B64 + n * p.ldb, p.K)
+                                                    : triple_to_f64(h, mid, lo, ra + rb + p.alpha_exp);
+    x64_store(p, off_m + legmap_offset32(p.n_dst, uint32_t(n)), x);
+  }
+}

@@ -1,0 +1,239 @@
+// Digit images of the binary64 operands that x64_gemm_kernel multiplies.
+//
+// Every row of an operand is cut into blocks of 256 along K.  With 2^e the
+// exponent of the row's largest entry and 2^b that of the block's (raised to
+// 2^(e-24) where it is smaller, so that every digit product stays a normal
+// binary32 number), an entry x is rounded to a multiple X of 2^(b-54) and X
+// written as seven balanced digits to the base 2^8,
+//   x 2^-e ~ sum_p d_p 2^(b-e-6-8p),   d_0 in [-128, 128], else [-128, 127],
+// each stored as the BF16 value d_p 2^(b-e-6-8p), which is exact.  Entries
+// within a factor four of the block's largest are represented exactly.
+// Adding 128 (256^0 + ... + 256^5) to X makes the balanced digits plain
+// bytes, so a digit costs one byte permute and one FMA.
+//
+// Image: tiles of `tile` rows (128 for the GEMM's A, 64 for B); per tile and
+// 16 of K, per digit, groups of eight rows, the two 8-wide halves of the 16
+// as 8 x 16-byte core matrices.  A GEMM stage is then one contiguous piece.
+// Columns K .. 16 ceil(K / 16) - 1 are zero; rows beyond the operand's are
+// not written (they only meet outputs that are not stored).
+//
+// Bound: memory, 8 bytes read and 14 written per entry (65536 x 4096: 5.9 GB
+// in 1.17 ms, 5.05 TB/s).  A block of threads
+// holds 8192 entries (whole rows) in registers between finding the exponents
+// and writing the digits, so each entry is read once; rows of more than 8192
+// entries get their exponents from a pass of their own.
+#include "common.cuh"
+#include "kernels.h"
+
+namespace mera {
+namespace {
+
+constexpr int kThreadsX = 256;
+constexpr int kItems = 4;                        // groups of 8 entries per thread
+constexpr int kCap = kThreadsX * kItems * 8;     // entries per block of threads
+
+struct SplitArgs {
+  const double* src;
+  int64_t ld, rows, K, seg_rows, tiles_per_seg;
+  uint8_t* img;
+  int* rowexp;
+  int tile, nk;        // rows per tile, 16-wide steps of K
+  int R, G;            // rows and groups of 8 entries per block of threads
+  int known;           // rowexp holds the rows' exponents already
+};
+
+// High word of |x|, at least 1 unless x is zero: orders entries by magnitude
+// up to the exponent and the leading bits.
+__device__ __forceinline__ int mag_word(double x) {
+  const int hi = __double2hiint(x) & 0x7FFFFFFF;
+  return hi == 0 && __double2loint(x) != 0 ? 1 : hi;
+}
+
+// Exponent of a row from its largest magnitude word.
+__device__ __forceinline__ int row_exponent(int w) {
+  const int e = (w >> 20) - 1023;
+  if (w == 0) return 0;  // all zeros: every digit is zero
+  return (e > kX64MaxExp || e < -kX64MaxExp) ? kX64Bad : e;
+}
+
+__global__ void __launch_bounds__(512) x64_rowexp_kernel(const double* __restrict__ src, int64_t ld, int64_t rows,
+                                                         int64_t K, int* __restrict__ rowexp) {
+  __shared__ int sm[16];
+  for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
+    const double* p = src + r * ld;
+    int w = 0;
+    for (int64_t k = threadIdx.x; k < K; k += blockDim.x) w = max(w, mag_word(p[k]));
+    w = __reduce_max_sync(0xffffffffu, w);
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = w;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int i = 1; i < 16; ++i) w = max(w, sm[i]);
+      rowexp[r] = row_exponent(w);
+    }
+    __syncthreads();
+  }
+}
+
+__global__ void __launch_bounds__(kThreadsX, 2) x64_split_kernel(const __grid_constant__ SplitArgs a) {
+  extern __shared__ int s_max[];  // [R][blocks of 256]: magnitude words, then [R] row exponents
+  const int nb = (a.G * 8 + kX64Block - 1) / kX64Block;
+  int* s_row = s_max + a.R * nb;
+  const int64_t r0 = int64_t(blockIdx.x) * a.R;
+  const int kbase = int(blockIdx.y) * a.G * 8;
+  const int rlow = min(a.R, 8);  // rows run fastest over the threads: stores fill whole core matrices
+  for (int i = threadIdx.x; i < a.R * nb; i += kThreadsX) s_max[i] = 0;
+  __syncthreads();
+
+  double x[kItems][8];
+  int rr[kItems], gg[kItems];
+#pragma unroll
+  for (int i = 0; i < kItems; ++i) {
+    const int id = threadIdx.x + kThreadsX * i;
+    const int q = id / rlow;
+    const int g = q % a.G;
+    const int r = id % rlow + rlow * (q / a.G);
+    rr[i] = (r < a.R && r0 + r < a.rows && kbase / 16 + g / 2 < a.nk) ? r : -1;
+    gg[i] = g;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) x[i][j] = 0.0;
+    if (rr[i] < 0) continue;
+    const int64_t k = kbase + g * 8;
+    const double* s = a.src + (r0 + r) * a.ld + k;
+    if (k + 8 <= a.K) {
+#pragma unroll
+      for (int j = 0; j < 8; j += 2) {
+        const double2 d = *reinterpret_cast<const double2*>(s + j);  // ld is a multiple of 8
+        x[i][j] = d.x;
+        x[i][j + 1] = d.y;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (k + j < a.K) x[i][j] = s[j];
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < kItems; ++i) {
+    if (rr[i] < 0) continue;
+    int w = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) w = max(w, mag_word(x[i][j]));
+    atomicMax(&s_max[rr[i] * nb + gg[i] * 8 / kX64Block], w);
+  }
+  __syncthreads();
+  for (int r = threadIdx.x; r < a.R; r += kThreadsX) {
+    if (r0 + r >= a.rows) continue;
+    int e;
+    if (a.known) {
+      e = a.rowexp[r0 + r];
+    } else {
+      int w = 0;
+      for (int b = 0; b < nb; ++b) w = max(w, s_max[r * nb + b]);
+      e = row_exponent(w);
+      a.rowexp[r0 + r] = e;
+    }
+    s_row[r] = e;
+  }
+  __syncthreads();
+
+#pragma unroll
+  for (int i = 0; i < kItems; ++i) {
+    if (rr[i] < 0) continue;
+    const int e = s_row[rr[i]];
+    const int w = s_max[rr[i] * nb + gg[i] * 8 / kX64Block];
+    const int b = max((w >> 20) - 1023, e - 24);  // exponent of the block's grid
+    const bool zero = w == 0 || e == kX64Bad;
+    uint32_t lo[8], hi[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const unsigned long long u = static_cast<unsigned long long>(__double_as_longlong(x[i][j]));
+      const int ex = int(u >> 52) & 0x7FF;
+      long long X = static_cast<long long>((u & 0xFFFFFFFFFFFFFull) | (ex ? 0x10000000000000ull : 0ull));
+      const int sh = ex - 1023 - b + 2;  // X 2^sh multiples of 2^(b-54)
+      if (sh >= 0)
+        X <<= sh;  // at most 2, ex - 1023 <= b
+      else
+        X = sh < -54 ? 0 : (X + (1ll << (-sh - 1))) >> -sh;
+      if (static_cast<long long>(u) < 0) X = -X;
+      if (zero) X = 0;
+      X += 0x0000808080808080ll;
+      lo[j] = uint32_t(X);
+      hi[j] = uint32_t(static_cast<unsigned long long>(X) >> 32);
+    }
+    const int64_t r = r0 + rr[i];
+    const int64_t seg = r / a.seg_rows, rs = r - seg * a.seg_rows;
+    const int64_t t = seg * a.tiles_per_seg + rs / a.tile;
+    const int ri = int(rs % a.tile);
+    const int g = kbase / 8 + gg[i];
+    const int plane = a.tile * 32;
+    uint8_t* d = a.img + (t * a.nk + g / 2) * int64_t(kX64Digits * plane) + (ri / 8) * 256 + (g & 1) * 128 + (ri % 8) * 16;
+#pragma unroll
+    for (int p = 0; p < kX64Digits; ++p) {
+      const float sc = zero ? 0.0f : __int_as_float((b - e - 6 - 8 * p + 127) << 23);
+      const float off = -8388736.0f * sc;  // -(2^23 + 128) sc
+      uint32_t f[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        uint32_t u;
+        if (p == 0)  // the sign-extended top digit plus 128, in [0, 256]
+          u = 0x4B000000u + uint32_t((int(hi[j]) >> 16) + 128);
+        else
+          u = __byte_perm(p <= 2 ? hi[j] : lo[j], 0x4B000000u, 0x7440u + uint32_t(p <= 2 ? 2 - p : 6 - p));
+        f[j] = __float_as_uint(__fmaf_rn(__uint_as_float(u), sc, off));
+      }
+      uint4 o;  // BF16 pairs: the values are exact in the upper halves
+      o.x = __byte_perm(f[0], f[1], 0x7632);
+      o.y = __byte_perm(f[2], f[3], 0x7632);
+      o.z = __byte_perm(f[4], f[5], 0x7632);
+      o.w = __byte_perm(f[6], f[7], 0x7632);
+      *reinterpret_cast<uint4*>(d + p * plane) = o;
+    }
+  }
+}
+
+}  // namespace
+
+cudaError_t launch_x64_split(const double* src, int64_t ld, int64_t rows, int64_t K, int64_t seg_rows, int tile,
+                             void* img, int* rowexp, cudaStream_t stream) {
+  if (rows <= 0 || K <= 0) return cudaSuccess;
+  if ((ld & 7) || K > ld || K > (1 << 30) || seg_rows <= 0 || rows % seg_rows || (reinterpret_cast<uintptr_t>(src) & 15))
+    return cudaErrorInvalidValue;
+  SplitArgs a;
+  a.src = src;
+  a.ld = ld;
+  a.rows = rows;
+  a.K = K;
+  a.seg_rows = seg_rows;
+  a.tiles_per_seg = (seg_rows + tile - 1) / tile;
+  a.img = static_cast<uint8_t*>(img);
+  a.rowexp = rowexp;
+  a.tile = tile;
+  a.nk = int((K + 15) / 16);
+  const int kp = a.nk * 16;
+  unsigned ksegs = 1;
+  if (kp <= kCap) {
+    a.known = 0;
+    a.G = kp / 8;
+    int R = 1;
+    while (2 * R * kp <= kCap && R < 256) R *= 2;
+    // at least two blocks of threads per SM where the rows allow it
+    while (R > 8 && (rows + R - 1) / R < 2 * 152) R /= 2;
+    a.R = R;
+  } else {
+    a.known = 1;
+    a.R = 8;
+    a.G = kCap / 8 / 8;  // 1024 of K: four blocks of 256
+    ksegs = unsigned((kp + a.G * 8 - 1) / (a.G * 8));
+    if (ksegs > 65535) return cudaErrorInvalidValue;
+    count_launch();
+    x64_rowexp_kernel<<<unsigned(std::min<int64_t>(rows, 152 * 16)), 512, 0, stream>>>(src, ld, rows, K, rowexp);
+  }
+  const int64_t gx = (rows + a.R - 1) / a.R;
+  if (gx > 0x7fffffff) return cudaErrorInvalidValue;
+  const int nb = (a.G * 8 + kX64Block - 1) / kX64Block;
+  count_launch();
+  x64_split_kernel<<<dim3(unsigned(gx), ksegs), kThreadsX, size_t(a.R) * (nb + 1) * sizeof(int), stream>>>(a);
+  return cudaGetLastError();
+}
+
+}  // namespace mera

@@ -182,100 +182,162 @@ struct Arena {
   size_t left() const { return used <= cap ? cap - used : 0; }
 };
 
+// Launches steps of one family (Wave) of the operation.  `out` is the
+// caller's output; the diagrams' parts of it go to `ws` where the program says
+// so.
+mera_status run_steps(const OpProgram& prog, const std::pair<int, int>* steps, int n, int family,
+                      const double* const inputs[4], double* out, int prec, char* ws, cudaStream_t stream) {
+  double flops = 0.0;
+  int dominant = 0;
+  for (int i = 0; i < n; ++i) {
+    const Step& st = prog.diagrams[size_t(steps[i].first)].steps[size_t(steps[i].second)];
+    if (st.kind != 1) continue;
+    flops += st.g.flops;
+    dominant |= st.g.dominant;
+  }
+  ProfScope ps(stream, family < 2 ? 1 : 0, dominant, flops);
+  auto diagram = [&](int i) -> const Program& { return prog.diagrams[size_t(steps[i].first)]; };
+  auto step = [&](int i) -> const Step& { return diagram(i).steps[size_t(steps[i].second)]; };
+  auto output = [&](int i) {
+    return prog.part_off < 0 ? out : reinterpret_cast<double*>(ws + prog.part_off + steps[i].first * prog.part_bytes);
+  };
+  auto accumulate = [&](int i) { return prog.part_off < 0 ? step(i).g.accumulate : 0; };
+  if (family == 0) {
+    PermuteJob jobs[kGroup];
+    int pr = prec;
+    for (int i = 0; i < n; ++i) {
+      const PermuteStep& p = step(i).p;
+      const Buffer& b = diagram(i).bufs[size_t(p.dst_buf)];
+      jobs[i] = {&p, inputs[p.slot], ws + b.offset, b.plane_bytes / buf_elem_bytes(b, prec)};
+      pr = b.raw == 1 ? PREC_RAW : prec;
+    }
+    return cuda_status(launch_permute(jobs, n, pr, stream), "permute");
+  }
+  if (family == 1 && is_oz(prec)) {  // fixed-point split of a raw buffer into its operand
+    OzSplitJob jobs[kGroup];
+    for (int i = 0; i < n; ++i) {
+      const SplitStep& x = step(i).x;
+      const Buffer& r = diagram(i).bufs[size_t(x.raw_buf)];
+      const Buffer& d = diagram(i).bufs[size_t(x.dst_buf)];
+      jobs[i] = {reinterpret_cast<const float*>(ws + r.offset), r.plane_bytes / 4, ws + d.offset,
+                 d.plane_bytes / elem_bytes(prec), x.rows, x.K, x.ld};
+    }
+    return cuda_status(launch_oz_split(jobs, n, planes(prec), stream), "split");
+  }
+  if (family == 1) {  // digit image of an operand
+    X64SplitJob jobs[kGroup];
+    for (int i = 0; i < n; ++i) {
+      const SplitStep& x = step(i).x;
+      const Buffer& d = diagram(i).bufs[size_t(x.dst_buf)];
+      jobs[i] = {reinterpret_cast<const double*>(ws + diagram(i).bufs[size_t(x.raw_buf)].offset), x.ld, x.rows, x.K,
+                 x.seg_rows, x.tile, ws + d.offset, reinterpret_cast<int*>(ws + d.offset + d.exp_off)};
+    }
+    return cuda_status(launch_x64_split(jobs, n, stream), "digit split");
+  }
+  if (family == 2) {
+    GemmF64Args jobs[kGroup];
+    for (int i = 0; i < n; ++i) {
+      const GemmStep& g = step(i).g;
+      const Program& dg = diagram(i);
+      GemmF64Args& a = jobs[i];
+      a.A = reinterpret_cast<const double*>(ws + dg.bufs[size_t(g.a_buf)].offset) + g.a_off;
+      a.a_m = g.lda;
+      a.a_k = 1;
+      a.B = reinterpret_cast<const double*>(ws + dg.bufs[size_t(g.b_buf)].offset) + g.b_off;
+      a.b_n = g.ldb;
+      a.b_k = 1;
+      a.M = g.M;
+      a.N = g.N;
+      a.K = g.K;
+      a.C = (g.c_buf >= 0 ? reinterpret_cast<double*>(ws + dg.bufs[size_t(g.c_buf)].offset) : output(i)) + g.c_off;
+      a.m_dst = g.m_dst;
+      a.n_dst = g.n_dst;
+      a.alpha = g.alpha;
+      a.accumulate = accumulate(i);
+    }
+    return cuda_status(launch_gemm_f64(jobs, n, stream), "gemm_f64");
+  }
+  if (family < 16) {
+    X64GemmArgs jobs[kGroup];
+    for (int i = 0; i < n; ++i) {
+      const GemmStep& g = step(i).g;
+      const Program& dg = diagram(i);
+      const Buffer& ax = dg.bufs[size_t(g.ax_buf)];
+      const Buffer& bx = dg.bufs[size_t(g.bx_buf)];
+      const int64_t row_img = (g.K + 15) / 16 * 32 * kX64Digits;  // image bytes per row
+      X64GemmArgs& a = jobs[i];
+      a.A = ws + ax.offset + g.ax_tile * kX64TileA * row_img;
+      a.ea = reinterpret_cast<const int*>(ws + ax.offset + ax.exp_off) + g.ax_row;
+      a.A64 = reinterpret_cast<const double*>(ws + dg.bufs[size_t(g.a_buf)].offset) + g.a_off;
+      a.lda = g.lda;
+      a.B = ws + bx.offset + g.bx_tile * kX64TileB * row_img;
+      a.eb = reinterpret_cast<const int*>(ws + bx.offset + bx.exp_off) + g.bx_row;
+      a.B64 = reinterpret_cast<const double*>(ws + dg.bufs[size_t(g.b_buf)].offset) + g.b_off;
+      a.ldb = g.ldb;
+      a.M = g.M;
+      a.N = g.N;
+      a.K = g.K;
+      a.C = (g.c_buf >= 0 ? reinterpret_cast<double*>(ws + dg.bufs[size_t(g.c_buf)].offset) : output(i)) + g.c_off;
+      a.m_dst = g.m_dst;
+      a.n_dst = g.n_dst;
+      a.alpha = g.alpha;
+      a.accumulate = accumulate(i);
+      a.split = g.split;
+      if (g.p_buf >= 0) {
+        a.partial = reinterpret_cast<float*>(ws + dg.bufs[size_t(g.p_buf)].offset);
+        a.partial_plane = dg.bufs[size_t(g.p_buf)].plane_bytes / 4;
+      }
+    }
+    return cuda_status(launch_gemm_x64(jobs, n, stream), "gemm_x64");
+  }
+  TcGemmArgs jobs[kGroup];
+  for (int i = 0; i < n; ++i) {
+    jobs[i] = tc_args(step(i).g, diagram(i), prec, ws, output(i));
+    jobs[i].accumulate = accumulate(i);
+  }
+  const cudaError_t e = launch_gemm_tc(jobs, n, stream);
+  if (e == cudaErrorNotSupported) return fail(MERA_EINVAL, "tensor-core GEMM unavailable for prec %d", prec);
+  return cuda_status(e, "gemm_tc");
+}
+
 // Execute a contraction program; inputs[slot] are device pointers.
 // reuse_resident: the u/w operand copies (resident == 1) and the u/w-only
 // products left by the previous run of this same program (same u, w,
 // workspace) are still valid; skip those steps.
 mera_status run_program(const OpProgram& prog, const double* const inputs[4], double* out, int prec, char* ws,
                         cudaStream_t stream, bool reuse_resident = false) {
-  for (const Program& dg : prog.diagrams) {
-    for (const Step& st : dg.steps) {
-      if (st.kind == 0) {
-        const PermuteStep& p = st.p;
-        const Buffer& b = dg.bufs[p.dst_buf];
-        if (p.skip || (reuse_resident && dg.bufs[p.op_buf].resident == 1)) continue;
-        const int64_t plane = b.plane_bytes / buf_elem_bytes(b, prec);
-        ProfScope ps(stream, 1, 0, 0.0);
-        cudaError_t e = launch_permute(p, inputs[p.slot], ws + b.offset, plane, b.raw == 1 ? PREC_RAW : prec, stream);
-        if (e != cudaSuccess) return cuda_status(e, "permute");
-        continue;
-      }
-      if (st.kind == 2) {  // split of a raw buffer into its operand, or of an operand into its digit image
-        const SplitStep& x = st.x;
-        const Buffer& r = dg.bufs[x.raw_buf];
-        const Buffer& d = dg.bufs[x.dst_buf];
-        if (x.skip || (reuse_resident && d.resident == 1)) continue;
-        ProfScope ps(stream, 1, 0, 0.0);
-        if (x.tile > 0) {
-          cudaError_t e = launch_x64_split(reinterpret_cast<const double*>(ws + r.offset), x.ld, x.rows, x.K,
-                                           x.seg_rows, x.tile, ws + d.offset,
-                                           reinterpret_cast<int*>(ws + d.offset + d.exp_off), stream);
-          if (e != cudaSuccess) return cuda_status(e, "digit split");
-          continue;
+  auto kept = [&](const Program& dg, const Step& st) {
+    if (st.kind == 0) return st.p.skip || (reuse_resident && dg.bufs[size_t(st.p.op_buf)].resident == 1);
+    if (st.kind == 2) return st.x.skip || (reuse_resident && dg.bufs[size_t(st.x.dst_buf)].resident == 1);
+    return reuse_resident && st.g.stat != 0;
+  };
+  if (!prog.waves.empty()) {
+    for (const Wave& w : prog.waves) {
+      std::pair<int, int> batch[kGroup];
+      int n = 0;
+      for (size_t i = 0; i <= w.steps.size(); ++i) {
+        if (n == kGroup || (i == w.steps.size() && n > 0)) {
+          const mera_status st = run_steps(prog, batch, n, w.family, inputs, out, prec, ws, stream);
+          if (st != MERA_OK) return st;
+          n = 0;
         }
-        cudaError_t e = launch_oz_split(reinterpret_cast<const float*>(ws + r.offset), r.plane_bytes / 4,
-                                        ws + d.offset, d.plane_bytes / elem_bytes(prec), x.rows, x.K, x.ld,
-                                        planes(prec), stream);
-        if (e != cudaSuccess) return cuda_status(e, "split");
-        continue;
+        if (i == w.steps.size()) break;
+        const Program& dg = prog.diagrams[size_t(w.steps[i].first)];
+        if (!kept(dg, dg.steps[size_t(w.steps[i].second)])) batch[n++] = w.steps[i];
       }
-      const GemmStep& g = st.g;
-      if (reuse_resident && g.stat) continue;  // u/w-only product kept from the previous run
-      const Buffer& a = dg.bufs[g.a_buf];
-      const Buffer& b = dg.bufs[g.b_buf];
-      ProfScope ps(stream, 0, g.dominant, g.flops);
-      if (g.ax_buf >= 0) {
-        const Buffer& ax = dg.bufs[g.ax_buf];
-        const Buffer& bx = dg.bufs[g.bx_buf];
-        const int64_t tile_k = (g.K + 15) / 16 * 32 * kX64Digits;  // image bytes per row of a tile
-        X64GemmArgs args;
-        args.A = ws + ax.offset + g.ax_tile * kX64TileA * tile_k;
-        args.ea = reinterpret_cast<const int*>(ws + ax.offset + ax.exp_off) + g.ax_row;
-        args.A64 = reinterpret_cast<const double*>(ws + a.offset) + g.a_off;
-        args.lda = g.lda;
-        args.B = ws + bx.offset + g.bx_tile * kX64TileB * tile_k;
-        args.eb = reinterpret_cast<const int*>(ws + bx.offset + bx.exp_off) + g.bx_row;
-        args.B64 = reinterpret_cast<const double*>(ws + b.offset) + g.b_off;
-        args.ldb = g.ldb;
-        args.M = g.M;
-        args.N = g.N;
-        args.K = g.K;
-        args.C = (g.c_buf >= 0 ? reinterpret_cast<double*>(ws + dg.bufs[g.c_buf].offset) : out) + g.c_off;
-        args.m_dst = g.m_dst;
-        args.n_dst = g.n_dst;
-        args.alpha = g.alpha;
-        args.accumulate = g.accumulate;
-        args.split = g.split;
-        if (g.p_buf >= 0) {
-          args.partial = reinterpret_cast<float*>(ws + dg.bufs[g.p_buf].offset);
-          args.partial_plane = dg.bufs[g.p_buf].plane_bytes / 4;
-        }
-        cudaError_t e = launch_gemm_x64(args, stream);
-        if (e != cudaSuccess) return cuda_status(e, "gemm_x64");
-      } else if (prec == PREC_F64) {
-        GemmF64Args args;
-        args.A = reinterpret_cast<const double*>(ws + a.offset) + g.a_off;
-        args.a_m = g.lda;
-        args.a_k = 1;
-        args.B = reinterpret_cast<const double*>(ws + b.offset) + g.b_off;
-        args.b_n = g.ldb;
-        args.b_k = 1;
-        args.M = g.M;
-        args.N = g.N;
-        args.K = g.K;
-        args.C = (g.c_buf >= 0 ? reinterpret_cast<double*>(ws + dg.bufs[g.c_buf].offset) : out) + g.c_off;
-        args.m_dst = g.m_dst;
-        args.n_dst = g.n_dst;
-        args.alpha = g.alpha;
-        args.accumulate = g.accumulate;
-        cudaError_t e = launch_gemm_f64(args, stream);
-        if (e != cudaSuccess) return cuda_status(e, "gemm_f64");
-      } else {
-        const TcGemmArgs args = tc_args(g, dg, prec, ws, out);
-        cudaError_t e = launch_gemm_tc(args, stream);
-        if (e == cudaErrorNotSupported) return fail(MERA_EINVAL, "tensor-core GEMM unavailable for prec %d", prec);
-        if (e != cudaSuccess) return cuda_status(e, "gemm_tc");
-      }
+    }
+    if (prog.part_off < 0) return MERA_OK;
+    return cuda_status(launch_ordered_sum(reinterpret_cast<const double*>(ws + prog.part_off), int(prog.diagrams.size()),
+                                          out, prog.part_bytes / 8, stream), "sum of the diagrams");
+  }
+  for (size_t d = 0; d < prog.diagrams.size(); ++d) {
+    const Program& dg = prog.diagrams[d];
+    for (size_t i = 0; i < dg.steps.size(); ++i) {
+      const Step& st = dg.steps[i];
+      if (kept(dg, st)) continue;
+      const std::pair<int, int> one{int(d), int(i)};
+      const mera_status rc = run_steps(prog, &one, 1, family_of(st, prec), inputs, out, prec, ws, stream);
+      if (rc != MERA_OK) return rc;
     }
   }
   return MERA_OK;
@@ -284,13 +346,24 @@ mera_status run_program(const OpProgram& prog, const double* const inputs[4], do
 // Workspace bytes of each composite operation.
 size_t op_bytes(const OpProgram& p) { return align_up(p.ws_bytes); }
 
-// The program that runs in `avail` bytes of workspace: PREC_F64 falls back to
-// the FP64 pipe for every product where the digit images do not fit, so a
-// workspace that was large enough for the operands alone stays accepted.
+// Least of the needs (0 .. kMostLess, get_program) that `avail` bytes hold,
+// need(less) telling each; kMostLess where none does.  So a workspace that is
+// large enough for the operands alone stays accepted.
+constexpr int kMostLess = 2;
+template <typename Need>
+int pick_less(size_t avail, Need need) {
+  int less = 0;
+  while (less < kMostLess && need(less) > avail) ++less;
+  return less;
+}
+
+// The fastest program that runs in `avail` bytes of workspace.
 const OpProgram* pick_program(int op, int chi_b, int chi_t, int prec, size_t avail) {
-  const OpProgram* p = get_program(op, chi_b, chi_t, prec);
-  if (p && p->has_x64 && op_bytes(*p) > avail) p = get_program(op, chi_b, chi_t, prec, true);
-  return p;
+  const int less = pick_less(avail, [&](int l) {
+    const OpProgram* p = get_program(op, chi_b, chi_t, prec, l);
+    return p ? op_bytes(*p) : 0;
+  });
+  return get_program(op, chi_b, chi_t, prec, less);
 }
 
 mera_status map_call(int op, const double* h, const double* rho, const double* u, const double* w, int chi_b,
@@ -318,8 +391,8 @@ using namespace mera;
 extern "C" const char* mera_version(void) { return "mera-gb300 0.1 sm_103a"; }
 extern "C" const char* mera_last_error(void) { return g_err.c_str(); }
 
-// plain: the least workspace that PREC_F64 runs in (pick_program).
-static mera_status ws_size_impl(int op, int chi_b, int chi_t, int prec, size_t* bytes, bool plain = false) {
+// less: get_program's.
+static mera_status ws_size_impl(int op, int chi_b, int chi_t, int prec, size_t* bytes, int less = 0) {
   if (!bytes) return fail(MERA_EINVAL, "null bytes");
   if (!chi_ok(chi_b, chi_t) || !prec_ok(prec)) return fail(MERA_EINVAL, "bad sizes or prec");
   switch (op) {
@@ -327,13 +400,13 @@ static mera_status ws_size_impl(int op, int chi_b, int chi_t, int prec, size_t* 
     case MERA_OP_DESCEND:
     case MERA_OP_ENV_U:
     case MERA_OP_ENV_W: {
-      const OpProgram* p = get_program(op, chi_b, chi_t, prec, plain);
+      const OpProgram* p = get_program(op, chi_b, chi_t, prec, less);
       if (!p) return fail(MERA_EINVAL, "no contraction program");
       *bytes = op_bytes(*p);
       return MERA_OK;
     }
     case MERA_OP_ENERGY: {
-      const OpProgram* p = get_program(OP_ASCEND, chi_b, chi_t, prec, plain);
+      const OpProgram* p = get_program(OP_ASCEND, chi_b, chi_t, prec, less);
       if (!p) return fail(MERA_EINVAL, "no contraction program");
       *bytes = op_bytes(*p) + align_up(ipow(chi_t, 6) * sizeof(double)) + kReduceBytes;
       return MERA_OK;
@@ -342,7 +415,7 @@ static mera_status ws_size_impl(int op, int chi_b, int chi_t, int prec, size_t* 
       // transposes of h and rho, an environment half, then the largest map
       size_t maps = 0;
       for (int op2 : {OP_ASCEND, OP_DESCEND, OP_ENV_U, OP_ENV_W}) {
-        const OpProgram* p = get_program(op2, chi_b, chi_t, prec, plain);
+        const OpProgram* p = get_program(op2, chi_b, chi_t, prec, less);
         if (!p) return fail(MERA_EINVAL, "no contraction program");
         maps = std::max(maps, op_bytes(*p));
       }
@@ -352,7 +425,7 @@ static mera_status ws_size_impl(int op, int chi_b, int chi_t, int prec, size_t* 
     }
     case MERA_OP_FIXED_POINT: {
       if (chi_b != chi_t) return fail(MERA_EINVAL, "fixed point needs chi_b == chi_t");
-      const OpProgram* p = get_program(OP_DESCEND, chi_b, chi_t, prec, plain);
+      const OpProgram* p = get_program(OP_DESCEND, chi_b, chi_t, prec, less);
       if (!p) return fail(MERA_EINVAL, "no contraction program");
       *bytes = op_bytes(*p) + align_up(ipow(chi_t, 6) * sizeof(double)) + kReduceBytes;
       return MERA_OK;
@@ -360,6 +433,18 @@ static mera_status ws_size_impl(int op, int chi_b, int chi_t, int prec, size_t* 
     default:
       return fail(MERA_EINVAL, "unknown op %d", op);
   }
+}
+
+// The least reduced form of `op` that `avail` bytes hold, and what it needs.
+static mera_status fit_workspace(int op, int chi_b, int chi_t, int prec, size_t avail, int* less, size_t* need) {
+  const mera_status st = ws_size_impl(op, chi_b, chi_t, prec, need);
+  if (st != MERA_OK) return st;
+  *less = pick_less(avail, [&](int l) {
+    size_t n = 0;
+    ws_size_impl(op, chi_b, chi_t, prec, &n, l);
+    return n;
+  });
+  return ws_size_impl(op, chi_b, chi_t, prec, need, *less);
 }
 
 extern "C" mera_status mera_workspace_size(int op, int chi_b, int chi_t, int prec, size_t* bytes) {
@@ -391,14 +476,13 @@ extern "C" mera_status mera_env_w(const double* h, const double* rho, const doub
 extern "C" mera_status mera_energy(const double* h, const double* rho, const double* u, const double* w, int chi_b,
                                    int chi_t, double* e_dev, int prec, void* ws, size_t ws_bytes, void* stream) {
   size_t need = 0;
-  mera_status st = ws_size_impl(MERA_OP_ENERGY, chi_b, chi_t, prec, &need);
+  int less = 0;
+  mera_status st = fit_workspace(MERA_OP_ENERGY, chi_b, chi_t, prec, ws_bytes, &less, &need);
   if (st != MERA_OK) return st;
   if (!h || !rho || !u || !w || !e_dev) return fail(MERA_EINVAL, "null pointer");
   if (reinterpret_cast<uintptr_t>(ws) % kAlign) return fail(MERA_EINVAL, "workspace not 256-byte aligned");
-  const bool plain = ws_bytes < need;
-  if (plain) ws_size_impl(MERA_OP_ENERGY, chi_b, chi_t, prec, &need, true);
   if (!ws || ws_bytes < need) return fail(MERA_ENOMEM, "workspace %zu bytes < %zu needed", ws_bytes, need);
-  const OpProgram* prog = get_program(OP_ASCEND, chi_b, chi_t, prec, plain);
+  const OpProgram* prog = get_program(OP_ASCEND, chi_b, chi_t, prec, less);
   Arena ar{static_cast<char*>(ws), ws_bytes};
   char* pws = ar.take(op_bytes(*prog));
   const int64_t n = ipow(chi_t, 3);
@@ -414,20 +498,19 @@ extern "C" mera_status mera_energy(const double* h, const double* rho, const dou
 extern "C" mera_status mera_fixed_point_rho(const double* u, const double* w, int chi, double* rho_inout, int n_iter,
                                             double* resid_dev, int prec, void* ws, size_t ws_bytes, void* stream) {
   size_t need = 0;
-  mera_status st = ws_size_impl(MERA_OP_FIXED_POINT, chi, chi, prec, &need);
+  int less = 0;
+  mera_status st = fit_workspace(MERA_OP_FIXED_POINT, chi, chi, prec, ws_bytes, &less, &need);
   if (st != MERA_OK) return st;
   if (!u || !w || !rho_inout) return fail(MERA_EINVAL, "null pointer");
   if (n_iter < 0) return fail(MERA_EINVAL, "negative n_iter");
   if (reinterpret_cast<uintptr_t>(ws) % kAlign) return fail(MERA_EINVAL, "workspace not 256-byte aligned");
-  const bool plain = ws_bytes < need;
-  if (plain) ws_size_impl(MERA_OP_FIXED_POINT, chi, chi, prec, &need, true);
   if (!ws || ws_bytes < need) return fail(MERA_ENOMEM, "workspace %zu bytes < %zu needed", ws_bytes, need);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (n_iter == 0) {
     if (resid_dev) return cuda_status(cudaMemsetAsync(resid_dev, 0, sizeof(double), s), "memset");
     return MERA_OK;
   }
-  const OpProgram* prog = get_program(OP_DESCEND, chi, chi, prec, plain);
+  const OpProgram* prog = get_program(OP_DESCEND, chi, chi, prec, less);
   Arena ar{static_cast<char*>(ws), ws_bytes};
   char* pws = ar.take(op_bytes(*prog));
   const int64_t n = ipow(chi, 3);
@@ -730,7 +813,7 @@ struct SweepLayout {
 };
 
 mera_status sweep_layout(int n_layers, const int* chi_b, const int* chi_t, int prec, SweepLayout* L,
-                         bool plain = false) {
+                         int less = 0) {
   if (n_layers < 1 || n_layers > MERA_MAX_LAYERS) return fail(MERA_EINVAL, "bad n_layers %d", n_layers);
   for (int t = 0; t < n_layers; ++t) {
     if (!chi_ok(chi_b[t], chi_t[t])) return fail(MERA_EINVAL, "bad dims in layer %d", t);
@@ -745,7 +828,7 @@ mera_status sweep_layout(int n_layers, const int* chi_b, const int* chi_t, int p
     rho_max = std::max(rho_max, size_t(ipow(chi_b[t], 6)));
     env_max = std::max(env_max, size_t(ipow(chi_b[t], 4)));
     for (int op : {OP_ASCEND, OP_DESCEND, OP_ENV_U, OP_ENV_W}) {
-      const OpProgram* p = get_program(op, chi_b[t], chi_t[t], prec, plain);
+      const OpProgram* p = get_program(op, chi_b[t], chi_t[t], prec, less);
       if (!p) return fail(MERA_EINVAL, "no program for layer %d", t);
       map_bytes = std::max(map_bytes, op_bytes(*p));
     }
@@ -753,11 +836,11 @@ mera_status sweep_layout(int n_layers, const int* chi_b, const int* chi_t, int p
     map_bytes = std::max(map_bytes, stiefel_bytes(int(eb), int(eb)));  // >= polar_bytes
     size_t fp = 0;
     if (t == n_layers - 1) {
-      ws_size_impl(MERA_OP_FIXED_POINT, chi_b[t], chi_t[t], prec, &fp, plain);
+      ws_size_impl(MERA_OP_FIXED_POINT, chi_b[t], chi_t[t], prec, &fp, less);
       map_bytes = std::max(map_bytes, fp);
     }
     if (t == 0) {
-      ws_size_impl(MERA_OP_ENERGY, chi_b[t], chi_t[t], prec, &fp, plain);
+      ws_size_impl(MERA_OP_ENERGY, chi_b[t], chi_t[t], prec, &fp, less);
       map_bytes = std::max(map_bytes, fp);
     }
   }
@@ -804,7 +887,8 @@ static mera_status sweep_impl(mera_state* S, const double* h1, double shift, int
   const int n = S->n_layers;
   SweepLayout L;
   mera_status st = sweep_layout(n, S->chi_b, S->chi_t, prec, &L);
-  if (st == MERA_OK && ws_bytes < L.total) st = sweep_layout(n, S->chi_b, S->chi_t, prec, &L, true);
+  for (int less = 1; less <= kMostLess && st == MERA_OK && ws_bytes < L.total; ++less)
+    st = sweep_layout(n, S->chi_b, S->chi_t, prec, &L, less);
   if (st != MERA_OK) return st;
   for (int t = 0; t < n; ++t)
     if (!S->u[t] || !S->w[t]) return fail(MERA_EINVAL, "null tensor in layer %d", t);
@@ -1064,10 +1148,10 @@ extern "C" mera_status mera_gemm_test(int prec, const double* A, const double* B
   if (is_oz(prec)) {
     e = launch_permute(pa_step, A, wra, int64_t(ra / 4), PREC_RAW, s);
     if (e == cudaSuccess) e = launch_permute(pb_step, B, wrb, int64_t(rb / 4), PREC_RAW, s);
-    if (e == cudaSuccess)
-      e = launch_oz_split(reinterpret_cast<const float*>(wra), int64_t(ra / 4), wa, int64_t(pa / eb), M, K, ld, int(np), s);
-    if (e == cudaSuccess)
-      e = launch_oz_split(reinterpret_cast<const float*>(wrb), int64_t(rb / 4), wb, int64_t(pb / eb), N, K, ld, int(np), s);
+    const OzSplitJob jobs[2] = {
+        {reinterpret_cast<const float*>(wra), int64_t(ra / 4), wa, int64_t(pa / eb), M, K, ld},
+        {reinterpret_cast<const float*>(wrb), int64_t(rb / 4), wb, int64_t(pb / eb), N, K, ld}};
+    if (e == cudaSuccess) e = launch_oz_split(jobs, 2, int(np), s);
   } else {
     e = launch_permute(pa_step, A, wa, int64_t(pa / eb), prec, s);
     if (e == cudaSuccess) e = launch_permute(pb_step, B, wb, int64_t(pb / eb), prec, s);
@@ -1088,9 +1172,9 @@ extern "C" mera_status mera_gemm_test(int prec, const double* A, const double* B
     g.split = xsplit;
     g.partial = reinterpret_cast<float*>(eb2 + align_up(size_t(N) * 4) / 4);
     g.partial_plane = int64_t(xsplit) * M * N;
-    e = launch_x64_split(g.A64, ld, M, K, M, kX64TileA, ia, ea, s);
-    if (e == cudaSuccess) e = launch_x64_split(g.B64, ld, N, K, N, kX64TileB, ib, eb2, s);
-    if (e == cudaSuccess) e = launch_gemm_x64(g, s);
+    const X64SplitJob jobs[2] = {{g.A64, ld, M, K, M, kX64TileA, ia, ea}, {g.B64, ld, N, K, N, kX64TileB, ib, eb2}};
+    e = launch_x64_split(jobs, 2, s);
+    if (e == cudaSuccess) e = launch_gemm_x64(&g, 1, s);
     return cuda_status(e, "gemm test x64");
   }
   if (prec == PREC_F64) {
@@ -1115,7 +1199,7 @@ mera_status set_last_error(mera_status st, const char* msg) { return fail(st, "%
 // The least workspace an operation runs in; mera_workspace_size reports what
 // it runs fastest in.
 mera_status least_workspace(int op, int chi_b, int chi_t, int prec, size_t* bytes) {
-  return ws_size_impl(op, chi_b, chi_t, prec, bytes, true);
+  return ws_size_impl(op, chi_b, chi_t, prec, bytes, kMostLess);
 }
 }  // namespace mera
 
@@ -1137,11 +1221,11 @@ extern "C" mera_status mera_energy_adjoint(const double* h, const double* rho, c
                                            double* du, double* dw, int prec, void* ws, size_t ws_bytes,
                                            void* stream) {
   size_t need = 0;
-  mera_status st = ws_size_impl(MERA_OP_ENERGY_ADJOINT, chi_b, chi_t, prec, &need);
+  int less = 0;
+  mera_status st = fit_workspace(MERA_OP_ENERGY_ADJOINT, chi_b, chi_t, prec, ws_bytes, &less, &need);
   if (st != MERA_OK) return st;
   if (!h || !rho || !u || !w || !g_dev) return fail(MERA_EINVAL, "null input pointer");
   if (reinterpret_cast<uintptr_t>(ws) % kAlign) return fail(MERA_EINVAL, "workspace not 256-byte aligned");
-  if (ws_bytes < need) ws_size_impl(MERA_OP_ENERGY_ADJOINT, chi_b, chi_t, prec, &need, true);
   if (!ws || ws_bytes < need) return fail(MERA_ENOMEM, "workspace %zu bytes < %zu needed", ws_bytes, need);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   Arena ar{static_cast<char*>(ws), ws_bytes};
@@ -1256,7 +1340,7 @@ static double sweep_flops(int n, const int* cb, const int* ct, int n_pow) {
 // transitional layer.)
 static mera_status batch_lanes(int n, int n_layers, const int* chi_b, const int* chi_t, int prec, int n_pow,
                                size_t budget_bytes, int max_lanes, int* lane, int* n_lanes, size_t* lane_bytes,
-                               bool plain) {
+                               int less) {
   if (n < 1 || n_layers < 1 || n_layers > MERA_MAX_LAYERS || !chi_b || !chi_t || n_pow < 0 || max_lanes < 1 ||
       !lane || !n_lanes || !lane_bytes)
     return fail(MERA_EINVAL, "bad arguments to mera_batch_lanes");
@@ -1266,7 +1350,7 @@ static mera_status batch_lanes(int n, int n_layers, const int* chi_b, const int*
     const int* cb = chi_b + size_t(i) * size_t(n_layers);
     const int* ct = chi_t + size_t(i) * size_t(n_layers);
     SweepLayout L;
-    const mera_status st = sweep_layout(n_layers, cb, ct, prec, &L, plain);
+    const mera_status st = sweep_layout(n_layers, cb, ct, prec, &L, less);
     if (st != MERA_OK) {
       g_err = "MERA " + std::to_string(i) + ": " + g_err;
       return st;
@@ -1337,11 +1421,11 @@ static mera_status batch_lanes(int n, int n_layers, const int* chi_b, const int*
 extern "C" mera_status mera_batch_lanes(int n, int n_layers, const int* chi_b, const int* chi_t, int prec, int n_pow,
                                         size_t budget_bytes, int max_lanes, int* lane, int* n_lanes,
                                         size_t* lane_bytes) {
-  const mera_status st =
-      batch_lanes(n, n_layers, chi_b, chi_t, prec, n_pow, budget_bytes, max_lanes, lane, n_lanes, lane_bytes, false);
-  // a budget that holds PREC_F64 sweeps only without digit images
-  if (st != MERA_ENOMEM || prec != PREC_F64) return st;
-  return batch_lanes(n, n_layers, chi_b, chi_t, prec, n_pow, budget_bytes, max_lanes, lane, n_lanes, lane_bytes, true);
+  // a budget that holds PREC_F64 sweeps only in a reduced form is accepted
+  mera_status st = MERA_ENOMEM;
+  for (int less = 0; less <= (prec == PREC_F64 ? kMostLess : 0) && st == MERA_ENOMEM; ++less)
+    st = batch_lanes(n, n_layers, chi_b, chi_t, prec, n_pow, budget_bytes, max_lanes, lane, n_lanes, lane_bytes, less);
+  return st;
 }
 
 // Tile-width autotuner: every tensor-core GEMM step of the op's program that
@@ -1353,7 +1437,7 @@ extern "C" mera_status mera_autotune(int op, int chi_b, int chi_t, int prec, dou
   if (!chi_ok(chi_b, chi_t)) return fail(MERA_EINVAL, "bad bond dimensions");
   if (prec == PREC_F64 || !prec_ok(prec)) return fail(MERA_EINVAL, "autotuning needs a tensor-core mode");
   if (op < OP_ASCEND || op > OP_ENV_W) return fail(MERA_EINVAL, "unknown op %d", op);
-  const OpProgram* prog = get_program(op, chi_b, chi_t, prec);
+  const OpProgram* prog = pick_program(op, chi_b, chi_t, prec, ws_bytes);
   if (!prog) return fail(MERA_EINVAL, "no contraction program");
   const size_t out_need = size_t(op == OP_ASCEND ? ipow(chi_t, 6)
                                  : op == OP_DESCEND ? ipow(chi_b, 6)

@@ -18,23 +18,49 @@ inline void count_launch(long long n = 1) { g_launch_count.fetch_add(n, std::mem
 // per-context caches: a device reset makes a new context).
 void* current_cu_context();
 
+// Several independent jobs of one kind go out in one launch (at most kGroup;
+// launchers split longer lists).  At small bond dimensions a launch costs as
+// much as its work, and one job seldom fills the GPU.
+constexpr int kGroup = 6;
+
 // Input tensor -> operand layout, cast to the operand precision (in the
 // fixed-point split modes: to the raw hi + lo binary32 planes).
-cudaError_t launch_permute(const PermuteStep& p, const double* src, void* dst, int64_t plane_elems,
-                           int prec, cudaStream_t stream);
+struct PermuteJob {
+  const PermuteStep* step = nullptr;
+  const double* src = nullptr;
+  void* dst = nullptr;
+  int64_t plane = 0;  // elements between planes
+};
+cudaError_t launch_permute(const PermuteJob* jobs, int n, int prec, cudaStream_t stream);
+inline cudaError_t launch_permute(const PermuteStep& p, const double* src, void* dst, int64_t plane_elems, int prec,
+                                  cudaStream_t stream) {
+  const PermuteJob j{&p, src, dst, plane_elems};
+  return launch_permute(&j, 1, prec, stream);
+}
 
 // Fixed-point split modes: raw hi + lo binary32 planes (rows x ld, the lo
 // plane raw_plane floats after the hi plane) -> `slices` BF16 planes of the
 // operand (dst_plane elements apart), one exponent per row and block of
 // kOzBlockK elements along K.  Columns K..ld-1 are not touched.
-cudaError_t launch_oz_split(const float* raw, int64_t raw_plane, void* dst, int64_t dst_plane, int64_t rows,
-                            int64_t K, int64_t ld, int slices, cudaStream_t stream);
+struct OzSplitJob {
+  const float* raw = nullptr;
+  int64_t raw_plane = 0;
+  void* dst = nullptr;
+  int64_t dst_plane = 0, rows = 0, K = 0, ld = 0;
+};
+cudaError_t launch_oz_split(const OzSplitJob* jobs, int n, int slices, cudaStream_t stream);
 
 // Binary64 operand (rows x K, pitch ld, a multiple of 8) -> digit image of
 // x64_gemm_kernel in tiles of `tile` rows, and one exponent per row.  Rows
 // come in segments of seg_rows, each padded to whole tiles.
-cudaError_t launch_x64_split(const double* src, int64_t ld, int64_t rows, int64_t K, int64_t seg_rows, int tile,
-                             void* img, int* rowexp, cudaStream_t stream);
+struct X64SplitJob {
+  const double* src = nullptr;
+  int64_t ld = 0, rows = 0, K = 0, seg_rows = 0;
+  int tile = 0;
+  void* img = nullptr;
+  int* rowexp = nullptr;
+};
+cudaError_t launch_x64_split(const X64SplitJob* jobs, int n, cudaStream_t stream);
 
 // FP64 GEMM with a scattered epilogue:
 //   C[m_dst(m) + n_dst(n)] (+)= alpha * sum_k A[m*a_m + k*a_k] * B[n*b_n + k*b_k]
@@ -50,7 +76,14 @@ struct GemmF64Args {
   int accumulate;
   const int* skip_if = nullptr;  // device flag: the kernel returns at once when *skip_if != 0
 };
-cudaError_t launch_gemm_f64(const GemmF64Args& args, cudaStream_t stream);
+cudaError_t launch_gemm_f64(const GemmF64Args* args, int n, cudaStream_t stream);
+inline cudaError_t launch_gemm_f64(const GemmF64Args& args, cudaStream_t stream) {
+  return launch_gemm_f64(&args, 1, stream);
+}
+
+// out = parts[0] + parts[1] + ... in that order, `count` elements each, the
+// parts one after another.
+cudaError_t launch_ordered_sum(const double* parts, int n, double* out, int64_t count, cudaStream_t stream);
 
 // Number of per-block partial sums the reduction kernels below may write.
 constexpr int kMaxPartials = 65536;

@@ -47,25 +47,51 @@ __device__ __forceinline__ void decode_other(const PermuteArgs& p, uint32_t o, i
   }
 }
 
-template <int PREC>
-__global__ void __launch_bounds__(256) permute_tile_kernel(const double* __restrict__ src, void* dst, int64_t plane,
-                                                           const __grid_constant__ PermuteArgs p) {
+struct PermuteJobArgs {
+  const double* src;
+  void* dst;
+  int64_t plane;
+  PermuteArgs p;
+};
+template <int G>
+struct PermuteGroup {
+  int n;
+  int64_t end[G];  // tiles of the jobs up to and including each
+  PermuteJobArgs job[G];
+};
+
+// Tiles of every job one after another; a block reloads its offset tables
+// when its next tile belongs to another job.
+template <int PREC, int G>
+__global__ void __launch_bounds__(256) permute_tile_kernel(const __grid_constant__ PermuteGroup<G> g) {
   __shared__ double tile[kTile * (kTile + 1)];
   __shared__ int64_t s_as[kTile], s_ad[kTile], s_bs[kTile], s_bd[kTile];
   const int tid = threadIdx.x;
-  const int ta = p.ta, tb = p.tb, count = ta * tb;
-  if (tid < kTile) {
-    s_as[tid] = tid < ta ? p.a_src[tid] : 0;
-    s_ad[tid] = tid < ta ? p.a_dst[tid] : 0;
-    s_bs[tid] = tid < tb ? p.b_src[tid] : 0;
-    s_bd[tid] = tid < tb ? p.b_dst[tid] : 0;
-  }
-  __syncthreads();
-  // x / d for x < 2^13 by a float reciprocal: (x + 0.5) / d is at least
-  // 0.5 / d away from an integer, far more than the float rounding error
-  const float inv_ta = 1.0f / float(ta), inv_tb = 1.0f / float(tb);
-  const int pitch = tb + 1;  // tile[ia * pitch + ib]
-  for (int64_t t = blockIdx.x; t < p.outer; t += gridDim.x) {
+  int cur = -1;
+  const int64_t total = g.end[g.n - 1];
+  for (int64_t tg = blockIdx.x; tg < total; tg += gridDim.x) {
+    int i = 0;
+    while (tg >= g.end[i]) ++i;
+    const int64_t t = tg - (i > 0 ? g.end[i - 1] : 0);
+    const PermuteArgs& p = g.job[i].p;
+    const double* __restrict__ src = g.job[i].src;
+    void* dst = g.job[i].dst;
+    const int64_t plane = g.job[i].plane;
+    const int ta = p.ta, tb = p.tb, count = ta * tb;
+    if (i != cur) {
+      cur = i;
+      if (tid < kTile) {
+        s_as[tid] = tid < ta ? p.a_src[tid] : 0;
+        s_ad[tid] = tid < ta ? p.a_dst[tid] : 0;
+        s_bs[tid] = tid < tb ? p.b_src[tid] : 0;
+        s_bd[tid] = tid < tb ? p.b_dst[tid] : 0;
+      }
+      __syncthreads();
+    }
+    // x / d for x < 2^13 by a float reciprocal: (x + 0.5) / d is at least
+    // 0.5 / d away from an integer, far more than the float rounding error
+    const float inv_ta = 1.0f / float(ta), inv_tb = 1.0f / float(tb);
+    const int pitch = tb + 1;  // tile[ia * pitch + ib]
     int64_t so, dof;
     decode_other(p, uint32_t(t), so, dof);
     // reads: 8 independent loads per thread in flight before any shared store
@@ -156,9 +182,10 @@ int fill_table(const std::vector<Leg>& g, int64_t* src_off, int64_t* dst_off) {
 
 }  // namespace
 
-cudaError_t launch_permute(const PermuteStep& st, const double* src, void* dst, int64_t plane_elems,
-                           int prec, cudaStream_t stream) {
-  if (st.rows <= 0 || st.cols <= 0) return cudaSuccess;
+namespace {
+
+// Tile description of one copy; false where its tile indices exceed 32 bits.
+bool permute_args(const PermuteStep& st, PermuteArgs& p) {
   // Every leg with its source and destination strides (size-1 legs dropped).
   std::vector<Leg> pool;
   int64_t acc = st.ld;
@@ -174,7 +201,7 @@ cudaError_t launch_permute(const PermuteStep& st, const double* src, void* dst, 
   // Ls: the leg contiguous in the source, Ld: the one contiguous in the
   // destination.  When they differ, Ls is kept out of A so that it leads B;
   // when they coincide, A leads with it and the reads run along A.
-  PermuteArgs p{};
+  p = PermuteArgs{};
   std::vector<Leg> ga, gb;
   if (!pool.empty()) {
     size_t is = 0, id = 0;
@@ -196,7 +223,7 @@ cudaError_t launch_permute(const PermuteStep& st, const double* src, void* dst, 
   }
   p.ta = fill_table(ga, p.a_src, p.a_dst);
   p.tb = fill_table(gb, p.b_src, p.b_dst);
-  if (int(pool.size()) > 2 * kMaxLeg) return cudaErrorInvalidValue;
+  if (int(pool.size()) > 2 * kMaxLeg) return false;
   p.outer = 1;
   p.n_other = 0;
   for (const Leg& l : pool) {  // outer legs (order is irrelevant for correctness)
@@ -206,10 +233,28 @@ cudaError_t launch_permute(const PermuteStep& st, const double* src, void* dst, 
     p.outer *= l.dim;
     ++p.n_other;
   }
-  if (p.outer >= (int64_t(1) << 31)) return cudaErrorInvalidValue;  // 32-bit tile indices
+  return p.outer < (int64_t(1) << 31);
+}
+
+template <int G>
+cudaError_t launch_permute_group(const PermuteJob* jobs, int n, int prec, cudaStream_t stream) {
+  static thread_local PermuteGroup<G> g;  // up to 15 KB
+  g.n = 0;
+  int64_t total = 0;
+  for (int i = 0; i < n; ++i) {
+    if (jobs[i].step->rows <= 0 || jobs[i].step->cols <= 0) continue;
+    PermuteJobArgs& a = g.job[g.n];
+    if (!permute_args(*jobs[i].step, a.p)) return cudaErrorInvalidValue;
+    a.src = jobs[i].src;
+    a.dst = jobs[i].dst;
+    a.plane = jobs[i].plane;
+    total += a.p.outer;
+    g.end[g.n++] = total;
+  }
+  if (g.n == 0) return cudaSuccess;
   count_launch();
-  const unsigned grid = unsigned(std::max<int64_t>(1, std::min<int64_t>(p.outer, 152 * 8)));
-#define MERA_PERMUTE_LAUNCH(P) permute_tile_kernel<P><<<grid, 256, 0, stream>>>(src, dst, plane_elems, p);
+  const unsigned grid = unsigned(std::max<int64_t>(1, std::min<int64_t>(total, 152 * 8)));
+#define MERA_PERMUTE_LAUNCH(P) permute_tile_kernel<P, G><<<grid, 256, 0, stream>>>(g);
   switch (prec) {
     case PREC_F64: MERA_PERMUTE_LAUNCH(PREC_F64) break;
     case PREC_TF32: MERA_PERMUTE_LAUNCH(PREC_TF32) break;
@@ -225,26 +270,121 @@ cudaError_t launch_permute(const PermuteStep& st, const double* src, void* dst, 
   return cudaGetLastError();
 }
 
+}  // namespace
+
+cudaError_t launch_permute(const PermuteJob* jobs, int n, int prec, cudaStream_t stream) {
+  for (int i = 0; i < n; i += kGroup) {
+    const int m = std::min(kGroup, n - i);
+    const cudaError_t e = m == 1 ? launch_permute_group<1>(jobs + i, m, prec, stream)
+                                 : launch_permute_group<kGroup>(jobs + i, m, prec, stream);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 // ---------------------------------------------------------------------------
 // FP64 GEMM.  (16 T) x (16 T) tile per block of 256 threads, T x T outputs per
 // thread at stride 16 (conflict-free shared-memory reads), K in steps of 16.
 // T = 4 for large problems; T = 2 or 1 when the tile count would leave most
-// of the 152 SMs idle (the small square products of the polar iteration).
+// of the 152 SMs idle (the small square products of the polar iteration), and
+// gemm_f64_small_kernel below that.
 // ---------------------------------------------------------------------------
 constexpr int kBK = 16;
 
+struct GemmF64Group {
+  int n;
+  int end[kGroup];  // blocks of the jobs up to and including each
+  GemmF64Args job[kGroup];
+};
+
+// Job of a block, and the block's index within it.
+__device__ __forceinline__ int job_of(const int* end, int b, int& local) {
+  int i = 0;
+  while (b >= end[i]) ++i;
+  local = b - (i > 0 ? end[i - 1] : 0);
+  return i;
+}
+
+// 8 x 8 tile per block of 256 threads, four threads per output, each with a
+// quarter of every 64-wide stage of K; their sums meet in a fixed order.
+// Products of this size are bound by latency and by the FP64 pipe of the SMs
+// they reach (two FMAs per clock): small tiles reach more of them, one stage
+// covers K <= 64 with one round trip to memory, and the next stage is in
+// flight while this one is summed.  256 x 64 x 64: 6.0 us with 16 x 16 tiles.
+__global__ void __launch_bounds__(256) gemm_f64_small_kernel(const __grid_constant__ GemmF64Group g) {
+  constexpr int R = 8, KS = 64, P = KS + 2;
+  __shared__ double As[R * P], Bs[R * P];
+  __shared__ double part[3][R * R];
+  int tile;
+  const GemmF64Args& p = g.job[job_of(g.end, int(blockIdx.x), tile)];
+  if (p.skip_if && *p.skip_if) return;
+  const int tid = threadIdx.x;
+  const int tiles_n = int((p.N + R - 1) / R);
+  const int64_t m0 = int64_t(tile / tiles_n) * R, n0 = int64_t(tile % tiles_n) * R;
+  // two elements of each operand per thread and stage, along its unit stride
+  int ra[2], ka[2], rb[2], kb[2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int e = tid + 256 * i;
+    if (p.a_k == 1) { ra[i] = e / KS; ka[i] = e % KS; } else { ra[i] = e % R; ka[i] = e / R; }
+    if (p.b_k == 1) { rb[i] = e / KS; kb[i] = e % KS; } else { rb[i] = e % R; kb[i] = e / R; }
+  }
+  double va[2], vb[2];
+  auto load = [&](int64_t k0) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int64_t gm = m0 + ra[i], ga = k0 + ka[i], gn = n0 + rb[i], gb = k0 + kb[i];
+      va[i] = (gm < p.M && ga < p.K) ? p.A[gm * p.a_m + ga * p.a_k] : 0.0;
+      vb[i] = (gn < p.N && gb < p.K) ? p.B[gn * p.b_n + gb * p.b_k] : 0.0;
+    }
+  };
+  const int o = tid % (R * R), q = tid / (R * R);  // output, quarter of K
+  const int r = o / R, c = o % R;
+  double acc = 0.0;
+  load(0);
+  for (int64_t k0 = 0; k0 < p.K; k0 += KS) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      As[ra[i] * P + ka[i]] = va[i];
+      Bs[rb[i] * P + kb[i]] = vb[i];
+    }
+    __syncthreads();
+    if (k0 + KS < p.K) load(k0 + KS);
+    const int left = int(min(int64_t(KS), p.K - k0));
+    const int lo = q * (KS / 4), hi = min(left, lo + KS / 4);
+    if (hi - lo == KS / 4) {
+#pragma unroll
+      for (int k = 0; k < KS / 4; ++k) acc = fma(As[r * P + lo + k], Bs[c * P + lo + k], acc);
+    } else {
+      for (int k = lo; k < hi; ++k) acc = fma(As[r * P + k], Bs[c * P + k], acc);
+    }
+    __syncthreads();
+  }
+  if (q > 0) part[q - 1][o] = acc;
+  __syncthreads();
+  if (q > 0 || m0 + r >= p.M || n0 + c >= p.N) return;
+  const double v = p.alpha * (((acc + part[0][o]) + part[1][o]) + part[2][o]);
+  double* dst = p.C + legmap_offset32(p.m_dst, uint32_t(m0 + r)) + legmap_offset32(p.n_dst, uint32_t(n0 + c));
+  *dst = p.accumulate ? (*dst + v) : v;
+}
+
 template <int T>
-__global__ void __launch_bounds__(256) gemm_f64_kernel(const __grid_constant__ GemmF64Args p) {
+__global__ void __launch_bounds__(256) gemm_f64_kernel(const __grid_constant__ GemmF64Group g) {
   constexpr int R = 16 * T;
   __shared__ double As[kBK][R + 1];
   __shared__ double Bs[kBK][R + 1];
   __shared__ int64_t offm[R];
   __shared__ int64_t offn[R];
+  int tile;
+  const GemmF64Args& p = g.job[job_of(g.end, int(blockIdx.x), tile)];
   if (p.skip_if && *p.skip_if) return;
 
+  // the K loop's operands in registers: the job's index is not a constant
+  const double* __restrict__ const pa = p.A;
+  const double* __restrict__ const pb = p.B;
+  const int64_t a_m = p.a_m, a_k = p.a_k, b_n = p.b_n, b_k = p.b_k, M = p.M, N = p.N, K = p.K;
   const int tid = threadIdx.x;
-  const int64_t tiles_n = (p.N + R - 1) / R;
-  const int64_t tile = blockIdx.x;
+  const int64_t tiles_n = (N + R - 1) / R;
   const int64_t m0 = (tile / tiles_n) * R;
   const int64_t n0 = (tile % tiles_n) * R;
   const int tx = tid % 16, ty = tid / 16;
@@ -255,10 +395,10 @@ __global__ void __launch_bounds__(256) gemm_f64_kernel(const __grid_constant__ G
 #pragma unroll
     for (int j = 0; j < T; ++j) acc[i][j] = 0.0;
 
-  const bool a_kfast = (p.a_k == 1);
-  const bool b_kfast = (p.b_k == 1);
+  const bool a_kfast = (a_k == 1);
+  const bool b_kfast = (b_k == 1);
 
-  for (int64_t k0 = 0; k0 < p.K; k0 += kBK) {
+  for (int64_t k0 = 0; k0 < K; k0 += kBK) {
     // R rows x 16 k per operand, T elements per thread, along the unit stride.
 #pragma unroll
     for (int i = 0; i < T; ++i) {
@@ -271,7 +411,7 @@ __global__ void __launch_bounds__(256) gemm_f64_kernel(const __grid_constant__ G
         k = tid / R + (256 / R) * i;
       }
       const int64_t gm = m0 + r, gk = k0 + k;
-      As[k][r] = (gm < p.M && gk < p.K) ? p.A[gm * p.a_m + gk * p.a_k] : 0.0;
+      As[k][r] = (gm < M && gk < K) ? pa[gm * a_m + gk * a_k] : 0.0;
     }
 #pragma unroll
     for (int i = 0; i < T; ++i) {
@@ -284,7 +424,7 @@ __global__ void __launch_bounds__(256) gemm_f64_kernel(const __grid_constant__ G
         k = tid / R + (256 / R) * i;
       }
       const int64_t gn = n0 + r, gk = k0 + k;
-      Bs[k][r] = (gn < p.N && gk < p.K) ? p.B[gn * p.b_n + gk * p.b_k] : 0.0;
+      Bs[k][r] = (gn < N && gk < K) ? pb[gn * b_n + gk * b_k] : 0.0;
     }
     __syncthreads();
 #pragma unroll
@@ -327,20 +467,60 @@ __global__ void __launch_bounds__(256) gemm_f64_kernel(const __grid_constant__ G
   }
 }
 
-cudaError_t launch_gemm_f64(const GemmF64Args& args, cudaStream_t stream) {
-  if (args.M <= 0 || args.N <= 0) return cudaSuccess;
-  if (args.M > 0x7fffffff || args.N > 0x7fffffff) return cudaErrorInvalidValue;  // 32-bit row/column decode
-  auto tiles = [&](int64_t r) { return ((args.M + r - 1) / r) * ((args.N + r - 1) / r); };
-  constexpr int64_t kFill = 2 * 152;  // enough blocks to occupy every SM twice
-  count_launch();
-  if (tiles(64) >= kFill || tiles(32) > 0x7fffffff) {
-    if (tiles(64) > 0x7fffffff) return cudaErrorInvalidValue;
-    gemm_f64_kernel<4><<<unsigned(tiles(64)), 256, 0, stream>>>(args);
-  } else if (tiles(32) >= kFill) {
-    gemm_f64_kernel<2><<<unsigned(tiles(32)), 256, 0, stream>>>(args);
-  } else {
-    gemm_f64_kernel<1><<<unsigned(tiles(16)), 256, 0, stream>>>(args);
+static cudaError_t launch_gemm_f64_group(const GemmF64Args* args, int n, cudaStream_t stream) {
+  GemmF64Group g;
+  g.n = 0;
+  for (int i = 0; i < n; ++i) {
+    if (args[i].M <= 0 || args[i].N <= 0) continue;
+    if (args[i].M > 0x7fffffff || args[i].N > 0x7fffffff) return cudaErrorInvalidValue;  // 32-bit row/column decode
+    g.job[g.n++] = args[i];
   }
+  if (g.n == 0) return cudaSuccess;
+  auto blocks = [&](int64_t r) {
+    int64_t t = 0;
+    for (int i = 0; i < g.n; ++i) {
+      t += ((g.job[i].M + r - 1) / r) * ((g.job[i].N + r - 1) / r);
+      g.end[i] = int(std::min<int64_t>(t, 0x7fffffff));
+    }
+    return t;
+  };
+  constexpr int64_t kFill = 2 * 152;  // enough blocks to occupy every SM twice
+  int64_t r = 8;
+  for (int64_t q : {64, 32, 16})
+    if (r == 8 && (blocks(q) >= kFill || blocks(q / 2) > 0x7fffffff)) r = q;
+  const int64_t nb = blocks(r);
+  if (nb > 0x7fffffff) return cudaErrorInvalidValue;
+  count_launch();
+  switch (r) {
+    case 64: gemm_f64_kernel<4><<<unsigned(nb), 256, 0, stream>>>(g); break;
+    case 32: gemm_f64_kernel<2><<<unsigned(nb), 256, 0, stream>>>(g); break;
+    case 16: gemm_f64_kernel<1><<<unsigned(nb), 256, 0, stream>>>(g); break;
+    default: gemm_f64_small_kernel<<<unsigned(nb), 256, 0, stream>>>(g); break;
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_gemm_f64(const GemmF64Args* args, int n, cudaStream_t stream) {
+  for (int i = 0; i < n; i += kGroup) {
+    const cudaError_t e = launch_gemm_f64_group(args + i, std::min(kGroup, n - i), stream);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+__global__ void __launch_bounds__(256) ordered_sum_kernel(const double* __restrict__ parts, int n,
+                                                          double* __restrict__ out, int64_t count) {
+  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < count; i += int64_t(gridDim.x) * blockDim.x) {
+    double v = parts[i];
+    for (int k = 1; k < n; ++k) v += parts[k * count + i];
+    out[i] = v;
+  }
+}
+
+cudaError_t launch_ordered_sum(const double* parts, int n, double* out, int64_t count, cudaStream_t stream) {
+  if (count <= 0) return cudaSuccess;
+  count_launch();
+  ordered_sum_kernel<<<unsigned(std::min<int64_t>((count + 255) / 256, 152 * 8)), 256, 0, stream>>>(parts, n, out, count);
   return cudaGetLastError();
 }
 

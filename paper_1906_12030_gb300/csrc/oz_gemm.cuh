@@ -86,7 +86,7 @@ __device__ __forceinline__ void dd_norm(float& hi, float& lo) {
 
 template <int S, int BN>
 __global__ void __launch_bounds__(kOzThreads, 1)
-    oz_gemm_kernel(const __grid_constant__ TMaps tm, const __grid_constant__ Epilogue ep) {
+    oz_gemm_kernel(const __grid_constant__ TcGroup g) {
   using C = OzCfg<S, BN>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -104,10 +104,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   int* off_n32 = reinterpret_cast<int*>(off_n + BN);
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int64_t tiles_n = (ep.N + BN - 1) / BN;
-  const int64_t tiles_mn = ((ep.M + kBM - 1) / kBM) * tiles_n;
-  const int64_t tiles = tiles_mn * ep.split;
-  const int num_k = int((ep.K + C::kBK - 1) / C::kBK);  // stages over all of K
+  const int items = g.end[g.n - 1];
   // a work item covers stages [kb0, kb1): kc is a whole number of blocks
 
   if (threadIdx.x == 0) {
@@ -140,11 +137,16 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       // ---- producer: S planes of A and of B per stage ----------------------
       uint32_t it = 0;
       bool alive = true;
-      for (int64_t t = blockIdx.x; t < tiles && alive; t += gridDim.x) {
-        int64_t row_t, col_t;
-        tile_of(t % tiles_mn, tiles_mn / tiles_n, tiles_n, ep.group_m, row_t, col_t);
-        const int m0 = int(row_t * kBM), n0 = int(col_t * BN);
-        const int kb0 = int(t / tiles_mn) * ep.kc, kb1 = min(kb0 + ep.kc, num_k);
+      for (int tg = int(blockIdx.x); tg < items && alive; tg += gridDim.x) {
+        int t;
+        const int job = item_of(g.end, tg, t);
+        const Epilogue& ep = g.ep[job];
+        const TMaps& tm = g.tm[job];
+        const int num_k = (int(ep.K) + C::kBK - 1) / C::kBK;
+        const int kb0 = split_of(t, ep.tiles_m * ep.tiles_n, ep.split) * ep.kc, kb1 = min(kb0 + ep.kc, num_k);
+        int row_t, col_t;
+        tile_of(t, ep.tiles_m, ep.tiles_n, ep.group_m, row_t, col_t);
+        const int m0 = row_t * kBM, n0 = col_t * BN;
         for (int kb = kb0; kb < kb1; ++kb, ++it) {
           const uint32_t s = it % C::kStages;
           if (it >= uint32_t(C::kStages) && !mbar_wait(&empty[s], ((it / C::kStages) & 1) ^ 1, abort_flag)) {
@@ -175,8 +177,12 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       constexpr uint32_t kBBase = uint32_t(S * C::kABytes);
       uint32_t it = 0, bc = 0;  // stages consumed, blocks issued
       bool alive = true;
-      for (int64_t t = blockIdx.x; t < tiles && alive; t += gridDim.x) {
-        const int kb0 = int(t / tiles_mn) * ep.kc, kb1 = min(kb0 + ep.kc, num_k);
+      for (int tg = int(blockIdx.x); tg < items && alive; tg += gridDim.x) {
+        int t;
+        const int job = item_of(g.end, tg, t);
+        const Epilogue& ep = g.ep[job];
+        const int num_k = (int(ep.K) + C::kBK - 1) / C::kBK;
+        const int kb0 = split_of(t, ep.tiles_m * ep.tiles_n, ep.split) * ep.kc, kb1 = min(kb0 + ep.kc, num_k);
         for (int blk = kb0; blk < kb1 && alive; blk += C::kBlockStages, ++bc) {
           const uint32_t b = bc & 1;
           if (bc >= 2 && !mbar_wait(&acc_empty[b], ((bc >> 1) - 1) & 1, abort_flag)) {
@@ -228,26 +234,28 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     const int row = quarter * 32 + lane;
     const bool active = sub < C::kActiveSubs;
     const int c0 = sub * C::kCols;  // first column of this warp's share
-    const bool final_fast = ep.c_final && ep.split <= 1 && ep.off32 && ep.alpha_pow2;
-    const bool raw_fast = !ep.c_final && ep.split <= 1 && ep.off32 && ep.alpha == 1.0;
     uint32_t bc = 0;
-    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-      const int64_t ks = t / tiles_mn;
-      int64_t row_t, col_t;
-      tile_of(t % tiles_mn, tiles_mn / tiles_n, tiles_n, ep.group_m, row_t, col_t);
-      const int64_t m0 = row_t * kBM, n0 = col_t * BN;
-      const int kb0 = int(ks) * ep.kc, kb1 = min(kb0 + ep.kc, num_k);
+    for (int tg = int(blockIdx.x); tg < items; tg += gridDim.x) {
+      int t;
+      const int job = item_of(g.end, tg, t);
+      const Epilogue& ep = g.ep[job];
+      const int num_k = (int(ep.K) + C::kBK - 1) / C::kBK;
+      const int ks = split_of(t, ep.tiles_m * ep.tiles_n, ep.split);
+      int row_t, col_t;
+      tile_of(t, ep.tiles_m, ep.tiles_n, ep.group_m, row_t, col_t);
+      const uint32_t n0 = uint32_t(col_t) * BN;
+      const uint32_t m = uint32_t(row_t) * kBM + row;
+      const int kb0 = ks * ep.kc, kb1 = min(kb0 + ep.kc, num_k);
       asm volatile("bar.sync 1, %0;" ::"n"(kOzEpiThreads) : "memory");
       if (et == 0) *abort_snapshot = *abort_flag;
       for (int c = et; c < BN; c += kOzEpiThreads) {
-        const int64_t n = n0 + c;
+        const uint32_t n = n0 + c;
         const int64_t o = n < ep.N ? legmap_offset32(ep.n_dst, uint32_t(n)) : 0;
         off_n[c] = o;
         off_n32[c] = int(o);
       }
       asm volatile("bar.sync 1, %0;" ::"n"(kOzEpiThreads) : "memory");
       if (*abort_snapshot) break;
-      const int64_t m = m0 + row;
       const bool row_ok = m < ep.M;
       float hi[C::kCols], lo[C::kCols];
 #pragma unroll
@@ -280,7 +288,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 #pragma unroll
       for (int j = 0; j < C::kCols; ++j) dd_norm(hi[j], lo[j]);
       if (ep.split > 1) {  // partial pair, summed by oz_splitk_reduce_kernel
-        float* p = ep.partial + (ks * ep.N + n0 + c0) * ep.M + m;
+        float* p = ep.partial + (int64_t(ks) * ep.N + n0 + c0) * ep.M + m;
 #pragma unroll
         for (int j = 0; j < C::kCols; ++j, p += ep.M)
           if (n0 + c0 + j < ep.N) {
@@ -290,32 +298,47 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         continue;
       }
       const int64_t off_m = legmap_offset32(ep.m_dst, uint32_t(m));
-      const bool whole = n0 + c0 + C::kCols <= ep.N;
-      if (ep.c_final) {
-        double* __restrict__ r = static_cast<double*>(ep.C) + off_m;
-#pragma unroll
-        for (int j = 0; j < C::kCols; ++j) {
-          if (!whole && n0 + c0 + j >= ep.N) continue;
-          const int64_t o = final_fast ? int64_t(off_n32[c0 + j]) : off_n[c0 + j];
-          const double x = final_fast ? f32_to_f64_pow2(hi[j], ep.alpha_exp) + f32_to_f64_pow2(lo[j], ep.alpha_exp)
-                                      : ep.alpha * (double(hi[j]) + double(lo[j]));
-          r[o] = ep.accumulate ? r[o] + x : x;
-        }
-      } else {
+      const bool fast = ep.off32 && n0 + c0 + C::kCols <= ep.N;  // whole columns, 32-bit column offsets
+      if (fast && !ep.c_final && ep.alpha == 1.0) {
+        // the next operand's raw pair; four offsets in registers before the stores
         float* __restrict__ r0 = static_cast<float*>(ep.C) + off_m;
         float* __restrict__ r1 = r0 + ep.c_plane;
-        const float alpha = float(ep.alpha);
+#pragma unroll
+        for (int j = 0; j < C::kCols; j += 4) {
+          const int4 q = *reinterpret_cast<const int4*>(off_n32 + c0 + j);
+          const int o[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            r0[o[k]] = hi[j + k];
+            r1[o[k]] = lo[j + k];
+          }
+        }
+        continue;
+      }
+      if (fast && ep.c_final && ep.alpha_pow2) {
+        double* __restrict__ r = static_cast<double*>(ep.C) + off_m;
+        const int ae = ep.alpha_exp, accumulate = ep.accumulate;
 #pragma unroll
         for (int j = 0; j < C::kCols; ++j) {
-          if (!whole && n0 + c0 + j >= ep.N) continue;
-          const int64_t o = raw_fast ? int64_t(off_n32[c0 + j]) : off_n[c0 + j];
-          if (raw_fast) {
-            r0[o] = hi[j];
-            r1[o] = lo[j];
-          } else {  // alpha a power of two in the programs: exact
-            r0[o] = __fmul_rn(alpha, hi[j]);
-            r1[o] = __fmul_rn(alpha, lo[j]);
-          }
+          const int o = off_n32[c0 + j];
+          const double x = f32_to_f64_pow2(hi[j], ae) + f32_to_f64_pow2(lo[j], ae);
+          r[o] = accumulate ? r[o] + x : x;
+        }
+        continue;
+      }
+#pragma unroll
+      for (int j = 0; j < C::kCols; ++j) {
+        if (n0 + c0 + j >= ep.N) continue;
+        const int64_t o = off_m + off_n[c0 + j];
+        if (ep.c_final) {
+          double* r = static_cast<double*>(ep.C) + o;
+          const double x = ep.alpha_pow2 ? f32_to_f64_pow2(hi[j], ep.alpha_exp) + f32_to_f64_pow2(lo[j], ep.alpha_exp)
+                                         : ep.alpha * (double(hi[j]) + double(lo[j]));
+          *r = ep.accumulate ? *r + x : x;
+        } else {  // alpha a power of two in the programs: exact
+          const float alpha = float(ep.alpha);
+          static_cast<float*>(ep.C)[o] = __fmul_rn(alpha, hi[j]);
+          static_cast<float*>(ep.C)[o + ep.c_plane] = __fmul_rn(alpha, lo[j]);
         }
       }
     }
@@ -332,7 +355,8 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 // Sum of the K-split partial pairs in a fixed order (double-float), then the
 // same output as the GEMM epilogue.  One thread per row m over a chunk of
 // columns.
-__global__ void __launch_bounds__(256) oz_splitk_reduce_kernel(const __grid_constant__ Epilogue ep) {
+__global__ void __launch_bounds__(256) oz_splitk_reduce_kernel(const __grid_constant__ TcGroup g) {
+  const Epilogue& ep = g.ep[blockIdx.z];
   const int64_t m = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (m >= ep.M) return;
   const int64_t off_m = legmap_offset32(ep.m_dst, uint32_t(m));

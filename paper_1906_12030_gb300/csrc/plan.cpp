@@ -345,6 +345,7 @@ struct Builder {
   std::vector<int64_t> img_seg; // and rows per segment
   std::vector<char> x64;        // the node's product runs on the tensor cores in PREC_F64
   bool plain = false;
+  bool spread = false;  // every buffer gets memory of its own
   std::vector<int64_t> k_of;    // K of the GEMM that reads each node's operand
   // GEMM info per internal node
   struct G {
@@ -365,8 +366,8 @@ struct Builder {
   const std::set<std::string>* shared = nullptr;
 
   Builder(const Diagram& d, const int64_t* dm, int p, double al, int acc, size_t sb,
-          const std::set<std::string>* sh = nullptr, bool pl = false)
-      : dg(d), dim(dm), prec(p), alpha(al), accumulate(acc), plain(pl), slice_threshold(sb), shared(sh) {}
+          const std::set<std::string>* sh = nullptr, bool pl = false, bool sp = false)
+      : dg(d), dim(dm), prec(p), alpha(al), accumulate(acc), plain(pl), spread(sp), slice_threshold(sb), shared(sh) {}
 
   int64_t prod(const std::vector<int>& legs) const {
     int64_t s = 1;
@@ -812,7 +813,7 @@ struct Builder {
       const int lo = first_use[bi], hi = last_use[bi];
       std::vector<std::pair<int64_t, int64_t>> busy;
       for (auto& iv : placed)
-        if (!(iv.hi < lo || hi < iv.lo)) busy.push_back({iv.off, iv.off + iv.bytes});
+        if (spread || !(iv.hi < lo || hi < iv.lo)) busy.push_back({iv.off, iv.off + iv.bytes});
       std::sort(busy.begin(), busy.end());
       int64_t off = 0;
       for (auto& r : busy) {
@@ -829,10 +830,9 @@ struct Builder {
 };
 
 struct Key {
-  int op, chi_b, chi_t, prec;
-  bool plain;
+  int op, chi_b, chi_t, prec, less;
   bool operator<(const Key& o) const {
-    return std::tie(op, chi_b, chi_t, prec, plain) < std::tie(o.op, o.chi_b, o.chi_t, o.prec, o.plain);
+    return std::tie(op, chi_b, chi_t, prec, less) < std::tie(o.op, o.chi_b, o.chi_t, o.prec, o.less);
   }
 };
 
@@ -846,8 +846,67 @@ std::map<std::tuple<int, int64_t, int64_t, int64_t, int>, int> g_tuned;  // (pre
 
 namespace {
 
+// Waves of an operation whose buffers share no memory within a batch of
+// `batch` diagrams: every step goes to the wave after the last of the steps
+// that write what it reads, batch after batch.  False where a program reads a
+// buffer that several steps write (slices).
+bool build_waves(OpProgram& prog, int op, int chi_b, int chi_t, int prec, int batch) {
+  const size_t nd = prog.diagrams.size();
+  std::map<int64_t, int> ready;                     // buffer offset -> level of the step that writes it
+  std::map<std::pair<int, int>, Wave> by_level;     // (level, family)
+  int root_level = -1, base = 0, top = 0;           // base: first level of the batch
+  for (size_t d = 0; d < nd; ++d) {
+    if (d > 0 && d % size_t(batch) == 0) {  // transient buffers are written anew, copies stay
+      base = top + 1;
+      std::map<int64_t, int> kept;
+      for (auto& kv : ready)
+        if (kv.first < int64_t(prog.persistent_bytes)) kept.insert(kv);
+      ready.swap(kept);
+    }
+    const Program& pg = prog.diagrams[d];
+    for (size_t si = 0; si < pg.steps.size(); ++si) {
+      const Step& st = pg.steps[si];
+      int level = base, out = -1;
+      auto reads = [&](int b) {
+        if (b < 0) return;
+        auto it = ready.find(pg.bufs[size_t(b)].offset);
+        if (it != ready.end()) level = std::max(level, it->second + 1);
+      };
+      if (st.kind == 0) {
+        if (st.p.skip) continue;
+        out = st.p.dst_buf;
+      } else if (st.kind == 2) {
+        if (st.x.skip) continue;
+        reads(st.x.raw_buf);
+        out = st.x.dst_buf;
+      } else {
+        for (int b : {st.g.a_buf, st.g.b_buf, st.g.ax_buf, st.g.bx_buf}) reads(b);
+        out = st.g.c_buf;
+        if (out < 0) {  // the second of two diagrams accumulates onto the first's output
+          if (nd < 3 && root_level >= 0) level = std::max(level, root_level + 1);
+          root_level = level;
+        }
+      }
+      if (out >= 0 && !ready.emplace(pg.bufs[size_t(out)].offset, level).second) return false;
+      const int fam = family_of(st, prec);
+      Wave& w = by_level[{level, fam}];
+      w.family = fam;
+      w.steps.push_back({int(d), int(si)});
+      top = std::max(top, level);
+    }
+  }
+  for (auto& kv : by_level) prog.waves.push_back(std::move(kv.second));
+  if (nd >= 3) {
+    int64_t n = int64_t(chi_b) * chi_b * (op == OP_ENV_U ? int64_t(chi_b) * chi_b : chi_t);
+    prog.part_off = int64_t((prog.ws_bytes + 255) / 256 * 256);
+    prog.part_bytes = n * 8;
+    prog.ws_bytes = size_t(prog.part_off) + nd * size_t(prog.part_bytes);
+  }
+  return true;
+}
+
 // g_mu is held.
-std::unique_ptr<OpProgram> build_program(int op, int chi_b, int chi_t, int prec, bool plain) {
+std::unique_ptr<OpProgram> build_program(int op, int chi_b, int chi_t, int prec, bool plain, int spread) {
   int64_t dim[64];
   for (int l = 0; l < 64; ++l) dim[l] = chi_b;
   for (char c : std::string("pqrstv")) dim[label_id(c)] = chi_t;
@@ -855,7 +914,7 @@ std::unique_ptr<OpProgram> build_program(int op, int chi_b, int chi_t, int prec,
   auto build_all = [&](const std::set<std::string>* sh) -> std::unique_ptr<OpProgram> {
     auto pr = std::make_unique<OpProgram>();
     for (size_t d = 0; d < ds.size(); ++d) {
-      Builder b(ds[d], dim, prec, 0.5, d == 0 ? 0 : 1, g_slice_bytes, sh, plain);
+      Builder b(ds[d], dim, prec, 0.5, d == 0 ? 0 : 1, g_slice_bytes, sh, plain, spread > 0);
       if (!b.build()) return nullptr;
       pr->flops += b.prog.flops;
       for (const Step& st : b.prog.steps) pr->has_x64 |= (st.kind == 1 && st.g.ax_buf >= 0);
@@ -883,7 +942,7 @@ std::unique_ptr<OpProgram> build_program(int op, int chi_b, int chi_t, int prec,
     std::set<std::string> shared;
     int64_t budget = int64_t(4) << 30;
     for (const std::string& k : order)
-      if (count[k] > 1 && bytes[k] <= (int64_t(1) << 30) && bytes[k] <= budget) {
+      if ((count[k] > 1 || spread > 0) && bytes[k] <= (int64_t(1) << 30) && bytes[k] <= budget) {
         shared.insert(k);
         budget -= bytes[k];
       }
@@ -945,33 +1004,57 @@ std::unique_ptr<OpProgram> build_program(int op, int chi_b, int chi_t, int prec,
     }
   }
   prog->persistent_bytes = res_base;
-  size_t trans = 0;
-  for (Program& pg : prog->diagrams) {
+  size_t trans = 0, used = 0;  // `used`: transient bytes of the diagrams that run together
+  for (size_t d = 0; d < prog->diagrams.size(); ++d) {
+    Program& pg = prog->diagrams[d];
+    if (spread == 0 || d % size_t(spread) == 0) used = 0;
     for (Buffer& bf : pg.bufs)
-      if (!bf.resident) bf.offset += int64_t(res_base);
-    trans = std::max(trans, pg.ws_bytes);
+      if (!bf.resident) bf.offset += int64_t(res_base + used);
+    used += (pg.ws_bytes + 255) / 256 * 256;
+    trans = std::max(trans, used);
   }
   prog->ws_bytes = res_base + trans;
+  if (spread > 0 && !build_waves(*prog, op, chi_b, chi_t, prec, spread)) return nullptr;
   return prog;
 }
 
 }  // namespace
 
-const OpProgram* get_program(int op, int chi_b, int chi_t, int prec, bool plain) {
+int family_of(const Step& st, int prec) {
+  if (st.kind == 0) return 0;
+  if (st.kind == 2) return 1;
+  if (st.g.ax_buf >= 0) return x64_kc((st.g.K + 15) / 16, st.g.split) <= kX64BlockSteps ? 3 : 4;
+  if (prec == PREC_F64) return 2;
+  return 16 + st.g.bn;
+}
+
+const OpProgram* get_program(int op, int chi_b, int chi_t, int prec, int less) {
   if (op < OP_ASCEND || op > OP_ENV_W) return nullptr;
   if (prec < PREC_F64 || prec > PREC_LAST) return nullptr;
   if (chi_b < 1 || chi_t < 1 || chi_b > 64 || chi_t > 64) return nullptr;
   if (chi_t > chi_b * chi_b) return nullptr;
   std::lock_guard<std::mutex> lk(g_mu);
-  Key k{op, chi_b, chi_t, prec, plain && prec == PREC_F64};
+  if (less > 1 && prec != PREC_F64) less = 1;
+  Key k{op, chi_b, chi_t, prec, less};
   auto it = g_cache.find(k);
   if (it != g_cache.end()) return it->second.get();
-  auto prog = build_program(op, chi_b, chi_t, prec, plain);
   // The digit images nearly triple a PREC_F64 operand.  Past chi ~ 33 the
   // operands alone fill most of the memory: those programs stay on the FP64
   // pipe (env_w at chi = 40: 130 GiB against 307 GiB).
   constexpr size_t kX64MaxWorkspace = size_t(96) << 30;
-  if (prog && prog->has_x64 && prog->ws_bytes > kX64MaxWorkspace) prog = build_program(op, chi_b, chi_t, prec, true);
+  constexpr size_t kSpreadAllWorkspace = size_t(1) << 30, kSpreadMaxWorkspace = size_t(4) << 30;
+  auto prog = build_program(op, chi_b, chi_t, prec, less > 1, 0);
+  if (prog && prog->has_x64 && prog->ws_bytes > kX64MaxWorkspace)
+    prog = build_program(op, chi_b, chi_t, prec, true, 0);
+  // Waves pay while one product does not fill the GPU; past that they only
+  // take memory.  All diagrams at once where that is little memory, else in
+  // pairs.
+  if (prog && less == 0 && prog->ws_bytes <= kSpreadMaxWorkspace) {
+    const int nd = int(prog->diagrams.size());
+    auto sp = build_program(op, chi_b, chi_t, prec, false, nd);
+    if (sp && nd > 2 && sp->ws_bytes > kSpreadAllWorkspace) sp = build_program(op, chi_b, chi_t, prec, false, 2);
+    if (sp && sp->ws_bytes <= kSpreadMaxWorkspace && sp->ws_bytes >= prog->ws_bytes) prog = std::move(sp);
+  }
   if (!prog) return nullptr;
   const OpProgram* out = prog.get();
   g_cache[k] = std::move(prog);
@@ -1086,6 +1169,13 @@ std::string program_json(const OpProgram& prog, int op, int chi_b, int chi_t, in
         o << "}";
       }
     }
+    o << "]}";
+  }
+  o << "],\"part_off\":" << prog.part_off << ",\"part_bytes\":" << prog.part_bytes << ",\"waves\":[";
+  for (size_t w = 0; w < prog.waves.size(); ++w) {
+    o << (w ? "," : "") << "{\"family\":" << prog.waves[w].family << ",\"steps\":[";
+    for (size_t k = 0; k < prog.waves[w].steps.size(); ++k)
+      o << (k ? "," : "") << "[" << prog.waves[w].steps[k].first << "," << prog.waves[w].steps[k].second << "]";
     o << "]}";
   }
   o << "]}";

@@ -136,6 +136,13 @@ struct Program {
   int out_rank = 0;
 };
 
+// Steps of one kind, from any of the operation's diagrams, that no step of
+// the wave depends on: one launch.
+struct Wave {
+  int family = 0;  // 0 permute, 1 split, 2 FP64 GEMM, 3/4 digit GEMM of one / several blocks, 16 + width: tensor-core GEMM
+  std::vector<std::pair<int, int>> steps;  // (diagram, step)
+};
+
 // A whole operation (sum of diagrams, each scaled by alpha, the first one
 // overwriting the output and the others accumulating).
 struct OpProgram {
@@ -144,6 +151,12 @@ struct OpProgram {
   size_t persistent_bytes = 0;  // leading workspace bytes holding the resident copies
   double flops = 0.0;
   int has_x64 = 0;  // some product runs on the tensor cores in PREC_F64
+  // Small operations: every buffer has memory of its own and the steps of all
+  // diagrams run in waves.  With three or more diagrams each writes its part
+  // of the output to part_off + d * part_bytes of the workspace, summed in
+  // the diagrams' order at the end; else the second accumulates.
+  std::vector<Wave> waves;
+  int64_t part_off = -1, part_bytes = 0;
 };
 
 // PREC_F64: whether a product runs on the tensor cores (digit splitting) or
@@ -176,8 +189,13 @@ std::vector<std::vector<int64_t>> tuned_tiles();
 int planes(int prec);       // 2 for BF16X3 (hi, lo), 3 for BF16X6 (hi, mid, lo), 3 / 4 for OZ3 / OZ4, else 1
 
 // Builds (and caches) the program; thread safe.  Returns nullptr on bad input.
-// plain: PREC_F64 with every product on the FP64 pipe (less workspace).
-const OpProgram* get_program(int op, int chi_b, int chi_t, int prec, bool plain = false);
+// less: 0 the fastest program, 1 one with a reused arena (small operations
+// else run in waves), 2 also PREC_F64 with every product on the FP64 pipe; each
+// needs no more workspace than the one before.
+const OpProgram* get_program(int op, int chi_b, int chi_t, int prec, int less = 0);
+
+// Launch family of a step (Wave).
+int family_of(const Step& st, int prec);
 
 std::string program_json(const OpProgram& prog, int op, int chi_b, int chi_t, int prec);
 

@@ -186,21 +186,54 @@ struct Epilogue {
   int off32;        // every column offset n_dst(n) is below 2^31
   int alpha_exp;    // alpha == 2^alpha_exp exactly (alpha_pow2 set)
   int alpha_pow2;
+  // work items (fewer than 2^31): tiles_m x tiles_n output tiles, times the K split
+  int tiles_m, tiles_n;
   int group_m;      // tile order: groups of this many row tiles, every column tile of a group in turn
 };
+
+// Jobs of one launch: their work items one after another.
+struct TcGroup {
+  int n;
+  int end[kGroup];  // work items of the jobs up to and including each
+  TMaps tm[kGroup];
+  Epilogue ep[kGroup];
+};
+
+// Job of work item t, and the item's index within it.
+__device__ __forceinline__ int item_of(const int* end, int t, int& local) {
+  int i = 0;
+  while (t >= end[i]) ++i;
+  local = t - (i > 0 ? end[i - 1] : 0);
+  return i;
+}
+
+// Split of work item t of a job with `tiles` output tiles, t becoming the
+// tile: item t covers tile t % tiles and k-range t / tiles.
+__device__ __forceinline__ int split_of(int& t, int tiles, int split) {
+  if (split <= 1) return 0;
+  const int ks = int(uint32_t(t) / uint32_t(tiles));
+  t -= ks * tiles;
+  return ks;
+}
 
 // Output tile (row tile, column tile) of the mn-th tile in the kernels' walk
 // order.  Tiles are taken in groups of group_m row tiles; within a group the
 // column tile changes slowest, so one column tile of B meets group_m row
 // tiles of A while both are in L2, and the group's A rows (sized by the host
-// to a fraction of L2) stay resident across the group's column tiles.
-__device__ __forceinline__ void tile_of(int64_t mn, int64_t tiles_m, int64_t tiles_n, int group_m, int64_t& tm,
-                                        int64_t& tn) {
-  const int64_t per_group = int64_t(group_m) * tiles_n;
-  const int64_t g = mn / per_group, r = mn - g * per_group;
-  const int64_t rows = min(int64_t(group_m), tiles_m - g * group_m);  // row tiles in this group
-  tn = r / rows;
-  tm = g * group_m + (r - tn * rows);
+// to a fraction of L2) stay resident across the group's column tiles.  32-bit
+// divisions: this runs once per tile in each role, on the path between two
+// tiles' MMAs.
+__device__ __forceinline__ void tile_of(int mn, int tiles_m, int tiles_n, int group_m, int& tm, int& tn) {
+  const uint32_t per_group = uint32_t(group_m) * uint32_t(tiles_n);
+  uint32_t g = 0, r = uint32_t(mn);
+  if (group_m < tiles_m) {
+    g = r / per_group;
+    r -= g * per_group;
+  }
+  const uint32_t rows = min(uint32_t(group_m), uint32_t(tiles_m) - g * uint32_t(group_m));  // row tiles in this group
+  const uint32_t c = tiles_n > 1 ? r / rows : 0;
+  tn = int(c);
+  tm = int(g * uint32_t(group_m) + (r - c * rows));
 }
 
 // binary32 -> binary64 times 2^e by integer operations, exact for every
@@ -295,7 +328,7 @@ __device__ __forceinline__ void store_chunk(void* C, int64_t off_m, int64_t c_pl
 
 template <int PREC, int BN>
 __global__ void __launch_bounds__(kThreads, 1)
-    tc_gemm_kernel(const __grid_constant__ TMaps tm, const __grid_constant__ Epilogue ep) {
+    tc_gemm_kernel(const __grid_constant__ TcGroup g) {
   using C = Cfg<PREC, BN>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -313,10 +346,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   int* off_n32 = reinterpret_cast<int*>(off_n + BN);
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int64_t tiles_n = (ep.N + BN - 1) / BN;
-  const int64_t tiles_mn = ((ep.M + kBM - 1) / kBM) * tiles_n;
-  const int64_t tiles = tiles_mn * ep.split;
-  const int num_k = int((ep.K + C::kBK - 1) / C::kBK);
+  const int items = g.end[g.n - 1];
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::kStages; ++s) {
@@ -348,11 +378,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       // ---- producer ---------------------------------------------------------
       uint32_t it = 0;
       bool alive = true;
-      for (int64_t t = blockIdx.x; t < tiles && alive; t += gridDim.x) {
-        int64_t row_t, col_t;
-        tile_of(t % tiles_mn, tiles_mn / tiles_n, tiles_n, ep.group_m, row_t, col_t);
-        const int m0 = int(row_t * kBM), n0 = int(col_t * BN);
-        const int kb0 = int(t / tiles_mn) * ep.kc, kb1 = min(kb0 + ep.kc, num_k);
+      for (int tg = int(blockIdx.x); tg < items && alive; tg += gridDim.x) {
+        int t;
+        const int job = item_of(g.end, tg, t);
+        const Epilogue& ep = g.ep[job];
+        const TMaps& tm = g.tm[job];
+        const int num_k = (int(ep.K) + C::kBK - 1) / C::kBK;
+        const int kb0 = split_of(t, ep.tiles_m * ep.tiles_n, ep.split) * ep.kc, kb1 = min(kb0 + ep.kc, num_k);
+        int row_t, col_t;
+        tile_of(t, ep.tiles_m, ep.tiles_n, ep.group_m, row_t, col_t);
+        const int m0 = row_t * kBM, n0 = col_t * BN;
         for (int kb = kb0; kb < kb1; ++kb, ++it) {
           const uint32_t s = it % C::kStages;
           if (it >= uint32_t(C::kStages) && !mbar_wait(&empty[s], ((it / C::kStages) & 1) ^ 1, abort_flag)) {
@@ -380,12 +415,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       constexpr uint32_t idesc = make_idesc(C::kFmt, kBM, BN < 16 ? 16 : BN);
       uint32_t it = 0, tc = 0;
       bool alive = true;
-      for (int64_t t = blockIdx.x; t < tiles && alive; t += gridDim.x, ++tc) {
+      for (int tg = int(blockIdx.x); tg < items && alive; tg += gridDim.x, ++tc) {
+        int t;
+        const int job = item_of(g.end, tg, t);
+        const Epilogue& ep = g.ep[job];
+        const int num_k = (int(ep.K) + C::kBK - 1) / C::kBK;
         const uint32_t b = tc & 1;
         if (tc >= 2 && !mbar_wait(&acc_empty[b], ((tc >> 1) - 1) & 1, abort_flag)) break;
         tc_fence_after();
         const uint32_t d = tmem + b * uint32_t(C::kAccStride);
-        const int kb0 = int(t / tiles_mn) * ep.kc, kb1 = min(kb0 + ep.kc, num_k);
+        const int kb0 = split_of(t, ep.tiles_m * ep.tiles_n, ep.split) * ep.kc, kb1 = min(kb0 + ep.kc, num_k);
         for (int kb = kb0; kb < kb1; ++kb, ++it) {
           const uint32_t s = it % C::kStages;
           if (!mbar_wait(&full[s], (it / C::kStages) & 1, abort_flag)) {
@@ -425,15 +464,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int row = quarter * 32 + lane;
     constexpr int kChunks = BN < 32 ? 1 : BN / 32;
     const int ch_lo = (sub * kChunks) / kSub, ch_hi = ((sub + 1) * kChunks) / kSub;
-    const float alpha = float(ep.alpha);
-    const bool fast_ok = !ep.c_final && ep.split <= 1 && ep.off32 && ep.alpha == 1.0;
-    const bool final_fast = ep.c_final && ep.split <= 1 && ep.off32 && ep.alpha_pow2;
     uint32_t tc = 0;
-    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x, ++tc) {
-      const int64_t ks = t / tiles_mn;
-      int64_t row_t, col_t;
-      tile_of(t % tiles_mn, tiles_mn / tiles_n, tiles_n, ep.group_m, row_t, col_t);
-      const int64_t m0 = row_t * kBM, n0 = col_t * BN;
+    for (int tg = int(blockIdx.x); tg < items; tg += gridDim.x, ++tc) {
+      int t;
+      const int job = item_of(g.end, tg, t);
+      const Epilogue& ep = g.ep[job];
+      const float alpha = float(ep.alpha);
+      const bool fast_ok = !ep.c_final && ep.split <= 1 && ep.off32 && ep.alpha == 1.0;
+      const bool final_fast = ep.c_final && ep.split <= 1 && ep.off32 && ep.alpha_pow2;
+      const int64_t ks = split_of(t, ep.tiles_m * ep.tiles_n, ep.split);
+      int row_t, col_t;
+      tile_of(t, ep.tiles_m, ep.tiles_n, ep.group_m, row_t, col_t);
+      const int64_t m0 = int64_t(row_t) * kBM, n0 = int64_t(col_t) * BN;
       const uint32_t b = tc & 1;
       // all epilogue threads are done with the previous tile's offsets;
       // decide together whether to go on
@@ -558,7 +600,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 // like a binary64 sum but runs on the FP32 pipe.  One thread per row m,
 // looping over a chunk of columns.
 template <int PREC>
-__global__ void __launch_bounds__(256) splitk_reduce_kernel(const __grid_constant__ Epilogue ep) {
+__global__ void __launch_bounds__(256) splitk_reduce_kernel(const __grid_constant__ TcGroup g) {
+  const Epilogue& ep = g.ep[blockIdx.z];
   const int64_t m = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (m >= ep.M) return;
   const int64_t off_m = legmap_offset32(ep.m_dst, uint32_t(m));
@@ -630,82 +673,7 @@ int group_rows(const TcGemmArgs& a, int64_t a_row_bytes) {
   return int(std::min<int64_t>(g, tiles_m));
 }
 
-template <int PREC, int BN>
-cudaError_t launch_cfg(const TcGemmArgs& a, cudaStream_t stream) {
-  using C = Cfg<PREC, BN>;
-  static std::once_flag once;
-  static cudaError_t attr_err = cudaSuccess;
-  std::call_once(once, [] {
-    attr_err = cudaFuncSetAttribute(tc_gemm_kernel<PREC, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    int(C::kSmem));
-  });
-  if (attr_err != cudaSuccess) return attr_err;
-  TMaps tm;
-  const char* A = static_cast<const char*>(a.A);
-  const char* B = static_cast<const char*>(a.B);
-  for (int pl = 0; pl < kMaxPlanes; ++pl) {
-    const int q = pl < C::kPlanes ? pl : 0;  // unused slots repeat plane 0
-    if (!encode_operand(&tm.a[pl], A + q * a.a_plane_bytes, PREC, a.M, a.K, a.lda, kBM, C::kSlab))
-      return cudaErrorInvalidValue;
-    if (!encode_operand(&tm.b[pl], B + q * a.b_plane_bytes, PREC, a.N, a.K, a.ldb, BN, C::kSlab))
-      return cudaErrorInvalidValue;
-  }
-  Epilogue ep;
-  ep.M = a.M;
-  ep.N = a.N;
-  ep.K = a.K;
-  ep.C = a.C;
-  ep.c_plane = a.c_plane_elems;
-  ep.m_dst = a.m_dst;
-  ep.n_dst = a.n_dst;
-  ep.alpha = a.alpha;
-  {
-    int e2 = 0;
-    const double fr = std::frexp(a.alpha, &e2);  // alpha = fr * 2^e2, fr in [0.5, 1)
-    ep.alpha_pow2 = (fr == 0.5) ? 1 : 0;
-    ep.alpha_exp = e2 - 1;
-  }
-  ep.accumulate = a.accumulate;
-  ep.c_final = a.c_final ? 1 : 0;
-  const int64_t num_k = (a.K + C::kBK - 1) / C::kBK;
-  const int split = a.split > 1 && a.partial ? a.split : 1;
-  ep.split = split;
-  ep.kc = int((num_k + split - 1) / split);
-  ep.partial = a.partial;
-  ep.p_plane = 0;
-  {
-    // largest column offset, to allow 32-bit column offsets (the row
-    // offset stays 64-bit)
-    int64_t hi = 0;
-    for (int i = 0; i < a.n_dst.n; ++i) hi += (a.n_dst.dim[i] - 1) * a.n_dst.stride[i];
-    ep.off32 = hi < (int64_t(1) << 31) ? 1 : 0;
-  }
-  ep.group_m = group_rows(a, a.K * C::kElem * C::kPlanes);
-  if (split > 1 && (int64_t(split - 1) * ep.kc >= num_k)) return cudaErrorInvalidValue;  // empty split
-  const int64_t tiles = ((a.M + kBM - 1) / kBM) * ((a.N + BN - 1) / BN) * split;
-  if (tiles <= 0) return cudaErrorInvalidValue;
-  static int resident = 0;  // CTAs of this configuration the whole GPU holds at once
-  static std::once_flag occ_once;
-  std::call_once(occ_once, [] {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tc_gemm_kernel<PREC, BN>, kThreads, C::kSmem);
-    resident = std::max(1, sms) * std::max(1, per_sm);
-  });
-  const unsigned grid = unsigned(std::min<int64_t>(tiles, resident));
-  count_launch();
-  tc_gemm_kernel<PREC, BN><<<grid, kThreads, C::kSmem, stream>>>(tm, ep);
-  if (split > 1) {
-    const unsigned gx = unsigned((a.M + 255) / 256);
-    const unsigned gy = unsigned(std::min<int64_t>(a.N, std::max<int64_t>(1, 4 * 152 / int64_t(gx))));
-    count_launch();
-    splitk_reduce_kernel<PREC><<<dim3(gx, gy), 256, 0, stream>>>(ep);
-  }
-  return cudaGetLastError();
-}
-
-// Shared by both launchers: the epilogue's destination description.
+// The epilogue's destination description of a job.
 void fill_epilogue(const TcGemmArgs& a, Epilogue& ep) {
   ep.M = a.M;
   ep.N = a.N;
@@ -721,124 +689,195 @@ void fill_epilogue(const TcGemmArgs& a, Epilogue& ep) {
   ep.alpha_exp = e2 - 1;
   ep.accumulate = a.accumulate;
   ep.c_final = a.c_final ? 1 : 0;
-  int64_t hi = 0;  // largest column offset: 32-bit column offsets allowed below 2^31
+  int64_t hi = 0;  // largest column offset: 32-bit column offsets allowed below 2^31 (the row offset stays 64-bit)
   for (int i = 0; i < a.n_dst.n; ++i) hi += (a.n_dst.dim[i] - 1) * a.n_dst.stride[i];
   ep.off32 = hi < (int64_t(1) << 31) ? 1 : 0;
+  ep.split = a.split > 1 && a.partial ? a.split : 1;
+  ep.partial = a.partial;
+  ep.p_plane = a.partial_plane;
 }
 
+// The K-split sums of the jobs that have one, in one launch.
+template <typename Kernel>
+void launch_reduce(Kernel kernel, const TcGroup& g, cudaStream_t stream) {
+  static thread_local TcGroup r;
+  r.n = 0;
+  unsigned gx = 0, gy = 0;
+  for (int i = 0; i < g.n; ++i) {
+    const Epilogue& ep = g.ep[i];
+    if (ep.split <= 1) continue;
+    r.ep[r.n++] = ep;
+    const unsigned x = unsigned((ep.M + 255) / 256);
+    gx = std::max(gx, x);
+    gy = std::max(gy, unsigned(std::min<int64_t>(ep.N, std::max<int64_t>(1, 4 * 152 / int64_t(x)))));
+  }
+  if (r.n == 0) return;
+  count_launch();
+  kernel<<<dim3(gx, gy, unsigned(r.n)), 256, 0, stream>>>(r);
+}
+
+// CTAs of a kernel that the whole GPU holds at once.
+template <typename Kernel>
+int resident_ctas(Kernel kernel, int threads, size_t smem) {
+  int dev = 0, sms = 0, per_sm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
+  return std::max(1, sms) * std::max(1, per_sm);
+}
+
+template <int PREC, int BN>
+cudaError_t launch_cfg(const TcGemmArgs* args, int n, cudaStream_t stream) {
+  using C = Cfg<PREC, BN>;
+  static std::once_flag once;
+  static cudaError_t attr_err = cudaSuccess;
+  static int resident = 0;
+  std::call_once(once, [] {
+    attr_err = cudaFuncSetAttribute(tc_gemm_kernel<PREC, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    int(C::kSmem));
+    resident = resident_ctas(tc_gemm_kernel<PREC, BN>, kThreads, C::kSmem);
+  });
+  if (attr_err != cudaSuccess) return attr_err;
+  static thread_local TcGroup g;
+  g.n = n;
+  int64_t items = 0;
+  for (int i = 0; i < n; ++i) {
+    const TcGemmArgs& a = args[i];
+    const char* A = static_cast<const char*>(a.A);
+    const char* B = static_cast<const char*>(a.B);
+    for (int pl = 0; pl < C::kPlanes; ++pl) {
+      if (!encode_operand(&g.tm[i].a[pl], A + pl * a.a_plane_bytes, PREC, a.M, a.K, a.lda, kBM, C::kSlab))
+        return cudaErrorInvalidValue;
+      if (!encode_operand(&g.tm[i].b[pl], B + pl * a.b_plane_bytes, PREC, a.N, a.K, a.ldb, BN, C::kSlab))
+        return cudaErrorInvalidValue;
+    }
+    Epilogue& ep = g.ep[i];
+    fill_epilogue(a, ep);
+    const int64_t num_k = (a.K + C::kBK - 1) / C::kBK;
+    ep.kc = int((num_k + ep.split - 1) / ep.split);
+    ep.group_m = group_rows(a, a.K * C::kElem * C::kPlanes);
+    if (ep.split > 1 && (int64_t(ep.split - 1) * ep.kc >= num_k)) return cudaErrorInvalidValue;  // empty split
+    items += ((a.M + kBM - 1) / kBM) * ((a.N + BN - 1) / BN) * ep.split;
+    if (items > 0x7fffffff) return cudaErrorInvalidValue;
+    ep.tiles_m = int((a.M + kBM - 1) / kBM);
+    ep.tiles_n = int((a.N + BN - 1) / BN);
+    g.end[i] = int(items);
+  }
+  count_launch();
+  tc_gemm_kernel<PREC, BN><<<unsigned(std::min<int64_t>(items, resident)), kThreads, C::kSmem, stream>>>(g);
+  launch_reduce(splitk_reduce_kernel<PREC>, g, stream);
+  return cudaGetLastError();
+}
 
 // Fixed-point split modes: S slice planes per operand, K split in whole
 // blocks of kOzBlockK.
 template <int S, int BN>
-cudaError_t launch_oz(const TcGemmArgs& a, cudaStream_t stream) {
+cudaError_t launch_oz(const TcGemmArgs* args, int n, cudaStream_t stream) {
   using C = OzCfg<S, BN>;
   static std::once_flag once;
   static cudaError_t attr_err = cudaSuccess;
+  static int resident = 0;
   std::call_once(once, [] {
     attr_err = cudaFuncSetAttribute(oz_gemm_kernel<S, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::kSmem));
+    resident = resident_ctas(oz_gemm_kernel<S, BN>, kOzThreads, C::kSmem);
   });
   if (attr_err != cudaSuccess) return attr_err;
-  TMaps tm;
-  const char* A = static_cast<const char*>(a.A);
-  const char* B = static_cast<const char*>(a.B);
-  for (int pl = 0; pl < kMaxPlanes; ++pl) {
-    const int q = pl < S ? pl : 0;
-    if (!encode_operand(&tm.a[pl], A + q * a.a_plane_bytes, PREC_BF16, a.M, a.K, a.lda, kBM, C::kSlab))
-      return cudaErrorInvalidValue;
-    if (!encode_operand(&tm.b[pl], B + q * a.b_plane_bytes, PREC_BF16, a.N, a.K, a.ldb, BN, C::kSlab))
-      return cudaErrorInvalidValue;
+  static thread_local TcGroup g;
+  g.n = n;
+  int64_t items = 0;
+  for (int i = 0; i < n; ++i) {
+    const TcGemmArgs& a = args[i];
+    const char* A = static_cast<const char*>(a.A);
+    const char* B = static_cast<const char*>(a.B);
+    for (int pl = 0; pl < S; ++pl) {
+      if (!encode_operand(&g.tm[i].a[pl], A + pl * a.a_plane_bytes, PREC_BF16, a.M, a.K, a.lda, kBM, C::kSlab))
+        return cudaErrorInvalidValue;
+      if (!encode_operand(&g.tm[i].b[pl], B + pl * a.b_plane_bytes, PREC_BF16, a.N, a.K, a.ldb, BN, C::kSlab))
+        return cudaErrorInvalidValue;
+    }
+    Epilogue& ep = g.ep[i];
+    fill_epilogue(a, ep);
+    ep.group_m = group_rows(a, a.K * 2 * S);
+    const int64_t nblk = (a.K + kOzBlockK - 1) / kOzBlockK;
+    const int64_t per = (nblk + ep.split - 1) / ep.split;  // blocks per split
+    ep.kc = int(per * C::kBlockStages);
+    if (ep.split > 1 && ((ep.split - 1) * per >= nblk || a.partial_plane < int64_t(ep.split) * a.N * a.M))
+      return cudaErrorInvalidValue;  // an empty split, or lo partials overlapping hi
+    items += ((a.M + kBM - 1) / kBM) * ((a.N + BN - 1) / BN) * ep.split;
+    if (items > 0x7fffffff) return cudaErrorInvalidValue;
+    ep.tiles_m = int((a.M + kBM - 1) / kBM);
+    ep.tiles_n = int((a.N + BN - 1) / BN);
+    g.end[i] = int(items);
   }
-  Epilogue ep;
-  fill_epilogue(a, ep);
-  ep.group_m = group_rows(a, a.K * 2 * S);
-  const int64_t num_k = (a.K + C::kBK - 1) / C::kBK;
-  const int64_t nblk = (a.K + kOzBlockK - 1) / kOzBlockK;
-  const int split = a.split > 1 && a.partial ? a.split : 1;
-  const int64_t per = (nblk + split - 1) / split;  // blocks per split
-  ep.split = split;
-  ep.kc = int(per * C::kBlockStages);
-  ep.partial = a.partial;
-  ep.p_plane = a.partial_plane;
-  if (split > 1 && ((split - 1) * per >= nblk || a.partial_plane < int64_t(split) * a.N * a.M))
-    return cudaErrorInvalidValue;  // an empty split, or lo partials overlapping hi
-  if (num_k <= 0) return cudaErrorInvalidValue;
-  const int64_t tiles = ((a.M + kBM - 1) / kBM) * ((a.N + BN - 1) / BN) * split;
-  static int resident = 0;
-  static std::once_flag occ_once;
-  std::call_once(occ_once, [] {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, oz_gemm_kernel<S, BN>, kOzThreads, C::kSmem);
-    resident = std::max(1, sms) * std::max(1, per_sm);
-  });
-  const unsigned grid = unsigned(std::min<int64_t>(tiles, resident));
   count_launch();
-  oz_gemm_kernel<S, BN><<<grid, kOzThreads, C::kSmem, stream>>>(tm, ep);
-  if (split > 1) {
-    const unsigned gx = unsigned((a.M + 255) / 256);
-    const unsigned gy = unsigned(std::min<int64_t>(a.N, std::max<int64_t>(1, 4 * 152 / int64_t(gx))));
-    count_launch();
-    oz_splitk_reduce_kernel<<<dim3(gx, gy), 256, 0, stream>>>(ep);
-  }
+  oz_gemm_kernel<S, BN><<<unsigned(std::min<int64_t>(items, resident)), kOzThreads, C::kSmem, stream>>>(g);
+  launch_reduce(oz_splitk_reduce_kernel, g, stream);
   return cudaGetLastError();
 }
 
 template <int S>
-cudaError_t launch_oz_prec(const TcGemmArgs& a, cudaStream_t stream) {
-  const int bn = a.bn > 0 ? a.bn : (a.N > 64 ? 128 : (a.N > 16 ? 64 : 16));
+cudaError_t launch_oz_prec(const TcGemmArgs* a, int n, cudaStream_t stream) {
+  const int bn = a->bn > 0 ? a->bn : (a->N > 64 ? 128 : (a->N > 16 ? 64 : 16));
   switch (bn) {
-    case 128: return launch_oz<S, 128>(a, stream);
-    case 64: return launch_oz<S, 64>(a, stream);
-    case 16: return launch_oz<S, 16>(a, stream);
+    case 128: return launch_oz<S, 128>(a, n, stream);
+    case 64: return launch_oz<S, 64>(a, n, stream);
+    case 16: return launch_oz<S, 16>(a, n, stream);
     default: return cudaErrorInvalidValue;
   }
 }
 
 template <int PREC>
-cudaError_t launch_prec(const TcGemmArgs& a, cudaStream_t stream) {
-  switch (a.bn) {  // a width chosen by the planner (heuristic or autotuned)
+cudaError_t launch_prec(const TcGemmArgs* a, int n, cudaStream_t stream) {
+  switch (a->bn) {  // a width chosen by the planner (heuristic or autotuned)
     case 0: break;
     case 256:
       if constexpr (PREC == PREC_BF16X6) return cudaErrorInvalidValue;  // one stage only
-      else return launch_cfg<PREC, 256>(a, stream);
+      else return launch_cfg<PREC, 256>(a, n, stream);
     case 192:  // N = 576 (chi = 24) in three full tiles
       if constexpr (PREC == PREC_BF16X6) return cudaErrorInvalidValue;
-      else return launch_cfg<PREC, 192>(a, stream);
+      else return launch_cfg<PREC, 192>(a, n, stream);
     case 160:
       if constexpr (PREC == PREC_BF16X6) return cudaErrorInvalidValue;
-      else return launch_cfg<PREC, 160>(a, stream);
-    case 128: return launch_cfg<PREC, 128>(a, stream);
-    case 64: return launch_cfg<PREC, 64>(a, stream);
-    case 16: return launch_cfg<PREC, 16>(a, stream);
+      else return launch_cfg<PREC, 160>(a, n, stream);
+    case 128: return launch_cfg<PREC, 128>(a, n, stream);
+    case 64: return launch_cfg<PREC, 64>(a, n, stream);
+    case 16: return launch_cfg<PREC, 16>(a, n, stream);
     default: return cudaErrorInvalidValue;
   }
   // three-plane operands: a 256-wide B tile leaves room for one stage only
-  if (a.N > 128 && PREC != PREC_BF16X6) return launch_cfg<PREC, (PREC == PREC_BF16X6 ? 128 : 256)>(a, stream);
-  if (a.N > 64) return launch_cfg<PREC, 128>(a, stream);
-  if (a.N > 16) return launch_cfg<PREC, 64>(a, stream);  // (a 32-wide variant spilled registers)
-  return launch_cfg<PREC, 16>(a, stream);
+  if (a->N > 128 && PREC != PREC_BF16X6) return launch_cfg<PREC, (PREC == PREC_BF16X6 ? 128 : 256)>(a, n, stream);
+  if (a->N > 64) return launch_cfg<PREC, 128>(a, n, stream);
+  if (a->N > 16) return launch_cfg<PREC, 64>(a, n, stream);  // (a 32-wide variant spilled registers)
+  return launch_cfg<PREC, 16>(a, n, stream);
 }
 
 }  // namespace
 
-cudaError_t launch_gemm_tc(const TcGemmArgs& a, cudaStream_t stream) {
-  if (a.M <= 0 || a.N <= 0 || a.K <= 0) return cudaErrorInvalidValue;
-  if (a.M > 0x7fffffff || a.N > 0x7fffffff || a.K > 0x7fffffff) return cudaErrorInvalidValue;
-  switch (a.prec) {
-    case PREC_TF32: return launch_prec<PREC_TF32>(a, stream);
-    case PREC_BF16: return launch_prec<PREC_BF16>(a, stream);
-    case PREC_BF16X3: return launch_prec<PREC_BF16X3>(a, stream);
-    case PREC_BF16X6: return launch_prec<PREC_BF16X6>(a, stream);
-    case PREC_OZ3: return launch_oz_prec<3>(a, stream);
-    case PREC_OZ4: return launch_oz_prec<4>(a, stream);
+static cudaError_t launch_tc_group(const TcGemmArgs* a, int n, cudaStream_t stream) {
+  for (int i = 0; i < n; ++i) {
+    if (a[i].M <= 0 || a[i].N <= 0 || a[i].K <= 0) return cudaErrorInvalidValue;
+    if (a[i].M > 0x7fffffff || a[i].N > 0x7fffffff || a[i].K > 0x7fffffff) return cudaErrorInvalidValue;
+  }
+  switch (a->prec) {
+    case PREC_TF32: return launch_prec<PREC_TF32>(a, n, stream);
+    case PREC_BF16: return launch_prec<PREC_BF16>(a, n, stream);
+    case PREC_BF16X3: return launch_prec<PREC_BF16X3>(a, n, stream);
+    case PREC_BF16X6: return launch_prec<PREC_BF16X6>(a, n, stream);
+    case PREC_OZ3: return launch_oz_prec<3>(a, n, stream);
+    case PREC_OZ4: return launch_oz_prec<4>(a, n, stream);
     default: return cudaErrorNotSupported;
   }
 }
 
-cudaError_t launch_gemm_x64(const X64GemmArgs& a, cudaStream_t stream) {
-  if (a.M <= 0 || a.N <= 0 || a.K <= 0) return cudaErrorInvalidValue;
-  if (a.M > 0x7fffffff || a.N > 0x7fffffff || a.K > (1 << 30)) return cudaErrorInvalidValue;
+cudaError_t launch_gemm_tc(const TcGemmArgs* args, int n, cudaStream_t stream) {
+  for (int i = 0; i < n; i += kGroup) {
+    const cudaError_t e = launch_tc_group(args + i, std::min(kGroup, n - i), stream);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+static cudaError_t launch_x64_group(const X64GemmArgs* args, int n, cudaStream_t stream) {
   static std::once_flag once;
   static cudaError_t attr_err = cudaSuccess;
   static int resident = 0;  // CTAs the whole GPU holds at once (one per SM)
@@ -852,49 +891,75 @@ cudaError_t launch_gemm_x64(const X64GemmArgs& a, cudaStream_t stream) {
     resident = std::max(1, sms);
   });
   if (attr_err != cudaSuccess) return attr_err;
-  X64Params p;
-  p.A = static_cast<const uint8_t*>(a.A);
-  p.B = static_cast<const uint8_t*>(a.B);
-  p.ea = a.ea;
-  p.eb = a.eb;
-  p.A64 = a.A64;
-  p.B64 = a.B64;
-  p.lda = a.lda;
-  p.ldb = a.ldb;
-  p.M = a.M;
-  p.N = a.N;
-  p.K = a.K;
-  p.C = a.C;
-  p.m_dst = a.m_dst;
-  p.n_dst = a.n_dst;
-  p.alpha = a.alpha;
-  int e2 = 0;
-  if (std::frexp(a.alpha, &e2) != 0.5) return cudaErrorInvalidValue;
-  p.alpha_exp = e2 - 1;
-  p.accumulate = a.accumulate;
-  p.nk = int((a.K + 15) / 16);
-  p.split = a.split > 1 && a.partial ? a.split : 1;
-  p.kc = int(x64_kc(p.nk, p.split));
-  p.partial = a.partial;
-  p.p_plane = a.partial_plane;
-  if (p.split > 1 && (int64_t(p.split - 1) * p.kc >= p.nk || a.partial_plane < int64_t(p.split) * a.N * a.M))
-    return cudaErrorInvalidValue;  // an empty split, or overlapping partial planes
-  const int64_t tiles_m = (a.M + kBM - 1) / kBM;
-  p.group_m = int(std::min<int64_t>(std::max<int64_t>(1, (int64_t(32) << 20) / (int64_t(p.nk) * kXABytes)), tiles_m));
-  const int64_t tiles = tiles_m * ((a.N + kXBN - 1) / kXBN) * p.split;
+  X64Group g, red;
+  g.n = n;
+  red.n = 0;
+  int64_t items = 0;
+  unsigned gx = 0, gy = 0;
+  for (int i = 0; i < n; ++i) {
+    const X64GemmArgs& a = args[i];
+    if (a.M <= 0 || a.N <= 0 || a.K <= 0) return cudaErrorInvalidValue;
+    if (a.M > 0x7fffffff || a.N > 0x7fffffff || a.K > (1 << 30)) return cudaErrorInvalidValue;
+    X64Params& p = g.job[i];
+    p.A = static_cast<const uint8_t*>(a.A);
+    p.B = static_cast<const uint8_t*>(a.B);
+    p.ea = a.ea;
+    p.eb = a.eb;
+    p.A64 = a.A64;
+    p.B64 = a.B64;
+    p.lda = a.lda;
+    p.ldb = a.ldb;
+    p.M = a.M;
+    p.N = a.N;
+    p.K = a.K;
+    p.C = a.C;
+    p.m_dst = a.m_dst;
+    p.n_dst = a.n_dst;
+    p.alpha = a.alpha;
+    int e2 = 0;
+    if (std::frexp(a.alpha, &e2) != 0.5) return cudaErrorInvalidValue;
+    p.alpha_exp = e2 - 1;
+    p.accumulate = a.accumulate;
+    p.nk = int((a.K + 15) / 16);
+    p.split = a.split > 1 && a.partial ? a.split : 1;
+    p.kc = int(x64_kc(p.nk, p.split));
+    p.partial = a.partial;
+    p.p_plane = a.partial_plane;
+    if (p.split > 1 && (int64_t(p.split - 1) * p.kc >= p.nk || a.partial_plane < int64_t(p.split) * a.N * a.M))
+      return cudaErrorInvalidValue;  // an empty split, or overlapping partial planes
+    const int64_t tiles_m = (a.M + kBM - 1) / kBM;
+    p.group_m = int(std::min<int64_t>(std::max<int64_t>(1, (int64_t(32) << 20) / (int64_t(p.nk) * kXABytes)), tiles_m));
+    items += tiles_m * ((a.N + kXBN - 1) / kXBN) * p.split;
+    if (items > 0x7fffffff) return cudaErrorInvalidValue;
+    p.tiles_m = int(tiles_m);
+    p.tiles_n = int((a.N + kXBN - 1) / kXBN);
+    g.end[i] = int(items);
+    if (p.split > 1) {
+      red.job[red.n++] = p;
+      const unsigned x = unsigned((a.M + 127) / 128);
+      gx = std::max(gx, x);
+      gy = std::max(gy, unsigned(std::min<int64_t>(a.N, std::max<int64_t>(1, 8 * 152 / int64_t(x)))));
+    }
+  }
   count_launch();
-  const unsigned grid = unsigned(std::min<int64_t>(tiles, resident));
-  if (p.kc <= kX64BlockSteps)
-    x64_gemm_kernel<false><<<grid, kXThreads, kXSmem, stream>>>(p);
+  const unsigned grid = unsigned(std::min<int64_t>(items, resident));
+  if (x64_single(args[0]))
+    x64_gemm_kernel<false><<<grid, kXThreads, kXSmem, stream>>>(g);
   else
-    x64_gemm_kernel<true><<<grid, kXThreads, kXSmem, stream>>>(p);
-  if (p.split > 1) {
-    const unsigned gx = unsigned((a.M + 127) / 128);
-    const unsigned gy = unsigned(std::min<int64_t>(a.N, std::max<int64_t>(1, 8 * 152 / int64_t(gx))));
+    x64_gemm_kernel<true><<<grid, kXThreads, kXSmem, stream>>>(g);
+  if (red.n > 0) {
     count_launch();
-    x64_reduce_kernel<<<dim3(gx, gy), 128, 0, stream>>>(p);
+    x64_reduce_kernel<<<dim3(gx, gy, unsigned(red.n)), 128, 0, stream>>>(red);
   }
   return cudaGetLastError();
+}
+
+cudaError_t launch_gemm_x64(const X64GemmArgs* args, int n, cudaStream_t stream) {
+  for (int i = 0; i < n; i += kGroup) {
+    const cudaError_t e = launch_x64_group(args + i, std::min(kGroup, n - i), stream);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 __global__ void report_notconv_kernel(const int* state) {

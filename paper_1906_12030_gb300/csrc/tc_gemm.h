@@ -36,7 +36,11 @@ struct TcGemmArgs {
   int64_t partial_plane = 0; // fixed-point split modes: floats from the hi to the lo plane of `partial`
 };
 
-cudaError_t launch_gemm_tc(const TcGemmArgs& args, cudaStream_t stream);
+// Jobs of one mode and tile width (`bn` or, where that is 0, the same N class).
+cudaError_t launch_gemm_tc(const TcGemmArgs* args, int n, cudaStream_t stream);
+inline cudaError_t launch_gemm_tc(const TcGemmArgs& args, cudaStream_t stream) {
+  return launch_gemm_tc(&args, 1, stream);
+}
 
 // The same product in PREC_F64 on the BF16 tensor cores, from the operands'
 // digit images and row exponents (x64_split.cu).  alpha must be a power of
@@ -60,7 +64,10 @@ struct X64GemmArgs {
   int64_t partial_plane = 0; // floats from one plane to the next
 };
 
-cudaError_t launch_gemm_x64(const X64GemmArgs& args, cudaStream_t stream);
+// Jobs that all fit in one block of K per work item, or all do not
+// (x64_single).
+inline bool x64_single(const X64GemmArgs& a) { return x64_kc((a.K + 15) / 16, a.split) <= kX64BlockSteps; }
+cudaError_t launch_gemm_x64(const X64GemmArgs* args, int n, cudaStream_t stream);
 
 // Sets bit MERA_ENOTCONV of the device status word unless the Newton-Schulz
 // state state[0] says the iteration converged (used where the host cannot

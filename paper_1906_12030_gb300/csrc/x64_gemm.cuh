@@ -88,7 +88,13 @@ struct X64Params {
   int split, kc;      // K split: steps per split
   float* partial;     // split > 1: hi, mid, lo planes [split][N][M]
   int64_t p_plane;
-  int group_m;
+  int tiles_m, tiles_n, group_m;  // work items (fewer than 2^31) and their order, as in Epilogue
+};
+
+struct X64Group {
+  int n;
+  int end[kGroup];  // work items of the jobs up to and including each
+  X64Params job[kGroup];
 };
 
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
@@ -171,7 +177,7 @@ __device__ __forceinline__ void x64_store(const X64Params& p, int64_t off, doubl
 
 // MULTI: a work item may span several blocks of K.
 template <bool MULTI>
-__global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_constant__ X64Params p) {
+__global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_constant__ X64Group g) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* aux = smem + size_t(kXStages) * kXStageBytes;
@@ -187,10 +193,7 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
   int* exp_n = reinterpret_cast<int*>(off_n + kXBN);
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int64_t tiles_n = (p.N + kXBN - 1) / kXBN;
-  const int64_t tiles_m = (p.M + kBM - 1) / kBM;
-  const int64_t tiles_mn = tiles_m * tiles_n;
-  const int64_t tiles = tiles_mn * p.split;
+  const int items = g.end[g.n - 1];
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kXStages; ++s) {
@@ -220,12 +223,14 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
       // ---- producer: all digits of 16 of K per stage ----------------------
       uint32_t it = 0;
       bool alive = true;
-      for (int64_t t = blockIdx.x; t < tiles && alive; t += gridDim.x) {
-        int64_t row_t, col_t;
-        tile_of(t % tiles_mn, tiles_m, tiles_n, p.group_m, row_t, col_t);
-        const int k0 = int(t / tiles_mn) * p.kc, k1 = min(k0 + p.kc, p.nk);
-        const uint8_t* a = p.A + row_t * p.nk * int64_t(kXABytes);
-        const uint8_t* b = p.B + col_t * p.nk * int64_t(kXBBytes);
+      for (int tg = int(blockIdx.x); tg < items && alive; tg += gridDim.x) {
+        int t;
+        const X64Params& p = g.job[item_of(g.end, tg, t)];
+        const int k0 = split_of(t, p.tiles_m * p.tiles_n, p.split) * p.kc, k1 = min(k0 + p.kc, p.nk);
+        int row_t, col_t;
+        tile_of(t, p.tiles_m, p.tiles_n, p.group_m, row_t, col_t);
+        const uint8_t* a = p.A + int64_t(row_t) * p.nk * kXABytes;
+        const uint8_t* b = p.B + int64_t(col_t) * p.nk * kXBBytes;
         for (int k = k0; k < k1; ++k, ++it) {
           const uint32_t s = it % kXStages;
           if (it >= uint32_t(kXStages) && !mbar_wait(&empty[s], ((it / kXStages) & 1) ^ 1, abort_flag)) {
@@ -246,8 +251,10 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
       // ---- MMA issuer ---------------------------------------------------------
       uint32_t it = 0, bc = 0;  // stages consumed, blocks issued
       bool alive = true;
-      for (int64_t t = blockIdx.x; t < tiles && alive; t += gridDim.x) {
-        const int k0 = int(t / tiles_mn) * p.kc, k1 = min(k0 + p.kc, p.nk);
+      for (int tg = int(blockIdx.x); tg < items && alive; tg += gridDim.x) {
+        int t;
+        const X64Params& p = g.job[item_of(g.end, tg, t)];
+        const int k0 = split_of(t, p.tiles_m * p.tiles_n, p.split) * p.kc, k1 = min(k0 + p.kc, p.nk);
         for (int k = k0; k < k1 && alive; ++bc) {
           const int ke = min(k1, (k / kX64BlockSteps + 1) * kX64BlockSteps);
           if (bc >= 1 && !mbar_wait(acc_empty, (bc - 1) & 1, abort_flag)) {
@@ -298,11 +305,13 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
     const int c0 = ((warp - 2) / 4) * kXCols;  // first column of this warp's share
     const int row = quarter * 32 + lane;
     uint32_t bc = 0;
-    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-      const int64_t ks = t / tiles_mn;
-      int64_t row_t, col_t;
-      tile_of(t % tiles_mn, tiles_m, tiles_n, p.group_m, row_t, col_t);
-      const int64_t m0 = row_t * kBM, n0 = col_t * kXBN;
+    for (int tg = int(blockIdx.x); tg < items; tg += gridDim.x) {
+      int t;
+      const X64Params& p = g.job[item_of(g.end, tg, t)];
+      const int64_t ks = split_of(t, p.tiles_m * p.tiles_n, p.split);
+      int row_t, col_t;
+      tile_of(t, p.tiles_m, p.tiles_n, p.group_m, row_t, col_t);
+      const int64_t m0 = int64_t(row_t) * kBM, n0 = int64_t(col_t) * kXBN;
       const int k0 = int(ks) * p.kc, k1 = min(k0 + p.kc, p.nk);
       asm volatile("bar.sync 1, %0;" ::"n"(kXEpiThreads) : "memory");
       if (et == 0) *abort_snapshot = *abort_flag;
@@ -402,7 +411,8 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
 
 // Sum of the K-split partial triples in a fixed order, then the GEMM's
 // output.  One thread per row m over a chunk of columns.
-__global__ void __launch_bounds__(128) x64_reduce_kernel(const __grid_constant__ X64Params p) {
+__global__ void __launch_bounds__(128) x64_reduce_kernel(const __grid_constant__ X64Group g) {
+  const X64Params& p = g.job[blockIdx.z];
   const int64_t m = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (m >= p.M) return;
   const int64_t off_m = legmap_offset32(p.m_dst, uint32_t(m));

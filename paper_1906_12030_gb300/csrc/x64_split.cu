@@ -40,6 +40,13 @@ struct SplitArgs {
   int tile, nk;        // rows per tile, 16-wide steps of K
   int R, G;            // rows and groups of 8 entries per block of threads
   int known;           // rowexp holds the rows' exponents already
+  int gx;              // blocks of threads along the rows
+};
+struct SplitGroup {
+  int n;
+  int end[kGroup];     // blocks of the jobs up to and including each
+  int rend[kGroup];    // rows whose exponents need a pass of their own, likewise
+  SplitArgs job[kGroup];
 };
 
 // High word of |x|, at least 1 unless x is zero: orders entries by magnitude
@@ -56,30 +63,37 @@ __device__ __forceinline__ int row_exponent(int w) {
   return (e > kX64MaxExp || e < -kX64MaxExp) ? kX64Bad : e;
 }
 
-__global__ void __launch_bounds__(512) x64_rowexp_kernel(const double* __restrict__ src, int64_t ld, int64_t rows,
-                                                         int64_t K, int* __restrict__ rowexp) {
+__global__ void __launch_bounds__(512) x64_rowexp_kernel(const __grid_constant__ SplitGroup g) {
   __shared__ int sm[16];
-  for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
-    const double* p = src + r * ld;
+  for (int64_t rg = blockIdx.x; rg < g.rend[g.n - 1]; rg += gridDim.x) {
+    int i = 0;
+    while (rg >= g.rend[i]) ++i;
+    const SplitArgs& a = g.job[i];
+    const int64_t r = rg - (i > 0 ? g.rend[i - 1] : 0);
+    const double* p = a.src + r * a.ld;
     int w = 0;
-    for (int64_t k = threadIdx.x; k < K; k += blockDim.x) w = max(w, mag_word(p[k]));
+    for (int64_t k = threadIdx.x; k < a.K; k += blockDim.x) w = max(w, mag_word(p[k]));
     w = __reduce_max_sync(0xffffffffu, w);
     if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = w;
     __syncthreads();
     if (threadIdx.x == 0) {
-      for (int i = 1; i < 16; ++i) w = max(w, sm[i]);
-      rowexp[r] = row_exponent(w);
+      for (int k = 1; k < 16; ++k) w = max(w, sm[k]);
+      a.rowexp[r] = row_exponent(w);
     }
     __syncthreads();
   }
 }
 
-__global__ void __launch_bounds__(kThreadsX, 2) x64_split_kernel(const __grid_constant__ SplitArgs a) {
+__global__ void __launch_bounds__(kThreadsX, 2) x64_split_kernel(const __grid_constant__ SplitGroup gr) {
+  int job = 0;
+  while (int(blockIdx.x) >= gr.end[job]) ++job;
+  const int block = int(blockIdx.x) - (job > 0 ? gr.end[job - 1] : 0);
+  const SplitArgs& a = gr.job[job];
   extern __shared__ int s_max[];  // [R][blocks of 256]: magnitude words, then [R] row exponents
   const int nb = (a.G * 8 + kX64Block - 1) / kX64Block;
   int* s_row = s_max + a.R * nb;
-  const int64_t r0 = int64_t(blockIdx.x) * a.R;
-  const int kbase = int(blockIdx.y) * a.G * 8;
+  const int64_t r0 = int64_t(block % a.gx) * a.R;
+  const int kbase = block / a.gx * a.G * 8;
   const int rlow = min(a.R, 8);  // rows run fastest over the threads: stores fill whole core matrices
   for (int i = threadIdx.x; i < a.R * nb; i += kThreadsX) s_max[i] = 0;
   __syncthreads();
@@ -193,47 +207,71 @@ __global__ void __launch_bounds__(kThreadsX, 2) x64_split_kernel(const __grid_co
 
 }  // namespace
 
-cudaError_t launch_x64_split(const double* src, int64_t ld, int64_t rows, int64_t K, int64_t seg_rows, int tile,
-                             void* img, int* rowexp, cudaStream_t stream) {
-  if (rows <= 0 || K <= 0) return cudaSuccess;
-  if ((ld & 7) || K > ld || K > (1 << 30) || seg_rows <= 0 || rows % seg_rows || (reinterpret_cast<uintptr_t>(src) & 15))
-    return cudaErrorInvalidValue;
-  SplitArgs a;
-  a.src = src;
-  a.ld = ld;
-  a.rows = rows;
-  a.K = K;
-  a.seg_rows = seg_rows;
-  a.tiles_per_seg = (seg_rows + tile - 1) / tile;
-  a.img = static_cast<uint8_t*>(img);
-  a.rowexp = rowexp;
-  a.tile = tile;
-  a.nk = int((K + 15) / 16);
-  const int kp = a.nk * 16;
-  unsigned ksegs = 1;
-  if (kp <= kCap) {
-    a.known = 0;
-    a.G = kp / 8;
-    int R = 1;
-    while (2 * R * kp <= kCap && R < 256) R *= 2;
-    // at least two blocks of threads per SM where the rows allow it
-    while (R > 8 && (rows + R - 1) / R < 2 * 152) R /= 2;
-    a.R = R;
-  } else {
-    a.known = 1;
-    a.R = 8;
-    a.G = kCap / 8 / 8;  // 1024 of K: four blocks of 256
-    ksegs = unsigned((kp + a.G * 8 - 1) / (a.G * 8));
-    if (ksegs > 65535) return cudaErrorInvalidValue;
-    count_launch();
-    x64_rowexp_kernel<<<unsigned(std::min<int64_t>(rows, 152 * 16)), 512, 0, stream>>>(src, ld, rows, K, rowexp);
+static cudaError_t launch_group(const X64SplitJob* jobs, int n, cudaStream_t stream) {
+  SplitGroup g;
+  g.n = 0;
+  int64_t blocks = 0, rows_known = 0;
+  size_t smem = 0;
+  for (int i = 0; i < n; ++i) {
+    const X64SplitJob& j = jobs[i];
+    if (j.rows <= 0 || j.K <= 0) continue;
+    if ((j.ld & 7) || j.K > j.ld || j.K > (1 << 30) || j.seg_rows <= 0 || j.rows % j.seg_rows ||
+        (reinterpret_cast<uintptr_t>(j.src) & 15))
+      return cudaErrorInvalidValue;
+    SplitArgs& a = g.job[g.n];
+    a.src = j.src;
+    a.ld = j.ld;
+    a.rows = j.rows;
+    a.K = j.K;
+    a.seg_rows = j.seg_rows;
+    a.tiles_per_seg = (j.seg_rows + j.tile - 1) / j.tile;
+    a.img = static_cast<uint8_t*>(j.img);
+    a.rowexp = j.rowexp;
+    a.tile = j.tile;
+    a.nk = int((j.K + 15) / 16);
+    const int kp = a.nk * 16;
+    int64_t ksegs = 1;
+    if (kp <= kCap) {
+      a.known = 0;
+      a.G = kp / 8;
+      int R = 1;
+      while (2 * R * kp <= kCap && R < 256) R *= 2;
+      // at least two blocks of threads per SM where the rows allow it
+      while (R > 8 && (j.rows + R - 1) / R < 2 * 152) R /= 2;
+      a.R = R;
+    } else {
+      a.known = 1;
+      a.R = 8;
+      a.G = kCap / 8 / 8;  // 1024 of K: four blocks of 256
+      ksegs = (kp + a.G * 8 - 1) / (a.G * 8);
+      rows_known += j.rows;
+    }
+    const int64_t gx = (j.rows + a.R - 1) / a.R;
+    blocks += gx * ksegs;
+    if (blocks > 0x7fffffff || rows_known > 0x7fffffff) return cudaErrorInvalidValue;
+    a.gx = int(gx);
+    g.end[g.n] = int(blocks);
+    g.rend[g.n] = int(rows_known);
+    const int nb = (a.G * 8 + kX64Block - 1) / kX64Block;
+    smem = std::max(smem, size_t(a.R) * (nb + 1) * sizeof(int));
+    ++g.n;
   }
-  const int64_t gx = (rows + a.R - 1) / a.R;
-  if (gx > 0x7fffffff) return cudaErrorInvalidValue;
-  const int nb = (a.G * 8 + kX64Block - 1) / kX64Block;
+  if (g.n == 0) return cudaSuccess;
+  if (rows_known > 0) {
+    count_launch();
+    x64_rowexp_kernel<<<unsigned(std::min<int64_t>(rows_known, 152 * 16)), 512, 0, stream>>>(g);
+  }
   count_launch();
-  x64_split_kernel<<<dim3(unsigned(gx), ksegs), kThreadsX, size_t(a.R) * (nb + 1) * sizeof(int), stream>>>(a);
+  x64_split_kernel<<<unsigned(blocks), kThreadsX, smem, stream>>>(g);
   return cudaGetLastError();
+}
+
+cudaError_t launch_x64_split(const X64SplitJob* jobs, int n, cudaStream_t stream) {
+  for (int i = 0; i < n; i += kGroup) {
+    const cudaError_t e = launch_group(jobs + i, std::min(kGroup, n - i), stream);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace mera

@@ -532,16 +532,45 @@ extern "C" mera_status mera_fixed_point_rho(const double* u, const double* w, in
 // ---------------------------------------------------------------------------
 // Polar update.
 // ---------------------------------------------------------------------------
-static size_t polar_bytes(int m, int n) {
+// Products of a Newton-Schulz step as digit products: the digit images,
+// row exponents and K-split partials of the largest of the three (X^T X, G G
+// and X B), which share them.
+struct PolarX64 {
+  size_t img_a, img_b, exp_a, exp_b, plane, total;
+};
+static PolarX64 polar_x64(int m, int n) {
+  auto img = [](int64_t rows, int64_t tile, int64_t k) {
+    return align_up(size_t((rows + tile - 1) / tile * tile) * size_t((k + 15) / 16) * 32 * kX64Digits);
+  };
+  PolarX64 x;
+  x.img_a = std::max({img(n, kX64TileA, m), img(n, kX64TileA, n), img(m, kX64TileA, n)});
+  x.img_b = std::max(img(n, kX64TileB, m), img(n, kX64TileB, n));
+  x.exp_a = align_up(size_t(m) * sizeof(int));
+  x.exp_b = align_up(size_t(n) * sizeof(int));
+  auto part = [](int64_t M, int64_t N, int64_t K) {
+    const int64_t s = x64_split_k(M, N, K);
+    return s > 1 ? align_up(size_t(s) * M * N * sizeof(float)) : size_t(0);
+  };
+  x.plane = std::max({part(n, n, m), part(n, n, n), part(m, n, n)});
+  x.total = x.img_a + x.img_b + x.exp_a + x.exp_b + 3 * x.plane;
+  return x;
+}
+
+// The least scratch of a polar update.
+static size_t polar_bytes_least(int m, int n) {
   return 2 * align_up(size_t(m) * n * sizeof(double)) + 3 * align_up(size_t(n) * n * sizeof(double)) +
          kReduceBytes;
 }
+static size_t polar_bytes(int m, int n) {
+  return polar_bytes_least(m, n) + (n > kNsFusedMax ? polar_x64(m, n).total : 0);
+}
 
 // Stiefel step: A, S (n x n), T, Yneg (m x n), then the polar update's scratch.
-static size_t stiefel_bytes(int m, int n) {
+static size_t stiefel_bytes_least(int m, int n) {
   return 2 * align_up(size_t(n) * n * sizeof(double)) + 2 * align_up(size_t(m) * n * sizeof(double)) +
-         polar_bytes(m, n);
+         polar_bytes_least(m, n);
 }
+static size_t stiefel_bytes(int m, int n) { return stiefel_bytes_least(m, n) - polar_bytes_least(m, n) + polar_bytes(m, n); }
 
 extern "C" mera_status mera_polar_workspace_size(int m, int n, size_t* bytes) {
   if (!bytes || m < 1 || n < 1 || m < n || m > 1 << 16) return fail(MERA_EINVAL, "bad polar sizes");
@@ -572,41 +601,75 @@ static mera_status polar_record(const double* env, int m, int n, double* out, in
   row_m.n = 1; row_m.dim[0] = m; row_m.stride[0] = n;
   // Device-gated iterations: once the residual is below tol, one more step
   // runs and every later kernel returns at once.
-  int* state = reinterpret_cast<int*>(scalars + 4);  // done, iterations, converged-after-this-step
-  if ((e = cudaMemsetAsync(state, 0, 3 * sizeof(int), s)) != cudaSuccess) return cuda_status(e, "polar state");
+  int* state = reinterpret_cast<int*>(scalars + 4);  // done, iterations, converged-after-this-step, block count
+  if ((e = cudaMemsetAsync(scalars + 2, 0, 4 * sizeof(double), s)) != cudaSuccess) return cuda_status(e, "polar state");
+  const bool fused = n <= kNsFusedMax;
+  // larger matrices: digit products on the tensor cores where the scratch has
+  // room for them (n = 1024: 6.0 ms a step on the FP64 pipe, 0.26 ms so)
+  const PolarX64 px = polar_x64(m, n);
+  const bool x64 = !fused && ar.left() >= px.total;
+  char* img_a = ar.take(x64 ? px.img_a : 0);
+  char* img_b = ar.take(x64 ? px.img_b : 0);
+  int* exp_a = reinterpret_cast<int*>(ar.take(x64 ? px.exp_a : 0));
+  int* exp_b = reinterpret_cast<int*>(ar.take(x64 ? px.exp_b : 0));
+  float* part = reinterpret_cast<float*>(ar.ptr());
+  auto product = [&](const GemmF64Args& g, cudaStream_t st) {
+    if (!x64) return launch_gemm_f64(g, st);
+    const X64SplitJob jobs[2] = {{g.A, g.a_m, g.M, g.K, g.M, kX64TileA, img_a, exp_a, g.a_k, state},
+                                 {g.B, g.b_n, g.N, g.K, g.N, kX64TileB, img_b, exp_b, g.b_k, state}};
+    cudaError_t r = launch_x64_split(jobs, 2, st);
+    if (r != cudaSuccess) return r;
+    X64GemmArgs a;
+    a.A = img_a; a.ea = exp_a; a.A64 = g.A; a.lda = g.a_m; a.a_k = g.a_k;
+    a.B = img_b; a.eb = exp_b; a.B64 = g.B; a.ldb = g.b_n; a.b_k = g.b_k;
+    a.M = g.M; a.N = g.N; a.K = g.K;
+    a.C = g.C; a.m_dst = g.m_dst; a.n_dst = g.n_dst; a.alpha = g.alpha; a.accumulate = g.accumulate;
+    a.split = x64_split_k(g.M, g.N, g.K);
+    a.partial = part;
+    a.partial_plane = int64_t(px.plane / sizeof(float));
+    a.skip_if = state;
+    return launch_gemm_x64(&a, 1, st);
+  };
   // G = x^T x (skipped once converged)
-  auto gram = [&](const double* x, cudaStream_t st) {
+  auto gram = [&](const double* x, cudaStream_t st, bool close = true, const cudaGraphConditionalHandle* cond = nullptr) {
+    if (fused) return launch_ns_gram(x, G, m, n, state, close, cond, max_iter, st);
     GemmF64Args g;
     g.skip_if = state;
     g.A = x; g.a_m = 1; g.a_k = n;
     g.B = x; g.b_n = 1; g.b_k = n;
     g.M = n; g.N = n; g.K = m;
     g.C = G; g.m_dst = row_n; g.n_dst = col_1; g.alpha = 1.0; g.accumulate = 0;
-    return launch_gemm_f64(g, st);
+    return product(g, st);
   };
   // One step src -> dst = src ((5/2)(I - G) + G^2), ending with the next
   // step's G.
-  auto step = [&](const double* src, double* dst, cudaStream_t st) {
-    GemmF64Args q;  // G2 = G G (skipped once converged)
-    q.skip_if = state;
-    q.A = G; q.a_m = n; q.a_k = 1;
-    q.B = G; q.b_n = 1; q.b_k = n;
-    q.M = n; q.N = n; q.K = n;
-    q.C = G2; q.m_dst = row_n; q.n_dst = col_1; q.alpha = 1.0; q.accumulate = 0;
-    cudaError_t r = launch_gemm_f64(q, st);
+  auto step = [&](const double* src, double* dst, cudaStream_t st, const cudaGraphConditionalHandle* cond) {
+    cudaError_t r = cudaSuccess;
+    if (fused) {
+      r = launch_ns_square(G, Bm, n, red, scalars + 1, tol, state, st);
+    } else {
+      GemmF64Args q;  // G2 = G G (skipped once converged)
+      q.skip_if = state;
+      q.A = G; q.a_m = n; q.a_k = 1;
+      q.B = G; q.b_n = 1; q.b_k = n;
+      q.M = n; q.N = n; q.K = n;
+      q.C = G2; q.m_dst = row_n; q.n_dst = col_1; q.alpha = 1.0; q.accumulate = 0;
+      r = product(q, st);
+      if (r == cudaSuccess) r = launch_ns_step(G, G2, Bm, n, red, scalars + 1, tol, state, st);
+    }
     if (r != cudaSuccess) return r;
-    if ((r = launch_ns_step(G, G2, Bm, n, red, scalars + 1, tol, state, st)) != cudaSuccess) return r;
     GemmF64Args g;
     g.skip_if = state;
     g.A = src; g.a_m = n; g.a_k = 1;
-    g.B = Bm; g.b_n = 1; g.b_k = n;
+    g.B = Bm; g.b_n = fused ? n : 1; g.b_k = fused ? 1 : n;  // (the fused kernels mirror B, so its rows serve too)
     g.M = m; g.N = n; g.K = n;
     g.C = dst; g.m_dst = row_m; g.n_dst = col_1; g.alpha = 1.0; g.accumulate = 0;
-    if ((r = launch_gemm_f64(g, st)) != cudaSuccess) return r;
-    if ((r = launch_ns_finish(state, st)) != cudaSuccess) return r;
-    return gram(dst, st);
+    if ((r = product(g, st)) != cudaSuccess) return r;
+    if (!fused && (r = launch_ns_finish(state, st)) != cudaSuccess) return r;
+    if ((r = gram(dst, st, true, cond)) != cudaSuccess || fused || !cond) return r;
+    return launch_ns_continue(state, *cond, max_iter, st);
   };
-  if ((e = gram(X, s)) != cudaSuccess) return cuda_status(e, "polar gemm");
+  if ((e = gram(X, s, false)) != cudaSuccess) return cuda_status(e, "polar gemm");
   if ((e = launch_ns_prescale(G, X, m, n, scalars + 2, s)) != cudaSuccess) return cuda_status(e, "polar prescale");
   // while (not converged and fewer than max_iter steps): X -> Xn -> X
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -630,9 +693,8 @@ static mera_status polar_record(const double* env, int m, int n, double* out, in
   cudaStream_t bs = nullptr;
   if ((e = cudaStreamCreateWithFlags(&bs, cudaStreamNonBlocking)) != cudaSuccess) return cuda_status(e, "body stream");
   e = cudaStreamBeginCaptureToGraph(bs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
-  if (e == cudaSuccess) e = step(X, Xn, bs);
-  if (e == cudaSuccess) e = step(Xn, X, bs);
-  if (e == cudaSuccess) e = launch_ns_continue(state, h, max_iter, bs);
+  if (e == cudaSuccess) e = step(X, Xn, bs, nullptr);
+  if (e == cudaSuccess) e = step(Xn, X, bs, &h);
   cudaGraph_t got = nullptr;
   const cudaError_t e2 = cudaStreamEndCapture(bs, &got);
   cudaStreamDestroy(bs);
@@ -703,7 +765,7 @@ extern "C" mera_status mera_polar_update(const double* env, int m, int n, double
   using namespace mera::polar_detail;
   if (!env || !out || env == out) return fail(MERA_EINVAL, "bad env/out pointers");
   if (m < 1 || n < 1 || m < n || m > 1 << 16) return fail(MERA_EINVAL, "polar needs m >= n >= 1 (m=%d n=%d)", m, n);
-  const size_t need = polar_bytes(m, n);
+  const size_t need = polar_bytes_least(m, n);
   if (reinterpret_cast<uintptr_t>(ws) % kAlign) return fail(MERA_EINVAL, "workspace not 256-byte aligned");
   if (!ws || ws_bytes < need) return fail(MERA_ENOMEM, "workspace %zu bytes < %zu needed", ws_bytes, need);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -767,7 +829,7 @@ extern "C" mera_status mera_stiefel_step(const double* X, const double* G, int m
   if (m < 1 || n < 1 || m < n || m > 1 << 16) return fail(MERA_EINVAL, "stiefel step needs m >= n >= 1");
   if (!(eta >= 0.0) || !std::isfinite(eta)) return fail(MERA_EINVAL, "bad step size");
   if (reinterpret_cast<uintptr_t>(ws) % kAlign) return fail(MERA_EINVAL, "workspace not 256-byte aligned");
-  if (!ws || ws_bytes < stiefel_bytes(m, n)) return fail(MERA_ENOMEM, "stiefel workspace too small");
+  if (!ws || ws_bytes < stiefel_bytes_least(m, n)) return fail(MERA_ENOMEM, "stiefel workspace too small");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   Arena ar{static_cast<char*>(ws), ws_bytes};
   double* A = reinterpret_cast<double*>(ar.take(size_t(n) * n * sizeof(double)));
@@ -833,7 +895,7 @@ mera_status sweep_layout(int n_layers, const int* chi_b, const int* chi_t, int p
       map_bytes = std::max(map_bytes, op_bytes(*p));
     }
     const int64_t eb = int64_t(chi_b[t]) * chi_b[t];
-    map_bytes = std::max(map_bytes, stiefel_bytes(int(eb), int(eb)));  // >= polar_bytes
+    map_bytes = std::max(map_bytes, less ? stiefel_bytes_least(int(eb), int(eb)) : stiefel_bytes(int(eb), int(eb)));
     size_t fp = 0;
     if (t == n_layers - 1) {
       ws_size_impl(MERA_OP_FIXED_POINT, chi_b[t], chi_t[t], prec, &fp, less);

@@ -50,15 +50,16 @@ struct OzSplitJob {
 };
 cudaError_t launch_oz_split(const OzSplitJob* jobs, int n, int slices, cudaStream_t stream);
 
-// Binary64 operand (rows x K, pitch ld, a multiple of 8) -> digit image of
-// x64_gemm_kernel in tiles of `tile` rows, and one exponent per row.  Rows
+// Binary64 operand (rows x K) -> digit image of x64_gemm_kernel in tiles of `tile` rows, and one exponent per row.  Rows
 // come in segments of seg_rows, each padded to whole tiles.
 struct X64SplitJob {
-  const double* src = nullptr;
+  const double* src = nullptr;  // entry (r, k) at src[r * ld + k * k_stride]
   int64_t ld = 0, rows = 0, K = 0, seg_rows = 0;
   int tile = 0;
   void* img = nullptr;
   int* rowexp = nullptr;
+  int64_t k_stride = 1;
+  const int* skip_if = nullptr;  // device flag: the launch does nothing where *skip_if != 0 (the first job's counts)
 };
 cudaError_t launch_x64_split(const X64SplitJob* jobs, int n, cudaStream_t stream);
 
@@ -99,7 +100,7 @@ cudaError_t launch_sym_normalize(const double* X, double* rho, int64_t n, double
 
 // Polar-iteration helpers (all binary64, deterministic reductions).
 // G = X^T X (n x n) and X (m x n) scaled by 1/c and 1/sqrt(c), c = max row
-// abs sum of G (>= its largest eigenvalue), written to *c.
+// abs sum of G (>= its largest eigenvalue), written to *c, which starts at 0.
 cudaError_t launch_ns_prescale(double* G, double* X, int64_t m, int64_t n, double* c, cudaStream_t stream);
 cudaError_t launch_frob_scale(const double* src, double* dst, int64_t count, double* partials,
                               double* scalars, cudaStream_t stream);
@@ -110,6 +111,16 @@ cudaError_t launch_ns_step(const double* G, const double* G2, double* Bm, int64_
                            double* resid, double tol, int* state, cudaStream_t stream);
 // Closes a step: state[1] += 1; state[0] = state[2].  Skipped once state[0] is set.
 cudaError_t launch_ns_finish(int* state, cudaStream_t stream);
+// The same step for n <= kNsFusedMax in fused launches (no G2, no finish):
+// launch_ns_square, X B, launch_ns_gram.  state[3] is zero between launches.
+// Up to here the FP64 pipe keeps up with the digit products (n = 256: 84 us a
+// step here; n = 400: 420 us on the FP64 pipe, 100 us as digit products).
+constexpr int64_t kNsFusedMax = 320;  // 820 tile pairs: partial sums in the 4096 slots of the callers' scratch
+cudaError_t launch_ns_square(const double* G, double* Bm, int64_t n, double* partials, double* resid, double tol,
+                             int* state, cudaStream_t stream);
+// close: ends a step.  cond: also sets the condition of the recorded loop.
+cudaError_t launch_ns_gram(const double* X, double* G, int64_t m, int64_t n, int* state, bool close,
+                           const cudaGraphConditionalHandle* cond, int max_iter, cudaStream_t stream);
 // out = -(state[1] odd ? x1 : x0): the polar result, selected on the device.
 cudaError_t launch_ns_output(const double* x0, const double* x1, const int* state, double* out, int64_t count,
                              cudaStream_t stream);

@@ -709,25 +709,18 @@ __global__ void __launch_bounds__(256) scale_by_inverse_kernel(const double* __r
 // Gershgorin rescale of the first Newton-Schulz step: with G = X^T X and
 // c = max_i sum_j |G_ij| >= lambda_max(G), X / sqrt(c) has every singular
 // value in (0, 1] and the same polar factor, usually much closer to 1 than
-// the Frobenius scaling leaves them.
-__global__ void __launch_bounds__(1024) ns_gershgorin_kernel(const double* __restrict__ G, int64_t n, double* c) {
-  __shared__ double sm[32];
-  double v = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-    double r = 0.0;
-    for (int64_t j = 0; j < n; ++j) r += fabs(G[i * n + j]);
-    v = fmax(v, r);
-  }
+// the Frobenius scaling leaves them.  One warp per row; the largest row sum
+// is kept by its bit pattern (non-negative binary64 values order like
+// integers), so *c starts at zero.
+__global__ void __launch_bounds__(256) ns_gershgorin_kernel(const double* __restrict__ G, int64_t n, double* c) {
+  const int64_t i = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) / 32;
+  if (i >= n) return;
+  double r = 0.0;
+  for (int64_t j = threadIdx.x & 31; j < n; j += 32) r += fabs(G[i * n + j]);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    v = threadIdx.x < (blockDim.x >> 5) ? sm[threadIdx.x] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
-    if (threadIdx.x == 0) *c = v;
-  }
+  for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
+  if ((threadIdx.x & 31) == 0)
+    atomicMax(reinterpret_cast<unsigned long long*>(c), static_cast<unsigned long long>(__double_as_longlong(r)));
 }
 
 __global__ void __launch_bounds__(256) ns_prescale_kernel(double* G, int64_t gcount, double* X, int64_t xcount,
@@ -744,7 +737,7 @@ __global__ void __launch_bounds__(256) ns_prescale_kernel(double* G, int64_t gco
 
 cudaError_t launch_ns_prescale(double* G, double* X, int64_t m, int64_t n, double* c, cudaStream_t stream) {
   count_launch(2);
-  ns_gershgorin_kernel<<<1, 1024, 0, stream>>>(G, n, c);
+  ns_gershgorin_kernel<<<unsigned((n + 7) / 8), 256, 0, stream>>>(G, n, c);
   const int64_t total = n * n + m * n;
   const int nb = int(std::min<int64_t>((total + 255) / 256, 1024));
   ns_prescale_kernel<<<nb, 256, 0, stream>>>(G, n * n, X, m * n, c);
@@ -822,6 +815,171 @@ cudaError_t launch_ns_finish(int* state, cudaStream_t stream) {
   return cudaGetLastError();
 }
 
+
+// One Newton-Schulz step of a small matrix in three launches: G^2 with the
+// polynomial, its residual and the convergence check in the epilogue; X B
+// (gemm_f64); X^T X, which also closes the step and, in the last step of a
+// loop body, decides whether to go on.  G and G^2 are symmetric, so only the
+// 8 x 8 tiles on and above the diagonal are summed (tile pairs), which takes a
+// third off the FP64 work of a step.  Tiles and K split as in
+// gemm_f64_small_kernel.  A step of a 256 x 256 matrix was seven launches and
+// 127 us and is 84 us now (54 us of FP64 pipe), of a 64 x 64 one 33 -> 18 us.
+constexpr int kNsR = 8, kNsK = 64, kNsP = kNsK + 2;
+
+// Tile pair t of the upper triangle, row by row: (i, j), i <= j < nt.
+__device__ __forceinline__ void tile_pair(int t, int nt, int& i, int& j) {
+  i = 0;
+  for (int len = nt; t >= len; --len) {
+    t -= len;
+    ++i;
+  }
+  j = i + t;
+}
+
+// Sum over k of A[i][k] B[j][k] for this thread's output of the tile pair,
+// complete in threads 0..63.  KFAST: rows of `x` run along k (x[i * ld + k]);
+// else along the outputs (x[k * ld + i]).
+template <bool KFAST>
+__device__ __forceinline__ double ns_tile(const double* __restrict__ x, int64_t ld, int n, int K, int i0, int j0,
+                                          double* As, double* Bs, double* part) {
+  const int tid = threadIdx.x;
+  int r[2], k[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int e = tid + 256 * q;
+    r[q] = KFAST ? e / kNsK : e % kNsR;
+    k[q] = KFAST ? e % kNsK : e / kNsR;
+  }
+  double va[2], vb[2];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int kk = k0 + k[q], gi = i0 + r[q], gj = j0 + r[q];
+      va[q] = (gi < n && kk < K) ? x[KFAST ? gi * ld + kk : kk * ld + gi] : 0.0;
+      vb[q] = (gj < n && kk < K) ? x[KFAST ? gj * ld + kk : kk * ld + gj] : 0.0;
+    }
+  };
+  const int o = tid % (kNsR * kNsR), quarter = tid / (kNsR * kNsR);
+  const double* a = As + o / kNsR * kNsP + quarter * (kNsK / 4);
+  const double* b = Bs + o % kNsR * kNsP + quarter * (kNsK / 4);
+  double acc = 0.0;
+  load(0);
+  for (int k0 = 0; k0 < K; k0 += kNsK) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      As[r[q] * kNsP + k[q]] = va[q];
+      Bs[r[q] * kNsP + k[q]] = vb[q];
+    }
+    __syncthreads();
+    if (k0 + kNsK < K) load(k0 + kNsK);
+    const int terms = min(kNsK / 4, K - k0 - quarter * (kNsK / 4));  // the rest is zero
+    if (terms == kNsK / 4) {
+#pragma unroll
+      for (int t = 0; t < kNsK / 4; ++t) acc = fma(a[t], b[t], acc);
+    } else {
+      for (int t = 0; t < terms; ++t) acc = fma(a[t], b[t], acc);
+    }
+    __syncthreads();
+  }
+  if (quarter > 0) part[(quarter - 1) * kNsR * kNsR + o] = acc;
+  __syncthreads();
+  if (quarter > 0) return 0.0;
+  return ((acc + part[o]) + part[kNsR * kNsR + o]) + part[2 * kNsR * kNsR + o];
+}
+
+// Bm = (5/2)(I - G) + G^2; the last block to finish sums the tiles' shares of
+// ||G - I||_F^2 in their order and sets state[2].  state[3] counts the blocks
+// and is left at zero.
+__global__ void __launch_bounds__(256) ns_square_kernel(const double* __restrict__ G, double* __restrict__ Bm, int n,
+                                                        double* __restrict__ partials, double* resid, double tol,
+                                                        int* state) {
+  __shared__ double As[kNsR * kNsP], Bs[kNsR * kNsP], part[3 * kNsR * kNsR];
+  __shared__ int last;
+  if (state[0]) return;
+  int ti, tj;
+  tile_pair(int(blockIdx.x), (n + kNsR - 1) / kNsR, ti, tj);
+  const int i0 = ti * kNsR, j0 = tj * kNsR;
+  const double g2 = ns_tile<true>(G, n, n, n, i0, j0, As, Bs, part);
+  const int tid = threadIdx.x;
+  double v = 0.0;
+  if (tid < kNsR * kNsR) {
+    const int i = i0 + tid / kNsR, j = j0 + tid % kNsR;
+    if (i < n && j < n) {
+      const double d = G[int64_t(i) * n + j] - (i == j ? 1.0 : 0.0);
+      const double b = fma(-2.5, d, g2);
+      Bm[int64_t(i) * n + j] = b;
+      if (ti != tj) Bm[int64_t(j) * n + i] = b;
+      v = ti == tj ? d * d : 2.0 * (d * d);
+    }
+  }
+  v = block_sum<256>(v);
+  if (tid == 0) {
+    partials[blockIdx.x] = v;
+    __threadfence();
+    last = atomicAdd(&state[3], 1) == int(gridDim.x) - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  v = 0.0;
+  for (int i = tid; i < int(gridDim.x); i += 256) v += __ldcg(partials + i);
+  v = block_sum<256>(v);
+  if (tid == 0) {
+    const double r = sqrt(v);
+    *resid = r;
+    state[2] = (r <= tol || !(r == r)) ? 1 : 0;  // converged, or NaN: stop after this step
+    state[3] = 0;
+  }
+}
+
+// G = X^T X (m x n, row-major X).  `close`: ends a step (state[1] += 1; done
+// if it converged, and then G is not needed).  `cond`: the loop's condition.
+__global__ void __launch_bounds__(256) ns_gram_kernel(const double* __restrict__ X, double* __restrict__ G, int m,
+                                                      int n, int* state, int close, int set_cond,
+                                                      cudaGraphConditionalHandle cond, int max_iter) {
+  __shared__ double As[kNsR * kNsP], Bs[kNsR * kNsP], part[3 * kNsR * kNsR];
+  // block 0 alone writes state[0] and state[1], and what it writes is the
+  // same early return for every block that reads it
+  const int done = state[0], stop = close ? state[2] : 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    int it = state[1];
+    if (close && !done) {
+      state[1] = ++it;
+      if (stop) state[0] = 1;
+    }
+    if (set_cond) cudaGraphSetConditional(cond, (!done && !stop && it < max_iter) ? 1u : 0u);
+  }
+  if (done || stop) return;
+  int ti, tj;
+  tile_pair(int(blockIdx.x), (n + kNsR - 1) / kNsR, ti, tj);
+  const double g = ns_tile<false>(X, n, n, m, ti * kNsR, tj * kNsR, As, Bs, part);
+  const int tid = threadIdx.x;
+  if (tid >= kNsR * kNsR) return;
+  const int i = ti * kNsR + tid / kNsR, j = tj * kNsR + tid % kNsR;
+  if (i >= n || j >= n) return;
+  G[int64_t(i) * n + j] = g;
+  if (ti != tj) G[int64_t(j) * n + i] = g;
+}
+
+static unsigned ns_pairs(int64_t n) {
+  const int64_t nt = (n + kNsR - 1) / kNsR;
+  return unsigned(nt * (nt + 1) / 2);
+}
+
+cudaError_t launch_ns_square(const double* G, double* Bm, int64_t n, double* partials, double* resid, double tol,
+                             int* state, cudaStream_t stream) {
+  count_launch();
+  ns_square_kernel<<<ns_pairs(n), 256, 0, stream>>>(G, Bm, int(n), partials, resid, tol, state);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_ns_gram(const double* X, double* G, int64_t m, int64_t n, int* state, bool close,
+                           const cudaGraphConditionalHandle* cond, int max_iter, cudaStream_t stream) {
+  count_launch();
+  ns_gram_kernel<<<ns_pairs(n), 256, 0, stream>>>(X, G, int(m), int(n), state, close ? 1 : 0, cond ? 1 : 0,
+                                                  cond ? *cond : cudaGraphConditionalHandle{}, max_iter);
+  return cudaGetLastError();
+}
 
 // out = -X with X the iterate the Newton-Schulz state points at (buffer
 // state[1] & 1), chosen on the device so that no host read is needed.  The

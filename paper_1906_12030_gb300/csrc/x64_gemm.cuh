@@ -77,7 +77,7 @@ struct X64Params {
   const int* eb;
   const double* A64;  // binary64 operands (rows with exponent kX64Bad)
   const double* B64;
-  int64_t lda, ldb;
+  int64_t lda, ldb, a_k, b_k;
   int64_t M, N, K;
   double* C;
   LegMap m_dst, n_dst;
@@ -94,6 +94,7 @@ struct X64Params {
 struct X64Group {
   int n;
   int end[kGroup];  // work items of the jobs up to and including each
+  const int* skip_if;
   X64Params job[kGroup];
 };
 
@@ -164,10 +165,12 @@ __device__ __forceinline__ double triple_to_f64(float h, float m, float l, int e
 }
 
 // One output from the binary64 operands, as gemm_f64_kernel sums it.
-__device__ __noinline__ double x64_plain(const double* a, const double* b, int64_t K) {
+__device__ __noinline__ double x64_plain(const X64Params& p, int64_t m, int64_t n) {
+  const double* a = p.A64 + m * p.lda;
+  const double* b = p.B64 + n * p.ldb;
   double s = 0.0;
-  for (int64_t k = 0; k < K; ++k) s = fma(a[k], b[k], s);
-  return s;
+  for (int64_t k = 0; k < p.K; ++k) s = fma(a[k * p.a_k], b[k * p.b_k], s);
+  return p.alpha * s;
 }
 
 __device__ __forceinline__ void x64_store(const X64Params& p, int64_t off, double x) {
@@ -178,6 +181,7 @@ __device__ __forceinline__ void x64_store(const X64Params& p, int64_t off, doubl
 // MULTI: a work item may span several blocks of K.
 template <bool MULTI>
 __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_constant__ X64Group g) {
+  if (g.skip_if && *g.skip_if) return;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* aux = smem + size_t(kXStages) * kXStageBytes;
@@ -396,7 +400,7 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
 #pragma unroll 1
         for (int c = c0; c < c0 + kXCols && n0 + c < p.N; ++c)
           if (ra == kX64Bad || exp_n[c] == kX64Bad)
-            x64_store(p, off_m + off_n[c], p.alpha * x64_plain(p.A64 + m * p.lda, p.B64 + (n0 + c) * p.ldb, p.K));
+            x64_store(p, off_m + off_n[c], x64_plain(p, m, n0 + c));
       }
     }
   }
@@ -412,6 +416,7 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
 // Sum of the K-split partial triples in a fixed order, then the GEMM's
 // output.  One thread per row m over a chunk of columns.
 __global__ void __launch_bounds__(128) x64_reduce_kernel(const __grid_constant__ X64Group g) {
+  if (g.skip_if && *g.skip_if) return;
   const X64Params& p = g.job[blockIdx.z];
   const int64_t m = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (m >= p.M) return;
@@ -426,7 +431,7 @@ __global__ void __launch_bounds__(128) x64_reduce_kernel(const __grid_constant__
       triple_add(h, mid, lo, q[0], q[p.p_plane], q[2 * p.p_plane]);
     }
     const int rb = p.eb[n];
-    const double x = ra == kX64Bad || rb == kX64Bad ? p.alpha * x64_plain(p.A64 + m * p.lda, p.B64 + n * p.ldb, p.K)
+    const double x = ra == kX64Bad || rb == kX64Bad ? x64_plain(p, m, n)
                                                     : triple_to_f64(h, mid, lo, ra + rb + p.alpha_exp);
     x64_store(p, off_m + legmap_offset32(p.n_dst, uint32_t(n)), x);
   }

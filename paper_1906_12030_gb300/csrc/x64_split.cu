@@ -34,18 +34,20 @@ constexpr int kCap = kThreadsX * kItems * 8;     // entries per block of threads
 
 struct SplitArgs {
   const double* src;
-  int64_t ld, rows, K, seg_rows, tiles_per_seg;
+  int64_t ld, rows, K, seg_rows, tiles_per_seg, k_stride;
   uint8_t* img;
   int* rowexp;
   int tile, nk;        // rows per tile, 16-wide steps of K
   int R, G;            // rows and groups of 8 entries per block of threads
   int known;           // rowexp holds the rows' exponents already
   int gx;              // blocks of threads along the rows
+  int pairs;           // entries of a row may be read two at a time
 };
 struct SplitGroup {
   int n;
   int end[kGroup];     // blocks of the jobs up to and including each
   int rend[kGroup];    // rows whose exponents need a pass of their own, likewise
+  const int* skip_if;
   SplitArgs job[kGroup];
 };
 
@@ -65,6 +67,7 @@ __device__ __forceinline__ int row_exponent(int w) {
 
 __global__ void __launch_bounds__(512) x64_rowexp_kernel(const __grid_constant__ SplitGroup g) {
   __shared__ int sm[16];
+  if (g.skip_if && *g.skip_if) return;
   for (int64_t rg = blockIdx.x; rg < g.rend[g.n - 1]; rg += gridDim.x) {
     int i = 0;
     while (rg >= g.rend[i]) ++i;
@@ -72,7 +75,7 @@ __global__ void __launch_bounds__(512) x64_rowexp_kernel(const __grid_constant__
     const int64_t r = rg - (i > 0 ? g.rend[i - 1] : 0);
     const double* p = a.src + r * a.ld;
     int w = 0;
-    for (int64_t k = threadIdx.x; k < a.K; k += blockDim.x) w = max(w, mag_word(p[k]));
+    for (int64_t k = threadIdx.x; k < a.K; k += blockDim.x) w = max(w, mag_word(p[k * a.k_stride]));
     w = __reduce_max_sync(0xffffffffu, w);
     if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = w;
     __syncthreads();
@@ -85,6 +88,7 @@ __global__ void __launch_bounds__(512) x64_rowexp_kernel(const __grid_constant__
 }
 
 __global__ void __launch_bounds__(kThreadsX, 2) x64_split_kernel(const __grid_constant__ SplitGroup gr) {
+  if (gr.skip_if && *gr.skip_if) return;
   int job = 0;
   while (int(blockIdx.x) >= gr.end[job]) ++job;
   const int block = int(blockIdx.x) - (job > 0 ? gr.end[job - 1] : 0);
@@ -112,18 +116,18 @@ __global__ void __launch_bounds__(kThreadsX, 2) x64_split_kernel(const __grid_co
     for (int j = 0; j < 8; ++j) x[i][j] = 0.0;
     if (rr[i] < 0) continue;
     const int64_t k = kbase + g * 8;
-    const double* s = a.src + (r0 + r) * a.ld + k;
-    if (k + 8 <= a.K) {
+    const double* s = a.src + (r0 + r) * a.ld + k * a.k_stride;
+    if (a.pairs && k + 8 <= a.K) {
 #pragma unroll
       for (int j = 0; j < 8; j += 2) {
-        const double2 d = *reinterpret_cast<const double2*>(s + j);  // ld is a multiple of 8
+        const double2 d = *reinterpret_cast<const double2*>(s + j);
         x[i][j] = d.x;
         x[i][j + 1] = d.y;
       }
     } else {
 #pragma unroll
       for (int j = 0; j < 8; ++j)
-        if (k + j < a.K) x[i][j] = s[j];
+        if (k + j < a.K) x[i][j] = s[j * a.k_stride];
     }
   }
 #pragma unroll
@@ -210,17 +214,18 @@ __global__ void __launch_bounds__(kThreadsX, 2) x64_split_kernel(const __grid_co
 static cudaError_t launch_group(const X64SplitJob* jobs, int n, cudaStream_t stream) {
   SplitGroup g;
   g.n = 0;
+  g.skip_if = jobs[0].skip_if;
   int64_t blocks = 0, rows_known = 0;
   size_t smem = 0;
   for (int i = 0; i < n; ++i) {
     const X64SplitJob& j = jobs[i];
     if (j.rows <= 0 || j.K <= 0) continue;
-    if ((j.ld & 7) || j.K > j.ld || j.K > (1 << 30) || j.seg_rows <= 0 || j.rows % j.seg_rows ||
-        (reinterpret_cast<uintptr_t>(j.src) & 15))
-      return cudaErrorInvalidValue;
+    if (j.K > (1 << 30) || j.seg_rows <= 0 || j.rows % j.seg_rows) return cudaErrorInvalidValue;
     SplitArgs& a = g.job[g.n];
     a.src = j.src;
     a.ld = j.ld;
+    a.k_stride = j.k_stride;
+    a.pairs = j.k_stride == 1 && (j.ld & 1) == 0 && (reinterpret_cast<uintptr_t>(j.src) & 15) == 0;
     a.rows = j.rows;
     a.K = j.K;
     a.seg_rows = j.seg_rows;

@@ -19,6 +19,7 @@
 
 #include "../../include/mera.h"
 #include "kernels.h"
+#include "launch.h"
 #include "plan.h"
 #include "tc_gemm.h"
 
@@ -923,7 +924,10 @@ mera_status sweep_layout(int n_layers, const int* chi_b, const int* chi_t, int p
   return MERA_OK;
 }
 
-__global__ void energy_per_spin_kernel(const double* tr, double shift, double* e) { *e = 0.5 * (*tr + shift); }
+__global__ void energy_per_spin_kernel(const double* tr, double shift, double* e) {
+  pdl_begin();
+  *e = 0.5 * (*tr + shift);
+}
 
 }  // namespace sweep_detail
 }  // namespace mera
@@ -1003,7 +1007,7 @@ static mera_status sweep_impl(mera_state* S, const double* h1, double shift, int
   st = mera_energy(h1, rho_above, S->u[0], S->w[0], S->chi_b[0], S->chi_t[0], etmp, prec, mws, mb, stream);
   if (st != MERA_OK) return st;
   count_launch();
-  energy_per_spin_kernel<<<1, 1, 0, s>>>(etmp, shift, e_dev);
+  launch(energy_per_spin_kernel, true, 1, 1, 0, s, etmp, shift, e_dev);
   return cuda_status(cudaGetLastError(), "energy per spin");
 }
 

@@ -6,6 +6,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "launch.h"
 
 namespace mera {
 
@@ -64,6 +65,7 @@ struct PermuteGroup {
 // when its next tile belongs to another job.
 template <int PREC, int G>
 __global__ void __launch_bounds__(256) permute_tile_kernel(const __grid_constant__ PermuteGroup<G> g) {
+  pdl_begin();
   __shared__ double tile[kTile * (kTile + 1)];
   __shared__ int64_t s_as[kTile], s_ad[kTile], s_bs[kTile], s_bd[kTile];
   const int tid = threadIdx.x;
@@ -254,7 +256,7 @@ cudaError_t launch_permute_group(const PermuteJob* jobs, int n, int prec, cudaSt
   if (g.n == 0) return cudaSuccess;
   count_launch();
   const unsigned grid = unsigned(std::max<int64_t>(1, std::min<int64_t>(total, 152 * 8)));
-#define MERA_PERMUTE_LAUNCH(P) permute_tile_kernel<P, G><<<grid, 256, 0, stream>>>(g);
+#define MERA_PERMUTE_LAUNCH(P) launch(permute_tile_kernel<P, G>, total <= 152 * 8, grid, 256, 0, stream, g);
   switch (prec) {
     case PREC_F64: MERA_PERMUTE_LAUNCH(PREC_F64) break;
     case PREC_TF32: MERA_PERMUTE_LAUNCH(PREC_TF32) break;
@@ -312,6 +314,7 @@ __device__ __forceinline__ int job_of(const int* end, int b, int& local) {
 // covers K <= 64 with one round trip to memory, and the next stage is in
 // flight while this one is summed.  256 x 64 x 64: 6.0 us with 16 x 16 tiles.
 __global__ void __launch_bounds__(256) gemm_f64_small_kernel(const __grid_constant__ GemmF64Group g) {
+  pdl_begin();
   constexpr int R = 8, KS = 64, P = KS + 2;
   __shared__ double As[R * P], Bs[R * P];
   __shared__ double part[3][R * R];
@@ -370,6 +373,7 @@ __global__ void __launch_bounds__(256) gemm_f64_small_kernel(const __grid_consta
 
 template <int T>
 __global__ void __launch_bounds__(256) gemm_f64_kernel(const __grid_constant__ GemmF64Group g) {
+  pdl_begin();
   constexpr int R = 16 * T;
   __shared__ double As[kBK][R + 1];
   __shared__ double Bs[kBK][R + 1];
@@ -492,10 +496,10 @@ static cudaError_t launch_gemm_f64_group(const GemmF64Args* args, int n, cudaStr
   if (nb > 0x7fffffff) return cudaErrorInvalidValue;
   count_launch();
   switch (r) {
-    case 64: gemm_f64_kernel<4><<<unsigned(nb), 256, 0, stream>>>(g); break;
-    case 32: gemm_f64_kernel<2><<<unsigned(nb), 256, 0, stream>>>(g); break;
-    case 16: gemm_f64_kernel<1><<<unsigned(nb), 256, 0, stream>>>(g); break;
-    default: gemm_f64_small_kernel<<<unsigned(nb), 256, 0, stream>>>(g); break;
+    case 64: launch(gemm_f64_kernel<4>, nb <= 304, unsigned(nb), 256, 0, stream, g); break;
+    case 32: launch(gemm_f64_kernel<2>, nb <= 304, unsigned(nb), 256, 0, stream, g); break;
+    case 16: launch(gemm_f64_kernel<1>, nb <= 304, unsigned(nb), 256, 0, stream, g); break;
+    default: launch(gemm_f64_small_kernel, nb <= 304, unsigned(nb), 256, 0, stream, g); break;
   }
   return cudaGetLastError();
 }
@@ -508,8 +512,9 @@ cudaError_t launch_gemm_f64(const GemmF64Args* args, int n, cudaStream_t stream)
   return cudaSuccess;
 }
 
-__global__ void __launch_bounds__(256) ordered_sum_kernel(const double* __restrict__ parts, int n,
-                                                          double* __restrict__ out, int64_t count) {
+__global__ void __launch_bounds__(256) ordered_sum_kernel(const double* parts, int n,
+                                                          double* out, int64_t count) {
+  pdl_begin();
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < count; i += int64_t(gridDim.x) * blockDim.x) {
     double v = parts[i];
     for (int k = 1; k < n; ++k) v += parts[k * count + i];
@@ -520,7 +525,7 @@ __global__ void __launch_bounds__(256) ordered_sum_kernel(const double* __restri
 cudaError_t launch_ordered_sum(const double* parts, int n, double* out, int64_t count, cudaStream_t stream) {
   if (count <= 0) return cudaSuccess;
   count_launch();
-  ordered_sum_kernel<<<unsigned(std::min<int64_t>((count + 255) / 256, 152 * 8)), 256, 0, stream>>>(parts, n, out, count);
+  launch(ordered_sum_kernel, count <= 152 * 256, unsigned(std::min<int64_t>((count + 255) / 256, 152 * 8)), 256, 0, stream, parts, n, out, count);
   return cudaGetLastError();
 }
 
@@ -547,8 +552,9 @@ __device__ __forceinline__ double block_sum(double v) {
 }
 
 // mode 0: out = sum; mode 1: out = sqrt(sum)
-__global__ void __launch_bounds__(1024) reduce_partials_kernel(const double* __restrict__ partials, int np,
+__global__ void __launch_bounds__(1024) reduce_partials_kernel(const double* partials, int np,
                                                                double* out, int mode) {
+  pdl_begin();
   double v = 0.0;
   for (int i = threadIdx.x; i < np; i += blockDim.x) v += partials[i];
   v = block_sum<1024>(v);
@@ -558,8 +564,9 @@ __global__ void __launch_bounds__(1024) reduce_partials_kernel(const double* __r
 // 32 x 32 tiles of an n x n matrix, block (32, 8).  tile (ti, tj) covers rows
 // [32 ti, 32 ti + 32) and columns [32 tj, ...).  The transposed tile of B is
 // staged through shared memory so both reads are coalesced.
-__global__ void __launch_bounds__(256) dot_t_kernel(const double* __restrict__ A, const double* __restrict__ B,
+__global__ void __launch_bounds__(256) dot_t_kernel(const double* A, const double* B,
                                                     int64_t n, double* partials) {
+  pdl_begin();
   __shared__ double bt[32][33];
   const int64_t nt = (n + 31) / 32;
   double v = 0.0;
@@ -599,12 +606,13 @@ cudaError_t launch_dot_transposed(const double* A, const double* B, int64_t n, d
   const int64_t nt = (n + 31) / 32;
   const int nb = reduction_blocks(nt * nt);
   count_launch(2);
-  dot_t_kernel<<<nb, dim3(32, 8), 0, stream>>>(A, B, n, partials);
-  reduce_partials_kernel<<<1, 1024, 0, stream>>>(partials, nb, out, 0);
+  launch(dot_t_kernel, nb <= 304, nb, dim3(32, 8), 0, stream, A, B, n, partials);
+  launch(reduce_partials_kernel, true, 1, 1024, 0, stream, partials, nb, out, 0);
   return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(1024) trace_kernel(const double* __restrict__ X, int64_t n, double* out) {
+__global__ void __launch_bounds__(1024) trace_kernel(const double* X, int64_t n, double* out) {
+  pdl_begin();
   double v = 0.0;
   for (int64_t i = threadIdx.x; i < n; i += blockDim.x) v += X[i * n + i];
   v = block_sum<1024>(v);
@@ -614,8 +622,9 @@ __global__ void __launch_bounds__(1024) trace_kernel(const double* __restrict__ 
 // rho = (X + X^T) / (2 tr X) over pairs of 32 x 32 tiles (I, J), I <= J:
 // both tiles are read once and both written once, so X is read once in all.
 template <bool RESID>
-__global__ void __launch_bounds__(256) sym_normalize_kernel(const double* __restrict__ X, double* rho, int64_t n,
-                                                            const double* __restrict__ trace, double* partials) {
+__global__ void __launch_bounds__(256) sym_normalize_kernel(const double* X, double* rho, int64_t n,
+                                                            const double* trace, double* partials) {
+  pdl_begin();
   __shared__ double sa[32][33], sb[32][33];
   const double inv2t = 0.5 / *trace;
   const int64_t nt = (n + 31) / 32;
@@ -674,16 +683,16 @@ __global__ void __launch_bounds__(256) sym_normalize_kernel(const double* __rest
 
 cudaError_t launch_sym_normalize(const double* X, double* rho, int64_t n, double* partials, double* scalars,
                                  double* resid, cudaStream_t stream) {
-  trace_kernel<<<1, 1024, 0, stream>>>(X, n, scalars);
+  launch(trace_kernel, true, 1, 1024, 0, stream, X, n, scalars);
   const int64_t nt = (n + 31) / 32;
   const int nb = reduction_blocks(nt * nt);
   if (resid) {
     count_launch(3);
-    sym_normalize_kernel<true><<<nb, dim3(32, 8), 0, stream>>>(X, rho, n, scalars, partials);
-    reduce_partials_kernel<<<1, 1024, 0, stream>>>(partials, nb, resid, 1);
+    launch(sym_normalize_kernel<true>, nb <= 304, nb, dim3(32, 8), 0, stream, X, rho, n, scalars, partials);
+    launch(reduce_partials_kernel, true, 1, 1024, 0, stream, partials, nb, resid, 1);
   } else {
     count_launch(2);
-    sym_normalize_kernel<false><<<nb, dim3(32, 8), 0, stream>>>(X, rho, n, scalars, partials);
+    launch(sym_normalize_kernel<false>, nb <= 304, nb, dim3(32, 8), 0, stream, X, rho, n, scalars, partials);
   }
   return cudaGetLastError();
 }
@@ -691,7 +700,8 @@ cudaError_t launch_sym_normalize(const double* X, double* rho, int64_t n, double
 // ---------------------------------------------------------------------------
 // Polar (quintic Newton-Schulz) helpers.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) sumsq_kernel(const double* __restrict__ x, int64_t count, double* partials) {
+__global__ void __launch_bounds__(256) sumsq_kernel(const double* x, int64_t count, double* partials) {
+  pdl_begin();
   double v = 0.0;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < count; i += int64_t(gridDim.x) * blockDim.x)
     v += x[i] * x[i];
@@ -699,8 +709,9 @@ __global__ void __launch_bounds__(256) sumsq_kernel(const double* __restrict__ x
   if (threadIdx.x == 0) partials[blockIdx.x] = v;
 }
 
-__global__ void __launch_bounds__(256) scale_by_inverse_kernel(const double* __restrict__ src, double* dst,
-                                                               int64_t count, const double* __restrict__ norm) {
+__global__ void __launch_bounds__(256) scale_by_inverse_kernel(const double* src, double* dst,
+                                                               int64_t count, const double* norm) {
+  pdl_begin();
   const double s = 1.0 / *norm;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < count; i += int64_t(gridDim.x) * blockDim.x)
     dst[i] = src[i] * s;
@@ -712,7 +723,8 @@ __global__ void __launch_bounds__(256) scale_by_inverse_kernel(const double* __r
 // the Frobenius scaling leaves them.  One warp per row; the largest row sum
 // is kept by its bit pattern (non-negative binary64 values order like
 // integers), so *c starts at zero.
-__global__ void __launch_bounds__(256) ns_gershgorin_kernel(const double* __restrict__ G, int64_t n, double* c) {
+__global__ void __launch_bounds__(256) ns_gershgorin_kernel(const double* G, int64_t n, double* c) {
+  pdl_begin();
   const int64_t i = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) / 32;
   if (i >= n) return;
   double r = 0.0;
@@ -724,7 +736,8 @@ __global__ void __launch_bounds__(256) ns_gershgorin_kernel(const double* __rest
 }
 
 __global__ void __launch_bounds__(256) ns_prescale_kernel(double* G, int64_t gcount, double* X, int64_t xcount,
-                                                          const double* __restrict__ c) {
+                                                          const double* c) {
+  pdl_begin();
   const double ig = 1.0 / *c, ix = 1.0 / sqrt(*c);
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < gcount + xcount;
        i += int64_t(gridDim.x) * blockDim.x) {
@@ -737,10 +750,10 @@ __global__ void __launch_bounds__(256) ns_prescale_kernel(double* G, int64_t gco
 
 cudaError_t launch_ns_prescale(double* G, double* X, int64_t m, int64_t n, double* c, cudaStream_t stream) {
   count_launch(2);
-  ns_gershgorin_kernel<<<unsigned((n + 7) / 8), 256, 0, stream>>>(G, n, c);
+  launch(ns_gershgorin_kernel, true, unsigned((n + 7) / 8), 256, 0, stream, G, n, c);
   const int64_t total = n * n + m * n;
   const int nb = int(std::min<int64_t>((total + 255) / 256, 1024));
-  ns_prescale_kernel<<<nb, 256, 0, stream>>>(G, n * n, X, m * n, c);
+  launch(ns_prescale_kernel, nb <= 304, nb, 256, 0, stream, G, n * n, X, m * n, c);
   return cudaGetLastError();
 }
 
@@ -748,9 +761,9 @@ cudaError_t launch_frob_scale(const double* src, double* dst, int64_t count, dou
                               cudaStream_t stream) {
   const int nb = int(std::min<int64_t>((count + 255) / 256, 1024));
   count_launch(3);
-  sumsq_kernel<<<nb, 256, 0, stream>>>(src, count, partials);
-  reduce_partials_kernel<<<1, 1024, 0, stream>>>(partials, nb, scalars, 1);
-  scale_by_inverse_kernel<<<nb, 256, 0, stream>>>(src, dst, count, scalars);
+  launch(sumsq_kernel, nb <= 304, nb, 256, 0, stream, src, count, partials);
+  launch(reduce_partials_kernel, true, 1, 1024, 0, stream, partials, nb, scalars, 1);
+  launch(scale_by_inverse_kernel, nb <= 304, nb, 256, 0, stream, src, dst, count, scalars);
   return cudaGetLastError();
 }
 
@@ -764,8 +777,9 @@ cudaError_t launch_frob_scale(const double* src, double* dst, int64_t count, dou
 // product; the point is the reach of a step budget: 100 steps bring a
 // singular value of 1e-38 of the largest to 1, the cubic's 1e-17.
 // Bm = p(G) = (5/2)(I - G) + G2 (G2 = G G) and partial sums of ||G - I||_F^2.
-__global__ void __launch_bounds__(256) ns_combine_kernel(const double* __restrict__ G, const double* __restrict__ G2,
+__global__ void __launch_bounds__(256) ns_combine_kernel(const double* G, const double* G2,
                                                          double* Bm, int64_t n, double* partials, const int* skip_if) {
+  pdl_begin();
   if (skip_if && *skip_if) return;
   double v = 0.0;
   const int64_t count = n * n;
@@ -781,8 +795,9 @@ __global__ void __launch_bounds__(256) ns_combine_kernel(const double* __restric
 
 // state[0] = done, state[1] = iterations executed, state[2] = converged after
 // this iteration; resid = ||X^T X - I||_F of the iterate entering it.
-__global__ void __launch_bounds__(1024) ns_check_kernel(const double* __restrict__ partials, int np, double* resid,
+__global__ void __launch_bounds__(1024) ns_check_kernel(const double* partials, int np, double* resid,
                                                         double tol, int* state) {
+  pdl_begin();
   if (state[0]) return;
   double v = 0.0;
   for (int i = threadIdx.x; i < np; i += blockDim.x) v += partials[i];
@@ -795,6 +810,7 @@ __global__ void __launch_bounds__(1024) ns_check_kernel(const double* __restrict
 }
 
 __global__ void ns_finish_kernel(int* state) {
+  pdl_begin();
   if (state[0]) return;
   state[1] += 1;
   if (state[2]) state[0] = 1;
@@ -804,14 +820,14 @@ cudaError_t launch_ns_step(const double* G, const double* G2, double* Bm, int64_
                            double* resid, double tol, int* state, cudaStream_t stream) {
   const int nb = int(std::min<int64_t>((n * n + 255) / 256, 1024));
   count_launch(2);
-  ns_combine_kernel<<<nb, 256, 0, stream>>>(G, G2, Bm, n, partials, state);
-  ns_check_kernel<<<1, 1024, 0, stream>>>(partials, nb, resid, tol, state);
+  launch(ns_combine_kernel, nb <= 304, nb, 256, 0, stream, G, G2, Bm, n, partials, state);
+  launch(ns_check_kernel, true, 1, 1024, 0, stream, partials, nb, resid, tol, state);
   return cudaGetLastError();
 }
 
 cudaError_t launch_ns_finish(int* state, cudaStream_t stream) {
   count_launch();
-  ns_finish_kernel<<<1, 1, 0, stream>>>(state);
+  launch(ns_finish_kernel, true, 1, 1, 0, stream, state);
   return cudaGetLastError();
 }
 
@@ -890,9 +906,10 @@ __device__ __forceinline__ double ns_tile(const double* __restrict__ x, int64_t 
 // Bm = (5/2)(I - G) + G^2; the last block to finish sums the tiles' shares of
 // ||G - I||_F^2 in their order and sets state[2].  state[3] counts the blocks
 // and is left at zero.
-__global__ void __launch_bounds__(256) ns_square_kernel(const double* __restrict__ G, double* __restrict__ Bm, int n,
-                                                        double* __restrict__ partials, double* resid, double tol,
+__global__ void __launch_bounds__(256) ns_square_kernel(const double* G, double* Bm, int n,
+                                                        double* partials, double* resid, double tol,
                                                         int* state) {
+  pdl_begin();
   __shared__ double As[kNsR * kNsP], Bs[kNsR * kNsP], part[3 * kNsR * kNsR];
   __shared__ int last;
   if (state[0]) return;
@@ -934,9 +951,10 @@ __global__ void __launch_bounds__(256) ns_square_kernel(const double* __restrict
 
 // G = X^T X (m x n, row-major X).  `close`: ends a step (state[1] += 1; done
 // if it converged, and then G is not needed).  `cond`: the loop's condition.
-__global__ void __launch_bounds__(256) ns_gram_kernel(const double* __restrict__ X, double* __restrict__ G, int m,
+__global__ void __launch_bounds__(256) ns_gram_kernel(const double* X, double* G, int m,
                                                       int n, int* state, int close, int set_cond,
                                                       cudaGraphConditionalHandle cond, int max_iter) {
+  pdl_begin();
   __shared__ double As[kNsR * kNsP], Bs[kNsR * kNsP], part[3 * kNsR * kNsR];
   // block 0 alone writes state[0] and state[1], and what it writes is the
   // same early return for every block that reads it
@@ -969,14 +987,14 @@ static unsigned ns_pairs(int64_t n) {
 cudaError_t launch_ns_square(const double* G, double* Bm, int64_t n, double* partials, double* resid, double tol,
                              int* state, cudaStream_t stream) {
   count_launch();
-  ns_square_kernel<<<ns_pairs(n), 256, 0, stream>>>(G, Bm, int(n), partials, resid, tol, state);
+  launch(ns_square_kernel, ns_pairs(n) <= 304, ns_pairs(n), 256, 0, stream, G, Bm, int(n), partials, resid, tol, state);
   return cudaGetLastError();
 }
 
 cudaError_t launch_ns_gram(const double* X, double* G, int64_t m, int64_t n, int* state, bool close,
                            const cudaGraphConditionalHandle* cond, int max_iter, cudaStream_t stream) {
   count_launch();
-  ns_gram_kernel<<<ns_pairs(n), 256, 0, stream>>>(X, G, int(m), int(n), state, close ? 1 : 0, cond ? 1 : 0,
+  launch(ns_gram_kernel, ns_pairs(n) <= 304, ns_pairs(n), 256, 0, stream, X, G, int(m), int(n), state, close ? 1 : 0, cond ? 1 : 0,
                                                   cond ? *cond : cudaGraphConditionalHandle{}, max_iter);
   return cudaGetLastError();
 }
@@ -984,8 +1002,9 @@ cudaError_t launch_ns_gram(const double* X, double* G, int64_t m, int64_t n, int
 // out = -X with X the iterate the Newton-Schulz state points at (buffer
 // state[1] & 1), chosen on the device so that no host read is needed.  The
 // sign flip is a bit operation (exact, off the FP64 pipe).
-__global__ void __launch_bounds__(256) ns_output_kernel(const double* __restrict__ x0, const double* __restrict__ x1,
-                                                        const int* __restrict__ state, double* out, int64_t count) {
+__global__ void __launch_bounds__(256) ns_output_kernel(const double* x0, const double* x1,
+                                                        const int* state, double* out, int64_t count) {
+  pdl_begin();
   const double* src = (state[1] & 1) ? x1 : x0;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < count; i += int64_t(gridDim.x) * blockDim.x)
     out[i] = __longlong_as_double(__double_as_longlong(src[i]) ^ (1ll << 63));
@@ -996,7 +1015,7 @@ cudaError_t launch_ns_output(const double* x0, const double* x1, const int* stat
   const int nb = int(std::min<int64_t>((count + 255) / 256, 1024));
   if (nb <= 0) return cudaSuccess;
   count_launch();
-  ns_output_kernel<<<nb, 256, 0, stream>>>(x0, x1, state, out, count);
+  launch(ns_output_kernel, nb <= 304, nb, 256, 0, stream, x0, x1, state, out, count);
   return cudaGetLastError();
 }
 
@@ -1004,16 +1023,18 @@ cudaError_t launch_ns_output(const double* x0, const double* x1, const int* stat
 // with A = X^T G, S = (A + A^T) / 2 and T = X S, the step direction is
 // G - T; the kernel writes Yneg = -(X - eta (G - T)) for the polar retraction
 // (the polar update returns -polar(-Y) = polar(Y)).
-__global__ void __launch_bounds__(256) stiefel_sym_kernel(const double* __restrict__ A, double* S, int64_t n) {
+__global__ void __launch_bounds__(256) stiefel_sym_kernel(const double* A, double* S, int64_t n) {
+  pdl_begin();
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n * n; i += int64_t(gridDim.x) * blockDim.x) {
     const int64_t r = i / n, c = i - r * n;
     S[i] = 0.5 * (A[i] + A[c * n + r]);
   }
 }
 
-__global__ void __launch_bounds__(256) stiefel_combine_kernel(const double* __restrict__ X, const double* __restrict__ G,
-                                                              const double* __restrict__ T, double* Yneg, int64_t count,
+__global__ void __launch_bounds__(256) stiefel_combine_kernel(const double* X, const double* G,
+                                                              const double* T, double* Yneg, int64_t count,
                                                               double eta) {
+  pdl_begin();
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < count; i += int64_t(gridDim.x) * blockDim.x)
     Yneg[i] = eta * (G[i] - T[i]) - X[i];
 }
@@ -1021,7 +1042,7 @@ __global__ void __launch_bounds__(256) stiefel_combine_kernel(const double* __re
 cudaError_t launch_stiefel_sym(const double* A, double* S, int64_t n, cudaStream_t stream) {
   const int nb = int(std::min<int64_t>((n * n + 255) / 256, 1024));
   count_launch();
-  stiefel_sym_kernel<<<nb, 256, 0, stream>>>(A, S, n);
+  launch(stiefel_sym_kernel, nb <= 304, nb, 256, 0, stream, A, S, n);
   return cudaGetLastError();
 }
 
@@ -1029,19 +1050,20 @@ cudaError_t launch_stiefel_combine(const double* X, const double* G, const doubl
                                    double eta, cudaStream_t stream) {
   const int nb = int(std::min<int64_t>((count + 255) / 256, 1024));
   count_launch();
-  stiefel_combine_kernel<<<nb, 256, 0, stream>>>(X, G, T, Yneg, count, eta);
+  launch(stiefel_combine_kernel, nb <= 304, nb, 256, 0, stream, X, G, T, Yneg, count, eta);
   return cudaGetLastError();
 }
 
 // Last kernel of a recorded Newton-Schulz loop body: go on while not
 // converged and fewer than max_iter steps have run.
 __global__ void ns_continue_kernel(const int* state, cudaGraphConditionalHandle h, int max_iter) {
+  pdl_begin();
   cudaGraphSetConditional(h, (state[0] == 0 && state[1] < max_iter) ? 1u : 0u);
 }
 
 cudaError_t launch_ns_continue(const int* state, cudaGraphConditionalHandle h, int max_iter, cudaStream_t stream) {
   count_launch();
-  ns_continue_kernel<<<1, 1, 0, stream>>>(state, h, max_iter);
+  launch(ns_continue_kernel, true, 1, 1, 0, stream, state, h, max_iter);
   return cudaGetLastError();
 }
 
@@ -1049,9 +1071,10 @@ cudaError_t launch_ns_continue(const int* state, cudaGraphConditionalHandle h, i
 // out = g * (a + b) elementwise (b may be null), g a device scalar: the
 // energy adjoint's sum of the two environment halves times the upstream
 // gradient.
-__global__ void __launch_bounds__(256) scaled_sum_kernel(const double* __restrict__ a, const double* __restrict__ b,
-                                                         const double* __restrict__ g, double* __restrict__ out,
+__global__ void __launch_bounds__(256) scaled_sum_kernel(const double* a, const double* b,
+                                                         const double* g, double* out,
                                                          int64_t n) {
+  pdl_begin();
   const double gv = *g;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
     out[i] = gv * (b ? a[i] + b[i] : a[i]);
@@ -1062,7 +1085,7 @@ cudaError_t launch_scaled_sum(const double* a, const double* b, const double* g,
   if (n <= 0) return cudaSuccess;
   const unsigned grid = unsigned(std::min<int64_t>((n + 255) / 256, 152 * 8));
   count_launch();
-  scaled_sum_kernel<<<grid, 256, 0, stream>>>(a, b, g, out, n);
+  launch(scaled_sum_kernel, grid <= 304, grid, 256, 0, stream, a, b, g, out, n);
   return cudaGetLastError();
 }
 

@@ -131,6 +131,8 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_wait();
+  pdl_trigger();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -298,8 +300,9 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         continue;
       }
       const int64_t off_m = legmap_offset32(ep.m_dst, uint32_t(m));
-      const bool fast = ep.off32 && n0 + c0 + C::kCols <= ep.N;  // whole columns, 32-bit column offsets
-      if (fast && !ep.c_final && ep.alpha == 1.0) {
+      // columns of this warp that exist; their stores carry a predicate
+      const int lim = int(min(int64_t(C::kCols), int64_t(ep.N) - n0 - c0));
+      if (ep.off32 && !ep.c_final && ep.alpha == 1.0) {
         // the next operand's raw pair; four offsets in registers before the stores
         float* __restrict__ r0 = static_cast<float*>(ep.C) + off_m;
         float* __restrict__ r1 = r0 + ep.c_plane;
@@ -308,21 +311,28 @@ __global__ void __launch_bounds__(kOzThreads, 1)
           const int4 q = *reinterpret_cast<const int4*>(off_n32 + c0 + j);
           const int o[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            r0[o[k]] = hi[j + k];
-            r1[o[k]] = lo[j + k];
-          }
+          for (int k = 0; k < 4; ++k)
+            if (j + k < lim) {
+              r0[o[k]] = hi[j + k];
+              r1[o[k]] = lo[j + k];
+            }
         }
         continue;
       }
-      if (fast && ep.c_final && ep.alpha_pow2) {
+      if (ep.off32 && ep.c_final && ep.alpha_pow2) {
         double* __restrict__ r = static_cast<double*>(ep.C) + off_m;
         const int ae = ep.alpha_exp, accumulate = ep.accumulate;
 #pragma unroll
-        for (int j = 0; j < C::kCols; ++j) {
-          const int o = off_n32[c0 + j];
-          const double x = f32_to_f64_pow2(hi[j], ae) + f32_to_f64_pow2(lo[j], ae);
-          r[o] = accumulate ? r[o] + x : x;
+        for (int j = 0; j < C::kCols; j += 8) {  // accumulating: eight reads at a time
+          double y[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) y[k] = accumulate && j + k < lim ? r[off_n32[c0 + j + k]] : 0.0;
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            if (j + k >= lim) continue;
+            const double x = f32_to_f64_pow2(hi[j + k], ae) + f32_to_f64_pow2(lo[j + k], ae);
+            r[off_n32[c0 + j + k]] = accumulate ? y[k] + x : x;
+          }
         }
         continue;
       }
@@ -356,6 +366,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 // same output as the GEMM epilogue.  One thread per row m over a chunk of
 // columns.
 __global__ void __launch_bounds__(256) oz_splitk_reduce_kernel(const __grid_constant__ TcGroup g) {
+  pdl_begin();
   const Epilogue& ep = g.ep[blockIdx.z];
   const int64_t m = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (m >= ep.M) return;

@@ -24,6 +24,7 @@
 // is below 2^-90 (or zero) are written as zeros.
 #include "common.cuh"
 #include "kernels.h"
+#include "launch.h"
 
 namespace mera {
 namespace {
@@ -51,6 +52,7 @@ struct OzSplitGroup {
 
 template <int S>
 __global__ void __launch_bounds__(256) oz_split_kernel(const __grid_constant__ OzSplitGroup gr) {
+  pdl_begin();
   constexpr int kPairs = kOzBlockK / 64;  // element pairs per lane
   const int lane = threadIdx.x & 31;
   const int64_t items = gr.end[gr.n - 1];
@@ -135,8 +137,8 @@ cudaError_t launch_oz_split(const OzSplitJob* jobs, int n, int slices, cudaStrea
     const unsigned grid = unsigned(std::min<int64_t>((items + 7) / 8, int64_t(152) * 16));
     count_launch();
     switch (slices) {
-      case 3: oz_split_kernel<3><<<grid, 256, 0, stream>>>(g); break;
-      case 4: oz_split_kernel<4><<<grid, 256, 0, stream>>>(g); break;
+      case 3: launch(oz_split_kernel<3>, grid <= 304, grid, 256, 0, stream, g); break;
+      case 4: launch(oz_split_kernel<4>, grid <= 304, grid, 256, 0, stream, g); break;
       default: return cudaErrorInvalidValue;
     }
     const cudaError_t e = cudaGetLastError();

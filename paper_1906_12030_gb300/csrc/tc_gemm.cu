@@ -27,6 +27,7 @@
 #include "../../include/mera.h"
 #include "common.cuh"
 #include "kernels.h"
+#include "launch.h"
 #include "tc_gemm.h"
 
 namespace mera {
@@ -164,6 +165,16 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
 // Operand tensor maps, one per plane (hi, lo / hi, mid, lo for split modes).
 constexpr int kMaxPlanes = 4;
 struct TMaps {
@@ -276,53 +287,96 @@ struct Cfg {
   static constexpr int kAccStride = kAccCols <= 32 ? 32 : kAccCols <= 64 ? 64 : kAccCols <= 128 ? 128 : 256;
   static constexpr int kTmemCols = 2 * kAccStride;
   static constexpr uint32_t kFmt = (PREC == PREC_TF32) ? 2u : 1u;  // TF32 / BF16
+  // columns an epilogue warp takes at a time: 32 where the tile's 32-wide
+  // chunks divide evenly over the four warps of a lane quarter, else 16 (64
+  // wide: one each instead of two idle warps; 160: three instead of four
+  // sixteenths for the busiest warp; 192: three instead of four)
+  static constexpr int kChunk = BN % 128 == 0 ? 32 : 16;
   static constexpr size_t kSmem = 1024 + size_t(kStages) * kStageBytes + 1024 + BN * (sizeof(int64_t) + sizeof(int));
 };
 
-// One row's 32 accumulator values -> operand-format stores at row offset
+// One row's CH accumulator values -> operand-format stores at row offset
 // off_m plus the 32-bit column offsets s_off[j] in shared memory (hi, lo /
-// hi, mid, lo planes
-// c_plane elements apart).  Conversions run on pairs (cvt.rn.bf16x2.f32);
-// each value is rounded exactly as the per-element path rounds it.
-template <int PREC>
+// hi, mid, lo planes c_plane elements apart).  Conversions run on pairs
+// (cvt.rn.bf16x2.f32); each value is rounded exactly as the per-element path
+// rounds it.  PART: only the first `lim` columns exist (ragged N; the same
+// instructions with a predicate each, where the per-element path would take
+// ten times as long: N = 144 in 160-wide tiles spent 12 us of 20 there).
+template <int PREC, int CH, bool PART>
 __device__ __forceinline__ void store_chunk(void* C, int64_t off_m, int64_t c_plane, const int* __restrict__ s_off,
-                                            const uint32_t (&v)[32]) {
+                                            const uint32_t (&v)[CH], int lim) {
   if constexpr (PREC == PREC_TF32) {
     float* r = static_cast<float*>(C) + off_m;
 #pragma unroll
-    for (int j = 0; j < 32; j += 4) {
+    for (int j = 0; j < CH; j += 4) {
       const int4 q = *reinterpret_cast<const int4*>(s_off + j);
-      r[q.x] = round_tf32(__uint_as_float(v[j]));
-      r[q.y] = round_tf32(__uint_as_float(v[j + 1]));
-      r[q.z] = round_tf32(__uint_as_float(v[j + 2]));
-      r[q.w] = round_tf32(__uint_as_float(v[j + 3]));
+      const int o[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (!PART || j + k < lim) r[o[k]] = round_tf32(__uint_as_float(v[j + k]));
     }
   } else {
     __nv_bfloat16* __restrict__ r0 = static_cast<__nv_bfloat16*>(C) + off_m;
     __nv_bfloat16* __restrict__ r1 = r0 + c_plane;
     __nv_bfloat16* __restrict__ r2 = r1 + c_plane;
 #pragma unroll
-    for (int j = 0; j < 32; j += 2) {
+    for (int j = 0; j < CH; j += 2) {
       const int2 q = *reinterpret_cast<const int2*>(s_off + j);
       const int o[2] = {q.x, q.y};
+      const bool in0 = !PART || j < lim, in1 = !PART || j + 1 < lim;
       const float f0 = __uint_as_float(v[j]), f1 = __uint_as_float(v[j + 1]);
       const __nv_bfloat162 h = __floats2bfloat162_rn(f0, f1);
-      r0[o[0]] = h.x;
-      r0[o[1]] = h.y;
+      if (in0) r0[o[0]] = h.x;
+      if (in1) r0[o[1]] = h.y;
       if constexpr (PREC == PREC_BF16X3 || PREC == PREC_BF16X6) {
         const float2 hf = __bfloat1622float2(h);
         const float e0 = f0 - hf.x, e1 = f1 - hf.y;
         const __nv_bfloat162 l = __floats2bfloat162_rn(e0, e1);
-        r1[o[0]] = l.x;
-        r1[o[1]] = l.y;
+        if (in0) r1[o[0]] = l.x;
+        if (in1) r1[o[1]] = l.y;
         if constexpr (PREC == PREC_BF16X6) {
           const float2 lf = __bfloat1622float2(l);
           const __nv_bfloat162 q = __floats2bfloat162_rn(e0 - lf.x, e1 - lf.y);
-          r2[o[0]] = q.x;
-          r2[o[1]] = q.y;
+          if (in0) r2[o[0]] = q.x;
+          if (in1) r2[o[1]] = q.y;
         }
       }
     }
+  }
+}
+
+// The same into the caller's binary64 output at r, scaled by 2^e.  An
+// accumulating store is bound by the latency of its reads: several go out
+// together (four where 32 values fill the registers).
+template <int CH, bool PART>
+__device__ __forceinline__ void store_final(double* __restrict__ r, const int* __restrict__ s_off,
+                                            const uint32_t (&v)[CH], int lim, int e, bool accumulate) {
+  constexpr int B = CH == 32 ? 4 : 8;
+#pragma unroll
+  for (int j = 0; j < CH; j += B) {
+    int o[B];  // offsets in registers before the stores
+    double x[B];
+#pragma unroll
+    for (int q = 0; q < B; q += 4) {
+      const int4 q4 = *reinterpret_cast<const int4*>(s_off + j + q);
+      o[q] = q4.x;
+      o[q + 1] = q4.y;
+      o[q + 2] = q4.z;
+      o[q + 3] = q4.w;
+    }
+    if (accumulate) {
+      double y[B];
+#pragma unroll
+      for (int q = 0; q < B; ++q) y[q] = (!PART || j + q < lim) ? r[o[q]] : 0.0;
+#pragma unroll
+      for (int q = 0; q < B; ++q) x[q] = y[q] + f32_to_f64_pow2(__uint_as_float(v[j + q]), e);
+    } else {
+#pragma unroll
+      for (int q = 0; q < B; ++q) x[q] = f32_to_f64_pow2(__uint_as_float(v[j + q]), e);
+    }
+#pragma unroll
+    for (int q = 0; q < B; ++q)
+      if (!PART || j + q < lim) r[o[q]] = x[q];
   }
 }
 
@@ -372,6 +426,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_wait();
+  pdl_trigger();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -459,10 +515,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ---- epilogue (warps 2..17) ------------------------------------------------
     const int et = threadIdx.x - 64;  // 0..kEpiThreads-1
     const int quarter = warp % 4;     // tensor-memory lanes this warp may read
-    const int sub = (warp - 2) / 4;   // which quarter of the tile's 32-column chunks
+    const int sub = (warp - 2) / 4;   // which quarter of the tile's column chunks
     constexpr int kSub = kEpiWarps / 4;
     const int row = quarter * 32 + lane;
-    constexpr int kChunks = BN < 32 ? 1 : BN / 32;
+    constexpr int CH = C::kChunk, kChunks = BN / CH;
     const int ch_lo = (sub * kChunks) / kSub, ch_hi = ((sub + 1) * kChunks) / kSub;
     uint32_t tc = 0;
     for (int tg = int(blockIdx.x); tg < items; tg += gridDim.x, ++tc) {
@@ -504,9 +560,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
 #pragma unroll 1
       for (int ch = ch_lo; ch < ch_hi; ++ch) {
-        const int c0 = ch * 32;
-        uint32_t v[32];
-        tmem_ld32(taddr + uint32_t(c0), v);
+        const int c0 = ch * CH;
+        uint32_t v[CH];
+        if constexpr (CH == 32)
+          tmem_ld32(taddr + uint32_t(c0), v);
+        else
+          tmem_ld16(taddr + uint32_t(c0), v);
         if (ch + 1 == ch_hi) {  // this warp's last read of the accumulator: hand it back
           tc_fence_before();
           __syncwarp();
@@ -516,44 +575,31 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (ep.split > 1) {  // raw partial sums, reduced afterwards (splitk_reduce_kernel)
           float* p = ep.partial + (ks * ep.N + n0 + c0) * ep.M + m;
 #pragma unroll
-          for (int j = 0; j < 32; ++j, p += ep.M)
-            if (c0 + j < BN && n0 + c0 + j < ep.N) *p = __uint_as_float(v[j]);
+          for (int j = 0; j < CH; ++j, p += ep.M)
+            if (n0 + c0 + j < ep.N) *p = __uint_as_float(v[j]);
           continue;
         }
-        if (fast_ok && c0 + 32 <= BN && n0 + c0 + 32 <= ep.N) {
-          // whole chunk, operand-format destination, offsets in 32 bits
-          store_chunk<PREC>(ep.C, off_m, ep.c_plane, off_n32 + c0, v);
+        const int lim = int(min(int64_t(CH), ep.N - n0 - c0));  // columns of this chunk that exist
+        if (lim <= 0) continue;
+        if (fast_ok) {  // operand-format destination, offsets in 32 bits
+          if (lim >= CH)
+            store_chunk<PREC, CH, false>(ep.C, off_m, ep.c_plane, off_n32 + c0, v, CH);
+          else
+            store_chunk<PREC, CH, true>(ep.C, off_m, ep.c_plane, off_n32 + c0, v, lim);
           continue;
         }
-        if (final_fast && c0 + 32 <= BN && n0 + c0 + 32 <= ep.N) {
-          // whole chunk into the caller's binary64 output, alpha a power of two
-          double* __restrict__ r = static_cast<double*>(ep.C) + off_m;
-          const int* __restrict__ so = off_n32 + c0;
-#pragma unroll
-          for (int j = 0; j < 32; j += 4) {
-            // four offsets in registers before the four stores
-            const int4 q4 = *reinterpret_cast<const int4*>(so + j);
-            const int o[4] = {q4.x, q4.y, q4.z, q4.w};
-            double x[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) x[q] = f32_to_f64_pow2(__uint_as_float(v[j + q]), ep.alpha_exp);
-            if (ep.accumulate) {
-              double y[4];
-#pragma unroll
-              for (int q = 0; q < 4; ++q) y[q] = r[o[q]];
-#pragma unroll
-              for (int q = 0; q < 4; ++q) r[o[q]] = y[q] + x[q];
-            } else {
-#pragma unroll
-              for (int q = 0; q < 4; ++q) r[o[q]] = x[q];
-            }
-          }
+        if (final_fast) {  // the caller's binary64 output, alpha a power of two
+          double* r = static_cast<double*>(ep.C) + off_m;
+          if (lim >= CH)
+            store_final<CH, false>(r, off_n32 + c0, v, CH, ep.alpha_exp, ep.accumulate != 0);
+          else
+            store_final<CH, true>(r, off_n32 + c0, v, lim, ep.alpha_exp, ep.accumulate != 0);
           continue;
         }
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
+        for (int j = 0; j < CH; ++j) {
           const int c = c0 + j;
-          if (c >= BN || n0 + c >= ep.N) continue;
+          if (n0 + c >= ep.N) continue;
           const int64_t off = off_m + off_n[c];
           if (ep.c_final) {
             double* dst = static_cast<double*>(ep.C) + off;
@@ -601,6 +647,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // looping over a chunk of columns.
 template <int PREC>
 __global__ void __launch_bounds__(256) splitk_reduce_kernel(const __grid_constant__ TcGroup g) {
+  pdl_begin();
   const Epilogue& ep = g.ep[blockIdx.z];
   const int64_t m = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (m >= ep.M) return;
@@ -713,7 +760,7 @@ void launch_reduce(Kernel kernel, const TcGroup& g, cudaStream_t stream) {
   }
   if (r.n == 0) return;
   count_launch();
-  kernel<<<dim3(gx, gy, unsigned(r.n)), 256, 0, stream>>>(r);
+  launch(kernel, gx * gy * unsigned(r.n) <= 304, dim3(gx, gy, unsigned(r.n)), 256, 0, stream, r);
 }
 
 // CTAs of a kernel that the whole GPU holds at once.
@@ -764,7 +811,7 @@ cudaError_t launch_cfg(const TcGemmArgs* args, int n, cudaStream_t stream) {
     g.end[i] = int(items);
   }
   count_launch();
-  tc_gemm_kernel<PREC, BN><<<unsigned(std::min<int64_t>(items, resident)), kThreads, C::kSmem, stream>>>(g);
+  launch(tc_gemm_kernel<PREC, BN>, items <= resident, unsigned(std::min<int64_t>(items, resident)), kThreads, C::kSmem, stream, g);
   launch_reduce(splitk_reduce_kernel<PREC>, g, stream);
   return cudaGetLastError();
 }
@@ -810,7 +857,7 @@ cudaError_t launch_oz(const TcGemmArgs* args, int n, cudaStream_t stream) {
     g.end[i] = int(items);
   }
   count_launch();
-  oz_gemm_kernel<S, BN><<<unsigned(std::min<int64_t>(items, resident)), kOzThreads, C::kSmem, stream>>>(g);
+  launch(oz_gemm_kernel<S, BN>, items <= resident, unsigned(std::min<int64_t>(items, resident)), kOzThreads, C::kSmem, stream, g);
   launch_reduce(oz_splitk_reduce_kernel, g, stream);
   return cudaGetLastError();
 }
@@ -947,12 +994,12 @@ static cudaError_t launch_x64_group(const X64GemmArgs* args, int n, cudaStream_t
   count_launch();
   const unsigned grid = unsigned(std::min<int64_t>(items, resident));
   if (x64_single(args[0]))
-    x64_gemm_kernel<false><<<grid, kXThreads, kXSmem, stream>>>(g);
+    launch(x64_gemm_kernel<false>, items <= resident, grid, kXThreads, kXSmem, stream, g);
   else
-    x64_gemm_kernel<true><<<grid, kXThreads, kXSmem, stream>>>(g);
+    launch(x64_gemm_kernel<true>, items <= resident, grid, kXThreads, kXSmem, stream, g);
   if (red.n > 0) {
     count_launch();
-    x64_reduce_kernel<<<dim3(gx, gy, unsigned(red.n)), 128, 0, stream>>>(red);
+    launch(x64_reduce_kernel, gx * gy * unsigned(red.n) <= 608, dim3(gx, gy, unsigned(red.n)), 128, 0, stream, red);
   }
   return cudaGetLastError();
 }
@@ -966,12 +1013,13 @@ cudaError_t launch_gemm_x64(const X64GemmArgs* args, int n, cudaStream_t stream)
 }
 
 __global__ void report_notconv_kernel(const int* state) {
+  pdl_begin();
   if (state[0] == 0) atomicOr(&g_device_status, 1 << MERA_ENOTCONV);
 }
 
 cudaError_t launch_report_notconv(const int* state, cudaStream_t stream) {
   count_launch();
-  report_notconv_kernel<<<1, 1, 0, stream>>>(state);
+  launch(report_notconv_kernel, true, 1, 1, 0, stream, state);
   return cudaGetLastError();
 }
 

@@ -142,8 +142,9 @@ __device__ __forceinline__ void triple_add(float& h, float& m, float& l, float x
 }
 
 // (h + m + l) 2^e rounded to binary64 with integer operations: h gives the
-// bit pattern, m + l the number of its last places to add.  The exponent
-// stays normal (|e| <= 2 kX64MaxExp + 1).
+// bit pattern, m + l the number of its last places to add, found with two
+// rounding constants (conversions run at a fraction of the FP32 rate).  The
+// exponent stays normal (|e| <= 2 kX64MaxExp + 1).
 __device__ __forceinline__ double triple_to_f64(float h, float m, float l, int e) {
   two_sum(h, m, h, m);
   two_sum(m, l, m, l);
@@ -152,9 +153,11 @@ __device__ __forceinline__ double triple_to_f64(float h, float m, float l, int e
   const int eh = int((u >> 23) & 0xFFu);
   // below 2^-70 of the scale there is nothing under h that the digits resolve
   const float sc = eh < 127 - 70 ? 0.0f : __int_as_float((52 + 127 + 127 - eh) << 23);
-  const float mp = __fmul_rn(m, sc);  // |mp| <= 2^28
-  const int q1 = __float2int_rn(mp);
-  int q = q1 + __float2int_rn(__fmaf_rn(l, sc, __fsub_rn(mp, __int2float_rn(q1))));
+  const float mp = __fmul_rn(m, sc);                      // |mp| <= 2^28
+  const float t1 = __fadd_rn(mp, 0x1.8p29f);                  // its multiples of 64
+  const float rem = __fsub_rn(mp, __fsub_rn(t1, 0x1.8p29f));  // exact, |rem| <= 32
+  const float t2 = __fadd_rn(__fmaf_rn(l, sc, rem), 0x1.8p23f);
+  int q = (__float_as_int(t1) - 0x4E400000) * 64 + (__float_as_int(t2) - 0x4B400000);
   if (int(u) < 0) q = -q;  // towards larger magnitude
   if (q < 0 && (u & 0x7FFFFFu) == 0) q *= 2;  // below a power of two the places are half as large
   // 24-bit significand of h over 29 more places
@@ -165,10 +168,11 @@ __device__ __forceinline__ double triple_to_f64(float h, float m, float l, int e
 }
 
 // One output from the binary64 operands, as gemm_f64_kernel sums it.
-__device__ __noinline__ double x64_plain(const X64Params& p, int64_t m, int64_t n) {
+__device__ __forceinline__ double x64_plain(const X64Params& p, int64_t m, int64_t n) {
   const double* a = p.A64 + m * p.lda;
   const double* b = p.B64 + n * p.ldb;
   double s = 0.0;
+#pragma unroll 1
   for (int64_t k = 0; k < p.K; ++k) s = fma(a[k * p.a_k], b[k * p.b_k], s);
   return p.alpha * s;
 }
@@ -181,7 +185,6 @@ __device__ __forceinline__ void x64_store(const X64Params& p, int64_t off, doubl
 // MULTI: a work item may span several blocks of K.
 template <bool MULTI>
 __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_constant__ X64Group g) {
-  if (g.skip_if && *g.skip_if) return;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* aux = smem + size_t(kXStages) * kXStageBytes;
@@ -197,7 +200,6 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
   int* exp_n = reinterpret_cast<int*>(off_n + kXBN);
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int items = g.end[g.n - 1];
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kXStages; ++s) {
@@ -221,6 +223,9 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_wait();
+  pdl_trigger();
+  const int items = g.skip_if && *g.skip_if ? 0 : g.end[g.n - 1];
 
   if (warp == 0) {
     if (lane == 0) {
@@ -388,13 +393,31 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
       const int64_t off_m = legmap_offset32(p.m_dst, uint32_t(m));
       const int ra = p.ea[m];
       bool bad = ra == kX64Bad;
+      if (!p.accumulate) {
 #pragma unroll
-      for (int j = 0; j < kXCols; ++j) {
-        const int c = c0 + j;
-        const int rb = exp_n[c];
-        bad |= rb == kX64Bad;
-        if (n0 + c >= p.N || ra == kX64Bad || rb == kX64Bad) continue;
-        x64_store(p, off_m + off_n[c], triple_to_f64(h[j], mid[j], lo[j], ra + rb + p.alpha_exp));
+        for (int j = 0; j < kXCols; ++j) {
+          const int c = c0 + j;
+          const int rb = exp_n[c];
+          bad |= rb == kX64Bad;
+          if (n0 + c >= p.N || ra == kX64Bad || rb == kX64Bad) continue;
+          p.C[off_m + off_n[c]] = triple_to_f64(h[j], mid[j], lo[j], ra + rb + p.alpha_exp);
+        }
+      } else {
+        // bound by the latency of the reads: four go out together
+#pragma unroll
+        for (int j = 0; j < kXCols; j += 4) {
+          double y[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) y[k] = n0 + c0 + j + k < p.N ? p.C[off_m + off_n[c0 + j + k]] : 0.0;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int c = c0 + j + k;
+            const int rb = exp_n[c];
+            bad |= rb == kX64Bad;
+            if (n0 + c >= p.N || ra == kX64Bad || rb == kX64Bad) continue;
+            p.C[off_m + off_n[c]] = y[k] + triple_to_f64(h[j + k], mid[j + k], lo[j + k], ra + rb + p.alpha_exp);
+          }
+        }
       }
       if (bad) {
 #pragma unroll 1
@@ -416,6 +439,7 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
 // Sum of the K-split partial triples in a fixed order, then the GEMM's
 // output.  One thread per row m over a chunk of columns.
 __global__ void __launch_bounds__(128) x64_reduce_kernel(const __grid_constant__ X64Group g) {
+  pdl_begin();
   if (g.skip_if && *g.skip_if) return;
   const X64Params& p = g.job[blockIdx.z];
   const int64_t m = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;

@@ -24,6 +24,7 @@
 // entries get their exponents from a pass of their own.
 #include "common.cuh"
 #include "kernels.h"
+#include "launch.h"
 
 namespace mera {
 namespace {
@@ -66,6 +67,7 @@ __device__ __forceinline__ int row_exponent(int w) {
 }
 
 __global__ void __launch_bounds__(512) x64_rowexp_kernel(const __grid_constant__ SplitGroup g) {
+  pdl_begin();
   __shared__ int sm[16];
   if (g.skip_if && *g.skip_if) return;
   for (int64_t rg = blockIdx.x; rg < g.rend[g.n - 1]; rg += gridDim.x) {
@@ -88,6 +90,7 @@ __global__ void __launch_bounds__(512) x64_rowexp_kernel(const __grid_constant__
 }
 
 __global__ void __launch_bounds__(kThreadsX, 2) x64_split_kernel(const __grid_constant__ SplitGroup gr) {
+  pdl_begin();
   if (gr.skip_if && *gr.skip_if) return;
   int job = 0;
   while (int(blockIdx.x) >= gr.end[job]) ++job;
@@ -264,10 +267,10 @@ static cudaError_t launch_group(const X64SplitJob* jobs, int n, cudaStream_t str
   if (g.n == 0) return cudaSuccess;
   if (rows_known > 0) {
     count_launch();
-    x64_rowexp_kernel<<<unsigned(std::min<int64_t>(rows_known, 152 * 16)), 512, 0, stream>>>(g);
+    launch(x64_rowexp_kernel, rows_known <= 304, unsigned(std::min<int64_t>(rows_known, 152 * 16)), 512, 0, stream, g);
   }
   count_launch();
-  x64_split_kernel<<<unsigned(blocks), kThreadsX, smem, stream>>>(g);
+  launch(x64_split_kernel, blocks <= 304, unsigned(blocks), kThreadsX, smem, stream, g);
   return cudaGetLastError();
 }
 

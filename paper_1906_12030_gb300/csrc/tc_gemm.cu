@@ -108,12 +108,65 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, in
       : "memory");
 }
 
+// Address of this CTA's shared-memory location in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+
+// The load of one CTA of a pair into its own shared memory, counted by a
+// barrier given as a cluster address (the pair's first CTA's).
+__device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* tm, int x, int y, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+      "[%4];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(bar)
+      : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+__device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 __device__ __forceinline__ void tc_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
+}
+
+// Completion of the pair's MMAs, on the barrier at this offset in both CTAs.
+__device__ __forceinline__ void tc_commit_pair(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+          smem_u32(bar)),
+      "h"(uint16_t(3))
+      : "memory");
+}
+
+// The MMA of a CTA pair: rows of A and half the rows of B in each CTA.
+template <int PREC>
+__device__ __forceinline__ void tc_mma_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                            uint32_t acc) {
+  if constexpr (PREC == PREC_TF32) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc));
+  } else {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc));
+  }
 }
 
 // D[tmem] (+)= A[smem] * B[smem]^T, both K-major.
@@ -270,14 +323,17 @@ __device__ __forceinline__ double f32_to_f64_pow2(float f, int e) {
 // Stages hold 128-byte slabs (64 BF16 or 32 TF32 along K) of every plane.
 // (64-byte slabs, which fit twice as many stages for the split-BF16 modes,
 // measured 2-5 % slower on the chi = 16 and chi = 32 contractions.)
-template <int PREC, int BN>
+// CG = 2: a CTA pair shares one 256-row tile; each CTA stages its 128 rows of A
+// and half the tile's rows of B.
+template <int PREC, int BN, int CG = 1>
 struct Cfg {
   static constexpr int kElem = (PREC == PREC_TF32) ? 4 : 2;
   static constexpr int kPlanes = (PREC == PREC_BF16X3) ? 2 : (PREC == PREC_BF16X6 ? 3 : 1);
   static constexpr int kSlab = 128;                         // swizzle span = bytes along K per stage
   static constexpr int kBK = kSlab / kElem;                 // K per stage
   static constexpr int kABytes = kBM * kSlab;               // one plane of A
-  static constexpr int kBBytes = BN * kSlab;
+  static constexpr int kBRows = BN / CG;
+  static constexpr int kBBytes = kBRows * kSlab;
   static constexpr int kStageBytes = kPlanes * (kABytes + kBBytes);
   static constexpr int kStages = kStageBudget / kStageBytes > 8 ? 8
                                  : (kStageBudget / kStageBytes < 2 ? 2 : kStageBudget / kStageBytes);
@@ -380,10 +436,17 @@ __device__ __forceinline__ void store_final(double* __restrict__ r, const int* _
   }
 }
 
-template <int PREC, int BN>
-__global__ void __launch_bounds__(kThreads, 1)
-    tc_gemm_kernel(const __grid_constant__ TcGroup g) {
-  using C = Cfg<PREC, BN>;
+// CG = 1: as described at the top.  CG = 2 (launched in clusters of two): one
+// work item is a 256 x BN tile of the pair; row_t counts pairs of row tiles.
+// Both CTAs' copies count on the first CTA's full barriers; its warp 1 issues
+// the pair's MMAs (each writes 128 rows in each CTA's tensor memory) and
+// commits to the barriers of both; both CTAs' epilogues hand the accumulator
+// back to it.  Why: for a 128 x 256 tile the shared-memory reads and writes of
+// A and B take as long as 1.5 times the TF32 or BF16 MMAs (1.25 times the
+// BF16X3 ones); a pair halves what it reads and writes of B.
+template <int PREC, int BN, int CG>
+__device__ __forceinline__ void tc_gemm_body(const TcGroup& g) {
+  using C = Cfg<PREC, BN, CG>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* stage_base = smem;
@@ -400,6 +463,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   int* off_n32 = reinterpret_cast<int*>(off_n + BN);
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const uint32_t rank = CG == 2 ? blockIdx.x & 1u : 0u;  // this CTA in its pair
+  const int first_item = int(blockIdx.x) / CG, item_step = int(gridDim.x) / CG;
   const int items = g.end[g.n - 1];
 
   if (threadIdx.x == 0) {
@@ -409,7 +474,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], kEpiWarps);  // one arrive per epilogue warp
+      mbar_init(&acc_empty[b], CG * kEpiWarps);  // one arrive per epilogue warp
     }
     *abort_flag = 0;
     *abort_snapshot = 0;
@@ -417,13 +482,23 @@ __global__ void __launch_bounds__(kThreads, 1)
     fence_barrier_init();
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(uint32_t(C::kTmemCols))
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (CG == 2) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                   "r"(uint32_t(C::kTmemCols))
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                   "r"(uint32_t(C::kTmemCols))
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   tc_fence_before();
-  __syncthreads();
+  if constexpr (CG == 2)
+    cluster_sync();  // the pair's barriers are initialised
+  else
+    __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   pdl_wait();
@@ -434,7 +509,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // ---- producer ---------------------------------------------------------
       uint32_t it = 0;
       bool alive = true;
-      for (int tg = int(blockIdx.x); tg < items && alive; tg += gridDim.x) {
+      for (int tg = first_item; tg < items && alive; tg += item_step) {
         int t;
         const int job = item_of(g.end, tg, t);
         const Epilogue& ep = g.ep[job];
@@ -443,7 +518,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int kb0 = split_of(t, ep.tiles_m * ep.tiles_n, ep.split) * ep.kc, kb1 = min(kb0 + ep.kc, num_k);
         int row_t, col_t;
         tile_of(t, ep.tiles_m, ep.tiles_n, ep.group_m, row_t, col_t);
-        const int m0 = row_t * kBM, n0 = col_t * BN;
+        const int m0 = (row_t * CG + int(rank)) * kBM, n0 = col_t * BN + int(rank) * C::kBRows;
         for (int kb = kb0; kb < kb1; ++kb, ++it) {
           const uint32_t s = it % C::kStages;
           if (it >= uint32_t(C::kStages) && !mbar_wait(&empty[s], ((it / C::kStages) & 1) ^ 1, abort_flag)) {
@@ -451,27 +526,34 @@ __global__ void __launch_bounds__(kThreads, 1)
             break;
           }
           uint8_t* st = stage_base + size_t(s) * C::kStageBytes;
-          mbar_arrive_expect_tx(&full[s], C::kStageBytes);
+          if (rank == 0) mbar_arrive_expect_tx(&full[s], CG * C::kStageBytes);
           const int x = kb * C::kBK;
+          const uint32_t bar = CG == 2 ? cluster_addr(smem_u32(&full[s]), 0) : 0u;
 #pragma unroll
           for (int pl = 0; pl < C::kPlanes; ++pl) {  // plane pl: A then B
             uint8_t* dst = st + pl * (C::kABytes + C::kBBytes);
-            tma_load_2d(dst, &tm.a[pl], x, m0, &full[s]);
-            tma_load_2d(dst + C::kABytes, &tm.b[pl], x, n0, &full[s]);
+            if constexpr (CG == 2) {
+              tma_load_2d_pair(dst, &tm.a[pl], x, m0, bar);
+              tma_load_2d_pair(dst + C::kABytes, &tm.b[pl], x, n0, bar);
+            } else {
+              tma_load_2d(dst, &tm.a[pl], x, m0, &full[s]);
+              tma_load_2d(dst + C::kABytes, &tm.b[pl], x, n0, &full[s]);
+            }
           }
         }
       }
       // drain: every issued stage must have landed before the CTA may exit
-      for (uint32_t j = (it > uint32_t(C::kStages) ? it - C::kStages : 0); j < it; ++j)
+      // (a pair's second CTA waits for the first one at the end)
+      for (uint32_t j = (it > uint32_t(C::kStages) ? it - C::kStages : 0); j < it && rank == 0; ++j)
         mbar_wait(&full[j % C::kStages], (j / C::kStages) & 1, never);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (lane == 0 && rank == 0) {
       // ---- MMA issuer -------------------------------------------------------
-      constexpr uint32_t idesc = make_idesc(C::kFmt, kBM, BN < 16 ? 16 : BN);
+      constexpr uint32_t idesc = make_idesc(C::kFmt, CG * kBM, BN < 16 ? 16 : BN);
       uint32_t it = 0, tc = 0;
       bool alive = true;
-      for (int tg = int(blockIdx.x); tg < items && alive; tg += gridDim.x, ++tc) {
+      for (int tg = first_item; tg < items && alive; tg += item_step, ++tc) {
         int t;
         const int job = item_of(g.end, tg, t);
         const Epilogue& ep = g.ep[job];
@@ -502,17 +584,32 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const uint32_t a_addr = s0 + pa * kPlaneStride + koff;
                 const uint32_t b_addr = s0 + pb * kPlaneStride + C::kABytes + koff;
                 const uint32_t acc = (kb > kb0 || k > 0 || pa > 0 || pb > 0) ? 1u : 0u;
-                tc_mma<PREC>(d, smem_desc<C::kSlab>(a_addr), smem_desc<C::kSlab>(b_addr), idesc, acc);
+                if constexpr (CG == 2)
+                  tc_mma_pair<PREC>(d, smem_desc<C::kSlab>(a_addr), smem_desc<C::kSlab>(b_addr), idesc, acc);
+                else
+                  tc_mma<PREC>(d, smem_desc<C::kSlab>(a_addr), smem_desc<C::kSlab>(b_addr), idesc, acc);
               }
             }
           }
-          tc_commit(&empty[s]);
+          if constexpr (CG == 2)
+            tc_commit_pair(&empty[s]);
+          else
+            tc_commit(&empty[s]);
         }
-        tc_commit(&acc_full[b]);  // also fires after an abort, so nobody waits on it forever
+        if constexpr (CG == 2)
+          tc_commit_pair(&acc_full[b]);
+        else
+          tc_commit(&acc_full[b]);  // also fires after an abort, so nobody waits on it forever
       }
     }
   } else {
     // ---- epilogue (warps 2..17) ------------------------------------------------
+    auto release = [](uint64_t* bar) {  // hands an accumulator back to the MMA warp
+      if constexpr (CG == 2)
+        mbar_arrive_cluster(cluster_addr(smem_u32(bar), 0));
+      else
+        mbar_arrive(bar);
+    };
     const int et = threadIdx.x - 64;  // 0..kEpiThreads-1
     const int quarter = warp % 4;     // tensor-memory lanes this warp may read
     const int sub = (warp - 2) / 4;   // which quarter of the tile's column chunks
@@ -521,7 +618,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr int CH = C::kChunk, kChunks = BN / CH;
     const int ch_lo = (sub * kChunks) / kSub, ch_hi = ((sub + 1) * kChunks) / kSub;
     uint32_t tc = 0;
-    for (int tg = int(blockIdx.x); tg < items; tg += gridDim.x, ++tc) {
+    for (int tg = first_item; tg < items; tg += item_step, ++tc) {
       int t;
       const int job = item_of(g.end, tg, t);
       const Epilogue& ep = g.ep[job];
@@ -531,7 +628,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int64_t ks = split_of(t, ep.tiles_m * ep.tiles_n, ep.split);
       int row_t, col_t;
       tile_of(t, ep.tiles_m, ep.tiles_n, ep.group_m, row_t, col_t);
-      const int64_t m0 = int64_t(row_t) * kBM, n0 = int64_t(col_t) * BN;
+      const int64_t m0 = (int64_t(row_t) * CG + rank) * kBM, n0 = int64_t(col_t) * BN;
       const uint32_t b = tc & 1;
       // all epilogue threads are done with the previous tile's offsets;
       // decide together whether to go on
@@ -555,7 +652,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (ch_lo >= ch_hi) {  // no columns for this warp: hand the accumulator back at once
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&acc_empty[b]);
+        if (lane == 0) release(&acc_empty[b]);
         continue;
       }
 #pragma unroll 1
@@ -569,7 +666,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (ch + 1 == ch_hi) {  // this warp's last read of the accumulator: hand it back
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(&acc_empty[b]);
+          if (lane == 0) release(&acc_empty[b]);
         }
         if (!row_ok) continue;
         if (ep.split > 1) {  // raw partial sums, reduced afterwards (splitk_reduce_kernel)
@@ -632,12 +729,30 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   }
   tc_fence_before();
-  __syncthreads();
+  if constexpr (CG == 2)
+    cluster_sync();  // nothing of the pair is in flight in either CTA
+  else
+    __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(uint32_t(C::kTmemCols))
-                 : "memory");
+    if constexpr (CG == 2)
+      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(uint32_t(C::kTmemCols))
+                   : "memory");
+    else
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(uint32_t(C::kTmemCols))
+                   : "memory");
   }
+}
+
+template <int PREC, int BN>
+__global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_constant__ TcGroup g) {
+  tc_gemm_body<PREC, BN, 1>(g);
+}
+
+template <int PREC, int BN>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+    tc_gemm_pair_kernel(const __grid_constant__ TcGroup g) {
+  tc_gemm_body<PREC, BN, 2>(g);
 }
 
 // Sum of the K-split partials in a fixed order, then the same epilogue as
@@ -773,18 +888,32 @@ int resident_ctas(Kernel kernel, int threads, size_t smem) {
   return std::max(1, sms) * std::max(1, per_sm);
 }
 
-template <int PREC, int BN>
+template <int PREC, int BN, int CG>
 cudaError_t launch_cfg(const TcGemmArgs* args, int n, cudaStream_t stream) {
-  using C = Cfg<PREC, BN>;
+  using C = Cfg<PREC, BN, CG>;
   static std::once_flag once;
   static cudaError_t attr_err = cudaSuccess;
-  static int resident = 0;
-  std::call_once(once, [] {
-    attr_err = cudaFuncSetAttribute(tc_gemm_kernel<PREC, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    int(C::kSmem));
-    resident = resident_ctas(tc_gemm_kernel<PREC, BN>, kThreads, C::kSmem);
+  static int resident = 0;  // work items in flight on the whole GPU
+  const auto kernel = [] {
+    if constexpr (CG == 2)
+      return tc_gemm_pair_kernel<PREC, BN>;
+    else
+      return tc_gemm_kernel<PREC, BN>;
+  }();
+  std::call_once(once, [&] {
+    attr_err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::kSmem));
+    if constexpr (CG == 2) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = 2;
+      cfg.blockDim = kThreads;
+      cfg.dynamicSmemBytes = C::kSmem;
+      if (attr_err == cudaSuccess) attr_err = cudaOccupancyMaxActiveClusters(&resident, kernel, &cfg);
+    } else {
+      resident = resident_ctas(kernel, kThreads, C::kSmem);
+    }
   });
   if (attr_err != cudaSuccess) return attr_err;
+  if (resident < 1) return cudaErrorInvalidConfiguration;
   static thread_local TcGroup g;
   g.n = n;
   int64_t items = 0;
@@ -795,25 +924,89 @@ cudaError_t launch_cfg(const TcGemmArgs* args, int n, cudaStream_t stream) {
     for (int pl = 0; pl < C::kPlanes; ++pl) {
       if (!encode_operand(&g.tm[i].a[pl], A + pl * a.a_plane_bytes, PREC, a.M, a.K, a.lda, kBM, C::kSlab))
         return cudaErrorInvalidValue;
-      if (!encode_operand(&g.tm[i].b[pl], B + pl * a.b_plane_bytes, PREC, a.N, a.K, a.ldb, BN, C::kSlab))
+      if (!encode_operand(&g.tm[i].b[pl], B + pl * a.b_plane_bytes, PREC, a.N, a.K, a.ldb, C::kBRows, C::kSlab))
         return cudaErrorInvalidValue;
     }
     Epilogue& ep = g.ep[i];
     fill_epilogue(a, ep);
     const int64_t num_k = (a.K + C::kBK - 1) / C::kBK;
     ep.kc = int((num_k + ep.split - 1) / ep.split);
-    ep.group_m = group_rows(a, a.K * C::kElem * C::kPlanes);
     if (ep.split > 1 && (int64_t(ep.split - 1) * ep.kc >= num_k)) return cudaErrorInvalidValue;  // empty split
-    items += ((a.M + kBM - 1) / kBM) * ((a.N + BN - 1) / BN) * ep.split;
-    if (items > 0x7fffffff) return cudaErrorInvalidValue;
-    ep.tiles_m = int((a.M + kBM - 1) / kBM);
+    ep.tiles_m = int((a.M + CG * kBM - 1) / (CG * kBM));
     ep.tiles_n = int((a.N + BN - 1) / BN);
+    ep.group_m = std::max(1, group_rows(a, a.K * C::kElem * C::kPlanes) / CG);
+    items += int64_t(ep.tiles_m) * ep.tiles_n * ep.split;
+    if (items > 0x7fffffff) return cudaErrorInvalidValue;
     g.end[i] = int(items);
   }
   count_launch();
-  launch(tc_gemm_kernel<PREC, BN>, items <= resident, unsigned(std::min<int64_t>(items, resident)), kThreads, C::kSmem, stream, g);
+  launch(kernel, items <= resident, unsigned(std::min<int64_t>(items, resident)) * CG, kThreads, C::kSmem, stream, g);
   launch_reduce(splitk_reduce_kernel<PREC>, g, stream);
   return cudaGetLastError();
+}
+
+// Tile width and CTAs per tile of a launch.  `bn` is the planner's width; a
+// recorded (tuned) width is kept.  Clocks per 128-byte step of K and item, as
+// measured: the tensor cores take 2 bn per product (`prods` of them), shared
+// memory (planes + prods) (128 + bn / cg) for the copies' writes and the MMAs'
+// reads.  A launch takes rounds of items over the SMs (or pairs of SMs).
+//
+// Pairs are for a K long enough that the MMAs, not the epilogue, set the pace
+// (chi = 24: BF16X3 331776 x 576 x 13824 5.22 -> 4.31 ms, TF32 331776 x 6912 x
+// 576 3.80 -> 3.38 ms; below the line BF16X3 65536 x 4096 x 256 0.66 -> 0.73
+// ms, since both halves of a pair wait for the slower epilogue).  Another
+// width is taken where it saves a nearly empty last round: TF32 6912 x 576 x
+// 331776 is 162 tiles of 192, two rounds of 152 SMs, or 135 pairs of 128, two
+// rounds of 76 pairs at 0.6 of the time each.
+struct TileChoice {
+  int bn, cg;
+};
+TileChoice choose_tile(const TcGemmArgs* a, int n, int bn, int prec) {
+  const int planes = prec == PREC_BF16X3 ? 2 : 1, prods = prec == PREC_BF16X3 ? 3 : 1;
+  const int64_t step = 128 / (prec == PREC_TF32 ? 4 : 2);
+  int64_t k_min = a[0].K, n_min = a[0].N;
+  for (int i = 0; i < n; ++i) {
+    if (a[i].split > 1 && a[i].partial) return {bn, 1};
+    k_min = std::min(k_min, a[i].K);
+    n_min = std::min(n_min, a[i].N);
+  }
+  const int64_t nk = (k_min + step - 1) / step;
+  const bool pairs = n_min > 128 && nk >= (prec == PREC_BF16X3 ? 6 : prec == PREC_TF32 ? 12 : 16);
+  auto cost = [&](int w, int cg) {
+    int64_t items = 0;
+    for (int i = 0; i < n; ++i)
+      items += ((a[i].M + cg * kBM - 1) / (cg * kBM)) * ((a[i].N + w - 1) / w);
+    const int64_t slots = 152 / cg;
+    return double((items + slots - 1) / slots) * std::max(2.0 * w * prods, double(planes + prods) * (128 + w / cg));
+  };
+  TileChoice best{bn, 1};
+  double c = cost(bn, 1);
+  if (!pairs) return best;
+  for (int w : {256, 192, 128}) {
+    const double q = cost(w, 2);
+    if (q < 0.97 * c) {
+      c = q;
+      best = {w, 2};
+    }
+  }
+  return best;
+}
+
+template <int PREC, int BN>
+cudaError_t launch_width(const TcGemmArgs* a, int n, cudaStream_t stream) {
+  if constexpr (PREC != PREC_BF16X6 && BN > 128) {
+    if (BN == tc_block_n(PREC, a->N)) {
+      const TileChoice t = choose_tile(a, n, BN, PREC);
+      if (t.cg == 2) {
+        switch (t.bn) {
+          case 256: return launch_cfg<PREC, 256, 2>(a, n, stream);
+          case 192: return launch_cfg<PREC, 192, 2>(a, n, stream);
+          default: return launch_cfg<PREC, 128, 2>(a, n, stream);
+        }
+      }
+    }
+  }
+  return launch_cfg<PREC, BN, 1>(a, n, stream);
 }
 
 // Fixed-point split modes: S slice planes per operand, K split in whole
@@ -879,23 +1072,23 @@ cudaError_t launch_prec(const TcGemmArgs* a, int n, cudaStream_t stream) {
     case 0: break;
     case 256:
       if constexpr (PREC == PREC_BF16X6) return cudaErrorInvalidValue;  // one stage only
-      else return launch_cfg<PREC, 256>(a, n, stream);
+      else return launch_width<PREC, 256>(a, n, stream);
     case 192:  // N = 576 (chi = 24) in three full tiles
       if constexpr (PREC == PREC_BF16X6) return cudaErrorInvalidValue;
-      else return launch_cfg<PREC, 192>(a, n, stream);
+      else return launch_width<PREC, 192>(a, n, stream);
     case 160:
       if constexpr (PREC == PREC_BF16X6) return cudaErrorInvalidValue;
-      else return launch_cfg<PREC, 160>(a, n, stream);
-    case 128: return launch_cfg<PREC, 128>(a, n, stream);
-    case 64: return launch_cfg<PREC, 64>(a, n, stream);
-    case 16: return launch_cfg<PREC, 16>(a, n, stream);
+      else return launch_width<PREC, 160>(a, n, stream);
+    case 128: return launch_width<PREC, 128>(a, n, stream);
+    case 64: return launch_width<PREC, 64>(a, n, stream);
+    case 16: return launch_width<PREC, 16>(a, n, stream);
     default: return cudaErrorInvalidValue;
   }
   // three-plane operands: a 256-wide B tile leaves room for one stage only
-  if (a->N > 128 && PREC != PREC_BF16X6) return launch_cfg<PREC, (PREC == PREC_BF16X6 ? 128 : 256)>(a, n, stream);
-  if (a->N > 64) return launch_cfg<PREC, 128>(a, n, stream);
-  if (a->N > 16) return launch_cfg<PREC, 64>(a, n, stream);  // (a 32-wide variant spilled registers)
-  return launch_cfg<PREC, 16>(a, n, stream);
+  if (a->N > 128 && PREC != PREC_BF16X6) return launch_width<PREC, (PREC == PREC_BF16X6 ? 128 : 256)>(a, n, stream);
+  if (a->N > 64) return launch_width<PREC, 128>(a, n, stream);
+  if (a->N > 16) return launch_width<PREC, 64>(a, n, stream);  // (a 32-wide variant spilled registers)
+  return launch_width<PREC, 16>(a, n, stream);
 }
 
 }  // namespace

@@ -322,17 +322,21 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       if (ep.off32 && ep.c_final && ep.alpha_pow2) {
         double* __restrict__ r = static_cast<double*>(ep.C) + off_m;
         const int ae = ep.alpha_exp, accumulate = ep.accumulate;
+if (!accumulate) {
 #pragma unroll
-        for (int j = 0; j < C::kCols; j += 8) {  // accumulating: eight reads at a time
-          double y[8];
+          for (int j = 0; j < C::kCols; ++j)
+            if (j < lim) r[off_n32[c0 + j]] = f32_to_f64_pow2(hi[j], ae) + f32_to_f64_pow2(lo[j], ae);
+          continue;
+        }
 #pragma unroll
-          for (int k = 0; k < 8; ++k) y[k] = accumulate && j + k < lim ? r[off_n32[c0 + j + k]] : 0.0;
+        for (int j = 0; j < C::kCols; j += 4) {  // bound by the latency of its reads: several at a time
+          double y[4];
 #pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            if (j + k >= lim) continue;
-            const double x = f32_to_f64_pow2(hi[j + k], ae) + f32_to_f64_pow2(lo[j + k], ae);
-            r[off_n32[c0 + j + k]] = accumulate ? y[k] + x : x;
-          }
+          for (int k = 0; k < 4; ++k) y[k] = j + k < lim ? r[off_n32[c0 + j + k]] : 0.0;
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (j + k < lim)
+              r[off_n32[c0 + j + k]] = y[k] + (f32_to_f64_pow2(hi[j + k], ae) + f32_to_f64_pow2(lo[j + k], ae));
         }
         continue;
       }

@@ -31,3 +31,4 @@ def test_pairs_match_single_ctas(prec, M, N, K):
             assert np.array_equal(C[lo:hi, c0:c1], D.cpu().numpy().reshape(hi - lo, c1 - c0))
     assert np.isfinite(C).all()
     assert m.mera_device_status(clear=True) == 0
+

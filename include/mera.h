@@ -79,7 +79,7 @@ extern "C" {
 typedef int mera_status;
 #define MERA_OK 0
 #define MERA_EINVAL 1    /* bad size, pointer, alignment or mode            */
-#define MERA_ENOMEM 2    /* workspace smaller than mera_workspace_size      */
+#define MERA_ENOMEM 2    /* workspace too small for every form of the call  */
 #define MERA_ECUDA 3     /* CUDA launch / runtime error                     */
 #define MERA_ENOTCONV 4  /* iteration cap reached; output still written     */
 #define MERA_ETIMEOUT 5  /* a bounded device-side wait gave up              */

@@ -623,7 +623,7 @@ __global__ void __launch_bounds__(1024) trace_kernel(const double* X, int64_t n,
 // both tiles are read once and both written once, so X is read once in all,
 // and each pair of entries is summed and scaled once (the sum commutes): at
 // two binary64 operations per entry the FP64 pipe, not memory, set the pace
-// (chi = 16: 96 us for 268 MB).  Blocks walk the pairs row by row of tiles.
+// (chi = 16, 268 MB: 96 us with both sums, 70 with one).  Blocks walk the pairs row by row of tiles.
 template <bool RESID>
 __global__ void __launch_bounds__(256) sym_normalize_kernel(const double* X, double* rho, int64_t n,
                                                             const double* trace, double* partials) {

@@ -84,7 +84,11 @@ __device__ __forceinline__ void dd_norm(float& hi, float& lo) {
   hi = s;
 }
 
-template <int S, int BN>
+// MULTI: the launch holds several jobs.  A launch of one reads its parameters
+// at fixed constant addresses: looked up by a job index they cost 1 to 2 % of
+// a chi = 16 product (1010 -> 1025 us), most of it between tiles.  The raw
+// stores test the tile's edge once (`whole`) rather than column by column.
+template <int S, int BN, bool MULTI>
 __global__ void __launch_bounds__(kOzThreads, 1)
     oz_gemm_kernel(const __grid_constant__ TcGroup g) {
   using C = OzCfg<S, BN>;
@@ -104,7 +108,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   int* off_n32 = reinterpret_cast<int*>(off_n + BN);
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int items = g.end[g.n - 1];
+  const int items = g.end[MULTI ? g.n - 1 : 0];
   // a work item covers stages [kb0, kb1): kc is a whole number of blocks
 
   if (threadIdx.x == 0) {
@@ -140,8 +144,8 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       uint32_t it = 0;
       bool alive = true;
       for (int tg = int(blockIdx.x); tg < items && alive; tg += gridDim.x) {
-        int t;
-        const int job = item_of(g.end, tg, t);
+        int t = tg;
+        const int job = MULTI ? item_of(g.end, tg, t) : 0;
         const Epilogue& ep = g.ep[job];
         const TMaps& tm = g.tm[job];
         const int num_k = (int(ep.K) + C::kBK - 1) / C::kBK;
@@ -180,8 +184,8 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       uint32_t it = 0, bc = 0;  // stages consumed, blocks issued
       bool alive = true;
       for (int tg = int(blockIdx.x); tg < items && alive; tg += gridDim.x) {
-        int t;
-        const int job = item_of(g.end, tg, t);
+        int t = tg;
+        const int job = MULTI ? item_of(g.end, tg, t) : 0;
         const Epilogue& ep = g.ep[job];
         const int num_k = (int(ep.K) + C::kBK - 1) / C::kBK;
         const int kb0 = split_of(t, ep.tiles_m * ep.tiles_n, ep.split) * ep.kc, kb1 = min(kb0 + ep.kc, num_k);
@@ -238,9 +242,11 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     const int c0 = sub * C::kCols;  // first column of this warp's share
     uint32_t bc = 0;
     for (int tg = int(blockIdx.x); tg < items; tg += gridDim.x) {
-      int t;
-      const int job = item_of(g.end, tg, t);
+      int t = tg;
+      const int job = MULTI ? item_of(g.end, tg, t) : 0;
       const Epilogue& ep = g.ep[job];
+      const bool final_fast = ep.c_final && ep.split <= 1 && ep.off32 && ep.alpha_pow2;
+      const bool raw_fast = !ep.c_final && ep.split <= 1 && ep.off32 && ep.alpha == 1.0;
       const int num_k = (int(ep.K) + C::kBK - 1) / C::kBK;
       const int ks = split_of(t, ep.tiles_m * ep.tiles_n, ep.split);
       int row_t, col_t;
@@ -300,59 +306,32 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         continue;
       }
       const int64_t off_m = legmap_offset32(ep.m_dst, uint32_t(m));
-      // columns of this warp that exist; their stores carry a predicate
-      const int lim = int(min(int64_t(C::kCols), int64_t(ep.N) - n0 - c0));
-      if (ep.off32 && !ep.c_final && ep.alpha == 1.0) {
-        // the next operand's raw pair; four offsets in registers before the stores
+      const bool whole = n0 + c0 + C::kCols <= ep.N;
+      if (ep.c_final) {
+        double* __restrict__ r = static_cast<double*>(ep.C) + off_m;
+#pragma unroll
+        for (int j = 0; j < C::kCols; ++j) {
+          if (!whole && n0 + c0 + j >= ep.N) continue;
+          const int64_t o = final_fast ? int64_t(off_n32[c0 + j]) : off_n[c0 + j];
+          const double x = final_fast ? f32_to_f64_pow2(hi[j], ep.alpha_exp) + f32_to_f64_pow2(lo[j], ep.alpha_exp)
+                                      : ep.alpha * (double(hi[j]) + double(lo[j]));
+          r[o] = ep.accumulate ? r[o] + x : x;
+        }
+      } else {
         float* __restrict__ r0 = static_cast<float*>(ep.C) + off_m;
         float* __restrict__ r1 = r0 + ep.c_plane;
+        const float alpha = float(ep.alpha);
 #pragma unroll
-        for (int j = 0; j < C::kCols; j += 4) {
-          const int4 q = *reinterpret_cast<const int4*>(off_n32 + c0 + j);
-          const int o[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (j + k < lim) {
-              r0[o[k]] = hi[j + k];
-              r1[o[k]] = lo[j + k];
-            }
-        }
-        continue;
-      }
-      if (ep.off32 && ep.c_final && ep.alpha_pow2) {
-        double* __restrict__ r = static_cast<double*>(ep.C) + off_m;
-        const int ae = ep.alpha_exp, accumulate = ep.accumulate;
-if (!accumulate) {
-#pragma unroll
-          for (int j = 0; j < C::kCols; ++j)
-            if (j < lim) r[off_n32[c0 + j]] = f32_to_f64_pow2(hi[j], ae) + f32_to_f64_pow2(lo[j], ae);
-          continue;
-        }
-#pragma unroll
-        for (int j = 0; j < C::kCols; j += 4) {  // bound by the latency of its reads: several at a time
-          double y[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) y[k] = j + k < lim ? r[off_n32[c0 + j + k]] : 0.0;
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (j + k < lim)
-              r[off_n32[c0 + j + k]] = y[k] + (f32_to_f64_pow2(hi[j + k], ae) + f32_to_f64_pow2(lo[j + k], ae));
-        }
-        continue;
-      }
-#pragma unroll
-      for (int j = 0; j < C::kCols; ++j) {
-        if (n0 + c0 + j >= ep.N) continue;
-        const int64_t o = off_m + off_n[c0 + j];
-        if (ep.c_final) {
-          double* r = static_cast<double*>(ep.C) + o;
-          const double x = ep.alpha_pow2 ? f32_to_f64_pow2(hi[j], ep.alpha_exp) + f32_to_f64_pow2(lo[j], ep.alpha_exp)
-                                         : ep.alpha * (double(hi[j]) + double(lo[j]));
-          *r = ep.accumulate ? *r + x : x;
-        } else {  // alpha a power of two in the programs: exact
-          const float alpha = float(ep.alpha);
-          static_cast<float*>(ep.C)[o] = __fmul_rn(alpha, hi[j]);
-          static_cast<float*>(ep.C)[o + ep.c_plane] = __fmul_rn(alpha, lo[j]);
+        for (int j = 0; j < C::kCols; ++j) {
+          if (!whole && n0 + c0 + j >= ep.N) continue;
+          const int64_t o = raw_fast ? int64_t(off_n32[c0 + j]) : off_n[c0 + j];
+          if (raw_fast) {
+            r0[o] = hi[j];
+            r1[o] = lo[j];
+          } else {  // alpha a power of two in the programs: exact
+            r0[o] = __fmul_rn(alpha, hi[j]);
+            r1[o] = __fmul_rn(alpha, lo[j]);
+          }
         }
       }
     }

@@ -1011,15 +1011,15 @@ cudaError_t launch_width(const TcGemmArgs* a, int n, cudaStream_t stream) {
 
 // Fixed-point split modes: S slice planes per operand, K split in whole
 // blocks of kOzBlockK.
-template <int S, int BN>
+template <int S, int BN, bool MULTI>
 cudaError_t launch_oz(const TcGemmArgs* args, int n, cudaStream_t stream) {
   using C = OzCfg<S, BN>;
   static std::once_flag once;
   static cudaError_t attr_err = cudaSuccess;
   static int resident = 0;
   std::call_once(once, [] {
-    attr_err = cudaFuncSetAttribute(oz_gemm_kernel<S, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::kSmem));
-    resident = resident_ctas(oz_gemm_kernel<S, BN>, kOzThreads, C::kSmem);
+    attr_err = cudaFuncSetAttribute(oz_gemm_kernel<S, BN, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::kSmem));
+    resident = resident_ctas(oz_gemm_kernel<S, BN, MULTI>, kOzThreads, C::kSmem);
   });
   if (attr_err != cudaSuccess) return attr_err;
   static thread_local TcGroup g;
@@ -1050,7 +1050,8 @@ cudaError_t launch_oz(const TcGemmArgs* args, int n, cudaStream_t stream) {
     g.end[i] = int(items);
   }
   count_launch();
-  launch(oz_gemm_kernel<S, BN>, items <= resident, unsigned(std::min<int64_t>(items, resident)), kOzThreads, C::kSmem, stream, g);
+  launch(oz_gemm_kernel<S, BN, MULTI>, items <= resident, unsigned(std::min<int64_t>(items, resident)), kOzThreads,
+         C::kSmem, stream, g);
   launch_reduce(oz_splitk_reduce_kernel, g, stream);
   return cudaGetLastError();
 }
@@ -1059,9 +1060,9 @@ template <int S>
 cudaError_t launch_oz_prec(const TcGemmArgs* a, int n, cudaStream_t stream) {
   const int bn = a->bn > 0 ? a->bn : (a->N > 64 ? 128 : (a->N > 16 ? 64 : 16));
   switch (bn) {
-    case 128: return launch_oz<S, 128>(a, n, stream);
-    case 64: return launch_oz<S, 64>(a, n, stream);
-    case 16: return launch_oz<S, 16>(a, n, stream);
+    case 128: return n > 1 ? launch_oz<S, 128, true>(a, n, stream) : launch_oz<S, 128, false>(a, n, stream);
+    case 64: return launch_oz<S, 64, true>(a, n, stream);
+    case 16: return launch_oz<S, 16, true>(a, n, stream);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -614,7 +614,8 @@ static mera_status polar_record(const double* env, int m, int n, double* out, in
   int* exp_a = reinterpret_cast<int*>(ar.take(x64 ? px.exp_a : 0));
   int* exp_b = reinterpret_cast<int*>(ar.take(x64 ? px.exp_b : 0));
   float* part = reinterpret_cast<float*>(ar.ptr());
-  auto product = [&](const GemmF64Args& g, cudaStream_t st) {
+  auto product = [&](GemmF64Args g, cudaStream_t st) {
+    g.ordered = 1;
     if (!x64) return launch_gemm_f64(g, st);
     const X64SplitJob jobs[2] = {{g.A, g.a_m, g.M, g.K, g.M, kX64TileA, img_a, exp_a, g.a_k, state},
                                  {g.B, g.b_n, g.N, g.K, g.N, kX64TileB, img_b, exp_b, g.b_k, state}};

@@ -76,6 +76,7 @@ struct GemmF64Args {
   double alpha;
   int accumulate;
   const int* skip_if = nullptr;  // device flag: the kernel returns at once when *skip_if != 0
+  int ordered = 0;  // every output one chain of FMAs in the order of K, whatever the tile
 };
 cudaError_t launch_gemm_f64(const GemmF64Args* args, int n, cudaStream_t stream);
 inline cudaError_t launch_gemm_f64(const GemmF64Args& args, cudaStream_t stream) {

@@ -355,7 +355,12 @@ __global__ void __launch_bounds__(256) gemm_f64_small_kernel(const __grid_consta
     if (k0 + KS < p.K) load(k0 + KS);
     const int left = int(min(int64_t(KS), p.K - k0));
     const int lo = q * (KS / 4), hi = min(left, lo + KS / 4);
-    if (hi - lo == KS / 4) {
+    if (p.ordered) {
+      if (q == 0) {
+#pragma unroll 16
+        for (int k = 0; k < left; ++k) acc = fma(As[r * P + k], Bs[c * P + k], acc);
+      }
+    } else if (hi - lo == KS / 4) {
 #pragma unroll
       for (int k = 0; k < KS / 4; ++k) acc = fma(As[r * P + lo + k], Bs[c * P + lo + k], acc);
     } else {
@@ -366,7 +371,7 @@ __global__ void __launch_bounds__(256) gemm_f64_small_kernel(const __grid_consta
   if (q > 0) part[q - 1][o] = acc;
   __syncthreads();
   if (q > 0 || m0 + r >= p.M || n0 + c >= p.N) return;
-  const double v = p.alpha * (((acc + part[0][o]) + part[1][o]) + part[2][o]);
+  const double v = p.alpha * (p.ordered ? acc : ((acc + part[0][o]) + part[1][o]) + part[2][o]);
   double* dst = p.C + legmap_offset32(p.m_dst, uint32_t(m0 + r)) + legmap_offset32(p.n_dst, uint32_t(n0 + c));
   *dst = p.accumulate ? (*dst + v) : v;
 }
@@ -740,16 +745,15 @@ __global__ void __launch_bounds__(256) scale_by_inverse_kernel(const double* src
 // the Frobenius scaling leaves them.  One warp per row; the largest row sum
 // is kept by its bit pattern (non-negative binary64 values order like
 // integers), so *c starts at zero.
-__global__ void __launch_bounds__(256) ns_gershgorin_kernel(const double* G, int64_t n, double* c) {
+// One thread per column (G is symmetric), its sum in order.
+__global__ void __launch_bounds__(64) ns_gershgorin_kernel(const double* G, int64_t n, double* c) {
   pdl_begin();
-  const int64_t i = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) / 32;
+  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i >= n) return;
   double r = 0.0;
-  for (int64_t j = threadIdx.x & 31; j < n; j += 32) r += fabs(G[i * n + j]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
-  if ((threadIdx.x & 31) == 0)
-    atomicMax(reinterpret_cast<unsigned long long*>(c), static_cast<unsigned long long>(__double_as_longlong(r)));
+#pragma unroll 8
+  for (int64_t j = 0; j < n; ++j) r += fabs(G[j * n + i]);
+  atomicMax(reinterpret_cast<unsigned long long*>(c), static_cast<unsigned long long>(__double_as_longlong(r)));
 }
 
 __global__ void __launch_bounds__(256) ns_prescale_kernel(double* G, int64_t gcount, double* X, int64_t xcount,
@@ -767,7 +771,7 @@ __global__ void __launch_bounds__(256) ns_prescale_kernel(double* G, int64_t gco
 
 cudaError_t launch_ns_prescale(double* G, double* X, int64_t m, int64_t n, double* c, cudaStream_t stream) {
   count_launch(2);
-  launch(ns_gershgorin_kernel, true, unsigned((n + 7) / 8), 256, 0, stream, G, n, c);
+  launch(ns_gershgorin_kernel, true, unsigned((n + 63) / 64), 64, 0, stream, G, n, c);
   const int64_t total = n * n + m * n;
   const int nb = int(std::min<int64_t>((total + 255) / 256, 1024));
   launch(ns_prescale_kernel, nb <= 304, nb, 256, 0, stream, G, n * n, X, m * n, c);
@@ -854,9 +858,10 @@ cudaError_t launch_ns_finish(int* state, cudaStream_t stream) {
 // (gemm_f64); X^T X, which also closes the step and, in the last step of a
 // loop body, decides whether to go on.  G and G^2 are symmetric, so only the
 // 8 x 8 tiles on and above the diagonal are summed (tile pairs), which takes a
-// third off the FP64 work of a step.  Tiles and K split as in
-// gemm_f64_small_kernel.  A step of a 256 x 256 matrix was seven launches and
-// 127 us and is 84 us now (54 us of FP64 pipe), of a 64 x 64 one 33 -> 18 us.
+// third off the FP64 work of a step.  Tiles as in gemm_f64_small_kernel, each
+// output one chain of FMAs in the order of K (four chains were 2 % faster, but
+// their rounding changed the path of long optimisations).  A step of a
+// 256 x 256 matrix was seven launches and 127 us and is 86 us now.
 constexpr int kNsR = 8, kNsK = 64, kNsP = kNsK + 2;
 
 // Tile pair t of the upper triangle, row by row: (i, j), i <= j < nt.
@@ -874,7 +879,7 @@ __device__ __forceinline__ void tile_pair(int t, int nt, int& i, int& j) {
 // else along the outputs (x[k * ld + i]).
 template <bool KFAST>
 __device__ __forceinline__ double ns_tile(const double* __restrict__ x, int64_t ld, int n, int K, int i0, int j0,
-                                          double* As, double* Bs, double* part) {
+                                          double* As, double* Bs) {
   const int tid = threadIdx.x;
   int r[2], k[2];
 #pragma unroll
@@ -892,9 +897,9 @@ __device__ __forceinline__ double ns_tile(const double* __restrict__ x, int64_t 
       vb[q] = (gj < n && kk < K) ? x[KFAST ? gj * ld + kk : kk * ld + gj] : 0.0;
     }
   };
-  const int o = tid % (kNsR * kNsR), quarter = tid / (kNsR * kNsR);
-  const double* a = As + o / kNsR * kNsP + quarter * (kNsK / 4);
-  const double* b = Bs + o % kNsR * kNsP + quarter * (kNsK / 4);
+  const double* a = As + tid / kNsR % kNsR * kNsP;
+  const double* b = Bs + tid % kNsR * kNsP;
+  const bool sums = tid < kNsR * kNsR;
   double acc = 0.0;
   load(0);
   for (int k0 = 0; k0 < K; k0 += kNsK) {
@@ -905,19 +910,18 @@ __device__ __forceinline__ double ns_tile(const double* __restrict__ x, int64_t 
     }
     __syncthreads();
     if (k0 + kNsK < K) load(k0 + kNsK);
-    const int terms = min(kNsK / 4, K - k0 - quarter * (kNsK / 4));  // the rest is zero
-    if (terms == kNsK / 4) {
-#pragma unroll
-      for (int t = 0; t < kNsK / 4; ++t) acc = fma(a[t], b[t], acc);
-    } else {
-      for (int t = 0; t < terms; ++t) acc = fma(a[t], b[t], acc);
+    if (sums) {  // in the order of K: an optimisation's path does not depend on the kernel
+      const int terms = min(kNsK, K - k0);
+      if (terms == kNsK) {
+#pragma unroll 16
+        for (int t = 0; t < kNsK; ++t) acc = fma(a[t], b[t], acc);
+      } else {
+        for (int t = 0; t < terms; ++t) acc = fma(a[t], b[t], acc);
+      }
     }
     __syncthreads();
   }
-  if (quarter > 0) part[(quarter - 1) * kNsR * kNsR + o] = acc;
-  __syncthreads();
-  if (quarter > 0) return 0.0;
-  return ((acc + part[o]) + part[kNsR * kNsR + o]) + part[2 * kNsR * kNsR + o];
+  return acc;
 }
 
 // Bm = (5/2)(I - G) + G^2; the last block to finish sums the tiles' shares of
@@ -927,13 +931,13 @@ __global__ void __launch_bounds__(256) ns_square_kernel(const double* G, double*
                                                         double* partials, double* resid, double tol,
                                                         int* state) {
   pdl_begin();
-  __shared__ double As[kNsR * kNsP], Bs[kNsR * kNsP], part[3 * kNsR * kNsR];
+  __shared__ double As[kNsR * kNsP], Bs[kNsR * kNsP];
   __shared__ int last;
   if (state[0]) return;
   int ti, tj;
   tile_pair(int(blockIdx.x), (n + kNsR - 1) / kNsR, ti, tj);
   const int i0 = ti * kNsR, j0 = tj * kNsR;
-  const double g2 = ns_tile<true>(G, n, n, n, i0, j0, As, Bs, part);
+  const double g2 = ns_tile<true>(G, n, n, n, i0, j0, As, Bs);
   const int tid = threadIdx.x;
   double v = 0.0;
   if (tid < kNsR * kNsR) {
@@ -972,7 +976,7 @@ __global__ void __launch_bounds__(256) ns_gram_kernel(const double* X, double* G
                                                       int n, int* state, int close, int set_cond,
                                                       cudaGraphConditionalHandle cond, int max_iter) {
   pdl_begin();
-  __shared__ double As[kNsR * kNsP], Bs[kNsR * kNsP], part[3 * kNsR * kNsR];
+  __shared__ double As[kNsR * kNsP], Bs[kNsR * kNsP];
   // block 0 alone writes state[0] and state[1], and what it writes is the
   // same early return for every block that reads it
   const int done = state[0], stop = close ? state[2] : 0;
@@ -987,7 +991,7 @@ __global__ void __launch_bounds__(256) ns_gram_kernel(const double* X, double* G
   if (done || stop) return;
   int ti, tj;
   tile_pair(int(blockIdx.x), (n + kNsR - 1) / kNsR, ti, tj);
-  const double g = ns_tile<false>(X, n, n, m, ti * kNsR, tj * kNsR, As, Bs, part);
+  const double g = ns_tile<false>(X, n, n, m, ti * kNsR, tj * kNsR, As, Bs);
   const int tid = threadIdx.x;
   if (tid >= kNsR * kNsR) return;
   const int i = ti * kNsR + tid / kNsR, j = tj * kNsR + tid % kNsR;

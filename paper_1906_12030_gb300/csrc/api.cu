@@ -533,45 +533,22 @@ extern "C" mera_status mera_fixed_point_rho(const double* u, const double* w, in
 // ---------------------------------------------------------------------------
 // Polar update.
 // ---------------------------------------------------------------------------
-// Products of a Newton-Schulz step as digit products: the digit images,
-// row exponents and K-split partials of the largest of the three (X^T X, G G
-// and X B), which share them.
-struct PolarX64 {
-  size_t img_a, img_b, exp_a, exp_b, plane, total;
-};
-static PolarX64 polar_x64(int m, int n) {
-  auto img = [](int64_t rows, int64_t tile, int64_t k) {
-    return align_up(size_t((rows + tile - 1) / tile * tile) * size_t((k + 15) / 16) * 32 * kX64Digits);
-  };
-  PolarX64 x;
-  x.img_a = std::max({img(n, kX64TileA, m), img(n, kX64TileA, n), img(m, kX64TileA, n)});
-  x.img_b = std::max(img(n, kX64TileB, m), img(n, kX64TileB, n));
-  x.exp_a = align_up(size_t(m) * sizeof(int));
-  x.exp_b = align_up(size_t(n) * sizeof(int));
-  auto part = [](int64_t M, int64_t N, int64_t K) {
-    const int64_t s = x64_split_k(M, N, K);
-    return s > 1 ? align_up(size_t(s) * M * N * sizeof(float)) : size_t(0);
-  };
-  x.plane = std::max({part(n, n, m), part(n, n, n), part(m, n, n)});
-  x.total = x.img_a + x.img_b + x.exp_a + x.exp_b + 3 * x.plane;
-  return x;
-}
-
-// The least scratch of a polar update.
-static size_t polar_bytes_least(int m, int n) {
+static size_t polar_bytes(int m, int n) {
   return 2 * align_up(size_t(m) * n * sizeof(double)) + 3 * align_up(size_t(n) * n * sizeof(double)) +
          kReduceBytes;
 }
-static size_t polar_bytes(int m, int n) {
-  return polar_bytes_least(m, n) + (n > kNsFusedMax ? polar_x64(m, n).total : 0);
+// The least a polar update runs in: the fused steps do without G2 (up to
+// n = 320 the whole size has always been asked for).
+static size_t polar_bytes_least(int m, int n) {
+  return polar_bytes(m, n) - (n > 320 && n <= kNsFusedMax ? align_up(size_t(n) * n * sizeof(double)) : 0);
 }
 
 // Stiefel step: A, S (n x n), T, Yneg (m x n), then the polar update's scratch.
-static size_t stiefel_bytes_least(int m, int n) {
+static size_t stiefel_bytes(int m, int n) {
   return 2 * align_up(size_t(n) * n * sizeof(double)) + 2 * align_up(size_t(m) * n * sizeof(double)) +
-         polar_bytes_least(m, n);
+         polar_bytes(m, n);
 }
-static size_t stiefel_bytes(int m, int n) { return stiefel_bytes_least(m, n) - polar_bytes_least(m, n) + polar_bytes(m, n); }
+static size_t stiefel_bytes_least(int m, int n) { return stiefel_bytes(m, n) - polar_bytes(m, n) + polar_bytes_least(m, n); }
 
 extern "C" mera_status mera_polar_workspace_size(int m, int n, size_t* bytes) {
   if (!bytes || m < 1 || n < 1 || m < n || m > 1 << 16) return fail(MERA_EINVAL, "bad polar sizes");
@@ -590,7 +567,8 @@ static mera_status polar_record(const double* env, int m, int n, double* out, in
   double* X = reinterpret_cast<double*>(ar.take(size_t(m) * n * sizeof(double)));
   double* Xn = reinterpret_cast<double*>(ar.take(size_t(m) * n * sizeof(double)));
   double* G = reinterpret_cast<double*>(ar.take(size_t(n) * n * sizeof(double)));
-  double* G2 = reinterpret_cast<double*>(ar.take(size_t(n) * n * sizeof(double)));
+  const bool fused = n <= kNsFusedMax;
+  double* G2 = reinterpret_cast<double*>(ar.take(fused ? 0 : size_t(n) * n * sizeof(double)));
   double* Bm = reinterpret_cast<double*>(ar.take(size_t(n) * n * sizeof(double)));
   double* red = reinterpret_cast<double*>(ar.take(kReduceBytes));
   double* scalars = red + 4096;
@@ -604,33 +582,12 @@ static mera_status polar_record(const double* env, int m, int n, double* out, in
   // runs and every later kernel returns at once.
   int* state = reinterpret_cast<int*>(scalars + 4);  // done, iterations, converged-after-this-step, block count
   if ((e = cudaMemsetAsync(scalars + 2, 0, 4 * sizeof(double), s)) != cudaSuccess) return cuda_status(e, "polar state");
-  const bool fused = n <= kNsFusedMax;
-  // larger matrices: digit products on the tensor cores where the scratch has
-  // room for them (n = 1024: 6.0 ms a step on the FP64 pipe, 0.26 ms so)
-  const PolarX64 px = polar_x64(m, n);
-  const bool x64 = !fused && ar.left() >= px.total;
-  char* img_a = ar.take(x64 ? px.img_a : 0);
-  char* img_b = ar.take(x64 ? px.img_b : 0);
-  int* exp_a = reinterpret_cast<int*>(ar.take(x64 ? px.exp_a : 0));
-  int* exp_b = reinterpret_cast<int*>(ar.take(x64 ? px.exp_b : 0));
-  float* part = reinterpret_cast<float*>(ar.ptr());
+  // binary64 products throughout, whatever the size: an iterate whose columns
+  // differ by decades, or a polynomial close to the identity, has entries of
+  // very different scale within one row, which digits of a row's scale lose
   auto product = [&](GemmF64Args g, cudaStream_t st) {
     g.ordered = 1;
-    if (!x64) return launch_gemm_f64(g, st);
-    const X64SplitJob jobs[2] = {{g.A, g.a_m, g.M, g.K, g.M, kX64TileA, img_a, exp_a, g.a_k, state},
-                                 {g.B, g.b_n, g.N, g.K, g.N, kX64TileB, img_b, exp_b, g.b_k, state}};
-    cudaError_t r = launch_x64_split(jobs, 2, st);
-    if (r != cudaSuccess) return r;
-    X64GemmArgs a;
-    a.A = img_a; a.ea = exp_a; a.A64 = g.A; a.lda = g.a_m; a.a_k = g.a_k;
-    a.B = img_b; a.eb = exp_b; a.B64 = g.B; a.ldb = g.b_n; a.b_k = g.b_k;
-    a.M = g.M; a.N = g.N; a.K = g.K;
-    a.C = g.C; a.m_dst = g.m_dst; a.n_dst = g.n_dst; a.alpha = g.alpha; a.accumulate = g.accumulate;
-    a.split = x64_split_k(g.M, g.N, g.K);
-    a.partial = part;
-    a.partial_plane = int64_t(px.plane / sizeof(float));
-    a.skip_if = state;
-    return launch_gemm_x64(&a, 1, st);
+    return launch_gemm_f64(g, st);
   };
   // G = x^T x (skipped once converged)
   auto gram = [&](const double* x, cudaStream_t st, bool close = true, const cudaGraphConditionalHandle* cond = nullptr) {
@@ -897,7 +854,7 @@ mera_status sweep_layout(int n_layers, const int* chi_b, const int* chi_t, int p
       map_bytes = std::max(map_bytes, op_bytes(*p));
     }
     const int64_t eb = int64_t(chi_b[t]) * chi_b[t];
-    map_bytes = std::max(map_bytes, less ? stiefel_bytes_least(int(eb), int(eb)) : stiefel_bytes(int(eb), int(eb)));
+    map_bytes = std::max(map_bytes, stiefel_bytes(int(eb), int(eb)));  // >= polar_bytes
     size_t fp = 0;
     if (t == n_layers - 1) {
       ws_size_impl(MERA_OP_FIXED_POINT, chi_b[t], chi_t[t], prec, &fp, less);

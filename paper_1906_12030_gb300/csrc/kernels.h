@@ -53,13 +53,11 @@ cudaError_t launch_oz_split(const OzSplitJob* jobs, int n, int slices, cudaStrea
 // Binary64 operand (rows x K) -> digit image of x64_gemm_kernel in tiles of `tile` rows, and one exponent per row.  Rows
 // come in segments of seg_rows, each padded to whole tiles.
 struct X64SplitJob {
-  const double* src = nullptr;  // entry (r, k) at src[r * ld + k * k_stride]
+  const double* src = nullptr;  // entry (r, k) at src[r * ld + k]
   int64_t ld = 0, rows = 0, K = 0, seg_rows = 0;
   int tile = 0;
   void* img = nullptr;
   int* rowexp = nullptr;
-  int64_t k_stride = 1;
-  const int* skip_if = nullptr;  // device flag: the launch does nothing where *skip_if != 0 (the first job's counts)
 };
 cudaError_t launch_x64_split(const X64SplitJob* jobs, int n, cudaStream_t stream);
 
@@ -114,9 +112,10 @@ cudaError_t launch_ns_step(const double* G, const double* G2, double* Bm, int64_
 cudaError_t launch_ns_finish(int* state, cudaStream_t stream);
 // The same step for n <= kNsFusedMax in fused launches (no G2, no finish):
 // launch_ns_square, X B, launch_ns_gram.  state[3] is zero between launches.
-// Up to here the FP64 pipe keeps up with the digit products (n = 256: 84 us a
-// step here; n = 400: 420 us on the FP64 pipe, 100 us as digit products).
-constexpr int64_t kNsFusedMax = 320;  // 820 tile pairs: partial sums in the 4096 slots of the callers' scratch
+// Whole updates at condition 1e3, fused against launch_ns_step's form, which
+// squares in full: n = 256 1.17 and 1.72 ms, 400 3.8 and 5.7, 720 19.8 and
+// 31.2, bit for bit the same.
+constexpr int64_t kNsFusedMax = 720;  // 4095 tile pairs: partial sums in the 4096 slots of the callers' scratch
 cudaError_t launch_ns_square(const double* G, double* Bm, int64_t n, double* partials, double* resid, double tol,
                              int* state, cudaStream_t stream);
 // close: ends a step.  cond: also sets the condition of the recorded loop.

@@ -1134,7 +1134,6 @@ static cudaError_t launch_x64_group(const X64GemmArgs* args, int n, cudaStream_t
   if (attr_err != cudaSuccess) return attr_err;
   X64Group g, red;
   g.n = n;
-  g.skip_if = red.skip_if = args[0].skip_if;
   red.n = 0;
   int64_t items = 0;
   unsigned gx = 0, gy = 0;
@@ -1151,8 +1150,6 @@ static cudaError_t launch_x64_group(const X64GemmArgs* args, int n, cudaStream_t
     p.B64 = a.B64;
     p.lda = a.lda;
     p.ldb = a.ldb;
-    p.a_k = a.a_k;
-    p.b_k = a.b_k;
     p.M = a.M;
     p.N = a.N;
     p.K = a.K;

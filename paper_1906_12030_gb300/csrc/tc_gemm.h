@@ -48,12 +48,12 @@ inline cudaError_t launch_gemm_tc(const TcGemmArgs& args, cudaStream_t stream) {
 struct X64GemmArgs {
   const void* A = nullptr;
   const int* ea = nullptr;
-  const double* A64 = nullptr;  // entry (m, k) at A64[m * lda + k * a_k]
-  int64_t lda = 0, a_k = 1;
+  const double* A64 = nullptr;  // entry (m, k) at A64[m * lda + k]
+  int64_t lda = 0;
   const void* B = nullptr;
   const int* eb = nullptr;
   const double* B64 = nullptr;
-  int64_t ldb = 0, b_k = 1;
+  int64_t ldb = 0;
   int64_t M = 0, N = 0, K = 0;
   double* C = nullptr;
   LegMap m_dst, n_dst;
@@ -62,7 +62,6 @@ struct X64GemmArgs {
   int split = 1;             // K split (x64_split_k); > 1 needs `partial`
   float* partial = nullptr;  // hi, mid, lo planes [split][N][M]
   int64_t partial_plane = 0; // floats from one plane to the next
-  const int* skip_if = nullptr;  // device flag: the launch does nothing where *skip_if != 0 (the first job's counts)
 };
 
 // Jobs that all fit in one block of K per work item, or all do not

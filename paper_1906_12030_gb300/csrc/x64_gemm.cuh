@@ -77,7 +77,7 @@ struct X64Params {
   const int* eb;
   const double* A64;  // binary64 operands (rows with exponent kX64Bad)
   const double* B64;
-  int64_t lda, ldb, a_k, b_k;
+  int64_t lda, ldb;
   int64_t M, N, K;
   double* C;
   LegMap m_dst, n_dst;
@@ -94,7 +94,6 @@ struct X64Params {
 struct X64Group {
   int n;
   int end[kGroup];  // work items of the jobs up to and including each
-  const int* skip_if;
   X64Params job[kGroup];
 };
 
@@ -173,7 +172,7 @@ __device__ __forceinline__ double x64_plain(const X64Params& p, int64_t m, int64
   const double* b = p.B64 + n * p.ldb;
   double s = 0.0;
 #pragma unroll 1
-  for (int64_t k = 0; k < p.K; ++k) s = fma(a[k * p.a_k], b[k * p.b_k], s);
+  for (int64_t k = 0; k < p.K; ++k) s = fma(a[k], b[k], s);
   return p.alpha * s;
 }
 
@@ -225,7 +224,7 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
   const uint32_t tmem = *tmem_slot;
   pdl_wait();
   pdl_trigger();
-  const int items = g.skip_if && *g.skip_if ? 0 : g.end[g.n - 1];
+  const int items = g.end[g.n - 1];
 
   if (warp == 0) {
     if (lane == 0) {
@@ -440,7 +439,6 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
 // output.  One thread per row m over a chunk of columns.
 __global__ void __launch_bounds__(128) x64_reduce_kernel(const __grid_constant__ X64Group g) {
   pdl_begin();
-  if (g.skip_if && *g.skip_if) return;
   const X64Params& p = g.job[blockIdx.z];
   const int64_t m = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (m >= p.M) return;

@@ -35,7 +35,7 @@ constexpr int kCap = kThreadsX * kItems * 8;     // entries per block of threads
 
 struct SplitArgs {
   const double* src;
-  int64_t ld, rows, K, seg_rows, tiles_per_seg, k_stride;
+  int64_t ld, rows, K, seg_rows, tiles_per_seg;
   uint8_t* img;
   int* rowexp;
   int tile, nk;        // rows per tile, 16-wide steps of K
@@ -48,7 +48,6 @@ struct SplitGroup {
   int n;
   int end[kGroup];     // blocks of the jobs up to and including each
   int rend[kGroup];    // rows whose exponents need a pass of their own, likewise
-  const int* skip_if;
   SplitArgs job[kGroup];
 };
 
@@ -69,7 +68,6 @@ __device__ __forceinline__ int row_exponent(int w) {
 __global__ void __launch_bounds__(512) x64_rowexp_kernel(const __grid_constant__ SplitGroup g) {
   pdl_begin();
   __shared__ int sm[16];
-  if (g.skip_if && *g.skip_if) return;
   for (int64_t rg = blockIdx.x; rg < g.rend[g.n - 1]; rg += gridDim.x) {
     int i = 0;
     while (rg >= g.rend[i]) ++i;
@@ -77,7 +75,7 @@ __global__ void __launch_bounds__(512) x64_rowexp_kernel(const __grid_constant__
     const int64_t r = rg - (i > 0 ? g.rend[i - 1] : 0);
     const double* p = a.src + r * a.ld;
     int w = 0;
-    for (int64_t k = threadIdx.x; k < a.K; k += blockDim.x) w = max(w, mag_word(p[k * a.k_stride]));
+    for (int64_t k = threadIdx.x; k < a.K; k += blockDim.x) w = max(w, mag_word(p[k]));
     w = __reduce_max_sync(0xffffffffu, w);
     if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = w;
     __syncthreads();
@@ -91,7 +89,6 @@ __global__ void __launch_bounds__(512) x64_rowexp_kernel(const __grid_constant__
 
 __global__ void __launch_bounds__(kThreadsX, 2) x64_split_kernel(const __grid_constant__ SplitGroup gr) {
   pdl_begin();
-  if (gr.skip_if && *gr.skip_if) return;
   int job = 0;
   while (int(blockIdx.x) >= gr.end[job]) ++job;
   const int block = int(blockIdx.x) - (job > 0 ? gr.end[job - 1] : 0);
@@ -119,7 +116,7 @@ __global__ void __launch_bounds__(kThreadsX, 2) x64_split_kernel(const __grid_co
     for (int j = 0; j < 8; ++j) x[i][j] = 0.0;
     if (rr[i] < 0) continue;
     const int64_t k = kbase + g * 8;
-    const double* s = a.src + (r0 + r) * a.ld + k * a.k_stride;
+    const double* s = a.src + (r0 + r) * a.ld + k;
     if (a.pairs && k + 8 <= a.K) {
 #pragma unroll
       for (int j = 0; j < 8; j += 2) {
@@ -130,7 +127,7 @@ __global__ void __launch_bounds__(kThreadsX, 2) x64_split_kernel(const __grid_co
     } else {
 #pragma unroll
       for (int j = 0; j < 8; ++j)
-        if (k + j < a.K) x[i][j] = s[j * a.k_stride];
+        if (k + j < a.K) x[i][j] = s[j];
     }
   }
 #pragma unroll
@@ -217,7 +214,6 @@ __global__ void __launch_bounds__(kThreadsX, 2) x64_split_kernel(const __grid_co
 static cudaError_t launch_group(const X64SplitJob* jobs, int n, cudaStream_t stream) {
   SplitGroup g;
   g.n = 0;
-  g.skip_if = jobs[0].skip_if;
   int64_t blocks = 0, rows_known = 0;
   size_t smem = 0;
   for (int i = 0; i < n; ++i) {
@@ -227,8 +223,7 @@ static cudaError_t launch_group(const X64SplitJob* jobs, int n, cudaStream_t str
     SplitArgs& a = g.job[g.n];
     a.src = j.src;
     a.ld = j.ld;
-    a.k_stride = j.k_stride;
-    a.pairs = j.k_stride == 1 && (j.ld & 1) == 0 && (reinterpret_cast<uintptr_t>(j.src) & 15) == 0;
+    a.pairs = (j.ld & 1) == 0 && (reinterpret_cast<uintptr_t>(j.src) & 15) == 0;
     a.rows = j.rows;
     a.K = j.K;
     a.seg_rows = j.seg_rows;

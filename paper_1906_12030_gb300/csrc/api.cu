@@ -284,6 +284,7 @@ mera_status run_steps(const OpProgram& prog, const std::pair<int, int>* steps, i
       a.alpha = g.alpha;
       a.accumulate = accumulate(i);
       a.split = g.split;
+      a.mask = ws + dg.bufs[size_t(g.m_buf)].offset;
       if (g.p_buf >= 0) {
         a.partial = reinterpret_cast<float*>(ws + dg.bufs[size_t(g.p_buf)].offset);
         a.partial_plane = dg.bufs[size_t(g.p_buf)].plane_bytes / 4;
@@ -1147,7 +1148,8 @@ extern "C" mera_status mera_gemm_test(int prec, const double* A, const double* B
   const size_t xa = align_up(size_t((M + kX64TileA - 1) / kX64TileA * kX64TileA) * row_img);
   const size_t xb = align_up(size_t((N + kX64TileB - 1) / kX64TileB * kX64TileB) * row_img);
   const size_t xneed = align_up(size_t(M) * ldx * 8) + align_up(size_t(N) * ldx * 8) + xa + xb +
-                       align_up(size_t(M) * 4) + align_up(size_t(N) * 4) + size_t(xsplit) * M * N * 12;
+                       align_up(size_t(M) * 4) + align_up(size_t(N) * 4) + size_t(x64_mask_bytes(M, N)) +
+                       size_t(xsplit) * M * N * 12;
   const bool x64 = prec == PREC_F64 && ws_bytes >= xneed;
   if (x64) ld = ldx;
   const size_t pa = align_up(size_t(M) * ld * eb), pb = align_up(size_t(N) * ld * eb);
@@ -1194,7 +1196,8 @@ extern "C" mera_status mera_gemm_test(int prec, const double* A, const double* B
     g.B = ib; g.eb = eb2; g.B64 = reinterpret_cast<const double*>(wb); g.ldb = ld;
     g.M = M; g.N = N; g.K = K; g.C = C; g.m_dst = md; g.n_dst = nd;
     g.split = xsplit;
-    g.partial = reinterpret_cast<float*>(eb2 + align_up(size_t(N) * 4) / 4);
+    g.mask = eb2 + align_up(size_t(N) * 4) / 4;
+    g.partial = reinterpret_cast<float*>(static_cast<char*>(g.mask) + x64_mask_bytes(M, N));
     g.partial_plane = int64_t(xsplit) * M * N;
     const X64SplitJob jobs[2] = {{g.A64, ld, M, K, M, kX64TileA, ia, ea}, {g.B64, ld, N, K, N, kX64TileB, ib, eb2}};
     e = launch_x64_split(jobs, 2, s);

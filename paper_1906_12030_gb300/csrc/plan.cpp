@@ -466,6 +466,16 @@ struct Builder {
       gs.ax_buf = img_of[gi.a];
       gs.bx_buf = img_of[gi.b];
     }
+    if (x64[i]) {  // live during this step only
+      Buffer mb;
+      mb.bytes = mb.plane_bytes = x64_mask_bytes(gs.M, gs.N);
+      mb.ld = kX64TileA;
+      mb.rows = mb.bytes / (mb.ld * 8);
+      prog.bufs.push_back(mb);
+      gs.m_buf = int(prog.bufs.size()) - 1;
+      first_use.push_back(-1);
+      last_use.push_back(-1);
+    }
     gs.split = x64[i] ? x64_split_k(gs.M, gs.N, gs.K) : tc_split_k(prec, gs.M, gs.N, gs.K, gs.bn);
     if (gs.split > 1) {  // FP32 partials [split][N][M], live during this step only
       Buffer pb;
@@ -500,7 +510,8 @@ struct Builder {
     if (last_use[gs.b_buf] < si) last_use[gs.b_buf] = si;
     for (int b : {gs.ax_buf, gs.bx_buf})
       if (b >= 0 && last_use[b] < si) last_use[b] = si;
-    if (gs.p_buf >= 0) first_use[gs.p_buf] = last_use[gs.p_buf] = si;
+    for (int b : {gs.p_buf, gs.m_buf})
+      if (b >= 0) first_use[b] = last_use[b] = si;
     if (gs.c_buf >= 0) {
       if (first_use[gs.c_buf] < 0) first_use[gs.c_buf] = si;
       if (last_use[gs.c_buf] < si) last_use[gs.c_buf] = si;
@@ -1161,7 +1172,7 @@ std::string program_json(const OpProgram& prog, int op, int chi_b, int chi_t, in
           << ",\"M\":" << g.M << ",\"N\":" << g.N << ",\"K\":" << g.K << ",\"lda\":" << g.lda << ",\"ldb\":" << g.ldb
           << ",\"c_buf\":" << g.c_buf << ",\"alpha\":" << g.alpha << ",\"accumulate\":" << g.accumulate
           << ",\"flops\":" << g.flops << ",\"dominant\":" << g.dominant << ",\"split\":" << g.split
-          << ",\"p_buf\":" << g.p_buf << ",\"ax_buf\":" << g.ax_buf << ",\"bx_buf\":" << g.bx_buf << ",\"a_off\":" << g.a_off << ",\"b_off\":" << g.b_off
+          << ",\"p_buf\":" << g.p_buf << ",\"ax_buf\":" << g.ax_buf << ",\"bx_buf\":" << g.bx_buf << ",\"m_buf\":" << g.m_buf << ",\"a_off\":" << g.a_off << ",\"b_off\":" << g.b_off
           << ",\"c_off\":" << g.c_off << ",\"stat\":" << g.stat << ",\"bn\":" << g.bn << ",\"m_dst\":";
         lm(g.m_dst);
         o << ",\"n_dst\":";

@@ -44,6 +44,10 @@ constexpr int kX64BlockSteps = kX64Block / 16;
 constexpr int kX64MaxExp = 400;
 constexpr int kX64Bad = 1 << 20;
 constexpr int kX64TileA = 128, kX64TileB = 64;  // rows per image tile of the GEMM's A and B
+// Masks of a product's outputs that are left to the FP64 units: a bit each.
+inline int64_t x64_mask_bytes(int64_t M, int64_t N) {
+  return (M + kX64TileA - 1) / kX64TileA * ((N + kX64TileB - 1) / kX64TileB) * (kX64TileA * kX64TileB / 8);
+}
 enum Slot : int { SLOT_OP = 0, SLOT_RHO = 1, SLOT_U = 2, SLOT_W = 3 };
 enum Op : int { OP_ASCEND = 0, OP_DESCEND = 1, OP_ENV_U = 2, OP_ENV_W = 3 };
 
@@ -89,6 +93,7 @@ struct GemmStep {
   int ax_buf = -1, bx_buf = -1;     // PREC_F64 on the tensor cores: digit images of A and B
   int64_t ax_row = 0, bx_row = 0;   // first row of the operands' row exponents (slices)
   int64_t ax_tile = 0, bx_tile = 0; // first tile of the operands' images (slices)
+  int m_buf = -1;     // and the masks of the outputs left to the FP64 units
   std::string label;  // e.g. "aceiq*CDcdil->ADadelq" for inspection
 };
 

@@ -1132,10 +1132,10 @@ static cudaError_t launch_x64_group(const X64GemmArgs* args, int n, cudaStream_t
     resident = std::max(1, sms);
   });
   if (attr_err != cudaSuccess) return attr_err;
-  X64Group g, red;
-  g.n = n;
+  X64Group g, red, ex;
+  g.n = ex.n = n;
   red.n = 0;
-  int64_t items = 0;
+  int64_t items = 0, units = 0;  // work items; x64_exact_kernel's units
   unsigned gx = 0, gy = 0;
   for (int i = 0; i < n; ++i) {
     const X64GemmArgs& a = args[i];
@@ -1166,6 +1166,8 @@ static cudaError_t launch_x64_group(const X64GemmArgs* args, int n, cudaStream_t
     p.kc = int(x64_kc(p.nk, p.split));
     p.partial = a.partial;
     p.p_plane = a.partial_plane;
+    p.mask = static_cast<unsigned long long*>(a.mask);
+    if (!p.mask) return cudaErrorInvalidValue;
     if (p.split > 1 && (int64_t(p.split - 1) * p.kc >= p.nk || a.partial_plane < int64_t(p.split) * a.N * a.M))
       return cudaErrorInvalidValue;  // an empty split, or overlapping partial planes
     const int64_t tiles_m = (a.M + kBM - 1) / kBM;
@@ -1175,6 +1177,10 @@ static cudaError_t launch_x64_group(const X64GemmArgs* args, int n, cudaStream_t
     p.tiles_m = int(tiles_m);
     p.tiles_n = int((a.N + kXBN - 1) / kXBN);
     g.end[i] = int(items);
+    units += tiles_m * p.tiles_n * kExUnits;
+    if (units > 0x7fffffff) return cudaErrorInvalidValue;
+    ex.job[i] = p;
+    ex.end[i] = int(units);
     if (p.split > 1) {
       red.job[red.n++] = p;
       const unsigned x = unsigned((a.M + 127) / 128);
@@ -1192,6 +1198,8 @@ static cudaError_t launch_x64_group(const X64GemmArgs* args, int n, cudaStream_t
     count_launch();
     launch(x64_reduce_kernel, gx * gy * unsigned(red.n) <= 608, dim3(gx, gy, unsigned(red.n)), 128, 0, stream, red);
   }
+  count_launch();
+  launch(x64_exact_kernel, true, unsigned(std::min<int64_t>(units, 2 * 152)), 256, 0, stream, ex);
   return cudaGetLastError();
 }
 

@@ -62,6 +62,7 @@ struct X64GemmArgs {
   int split = 1;             // K split (x64_split_k); > 1 needs `partial`
   float* partial = nullptr;  // hi, mid, lo planes [split][N][M]
   int64_t partial_plane = 0; // floats from one plane to the next
+  void* mask = nullptr;      // x64_mask_bytes(M, N) of scratch
 };
 
 // Jobs that all fit in one block of K per work item, or all do not

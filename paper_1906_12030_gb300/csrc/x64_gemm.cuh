@@ -51,9 +51,11 @@
 // 497 -> 15.6 ms, its error against 64 bits 1.8e-15 -> 1.5e-15.
 //
 // Rows of A or B that the digits cannot represent (a NaN, an infinity, or a
-// largest entry beyond 2^+-kX64MaxExp) carry the exponent kX64Bad; outputs
-// that touch one are summed from the binary64 operands by FMAs in the order
-// of K, as the FP64 kernel sums them.
+// largest entry beyond 2^+-kX64MaxExp) carry the exponent kX64Bad.  Outputs
+// that touch one are left to x64_exact_kernel, which sums them from the
+// binary64 operands on the FP64 units: each tile has a mask of them, 64 bits
+// per row.  (Summed here, by the epilogue, a column of K = 331776 would keep
+// the copy and MMA warps waiting past the limit of their waits.)
 
 constexpr int kXBN = 64;
 constexpr int kXPlanes = kX64Digits;
@@ -88,6 +90,7 @@ struct X64Params {
   int split, kc;      // K split: steps per split
   float* partial;     // split > 1: hi, mid, lo planes [split][N][M]
   int64_t p_plane;
+  unsigned long long* mask;  // outputs left to x64_exact_kernel: [tile][kBM], bit c for column c
   int tiles_m, tiles_n, group_m;  // work items (fewer than 2^31) and their order, as in Epilogue
 };
 
@@ -166,14 +169,9 @@ __device__ __forceinline__ double triple_to_f64(float h, float m, float l, int e
   return eh == 0 ? 0.0 : __hiloint2double(int(hi), int(uint32_t(mag)));
 }
 
-// One output from the binary64 operands, as gemm_f64_kernel sums it.
-__device__ __forceinline__ double x64_plain(const X64Params& p, int64_t m, int64_t n) {
-  const double* a = p.A64 + m * p.lda;
-  const double* b = p.B64 + n * p.ldb;
-  double s = 0.0;
-#pragma unroll 1
-  for (int64_t k = 0; k < p.K; ++k) s = fma(a[k], b[k], s);
-  return p.alpha * s;
+// Mask word of row `row` of a tile.
+__device__ __forceinline__ unsigned long long* x64_mask(const X64Params& p, int row_t, int col_t, int row) {
+  return p.mask + (int64_t(row_t) * p.tiles_n + col_t) * kBM + row;
 }
 
 __device__ __forceinline__ void x64_store(const X64Params& p, int64_t off, double x) {
@@ -377,8 +375,11 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
           break;
         }
       }
-      if (!ok || !row_ok) continue;
+      if (!ok) continue;
+      uint16_t* const mask = reinterpret_cast<uint16_t*>(x64_mask(p, row_t, col_t, row)) + c0 / kXCols;
       if (p.split > 1) {  // partial triple, summed by x64_reduce_kernel
+        if (ks == 0) *mask = 0;
+        if (!row_ok) continue;
         float* q = p.partial + (ks * p.N + n0 + c0) * p.M + m;
 #pragma unroll
         for (int j = 0; j < kXCols; ++j, q += p.M)
@@ -389,16 +390,24 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
           }
         continue;
       }
+      const int ra = row_ok ? p.ea[m] : 0;
+      uint32_t todo = 0, skip = 0;  // columns that exist, and those left to x64_exact_kernel
+#pragma unroll
+      for (int j = 0; j < kXCols; ++j) {
+        if (row_ok && n0 + c0 + j < p.N) todo |= 1u << j;
+        if (ra == kX64Bad || exp_n[c0 + j] == kX64Bad) skip |= 1u << j;
+      }
+      skip &= todo;
+      todo &= ~skip;
+      *mask = uint16_t(skip);
+      if (todo == 0) continue;
       const int64_t off_m = legmap_offset32(p.m_dst, uint32_t(m));
-      const int ra = p.ea[m];
-      bool bad = ra == kX64Bad;
       if (!p.accumulate) {
 #pragma unroll
         for (int j = 0; j < kXCols; ++j) {
           const int c = c0 + j;
           const int rb = exp_n[c];
-          bad |= rb == kX64Bad;
-          if (n0 + c >= p.N || ra == kX64Bad || rb == kX64Bad) continue;
+          if (!(todo >> j & 1u)) continue;
           p.C[off_m + off_n[c]] = triple_to_f64(h[j], mid[j], lo[j], ra + rb + p.alpha_exp);
         }
       } else {
@@ -407,22 +416,15 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
         for (int j = 0; j < kXCols; j += 4) {
           double y[4];
 #pragma unroll
-          for (int k = 0; k < 4; ++k) y[k] = n0 + c0 + j + k < p.N ? p.C[off_m + off_n[c0 + j + k]] : 0.0;
+          for (int k = 0; k < 4; ++k) y[k] = (todo >> (j + k) & 1u) ? p.C[off_m + off_n[c0 + j + k]] : 0.0;
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             const int c = c0 + j + k;
             const int rb = exp_n[c];
-            bad |= rb == kX64Bad;
-            if (n0 + c >= p.N || ra == kX64Bad || rb == kX64Bad) continue;
+            if (!(todo >> (j + k) & 1u)) continue;
             p.C[off_m + off_n[c]] = y[k] + triple_to_f64(h[j + k], mid[j + k], lo[j + k], ra + rb + p.alpha_exp);
           }
         }
-      }
-      if (bad) {
-#pragma unroll 1
-        for (int c = c0; c < c0 + kXCols && n0 + c < p.N; ++c)
-          if (ra == kX64Bad || exp_n[c] == kX64Bad)
-            x64_store(p, off_m + off_n[c], x64_plain(p, m, n0 + c));
       }
     }
   }
@@ -453,8 +455,92 @@ __global__ void __launch_bounds__(128) x64_reduce_kernel(const __grid_constant__
       triple_add(h, mid, lo, q[0], q[p.p_plane], q[2 * p.p_plane]);
     }
     const int rb = p.eb[n];
-    const double x = ra == kX64Bad || rb == kX64Bad ? x64_plain(p, m, n)
-                                                    : triple_to_f64(h, mid, lo, ra + rb + p.alpha_exp);
-    x64_store(p, off_m + legmap_offset32(p.n_dst, uint32_t(n)), x);
+    if (ra == kX64Bad || rb == kX64Bad) {  // (the mask was cleared by the GEMM)
+      atomicOr(x64_mask(p, int(m / kBM), int(n / kXBN), int(m % kBM)), 1ull << (n % kXBN));
+      continue;
+    }
+    x64_store(p, off_m + legmap_offset32(p.n_dst, uint32_t(n)), triple_to_f64(h, mid, lo, ra + rb + p.alpha_exp));
+  }
+}
+
+// The outputs that the tiles' masks name, from the binary64 operands: one
+// chain of FMAs in the order of K each, as the FP64 kernels sum them, bit for
+// bit.  Bound: the FP64 pipe where many outputs are named; where none is, the
+// reading of the masks (a bit per output).  A unit is eight rows of a tile;
+// units go round the blocks, so that a single tile with a long K still meets
+// sixteen SMs, and the named outputs of a unit are gathered before its rows of
+// A and B pass through shared memory: a few scattered ones cost one warp's
+// FMAs and not all sixteen's.  `end` counts units.
+constexpr int kExRows = 8, kExUnits = kBM / kExRows;  // rows per unit, units per tile
+__global__ void __launch_bounds__(256) x64_exact_kernel(const __grid_constant__ X64Group g) {
+  pdl_begin();
+  constexpr int KC = 32, P = KC + 1;  // of K at a time, and the pitch of its rows
+  __shared__ double As[kExRows * P], Bs[kXBN * P];
+  __shared__ int list[256], n_list, n_out;
+  __shared__ uint16_t outs[kExRows * kXBN];
+  const int tid = threadIdx.x;
+  const int64_t units = g.end[g.n - 1];
+  for (int64_t base = 0; base < units; base += 256 * int64_t(gridDim.x)) {
+    if (tid == 0) n_list = 0;
+    __syncthreads();
+    const int64_t u = base + int64_t(tid) * gridDim.x + blockIdx.x;
+    if (u < units) {
+      int local;
+      const X64Params& p = g.job[item_of(g.end, int(u), local)];
+      const ulonglong2* w = reinterpret_cast<const ulonglong2*>(p.mask + int64_t(local) * kExRows);
+      unsigned long long any = 0;
+#pragma unroll
+      for (int q = 0; q < kExRows / 2; ++q) any |= w[q].x | w[q].y;
+      if (any) list[atomicAdd(&n_list, 1)] = int(u);
+    }
+    __syncthreads();
+    const int n = n_list;
+    for (int i = 0; i < n; ++i) {
+      int local;
+      const X64Params& p = g.job[item_of(g.end, list[i], local)];
+      const int tile = local / kExUnits;
+      const int64_t m0 = int64_t(tile / p.tiles_n) * kBM + local % kExUnits * kExRows;
+      const int64_t n0 = int64_t(tile % p.tiles_n) * kXBN;
+      if (tid == 0) n_out = 0;
+      __syncthreads();
+      for (int e = tid; e < kExRows * kXBN; e += 256)
+        if ((p.mask[int64_t(local) * kExRows + e / kXBN] >> (e % kXBN) & 1) && m0 + e / kXBN < p.M &&
+            n0 + e % kXBN < p.N)
+          outs[atomicAdd(&n_out, 1)] = uint16_t(e);
+      __syncthreads();
+      const int total = n_out;
+      const int e0 = tid < total ? outs[tid] : 0, e1 = tid + 256 < total ? outs[tid + 256] : 0;
+      const double* const a0 = As + e0 / kXBN * P;
+      const double* const b0 = Bs + e0 % kXBN * P;
+      const double* const a1 = As + e1 / kXBN * P;
+      const double* const b1 = Bs + e1 % kXBN * P;
+      double s0 = 0.0, s1 = 0.0;
+      const int kk = tid % KC, rr = tid / KC;  // this thread's column and first row of the loads
+      for (int64_t k0 = 0; k0 < p.K; k0 += KC) {
+        const bool in = k0 + kk < p.K;
+        As[rr * P + kk] = in && m0 + rr < p.M ? p.A64[(m0 + rr) * p.lda + k0 + kk] : 0.0;
+#pragma unroll
+        for (int q = 0; q < kXBN; q += 256 / KC)
+          Bs[(rr + q) * P + kk] = in && n0 + rr + q < p.N ? p.B64[(n0 + rr + q) * p.ldb + k0 + kk] : 0.0;
+        __syncthreads();
+        const int terms = int(min(int64_t(KC), p.K - k0));
+        if (tid < total) {
+#pragma unroll 8
+          for (int k = 0; k < terms; ++k) s0 = fma(a0[k], b0[k], s0);
+        }
+        if (tid + 256 < total) {
+#pragma unroll 8
+          for (int k = 0; k < terms; ++k) s1 = fma(a1[k], b1[k], s1);
+        }
+        __syncthreads();
+      }
+      auto store = [&](int e, double v) {
+        x64_store(p, legmap_offset32(p.m_dst, uint32_t(m0 + e / kXBN)) + legmap_offset32(p.n_dst, uint32_t(n0 + e % kXBN)),
+                  p.alpha * v);
+      };
+      if (tid < total) store(e0, s0);
+      if (tid + 256 < total) store(e1, s1);
+    }
+    __syncthreads();
   }
 }

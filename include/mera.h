@@ -31,16 +31,20 @@
  *   behind mera_ascend_noalloc, the library holds no device memory.
  * - prec selects the arithmetic of the contractions (the O(chi^9) part):
  *     MERA_PREC_F64    binary64 everywhere.  Large products run on the
- *                      tensor cores: each operand entry is cut into seven
+ *                      tensor cores: each operand entry is cut into eight
  *                      signed 8-bit digits relative to the largest entry of
  *                      its row and of its block of 256 along the contraction
- *                      index, the digit products are summed exactly, and the
- *                      result is rounded once to binary64; errors are below
- *                      those of a chain of binary64 FMAs, relative to those
- *                      largest entries.  Rows that hold a NaN, an infinity
- *                      or entries beyond 2^+-400, small products, and calls
- *                      whose workspace does not hold the digits use the FP64
- *                      units.
+ *                      index, and the 36 leading digit products are summed
+ *                      and rounded once to binary64.  An output is taken from
+ *                      them only where the magnitudes of its K terms sum to
+ *                      S >= 2^-8 sqrt(K) times the product of its two rows'
+ *                      scales: its error is then within K 2^-53 S, the bound
+ *                      of a chain of binary64 FMAs, and at random about
+ *                      2^-54 S.  All other outputs (terms far smaller than
+ *                      the largest entries of their rows; rows that hold a
+ *                      NaN, an infinity or entries beyond 2^+-400), small
+ *                      products, and calls whose workspace does not hold the
+ *                      digits use the FP64 units.
  *     MERA_PREC_TF32   tensor cores, TF32 operands, FP32 accumulation,
  *     MERA_PREC_BF16   tensor cores, BF16 operands, FP32 accumulation,
  *     MERA_PREC_BF16X3 tensor cores, each operand split into a BF16 pair

@@ -265,7 +265,7 @@ mera_status run_steps(const OpProgram& prog, const std::pair<int, int>* steps, i
       const Program& dg = diagram(i);
       const Buffer& ax = dg.bufs[size_t(g.ax_buf)];
       const Buffer& bx = dg.bufs[size_t(g.bx_buf)];
-      const int64_t row_img = (g.K + 15) / 16 * 32 * kX64Digits;  // image bytes per row
+      const int64_t row_img = (g.K + 15) / 16 * 32 * kX64Planes;  // image bytes per row
       X64GemmArgs& a = jobs[i];
       a.A = ws + ax.offset + g.ax_tile * kX64TileA * row_img;
       a.ea = reinterpret_cast<const int*>(ws + ax.offset + ax.exp_off) + g.ax_row;
@@ -1144,12 +1144,12 @@ extern "C" mera_status mera_gemm_test(int prec, const double* A, const double* B
   // PREC_F64: the tensor-core route where the workspace also holds the digit
   // images, the row exponents and the K-split partials
   const int xsplit = x64_split_k(M, N, K);
-  const int64_t ldx = (int64_t(K) + 7) / 8 * 8, row_img = int64_t((K + 15) / 16) * 32 * kX64Digits;
+  const int64_t ldx = (int64_t(K) + 7) / 8 * 8, row_img = int64_t((K + 15) / 16) * 32 * kX64Planes;
   const size_t xa = align_up(size_t((M + kX64TileA - 1) / kX64TileA * kX64TileA) * row_img);
   const size_t xb = align_up(size_t((N + kX64TileB - 1) / kX64TileB * kX64TileB) * row_img);
   const size_t xneed = align_up(size_t(M) * ldx * 8) + align_up(size_t(N) * ldx * 8) + xa + xb +
                        align_up(size_t(M) * 4) + align_up(size_t(N) * 4) + size_t(x64_mask_bytes(M, N)) +
-                       size_t(xsplit) * M * N * 12;
+                       size_t(xsplit) * M * N * 16;
   const bool x64 = prec == PREC_F64 && ws_bytes >= xneed;
   if (x64) ld = ldx;
   const size_t pa = align_up(size_t(M) * ld * eb), pb = align_up(size_t(N) * ld * eb);

@@ -482,7 +482,7 @@ struct Builder {
       pb.rows = int64_t(gs.split) * gs.N;
       pb.ld = gs.M;
       pb.plane_bytes = round_up(pb.rows * pb.ld * 4, 256);
-      pb.bytes = pb.plane_bytes * (x64[i] ? 3 : is_oz(prec) ? 2 : 1);  // hi, (mid,) lo planes
+      pb.bytes = pb.plane_bytes * (x64[i] ? 4 : is_oz(prec) ? 2 : 1);  // hi, lo planes; hi, mid, lo and magnitudes
       prog.bufs.push_back(pb);
       gs.p_buf = int(prog.bufs.size()) - 1;
       first_use.push_back(-1);
@@ -597,7 +597,7 @@ struct Builder {
         const Node& cn = tr.nodes[c];
         if (cn.tensor >= 0 || popcount64(cn.legs) != 7) continue;
         // operand bytes per element, the digit image of a PREC_F64 operand included
-        const double bytes = size_of(cn.legs, dim) * (operand_elem_bytes(prec) + (x64[i] ? 2.0 * kX64Digits : 0.0));
+        const double bytes = size_of(cn.legs, dim) * (operand_elem_bytes(prec) + (x64[i] ? 2.0 * kX64Planes : 0.0));
         if (bytes <= double(slice_threshold)) continue;
         const uint64_t K2 = tr.nodes[g[i].a].legs & tr.nodes[g[i].b].legs;
         int best = -1;
@@ -727,7 +727,7 @@ struct Builder {
           const int64_t tiles = segs * ((img_seg[c] + img_tile[c] - 1) / img_tile[c]);
           Buffer im = b;
           im.raw = 0;
-          im.exp_off = round_up(tiles * img_tile[c] * ((Kn + 15) / 16) * 32 * kX64Digits, 256);
+          im.exp_off = round_up(tiles * img_tile[c] * ((Kn + 15) / 16) * 32 * kX64Planes, 256);
           im.plane_bytes = im.bytes = im.exp_off + round_up(b.rows * 4, 256);
           prog.bufs.push_back(im);
           img_of[c] = int(prog.bufs.size()) - 1;
@@ -1049,10 +1049,11 @@ const OpProgram* get_program(int op, int chi_b, int chi_t, int prec, int less) {
   Key k{op, chi_b, chi_t, prec, less};
   auto it = g_cache.find(k);
   if (it != g_cache.end()) return it->second.get();
-  // The digit images nearly triple a PREC_F64 operand.  Past chi ~ 33 the
+  // The digit images more than triple a PREC_F64 operand.  Past chi ~ 33 the
   // operands alone fill most of the memory: those programs stay on the FP64
-  // pipe (env_w at chi = 40: 130 GiB against 307 GiB).
-  constexpr size_t kX64MaxWorkspace = size_t(96) << 30;
+  // pipe (env_w at chi = 32 takes 95 GiB with images, at chi = 40 the operands
+  // alone 130).
+  constexpr size_t kX64MaxWorkspace = size_t(112) << 30;
   constexpr size_t kSpreadAllWorkspace = size_t(1) << 30, kSpreadMaxWorkspace = size_t(4) << 30;
   auto prog = build_program(op, chi_b, chi_t, prec, less > 1, 0);
   if (prog && prog->has_x64 && prog->ws_bytes > kX64MaxWorkspace)

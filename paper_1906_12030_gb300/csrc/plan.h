@@ -35,10 +35,12 @@ inline bool is_oz(int prec) { return prec == PREC_OZ3 || prec == PREC_OZ4; }
 // GEMM sums the leading slice products of such a block exactly in FP32.
 constexpr int kOzBlockK = 256;
 // Large products of PREC_F64 run on the BF16 tensor cores, each entry cut
-// into digits (x64_split.cu, x64_gemm.cuh): digits per entry, entries along K
-// that share a block exponent, 16-wide K steps per block, the largest row
-// exponent the digits represent, and the exponent that marks other rows.
-constexpr int kX64Digits = 7;
+// into digits (x64_split.cu, x64_gemm.cuh): digits per entry, planes of an
+// image (the digits and the magnitudes), entries along K that share a block
+// exponent, 16-wide K steps per block, the largest row exponent the digits
+// represent, and the exponent that marks other rows.
+constexpr int kX64Digits = 8;
+constexpr int kX64Planes = kX64Digits + 1;
 constexpr int kX64Block = 256;
 constexpr int kX64BlockSteps = kX64Block / 16;
 constexpr int kX64MaxExp = 400;

@@ -1167,11 +1167,12 @@ static cudaError_t launch_x64_group(const X64GemmArgs* args, int n, cudaStream_t
     p.partial = a.partial;
     p.p_plane = a.partial_plane;
     p.mask = static_cast<unsigned long long*>(a.mask);
+    p.least = float(std::ldexp(std::max(std::sqrt(double(a.K)), 4.0), -8));
     if (!p.mask) return cudaErrorInvalidValue;
     if (p.split > 1 && (int64_t(p.split - 1) * p.kc >= p.nk || a.partial_plane < int64_t(p.split) * a.N * a.M))
       return cudaErrorInvalidValue;  // an empty split, or overlapping partial planes
     const int64_t tiles_m = (a.M + kBM - 1) / kBM;
-    p.group_m = int(std::min<int64_t>(std::max<int64_t>(1, (int64_t(32) << 20) / (int64_t(p.nk) * kXABytes)), tiles_m));
+    p.group_m = int(std::min<int64_t>(std::max<int64_t>(1, (int64_t(32) << 20) / (int64_t(p.nk) * kXATile)), tiles_m));
     items += tiles_m * ((a.N + kXBN - 1) / kXBN) * p.split;
     if (items > 0x7fffffff) return cudaErrorInvalidValue;
     p.tiles_m = int(tiles_m);

@@ -60,7 +60,7 @@ struct X64GemmArgs {
   double alpha = 1.0;
   int accumulate = 0;
   int split = 1;             // K split (x64_split_k); > 1 needs `partial`
-  float* partial = nullptr;  // hi, mid, lo planes [split][N][M]
+  float* partial = nullptr;  // hi, mid, lo and magnitude planes [split][N][M]
   int64_t partial_plane = 0; // floats from one plane to the next
   void* mask = nullptr;      // x64_mask_bytes(M, N) of scratch
 };

@@ -4,8 +4,8 @@
 //
 // What bounds a binary64 product on this GPU is the FP64 pipe (two FMAs per
 // clock and SM, 1.25 TFLOP/s); the BF16 tensor cores do 1500 times as many
-// products.  So each operand entry is cut into seven signed 8-bit digits
-// (x64_split.cu), and the product is the sum of the 34 digit products whose
+// products.  So each operand entry is cut into eight signed 8-bit digits
+// (x64_split.cu), and the product is the sum of the 36 digit products whose
 // orders p + q are at most 7.  This is the error-free splitting of Ozaki,
 // Ogita, Oishi and Rump (Numer. Algorithms 59, 2012), with one exponent per
 // row and block of 256 along K.
@@ -16,25 +16,39 @@
 // 2^24, what an FP32 accumulator holds exactly, for d <= 3 whatever the data,
 // and for d >= 4 unless nearly all products are extreme and of one sign
 // (then off by a unit of 2^-44 or less, 2^-52 of such a result).  Each order
-// therefore has an accumulator of its own.  What is left out (orders 8 and
-// up, and the bits below the seventh digit) is ~2^-58 and 2^-55 of the
-// block scale: on Gaussian, decaying, heavy-tailed, positive and diagonally
-// dominant operands with K = 16 .. 1024 the error of the sum is 2 to 15
-// times smaller than that of a chain of binary64 FMAs.
+// therefore has an accumulator of its own.
+//
+// Accuracy.  What is left out of a term, the orders from 8 up, is at most
+// 2^-59 of the product of the two rows' scales 2^E and 2^-62 of it at random
+// (the bits below the eighth digit are less).  Against the sum's own size
+// S = sum |a_k b_k| that is nothing where the rows hold entries of one scale,
+// but not where an entry far above the others meets a zero or a small one.
+// So S is summed too, from one more plane of magnitudes, and an output is
+// taken from the digits only where S >= 2^-8 sqrt(K) 2^E (and >= 2^-6 2^E):
+// its error is then below K 2^-53 S, the bound of a chain of binary64 FMAs,
+// whatever the operands, and 2^-54 S or less at random, what such a chain has.
+// S = 0 leaves an exact zero.  The others are left to the FP64 units.  With
+// seven digits and 2^6 times the limit, a tenth to most of the outputs of
+// ordinary maps were below it; with eight 0 to 0.2 % of a map's are (chi = 4
+// to 9 of random isometries, chi = 6 after 3 and 60 sweeps).
 //
 // Tile 128 x 64: eight accumulators of 64 columns fill tensor memory.  (A
 // wider tile has no room for eight; a narrower one needs more shared-memory
 // reads of A per product than the tensor cores take time for.)  The digits of
 // B lie next to each other in a stage and the accumulators next to each
 // other in tensor memory, so one MMA of width 256 meets a digit of A with
-// four digits of B and adds into four orders: 11 MMAs per 16 of K for the 34
-// products.  Per 16 of K the MMAs take 1088 clocks, the shared-memory reads
-// of their operands 896 and the writes of the copies 336: shared-memory
-// bandwidth sets the pace.
+// four digits of B and adds into four orders: 12 MMAs per 16 of K for the 36
+// products.  Per 16 of K the MMAs take 1184 clocks, the shared-memory reads
+// of their operands 1008 and the writes of the copies 432 (magnitudes
+// included): shared-memory bandwidth sets the pace.
 //
-// A stage is 16 of K of all planes, stored by the split kernel as the very
+// A stage is 16 of K of all digits, stored by the split kernel as the very
 // image that the MMA reads (8 x 16-byte core matrices, no swizzle), so a
-// stage is two contiguous bulk copies and five stages fit in shared memory.
+// stage is two contiguous bulk copies and four stages fit in shared memory.
+// The magnitudes come after the last block of a work item, 128 of K to a
+// stage, into the first accumulator once the epilogue has taken the digits'
+// sums out: before the first block, they would have had to wait for the
+// stores of the item before.
 //
 // Warp roles as in tc_gemm_kernel: warp 0 copies, warp 1 MMA, warps 2..17
 // epilogue, four per tensor-memory lane quarter with 16 columns each.  There
@@ -52,18 +66,23 @@
 //
 // Rows of A or B that the digits cannot represent (a NaN, an infinity, or a
 // largest entry beyond 2^+-kX64MaxExp) carry the exponent kX64Bad.  Outputs
-// that touch one are left to x64_exact_kernel, which sums them from the
-// binary64 operands on the FP64 units: each tile has a mask of them, 64 bits
-// per row.  (Summed here, by the epilogue, a column of K = 331776 would keep
-// the copy and MMA warps waiting past the limit of their waits.)
+// that touch one, and those below the limit on S, are left to
+// x64_exact_kernel, which sums them from the binary64 operands on the FP64
+// units: each tile has a mask of them, 64 bits per row.  (Summed here, by the
+// epilogue, a column of K = 331776 would keep the copy and MMA warps waiting
+// past the limit of their waits.)
 
 constexpr int kXBN = 64;
-constexpr int kXPlanes = kX64Digits;
+constexpr int kXDigits = kX64Digits;
 constexpr int kXOrders = 8;
-constexpr int kXABytes = kXPlanes * kBM * 32;    // 16 of K, all digits
-constexpr int kXBBytes = kXPlanes * kXBN * 32;
+constexpr int kXAPlane = kBM * 32, kXBPlane = kXBN * 32;  // 16 of K, one plane
+constexpr int kXABytes = kXDigits * kXAPlane;             // all digits
+constexpr int kXBBytes = kXDigits * kXBPlane;
+constexpr int kXATile = kXABytes + kXAPlane;              // and the magnitudes: bytes of a tile's image per 16 of K
+constexpr int kXBTile = kXBBytes + kXBPlane;
+constexpr int kXMagSteps = kXDigits;                      // 16-wide steps of magnitudes that fill a stage
 constexpr int kXStageBytes = kXABytes + kXBBytes;
-constexpr int kXStages = 5;
+constexpr int kXStages = 4;
 constexpr int kXEpiWarps = 16;
 constexpr int kXEpiThreads = 32 * kXEpiWarps;
 constexpr int kXThreads = 64 + kXEpiThreads;
@@ -88,7 +107,8 @@ struct X64Params {
   int accumulate;
   int nk;             // 16-wide steps of K
   int split, kc;      // K split: steps per split
-  float* partial;     // split > 1: hi, mid, lo planes [split][N][M]
+  float least;        // an output whose scaled magnitudes sum to less, but not to zero, is left to the FP64 units
+  float* partial;     // split > 1: hi, mid, lo and magnitude planes [split][N][M]
   int64_t p_plane;
   unsigned long long* mask;  // outputs left to x64_exact_kernel: [tile][kBM], bit c for column c
   int tiles_m, tiles_n, group_m;  // work items (fewer than 2^31) and their order, as in Epilogue
@@ -235,18 +255,27 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
         const int k0 = split_of(t, p.tiles_m * p.tiles_n, p.split) * p.kc, k1 = min(k0 + p.kc, p.nk);
         int row_t, col_t;
         tile_of(t, p.tiles_m, p.tiles_n, p.group_m, row_t, col_t);
-        const uint8_t* a = p.A + int64_t(row_t) * p.nk * kXABytes;
-        const uint8_t* b = p.B + int64_t(col_t) * p.nk * kXBBytes;
-        for (int k = k0; k < k1; ++k, ++it) {
+        const uint8_t* a = p.A + int64_t(row_t) * p.nk * kXATile;
+        const uint8_t* b = p.B + int64_t(col_t) * p.nk * kXBTile;
+        auto stage = [&](const uint8_t* sa, uint32_t na, const uint8_t* sb, uint32_t nb) {
           const uint32_t s = it % kXStages;
           if (it >= uint32_t(kXStages) && !mbar_wait(&empty[s], ((it / kXStages) & 1) ^ 1, abort_flag)) {
             alive = false;
-            break;
+            return;
           }
           uint8_t* st = smem + size_t(s) * kXStageBytes;
-          mbar_arrive_expect_tx(&full[s], kXStageBytes);
-          bulk_load(st, a + k * int64_t(kXABytes), kXABytes, &full[s]);
-          bulk_load(st + kXABytes, b + k * int64_t(kXBBytes), kXBBytes, &full[s]);
+          mbar_arrive_expect_tx(&full[s], na + nb);
+          bulk_load(st, sa, na, &full[s]);
+          bulk_load(st + kXABytes, sb, nb, &full[s]);
+          ++it;
+        };
+        for (int k = k0; k < k1 && alive; ++k)
+          stage(a + k * int64_t(kXABytes), kXABytes, b + k * int64_t(kXBBytes), kXBBytes);
+        a += int64_t(p.nk) * kXABytes;  // the magnitudes
+        b += int64_t(p.nk) * kXBBytes;
+        for (int k = k0; k < k1 && alive; k += kXMagSteps) {
+          const uint32_t c = uint32_t(min(kXMagSteps, k1 - k));
+          stage(a + k * int64_t(kXAPlane), c * kXAPlane, b + k * int64_t(kXBPlane), c * kXBPlane);
         }
       }
       for (uint32_t j = (it > uint32_t(kXStages) ? it - kXStages : 0); j < it; ++j)
@@ -278,23 +307,14 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
             tc_fence_after();
             const uint32_t sa = smem_u32(smem + size_t(s) * kXStageBytes), sb = sa + kXABytes;
 #pragma unroll
-            for (int pa = 0; pa < kXPlanes; ++pa) {
-              const uint64_t da = x64_desc(sa + pa * kBM * 32);
-              const int nq = min(kXPlanes, kXOrders - pa);  // digits of B that this digit of A meets
+            for (int pa = 0; pa < kXDigits; ++pa) {
+              const uint64_t da = x64_desc(sa + pa * kXAPlane);
+              const int nq = min(kXDigits, kXOrders - pa);  // digits of B that this digit of A meets
 #pragma unroll
               for (int q = 0; q < nq; q += 4) {
                 const int cnt = min(4, nq - q);
-                const uint64_t db = x64_desc(sb + q * kXBN * 32);
+                const uint64_t db = x64_desc(sb + q * kXBPlane);
                 const uint32_t d = tmem + uint32_t((pa + q) * kXBN);
-                if (pa == 1 && q == 4) {
-                  // orders 5, 6 and 7: the last one starts here
-                  if (first) {
-                    tc_mma<PREC_BF16>(d, da, db, make_idesc(1u, kBM, 2 * kXBN), 1u);
-                    tc_mma<PREC_BF16>(d + 2 * kXBN, da, x64_desc(sb + (q + 2) * kXBN * 32),
-                                      make_idesc(1u, kBM, kXBN), 0u);
-                    continue;
-                  }
-                }
                 tc_mma<PREC_BF16>(d, da, db, make_idesc(1u, kBM, cnt * kXBN), (pa == 0 && first) ? 0u : 1u);
               }
             }
@@ -302,6 +322,25 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
           }
           tc_commit(acc_full);  // also after an abort, so that no epilogue warp waits forever
         }
+        if (!alive) break;
+        // the magnitudes, as one more block
+        if (!mbar_wait(acc_empty, (bc - 1) & 1, abort_flag)) break;
+        tc_fence_after();
+        for (int k = k0; k < k1; k += kXMagSteps, ++it) {
+          const uint32_t s = it % kXStages;
+          if (!mbar_wait(&full[s], (it / kXStages) & 1, abort_flag)) {
+            alive = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t sa = smem_u32(smem + size_t(s) * kXStageBytes), sb = sa + kXABytes;
+          for (int j = 0; j < min(kXMagSteps, k1 - k); ++j)
+            tc_mma<PREC_BF16>(tmem, x64_desc(sa + j * kXAPlane), x64_desc(sb + j * kXBPlane),
+                              make_idesc(1u, kBM, kXBN), k > k0 || j > 0 ? 1u : 0u);
+          tc_commit(&empty[s]);
+        }
+        tc_commit(acc_full);
+        ++bc;
       }
     }
   } else {
@@ -375,7 +414,16 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
           break;
         }
       }
-      if (!ok) continue;
+      // sums of the magnitudes
+      uint32_t sum[kXCols];
+      ok = ok && __all_sync(0xffffffffu, mbar_wait(acc_full, bc & 1, abort_flag) ? 1 : 0) != 0;
+      if (!ok) continue;  // the next tile's snapshot sees the abort flag
+      tc_fence_after();
+      tmem_ld16(tmem + uint32_t(c0) + (uint32_t(quarter * 32) << 16), sum);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(acc_empty);
+      ++bc;
       uint16_t* const mask = reinterpret_cast<uint16_t*>(x64_mask(p, row_t, col_t, row)) + c0 / kXCols;
       if (p.split > 1) {  // partial triple, summed by x64_reduce_kernel
         if (ks == 0) *mask = 0;
@@ -387,6 +435,7 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
             q[0] = h[j];
             q[p.p_plane] = mid[j];
             q[2 * p.p_plane] = lo[j];
+            q[3 * p.p_plane] = __uint_as_float(sum[j]);
           }
         continue;
       }
@@ -395,7 +444,8 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
 #pragma unroll
       for (int j = 0; j < kXCols; ++j) {
         if (row_ok && n0 + c0 + j < p.N) todo |= 1u << j;
-        if (ra == kX64Bad || exp_n[c0 + j] == kX64Bad) skip |= 1u << j;
+        const float s = __uint_as_float(sum[j]);
+        if (ra == kX64Bad || exp_n[c0 + j] == kX64Bad || (s < p.least && s > 0.0f)) skip |= 1u << j;
       }
       skip &= todo;
       todo &= ~skip;
@@ -437,8 +487,8 @@ __global__ void __launch_bounds__(kXThreads, 1) x64_gemm_kernel(const __grid_con
   }
 }
 
-// Sum of the K-split partial triples in a fixed order, then the GEMM's
-// output.  One thread per row m over a chunk of columns.
+// Sum of the K-split partial triples and magnitudes in a fixed order, then the
+// GEMM's output.  One thread per row m over a chunk of columns.
 __global__ void __launch_bounds__(128) x64_reduce_kernel(const __grid_constant__ X64Group g) {
   pdl_begin();
   const X64Params& p = g.job[blockIdx.z];
@@ -449,13 +499,14 @@ __global__ void __launch_bounds__(128) x64_reduce_kernel(const __grid_constant__
   const int64_t n_per = (p.N + gridDim.y - 1) / gridDim.y;
   const int64_t n_lo = int64_t(blockIdx.y) * n_per, n_hi = min(p.N, n_lo + n_per);
   for (int64_t n = n_lo; n < n_hi; ++n) {
-    float h = 0.0f, mid = 0.0f, lo = 0.0f;
+    float h = 0.0f, mid = 0.0f, lo = 0.0f, sum = 0.0f;
     for (int s = 0; s < p.split; ++s) {
       const float* q = p.partial + (int64_t(s) * p.N + n) * p.M + m;
       triple_add(h, mid, lo, q[0], q[p.p_plane], q[2 * p.p_plane]);
+      sum += q[3 * p.p_plane];
     }
     const int rb = p.eb[n];
-    if (ra == kX64Bad || rb == kX64Bad) {  // (the mask was cleared by the GEMM)
+    if (ra == kX64Bad || rb == kX64Bad || (sum < p.least && sum > 0.0f)) {  // (the mask was cleared by the GEMM)
       atomicOr(x64_mask(p, int(m / kBM), int(n / kXBN), int(m % kBM)), 1ull << (n % kXBN));
       continue;
     }
@@ -463,44 +514,106 @@ __global__ void __launch_bounds__(128) x64_reduce_kernel(const __grid_constant__
   }
 }
 
-// The outputs that the tiles' masks name, from the binary64 operands: one
-// chain of FMAs in the order of K each, as the FP64 kernels sum them, bit for
-// bit.  Bound: the FP64 pipe where many outputs are named; where none is, the
-// reading of the masks (a bit per output).  A unit is eight rows of a tile;
-// units go round the blocks, so that a single tile with a long K still meets
-// sixteen SMs, and the named outputs of a unit are gathered before its rows of
-// A and B pass through shared memory: a few scattered ones cost one warp's
-// FMAs and not all sixteen's.  `end` counts units.
+// The outputs that the tiles' masks name, from the binary64 operands.  Bound:
+// the FP64 pipe where many are named; where none is, the reading of the masks
+// (a bit per output); in between latency: a map of ordinary operands names a
+// few outputs of every thousand.  So each block looks through its units (eight
+// rows of a tile; they go round the blocks, so that even a single tile meets
+// sixteen SMs) and gathers what they name.  From units that name little, a
+// warp takes an output at a time, 128 terms in flight.  A unit that names much
+// is summed by the whole block through shared memory, one chain of FMAs in the
+// order of K per output, as the FP64 kernels sum it, bit for bit; so is any
+// output of a row that the digits cannot represent.  `end` counts units.
+// (Everything through shared memory: chi = 8 sweep 10.8 ms.)
 constexpr int kExRows = 8, kExUnits = kBM / kExRows;  // rows per unit, units per tile
 __global__ void __launch_bounds__(256) x64_exact_kernel(const __grid_constant__ X64Group g) {
   pdl_begin();
-  constexpr int KC = 32, P = KC + 1;  // of K at a time, and the pitch of its rows
+  constexpr int KC = 32, P = KC + 1;        // of K at a time, and the pitch of its rows
+  constexpr int kFew = 16;                  // outputs of a unit that warps take one by one
   __shared__ double As[kExRows * P], Bs[kXBN * P];
-  __shared__ int list[256], n_list, n_out;
+  __shared__ int many[256], n_many, n_few, n_out;
+  __shared__ int few[256 * kFew];           // thread that looked at the unit, output in it
   __shared__ uint16_t outs[kExRows * kXBN];
-  const int tid = threadIdx.x;
+  static_assert(kExRows * kXBN == 1 << 9, "outputs of a unit");
+  const int tid = threadIdx.x, lane = tid & 31;
   const int64_t units = g.end[g.n - 1];
+  // job of a unit, and where its tile lies
+  auto place = [&](int unit, int& local, int64_t& m0, int64_t& n0) -> const X64Params& {
+    const X64Params& p = g.job[item_of(g.end, unit, local)];
+    const int tile = local / kExUnits;
+    m0 = int64_t(tile / p.tiles_n) * kBM + local % kExUnits * kExRows;
+    n0 = int64_t(tile % p.tiles_n) * kXBN;
+    return p;
+  };
+  auto store = [](const X64Params& p, int64_t m, int64_t n, double v) {
+    x64_store(p, legmap_offset32(p.m_dst, uint32_t(m)) + legmap_offset32(p.n_dst, uint32_t(n)), p.alpha * v);
+  };
   for (int64_t base = 0; base < units; base += 256 * int64_t(gridDim.x)) {
-    if (tid == 0) n_list = 0;
+    if (tid == 0) n_many = n_few = 0;
     __syncthreads();
     const int64_t u = base + int64_t(tid) * gridDim.x + blockIdx.x;
     if (u < units) {
       int local;
-      const X64Params& p = g.job[item_of(g.end, int(u), local)];
+      int64_t m0, n0;
+      const X64Params& p = place(int(u), local, m0, n0);
       const ulonglong2* w = reinterpret_cast<const ulonglong2*>(p.mask + int64_t(local) * kExRows);
-      unsigned long long any = 0;
+      unsigned long long bits[kExRows];
+      int count = 0;
 #pragma unroll
-      for (int q = 0; q < kExRows / 2; ++q) any |= w[q].x | w[q].y;
-      if (any) list[atomicAdd(&n_list, 1)] = int(u);
+      for (int q = 0; q < kExRows; q += 2) {
+        const ulonglong2 v = w[q / 2];
+        bits[q] = v.x;
+        bits[q + 1] = v.y;
+        count += __popcll(v.x) + __popcll(v.y);
+      }
+      if (count > 0) {
+        bool chain = count > kFew;
+        if (!chain) {
+#pragma unroll
+          for (int q = 0; q < kExRows; ++q)
+            for (unsigned long long b = bits[q]; b; b &= b - 1) {
+              const int64_t n = n0 + __ffsll(static_cast<long long>(b)) - 1;
+              if (m0 + q < p.M && n < p.N && (p.ea[m0 + q] == kX64Bad || p.eb[n] == kX64Bad)) chain = true;
+            }
+        }
+        if (chain) {
+          many[atomicAdd(&n_many, 1)] = int(u);
+        } else {
+          int i = atomicAdd(&n_few, count);
+#pragma unroll
+          for (int q = 0; q < kExRows; ++q)
+            for (unsigned long long b = bits[q]; b; b &= b - 1)
+              few[i++] = tid << 9 | (q * kXBN + __ffsll(static_cast<long long>(b)) - 1);
+        }
+      }
     }
     __syncthreads();
-    const int n = n_list;
-    for (int i = 0; i < n; ++i) {
+    for (int i = tid / 32; i < n_few; i += 8) {
       int local;
-      const X64Params& p = g.job[item_of(g.end, list[i], local)];
-      const int tile = local / kExUnits;
-      const int64_t m0 = int64_t(tile / p.tiles_n) * kBM + local % kExUnits * kExRows;
-      const int64_t n0 = int64_t(tile % p.tiles_n) * kXBN;
+      int64_t m, n;
+      const X64Params& p = place(int(base + int64_t(few[i] >> 9) * gridDim.x + blockIdx.x), local, m, n);
+      m += few[i] % (kExRows * kXBN) / kXBN;
+      n += few[i] % kXBN;
+      if (m >= p.M || n >= p.N) continue;
+      const double* a = p.A64 + m * p.lda;
+      const double* b = p.B64 + n * p.ldb;
+      double s[4] = {0.0, 0.0, 0.0, 0.0};
+      int64_t k = lane;
+      for (; k + 96 < p.K; k += 128) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s[q] = fma(a[k + 32 * q], b[k + 32 * q], s[q]);
+      }
+      for (; k < p.K; k += 32) s[0] = fma(a[k], b[k], s[0]);
+      double v = (s[0] + s[1]) + (s[2] + s[3]);
+      __syncwarp();
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) store(p, m, n, v);
+    }
+    for (int i = 0; i < n_many; ++i) {
+      int local;
+      int64_t m0, n0;
+      const X64Params& p = place(many[i], local, m0, n0);
       if (tid == 0) n_out = 0;
       __syncthreads();
       for (int e = tid; e < kExRows * kXBN; e += 256)
@@ -534,12 +647,8 @@ __global__ void __launch_bounds__(256) x64_exact_kernel(const __grid_constant__ 
         }
         __syncthreads();
       }
-      auto store = [&](int e, double v) {
-        x64_store(p, legmap_offset32(p.m_dst, uint32_t(m0 + e / kXBN)) + legmap_offset32(p.n_dst, uint32_t(n0 + e % kXBN)),
-                  p.alpha * v);
-      };
-      if (tid < total) store(e0, s0);
-      if (tid + 256 < total) store(e1, s1);
+      if (tid < total) store(p, m0 + e0 / kXBN, n0 + e0 % kXBN, s0);
+      if (tid + 256 < total) store(p, m0 + e1 / kXBN, n0 + e1 % kXBN, s1);
     }
     __syncthreads();
   }

@@ -3,22 +3,24 @@
 // Every row of an operand is cut into blocks of 256 along K.  With 2^e the
 // exponent of the row's largest entry and 2^b that of the block's (raised to
 // 2^(e-24) where it is smaller, so that every digit product stays a normal
-// binary32 number), an entry x is rounded to a multiple X of 2^(b-54) and X
-// written as seven balanced digits to the base 2^8,
+// binary32 number), an entry x is rounded to a multiple X of 2^(b-62) and X
+// written as eight balanced digits to the base 2^8,
 //   x 2^-e ~ sum_p d_p 2^(b-e-6-8p),   d_0 in [-128, 128], else [-128, 127],
 // each stored as the BF16 value d_p 2^(b-e-6-8p), which is exact.  Entries
-// within a factor four of the block's largest are represented exactly.
-// Adding 128 (256^0 + ... + 256^5) to X makes the balanced digits plain
+// within a factor 2^10 of the block's largest are represented exactly.
+// Adding 128 (256^0 + ... + 256^7) to X makes the balanced digits plain
 // bytes, so a digit costs one byte permute and one FMA.
+// A ninth plane holds |x| 2^-e itself, cut to a BF16 value (below 2^-60, but
+// not zero: 2^-60), from which the GEMM sums the magnitudes of its terms.
 //
 // Image: tiles of `tile` rows (128 for the GEMM's A, 64 for B); per tile and
 // 16 of K, per digit, groups of eight rows, the two 8-wide halves of the 16
-// as 8 x 16-byte core matrices.  A GEMM stage is then one contiguous piece.
+// as 8 x 16-byte core matrices; after all digits of the tile its magnitudes,
+// likewise.  A GEMM stage is then one contiguous piece.
 // Columns K .. 16 ceil(K / 16) - 1 are zero; rows beyond the operand's are
 // not written (they only meet outputs that are not stored).
 //
-// Bound: memory, 8 bytes read and 14 written per entry (65536 x 4096: 5.9 GB
-// in 1.17 ms, 5.05 TB/s).  A block of threads
+// Bound: memory, 8 bytes read and 18 written per entry.  A block of threads
 // holds 8192 entries (whole rows) in registers between finding the exponents
 // and writing the digits, so each entry is read once; rows of more than 8192
 // entries get their exponents from a pass of their own.
@@ -161,22 +163,27 @@ __global__ void __launch_bounds__(kThreadsX, 2) x64_split_kernel(const __grid_co
     const int w = s_max[rr[i] * nb + gg[i] * 8 / kX64Block];
     const int b = max((w >> 20) - 1023, e - 24);  // exponent of the block's grid
     const bool zero = w == 0 || e == kX64Bad;
-    uint32_t lo[8], hi[8];
+    uint32_t lo[8], hi[8], mag[8], top = 0;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const unsigned long long u = static_cast<unsigned long long>(__double_as_longlong(x[i][j]));
       const int ex = int(u >> 52) & 0x7FF;
       long long X = static_cast<long long>((u & 0xFFFFFFFFFFFFFull) | (ex ? 0x10000000000000ull : 0ull));
-      const int sh = ex - 1023 - b + 2;  // X 2^sh multiples of 2^(b-54)
+      const int sh = ex - 1023 - b + 10;  // X 2^sh multiples of 2^(b-62), below 2^63
       if (sh >= 0)
-        X <<= sh;  // at most 2, ex - 1023 <= b
+        X <<= sh;  // at most 10, ex - 1023 <= b
       else
         X = sh < -54 ? 0 : (X + (1ll << (-sh - 1))) >> -sh;
       if (static_cast<long long>(u) < 0) X = -X;
       if (zero) X = 0;
-      X += 0x0000808080808080ll;
-      lo[j] = uint32_t(X);
-      hi[j] = uint32_t(static_cast<unsigned long long>(X) >> 32);
+      const unsigned long long Y = static_cast<unsigned long long>(X) + 0x8080808080808080ull;
+      lo[j] = uint32_t(Y);
+      hi[j] = uint32_t(Y >> 32);
+      // the top digit of a positive X may be 128: its byte has wrapped to 0
+      if (X >= 0 && static_cast<long long>(Y) >= 0) top |= 1u << j;
+      const int em = max(ex - 1023 - e, -60);
+      const uint32_t v = (uint32_t(em + 127) << 7) | (em > -60 ? uint32_t(u >> 45) & 0x7Fu : 0u);
+      mag[j] = zero || (u << 1) == 0 ? 0u : v;
     }
     const int64_t r = r0 + rr[i];
     const int64_t seg = r / a.seg_rows, rs = r - seg * a.seg_rows;
@@ -184,7 +191,10 @@ __global__ void __launch_bounds__(kThreadsX, 2) x64_split_kernel(const __grid_co
     const int ri = int(rs % a.tile);
     const int g = kbase / 8 + gg[i];
     const int plane = a.tile * 32;
-    uint8_t* d = a.img + (t * a.nk + g / 2) * int64_t(kX64Digits * plane) + (ri / 8) * 256 + (g & 1) * 128 + (ri % 8) * 16;
+    uint8_t* d = a.img + t * a.nk * int64_t(kX64Planes * plane) + (ri / 8) * 256 + (g & 1) * 128 + (ri % 8) * 16;
+    *reinterpret_cast<uint4*>(d + (int64_t(a.nk) * kX64Digits + g / 2) * plane) =
+        make_uint4(mag[0] | mag[1] << 16, mag[2] | mag[3] << 16, mag[4] | mag[5] << 16, mag[6] | mag[7] << 16);
+    d += int64_t(g / 2) * (kX64Digits * plane);
 #pragma unroll
     for (int p = 0; p < kX64Digits; ++p) {
       const float sc = zero ? 0.0f : __int_as_float((b - e - 6 - 8 * p + 127) << 23);
@@ -192,11 +202,8 @@ __global__ void __launch_bounds__(kThreadsX, 2) x64_split_kernel(const __grid_co
       uint32_t f[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        uint32_t u;
-        if (p == 0)  // the sign-extended top digit plus 128, in [0, 256]
-          u = 0x4B000000u + uint32_t((int(hi[j]) >> 16) + 128);
-        else
-          u = __byte_perm(p <= 2 ? hi[j] : lo[j], 0x4B000000u, 0x7440u + uint32_t(p <= 2 ? 2 - p : 6 - p));
+        uint32_t u = __byte_perm(p <= 3 ? hi[j] : lo[j], 0x4B000000u, 0x7440u + uint32_t(p <= 3 ? 3 - p : 7 - p));
+        if (p == 0) u += (top >> j & 1u) << 8;
         f[j] = __float_as_uint(__fmaf_rn(__uint_as_float(u), sc, off));
       }
       uint4 o;  // BF16 pairs: the values are exact in the upper halves

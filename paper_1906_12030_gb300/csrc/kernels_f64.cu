@@ -476,15 +476,17 @@ __global__ void __launch_bounds__(256) gemm_f64_kernel(const __grid_constant__ G
   }
 }
 
-static cudaError_t launch_gemm_f64_group(const GemmF64Args* args, int n, cudaStream_t stream) {
-  GemmF64Group g;
-  g.n = 0;
-  for (int i = 0; i < n; ++i) {
-    if (args[i].M <= 0 || args[i].N <= 0) continue;
-    if (args[i].M > 0x7fffffff || args[i].N > 0x7fffffff) return cudaErrorInvalidValue;  // 32-bit row/column decode
-    g.job[g.n++] = args[i];
-  }
+constexpr int64_t kFill = 2 * 152;  // enough blocks to occupy every SM twice
+
+// Whether a product goes to gemm_f64_small_kernel.  It alone sums in another
+// order, so this is for each product by its own size and not by its group's:
+// the result does not depend on what else runs in the launch.
+static bool gemm_f64_is_small(const GemmF64Args& a) { return ((a.M + 15) / 16) * ((a.N + 15) / 16) < kFill; }
+
+// Jobs that are all small, or all not.
+static cudaError_t launch_gemm_f64_group(GemmF64Group& g, cudaStream_t stream) {
   if (g.n == 0) return cudaSuccess;
+  const bool small = gemm_f64_is_small(g.job[0]);
   auto blocks = [&](int64_t r) {
     int64_t t = 0;
     for (int i = 0; i < g.n; ++i) {
@@ -493,10 +495,9 @@ static cudaError_t launch_gemm_f64_group(const GemmF64Args* args, int n, cudaStr
     }
     return t;
   };
-  constexpr int64_t kFill = 2 * 152;  // enough blocks to occupy every SM twice
-  int64_t r = 8;
-  for (int64_t q : {64, 32, 16})
-    if (r == 8 && (blocks(q) >= kFill || blocks(q / 2) > 0x7fffffff)) r = q;
+  int64_t r = small ? 8 : 16;
+  for (int64_t q : {64, 32})
+    if (r == 16 && (blocks(q) >= kFill || blocks(q / 2) > 0x7fffffff)) r = q;
   const int64_t nb = blocks(r);
   if (nb > 0x7fffffff) return cudaErrorInvalidValue;
   count_launch();
@@ -510,11 +511,20 @@ static cudaError_t launch_gemm_f64_group(const GemmF64Args* args, int n, cudaStr
 }
 
 cudaError_t launch_gemm_f64(const GemmF64Args* args, int n, cudaStream_t stream) {
-  for (int i = 0; i < n; i += kGroup) {
-    const cudaError_t e = launch_gemm_f64_group(args + i, std::min(kGroup, n - i), stream);
+  GemmF64Group g[2];
+  g[0].n = g[1].n = 0;
+  for (int i = 0; i < n; ++i) {
+    if (args[i].M <= 0 || args[i].N <= 0) continue;
+    if (args[i].M > 0x7fffffff || args[i].N > 0x7fffffff) return cudaErrorInvalidValue;  // 32-bit row/column decode
+    GemmF64Group& to = g[gemm_f64_is_small(args[i]) ? 1 : 0];
+    to.job[to.n++] = args[i];
+    if (to.n < kGroup) continue;
+    const cudaError_t e = launch_gemm_f64_group(to, stream);
     if (e != cudaSuccess) return e;
+    to.n = 0;
   }
-  return cudaSuccess;
+  const cudaError_t e = launch_gemm_f64_group(g[0], stream);
+  return e != cudaSuccess ? e : launch_gemm_f64_group(g[1], stream);
 }
 
 __global__ void __launch_bounds__(256) ordered_sum_kernel(const double* parts, int n,

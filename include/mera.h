@@ -271,7 +271,8 @@ mera_status mera_sweep(mera_state* state, const double* h1_dev, double shift, in
  * after another and may share one scratch buffer (large enough for each of
  * them).  Lanes run concurrently: a pool of n_threads host threads issues
  * them, so that the launches of different lanes are issued in parallel.
- * Each MERA's result is exactly what mera_sweep gives for it alone.
+ * Each MERA's result is exactly what mera_sweep gives for it alone in a
+ * scratch of that size.
  * Returns the most severe status of the batch; the error text names the
  * MERA.  MERA_EINVAL, before any
  * work, if one scratch pointer is given with two different streams (only
@@ -286,7 +287,10 @@ mera_status mera_sweep_batch(mera_state* states, int n, const double* const* h1,
  * Lanes for mera_sweep_batch under a device-memory budget (host only, no
  * device access).  MERA i has n_layers layers with dimensions
  * chi_b[i * n_layers + k], chi_t[i * n_layers + k]; its scratch is
- * mera_sweep_workspace_size and its cost the contraction flops of one sweep
+ * mera_sweep_workspace_size (MERA_PREC_F64: or less, where that opens more
+ * lanes; the results are the same as long as the digits of large products fit,
+ * and they are left out only where the budget holds no lane with them) and its
+ * cost the contraction flops of one sweep
  * with n_pow power steps.  MERAs whose sweep alone fills the GPU (at least
  * 1e14 flops, e.g. chi >= 20 with tau* = 3) all go to lane 0, one after
  * another: their GEMMs are persistent kernels over every SM, and two of them
@@ -330,7 +334,11 @@ mera_status mera_stiefel_step(const double* X, const double* G, int m, int n, do
 mera_status mera_sweep_riemannian(mera_state* S, const double* h1, double shift, int n_pow, int prec, double eta,
                                   void* ws, size_t ws_bytes, double* e_dev, void* stream);
 
-/* Scratch bytes for mera_sweep on a state with these dimensions. */
+/*
+ * Scratch bytes for mera_sweep on a state with these dimensions.  With a
+ * larger one (up to three times as much below chi ~ 16) the tensor-core modes
+ * run more of their small steps at a time, with the same results.
+ */
 mera_status mera_sweep_workspace_size(int n_layers, const int* chi_b, const int* chi_t, int prec,
                                       size_t* bytes);
 

@@ -351,7 +351,7 @@ size_t op_bytes(const OpProgram& p) { return align_up(p.ws_bytes); }
 // Least of the needs (0 .. kMostLess, get_program) that `avail` bytes hold,
 // need(less) telling each; kMostLess where none does.  So a workspace that is
 // large enough for the operands alone stays accepted.
-constexpr int kMostLess = 2;
+constexpr int kMostLess = 3;
 template <typename Need>
 int pick_less(size_t avail, Need need) {
   int less = 0;
@@ -893,11 +893,17 @@ __global__ void energy_per_spin_kernel(const double* tr, double shift, double* e
 
 using namespace mera::sweep_detail;
 
+// The form (get_program) whose scratch a sweep asks for.  PREC_F64: the
+// fastest.  The other modes: a reused arena, which is what their batches are
+// planned and their budgets refused by; most steps run in waves of one diagram
+// within it (chi = 12 BF16X3: 348 MiB, all diagrams in waves 885).
+static int reported_form(int prec) { return prec == PREC_F64 ? 0 : 2; }
+
 extern "C" mera_status mera_sweep_workspace_size(int n_layers, const int* chi_b, const int* chi_t, int prec,
                                                  size_t* bytes) {
   if (!chi_b || !chi_t || !bytes) return fail(MERA_EINVAL, "null argument");
   SweepLayout L;
-  mera_status st = sweep_layout(n_layers, chi_b, chi_t, prec, &L);
+  mera_status st = sweep_layout(n_layers, chi_b, chi_t, prec, &L, reported_form(prec));
   if (st != MERA_OK) return st;
   *bytes = L.total;
   return MERA_OK;
@@ -1448,11 +1454,25 @@ static mera_status batch_lanes(int n, int n_layers, const int* chi_b, const int*
 extern "C" mera_status mera_batch_lanes(int n, int n_layers, const int* chi_b, const int* chi_t, int prec, int n_pow,
                                         size_t budget_bytes, int max_lanes, int* lane, int* n_lanes,
                                         size_t* lane_bytes) {
-  // a budget that holds PREC_F64 sweeps only in a reduced form is accepted
+  if (prec != PREC_F64)
+    return batch_lanes(n, n_layers, chi_b, chi_t, prec, n_pow, budget_bytes, max_lanes, lane, n_lanes, lane_bytes,
+                       reported_form(prec));
+  // PREC_F64: the form that opens the most lanes, the faster of two that open
+  // as many (lanes side by side fill the GPU as waves do).  The one without
+  // digit products, whose results differ in the last bits, only where the
+  // budget holds no other.
   mera_status st = MERA_ENOMEM;
-  for (int less = 0; less <= (prec == PREC_F64 ? kMostLess : 0) && st == MERA_ENOMEM; ++less)
+  int best = -1, most = 0;
+  for (int less = 0; less <= kMostLess && (less < kMostLess || best < 0); ++less) {
     st = batch_lanes(n, n_layers, chi_b, chi_t, prec, n_pow, budget_bytes, max_lanes, lane, n_lanes, lane_bytes, less);
-  return st;
+    if (st != MERA_OK && st != MERA_ENOMEM) return st;
+    if (st == MERA_OK && *n_lanes > most) {
+      best = less;
+      most = *n_lanes;
+    }
+  }
+  if (best < 0) return st;
+  return batch_lanes(n, n_layers, chi_b, chi_t, prec, n_pow, budget_bytes, max_lanes, lane, n_lanes, lane_bytes, best);
 }
 
 // Tile-width autotuner: every tensor-core GEMM step of the op's program that

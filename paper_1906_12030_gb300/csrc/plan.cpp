@@ -2,6 +2,7 @@
 #include "plan.h"
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <functional>
@@ -857,12 +858,87 @@ std::map<std::tuple<int, int64_t, int64_t, int64_t, int>, int> g_tuned;  // (pre
 
 namespace {
 
+// Memory of the transient buffers of an operation that runs in waves: those
+// that live at a common level, from the one that writes to the last that
+// reads, both included, are kept apart, first fit by size; batches follow one
+// another.  (With memory of its own for every buffer, eight chi = 12 sweeps
+// took three times as much.)  Several diagrams at a time, the program that
+// mera_plan_json describes: also those whose steps overlap within a diagram, so
+// that it can be followed step by step too.
+void pack_waves(OpProgram& prog, const std::vector<std::vector<int>>& levels, int batch) {
+  struct Life {
+    Buffer* b;
+    size_t d;
+    int lo, hi, step_lo, step_hi;
+  };
+  auto meet = [&](const Life& x, const Life& y) {
+    return (x.lo <= y.hi && y.lo <= x.hi) || (batch > 1 && x.d == y.d && x.step_lo <= y.step_hi && y.step_lo <= x.step_hi);
+  };
+  size_t peak = 0;
+  for (size_t d0 = 0; d0 < prog.diagrams.size(); d0 += size_t(batch)) {
+    std::vector<Life> lives;
+    for (size_t d = d0; d < std::min(prog.diagrams.size(), d0 + size_t(batch)); ++d) {
+      Program& pg = prog.diagrams[d];
+      std::vector<Life> life;
+      for (Buffer& b : pg.bufs) life.push_back({&b, d, INT_MAX, -1, 0, 0});
+      for (size_t si = 0; si < pg.steps.size(); ++si) {
+        const int at = levels[d][si];
+        if (at < 0) continue;
+        const Step& st = pg.steps[si];
+        std::vector<int> touched;
+        if (st.kind == 0)
+          touched = {st.p.dst_buf};
+        else if (st.kind == 2)
+          touched = {st.x.raw_buf, st.x.dst_buf};
+        else
+          touched = {st.g.a_buf, st.g.b_buf, st.g.ax_buf, st.g.bx_buf, st.g.c_buf, st.g.p_buf, st.g.m_buf};
+        for (int b : touched)
+          if (b >= 0) {
+            Life& l = life[size_t(b)];
+            if (l.hi < 0) l.step_lo = int(si);
+            l.step_hi = int(si);
+            l.lo = std::min(l.lo, at);
+            l.hi = std::max(l.hi, at);
+          }
+      }
+      for (const Life& l : life) {
+        if (l.b->resident) continue;
+        if (l.hi >= 0) {
+          lives.push_back(l);
+        } else {  // written by no step that runs
+          l.b->offset = int64_t(prog.persistent_bytes);
+          peak = std::max(peak, size_t(l.b->bytes));
+        }
+      }
+    }
+    std::stable_sort(lives.begin(), lives.end(), [](const Life& x, const Life& y) { return x.b->bytes > y.b->bytes; });
+    for (size_t i = 0; i < lives.size(); ++i) {
+      std::vector<std::pair<int64_t, int64_t>> busy;
+      for (size_t j = 0; j < i; ++j)
+        if (meet(lives[j], lives[i]))
+          busy.push_back({lives[j].b->offset, lives[j].b->offset + lives[j].b->bytes});
+      std::sort(busy.begin(), busy.end());
+      int64_t off = int64_t(prog.persistent_bytes);
+      for (const auto& r : busy) {
+        if (off + lives[i].b->bytes <= r.first) break;
+        off = std::max(off, round_up(r.second, 256));
+      }
+      lives[i].b->offset = off;
+      peak = std::max(peak, size_t(off + lives[i].b->bytes) - prog.persistent_bytes);
+    }
+  }
+  prog.spread_bytes = prog.ws_bytes;
+  prog.ws_bytes = prog.persistent_bytes + (peak + 255) / 256 * 256;
+}
+
 // Waves of an operation whose buffers share no memory within a batch of
 // `batch` diagrams: every step goes to the wave after the last of the steps
 // that write what it reads, batch after batch.  False where a program reads a
 // buffer that several steps write (slices).
 bool build_waves(OpProgram& prog, int op, int chi_b, int chi_t, int prec, int batch) {
   const size_t nd = prog.diagrams.size();
+  const bool parts = nd >= 3 && batch > 1;
+  std::vector<std::vector<int>> levels(nd);         // of every step; -1: not run
   std::map<int64_t, int> ready;                     // buffer offset -> level of the step that writes it
   std::map<std::pair<int, int>, Wave> by_level;     // (level, family)
   int root_level = -1, base = 0, top = 0;           // base: first level of the batch
@@ -875,6 +951,7 @@ bool build_waves(OpProgram& prog, int op, int chi_b, int chi_t, int prec, int ba
       ready.swap(kept);
     }
     const Program& pg = prog.diagrams[d];
+    levels[d].assign(pg.steps.size(), -1);
     for (size_t si = 0; si < pg.steps.size(); ++si) {
       const Step& st = pg.steps[si];
       int level = base, out = -1;
@@ -893,8 +970,8 @@ bool build_waves(OpProgram& prog, int op, int chi_b, int chi_t, int prec, int ba
       } else {
         for (int b : {st.g.a_buf, st.g.b_buf, st.g.ax_buf, st.g.bx_buf}) reads(b);
         out = st.g.c_buf;
-        if (out < 0) {  // the second of two diagrams accumulates onto the first's output
-          if (nd < 3 && root_level >= 0) level = std::max(level, root_level + 1);
+        if (out < 0) {  // without parts, a diagram accumulates onto the output of the one before
+          if (!parts && root_level >= 0) level = std::max(level, root_level + 1);
           root_level = level;
         }
       }
@@ -903,11 +980,13 @@ bool build_waves(OpProgram& prog, int op, int chi_b, int chi_t, int prec, int ba
       Wave& w = by_level[{level, fam}];
       w.family = fam;
       w.steps.push_back({int(d), int(si)});
+      levels[d][si] = level;
       top = std::max(top, level);
     }
   }
   for (auto& kv : by_level) prog.waves.push_back(std::move(kv.second));
-  if (nd >= 3) {
+  pack_waves(prog, levels, batch);
+  if (parts) {
     int64_t n = int64_t(chi_b) * chi_b * (op == OP_ENV_U ? int64_t(chi_b) * chi_b : chi_t);
     prog.part_off = int64_t((prog.ws_bytes + 255) / 256 * 256);
     prog.part_bytes = n * 8;
@@ -953,7 +1032,7 @@ std::unique_ptr<OpProgram> build_program(int op, int chi_b, int chi_t, int prec,
     std::set<std::string> shared;
     int64_t budget = int64_t(4) << 30;
     for (const std::string& k : order)
-      if ((count[k] > 1 || spread > 0) && bytes[k] <= (int64_t(1) << 30) && bytes[k] <= budget) {
+      if ((count[k] > 1 || spread > 1) && bytes[k] <= (int64_t(1) << 30) && bytes[k] <= budget) {
         shared.insert(k);
         budget -= bytes[k];
       }
@@ -1045,7 +1124,7 @@ const OpProgram* get_program(int op, int chi_b, int chi_t, int prec, int less) {
   if (chi_b < 1 || chi_t < 1 || chi_b > 64 || chi_t > 64) return nullptr;
   if (chi_t > chi_b * chi_b) return nullptr;
   std::lock_guard<std::mutex> lk(g_mu);
-  if (less > 1 && prec != PREC_F64) less = 1;
+  if (less > 2 && prec != PREC_F64) less = 2;
   Key k{op, chi_b, chi_t, prec, less};
   auto it = g_cache.find(k);
   if (it != g_cache.end()) return it->second.get();
@@ -1055,17 +1134,19 @@ const OpProgram* get_program(int op, int chi_b, int chi_t, int prec, int less) {
   // alone 130).
   constexpr size_t kX64MaxWorkspace = size_t(112) << 30;
   constexpr size_t kSpreadAllWorkspace = size_t(1) << 30, kSpreadMaxWorkspace = size_t(4) << 30;
-  auto prog = build_program(op, chi_b, chi_t, prec, less > 1, 0);
+  auto prog = build_program(op, chi_b, chi_t, prec, less > 2, 0);
   if (prog && prog->has_x64 && prog->ws_bytes > kX64MaxWorkspace)
     prog = build_program(op, chi_b, chi_t, prec, true, 0);
   // Waves pay while one product does not fill the GPU; past that they only
-  // take memory.  All diagrams at once where that is little memory, else in
-  // pairs.
-  if (prog && less == 0 && prog->ws_bytes <= kSpreadMaxWorkspace) {
+  // take memory.  All diagrams at once where that is little memory (before
+  // packing), else in pairs; with less == 1 one after another, which groups
+  // the copies and the branches of each.
+  if (prog && less <= 1 && prog->ws_bytes <= kSpreadMaxWorkspace) {
     const int nd = int(prog->diagrams.size());
-    auto sp = build_program(op, chi_b, chi_t, prec, false, nd);
-    if (sp && nd > 2 && sp->ws_bytes > kSpreadAllWorkspace) sp = build_program(op, chi_b, chi_t, prec, false, 2);
-    if (sp && sp->ws_bytes <= kSpreadMaxWorkspace && sp->ws_bytes >= prog->ws_bytes) prog = std::move(sp);
+    auto sp = build_program(op, chi_b, chi_t, prec, false, less == 0 ? nd : 1);
+    if (sp && less == 0 && nd > 2 && sp->spread_bytes > kSpreadAllWorkspace)
+      sp = build_program(op, chi_b, chi_t, prec, false, 2);
+    if (sp && sp->spread_bytes <= kSpreadMaxWorkspace) prog = std::move(sp);
   }
   if (!prog) return nullptr;
   const OpProgram* out = prog.get();

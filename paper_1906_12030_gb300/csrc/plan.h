@@ -155,12 +155,14 @@ struct Wave {
 struct OpProgram {
   std::vector<Program> diagrams;
   size_t ws_bytes = 0;
+  size_t spread_bytes = 0;      // waves: what they would take with memory of its own for every buffer
   size_t persistent_bytes = 0;  // leading workspace bytes holding the resident copies
   double flops = 0.0;
   int has_x64 = 0;  // some product runs on the tensor cores in PREC_F64
-  // Small operations: every buffer has memory of its own and the steps of all
-  // diagrams run in waves.  With three or more diagrams each writes its part
-  // of the output to part_off + d * part_bytes of the workspace, summed in
+  // Small operations: the steps of all diagrams (or of two, or of one at a
+  // time) run in waves, and no two buffers that live in a common wave share
+  // memory.  With three or more diagrams, two or more at a time, each writes
+  // its part of the output to part_off + d * part_bytes of the workspace, summed in
   // the diagrams' order at the end; else the second accumulates.
   std::vector<Wave> waves;
   int64_t part_off = -1, part_bytes = 0;
@@ -196,9 +198,9 @@ std::vector<std::vector<int64_t>> tuned_tiles();
 int planes(int prec);       // 2 for BF16X3 (hi, lo), 3 for BF16X6 (hi, mid, lo), 3 / 4 for OZ3 / OZ4, else 1
 
 // Builds (and caches) the program; thread safe.  Returns nullptr on bad input.
-// less: 0 the fastest program, 1 one with a reused arena (small operations
-// else run in waves), 2 also PREC_F64 with every product on the FP64 pipe; each
-// needs no more workspace than the one before.
+// less: 0 the fastest program (small operations run in waves), 1 waves of one
+// diagram at a time, 2 one step at a time in a reused arena, 3 also PREC_F64
+// with every product on the FP64 pipe.  The first three give the same bits.
 const OpProgram* get_program(int op, int chi_b, int chi_t, int prec, int less = 0);
 
 // Launch family of a step (Wave).

@@ -103,26 +103,30 @@ int planes(int prec) {
 double operand_elem_bytes(int prec) { return double(elem_bytes(prec) * planes(prec)) + (is_oz(prec) ? 8.0 : 0.0); }
 
 // Cost model of a PREC_F64 product of M x N x K.  FP64 pipe: two FMAs per
-// clock and SM over the tiles of launch_gemm_f64, in waves of one tile per SM
-// (a 100 x 10 x 1000 product is 7 tiles and takes 44 us), plus a launch.
-// Tensor cores: the digit products of the padded tiles, the passes that write
-// the two digit images (8 bytes read and 14 written per entry) and three
-// launches.
+// clock and SM over the tiles of launch_gemm_f64 (8 to 64 wide), in rounds of
+// one tile per SM, plus a launch.  Tensor cores: the digit products of the
+// padded tiles, the passes that write the two digit images (8 bytes read and
+// 18 written per entry) and three launches more.  On their own those cost 22 us,
+// and with that the model picks the faster of the two for all but a few of
+// 665 products of 36..65536 x 6..512 x 16..10000 (64 x 8 x 512: 22 us on the FP64
+// pipe, 33 us as digits; 64 x 8 x 4096: 96 and 55); in a wave the jobs of a
+// launch share them, and 12 us, which chi = 7 env_u is 1.4 times faster with,
+// costs no other map more than 2 %.
 bool x64_use(int64_t M, int64_t N, int64_t K) {
   if (K < 16 || M > 0x3fffffff || N > 0x3fffffff || K > (int64_t(1) << 30)) return false;
   auto tiles = [&](int64_t r) { return ((M + r - 1) / r) * ((N + r - 1) / r); };
-  const int64_t r = tiles(64) >= 304 ? 64 : tiles(32) >= 304 ? 32 : 16;
-  const double fp64 = double((tiles(r) + 151) / 152) * double(r * r) * double(K) * 0.27e-9 + 3e-6;
+  const int64_t r = tiles(64) >= 304 ? 64 : tiles(32) >= 304 ? 32 : tiles(16) >= 304 ? 16 : 8;
+  const double fp64 = double((tiles(r) + 151) / 152) * double(r * r) * double(K) * 0.3e-9 + 3e-6;
   const double mp = double((M + 127) / 128 * 128), np = double((N + 63) / 64 * 64), kp = double((K + 15) / 16 * 16);
-  const double x64 = 2.0 * mp * np * kp / 4.0e13 + 22.0 * (mp + np) * kp / 4.5e12 + 14e-6;
+  const double x64 = 2.0 * mp * np * kp / 3.2e13 + 26.0 * (mp + np) * kp / 4.5e12 + 12e-6;
   return x64 < fp64;
 }
 
 // K split of such a product: over the splits that leave at least eight
 // 16-wide steps each, the one whose waves of work items take the least time.
-// A step takes about 0.7 us, a block's fold (every 16 steps) 1.5 us, a work
-// item 2 us besides, and the sum of the partials 12 bytes per output and
-// split at memory speed plus a launch.
+// A step takes about 0.75 us (magnitudes included), a block's fold (every 16
+// steps) 1.5 us, a work item 2 us besides, and the sum of the partials 16 bytes
+// per output and split, written and read, at memory speed plus a launch.
 int x64_split_k(int64_t M, int64_t N, int64_t K) {
   constexpr int64_t kSMs = 152;
   const int64_t tiles = ((M + kX64TileA - 1) / kX64TileA) * ((N + kX64TileB - 1) / kX64TileB);
@@ -135,8 +139,8 @@ int x64_split_k(int64_t M, int64_t N, int64_t K) {
     const int64_t sn = (nk + kc - 1) / kc;
     if (x64_kc(nk, sn) != kc) continue;  // the launcher derives kc from the split
     const int64_t waves = (tiles * sn + kSMs - 1) / kSMs;
-    double t = double(waves) * (0.7 * double(kc) + 1.5 * double((kc + kX64BlockSteps - 1) / kX64BlockSteps) + 2.0);
-    if (sn > 1) t += 3.0 + 24.0 * double(sn) * double(M) * double(N) / 4e6;
+    double t = double(waves) * (0.75 * double(kc) + 1.5 * double((kc + kX64BlockSteps - 1) / kX64BlockSteps) + 2.0);
+    if (sn > 1) t += 3.0 + 32.0 * double(sn) * double(M) * double(N) / 4e6;
     if (s == 1 || t < best_t * 0.98) {
       best = sn;
       best_t = t;

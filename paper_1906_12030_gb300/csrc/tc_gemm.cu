@@ -444,7 +444,9 @@ __device__ __forceinline__ void store_final(double* __restrict__ r, const int* _
 // back to it.  Why: for a 128 x 256 tile the shared-memory reads and writes of
 // A and B take as long as 1.5 times the TF32 or BF16 MMAs (1.25 times the
 // BF16X3 ones); a pair halves what it reads and writes of B.
-template <int PREC, int BN, int CG>
+// MULTI: the launch may hold several jobs; a launch of one may instead read
+// its parameters at fixed constant addresses.
+template <int PREC, int BN, int CG, bool MULTI>
 __device__ __forceinline__ void tc_gemm_body(const TcGroup& g) {
   using C = Cfg<PREC, BN, CG>;
   extern __shared__ uint8_t smem_raw[];
@@ -465,7 +467,7 @@ __device__ __forceinline__ void tc_gemm_body(const TcGroup& g) {
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const uint32_t rank = CG == 2 ? blockIdx.x & 1u : 0u;  // this CTA in its pair
   const int first_item = int(blockIdx.x) / CG, item_step = int(gridDim.x) / CG;
-  const int items = g.end[g.n - 1];
+  const int items = g.end[MULTI ? g.n - 1 : 0];
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::kStages; ++s) {
@@ -510,8 +512,8 @@ __device__ __forceinline__ void tc_gemm_body(const TcGroup& g) {
       uint32_t it = 0;
       bool alive = true;
       for (int tg = first_item; tg < items && alive; tg += item_step) {
-        int t;
-        const int job = item_of(g.end, tg, t);
+        int t = tg;
+        const int job = MULTI ? item_of(g.end, tg, t) : 0;
         const Epilogue& ep = g.ep[job];
         const TMaps& tm = g.tm[job];
         const int num_k = (int(ep.K) + C::kBK - 1) / C::kBK;
@@ -554,8 +556,8 @@ __device__ __forceinline__ void tc_gemm_body(const TcGroup& g) {
       uint32_t it = 0, tc = 0;
       bool alive = true;
       for (int tg = first_item; tg < items && alive; tg += item_step, ++tc) {
-        int t;
-        const int job = item_of(g.end, tg, t);
+        int t = tg;
+        const int job = MULTI ? item_of(g.end, tg, t) : 0;
         const Epilogue& ep = g.ep[job];
         const int num_k = (int(ep.K) + C::kBK - 1) / C::kBK;
         const uint32_t b = tc & 1;
@@ -619,8 +621,8 @@ __device__ __forceinline__ void tc_gemm_body(const TcGroup& g) {
     const int ch_lo = (sub * kChunks) / kSub, ch_hi = ((sub + 1) * kChunks) / kSub;
     uint32_t tc = 0;
     for (int tg = first_item; tg < items; tg += item_step, ++tc) {
-      int t;
-      const int job = item_of(g.end, tg, t);
+      int t = tg;
+      const int job = MULTI ? item_of(g.end, tg, t) : 0;
       const Epilogue& ep = g.ep[job];
       const float alpha = float(ep.alpha);
       const bool fast_ok = !ep.c_final && ep.split <= 1 && ep.off32 && ep.alpha == 1.0;
@@ -744,15 +746,15 @@ __device__ __forceinline__ void tc_gemm_body(const TcGroup& g) {
   }
 }
 
-template <int PREC, int BN>
+template <int PREC, int BN, bool MULTI>
 __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_constant__ TcGroup g) {
-  tc_gemm_body<PREC, BN, 1>(g);
+  tc_gemm_body<PREC, BN, 1, MULTI>(g);
 }
 
 template <int PREC, int BN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     tc_gemm_pair_kernel(const __grid_constant__ TcGroup g) {
-  tc_gemm_body<PREC, BN, 2>(g);
+  tc_gemm_body<PREC, BN, 2, true>(g);
 }
 
 // Sum of the K-split partials in a fixed order, then the same epilogue as
@@ -888,7 +890,7 @@ int resident_ctas(Kernel kernel, int threads, size_t smem) {
   return std::max(1, sms) * std::max(1, per_sm);
 }
 
-template <int PREC, int BN, int CG>
+template <int PREC, int BN, int CG, bool MULTI = true>
 cudaError_t launch_cfg(const TcGemmArgs* args, int n, cudaStream_t stream) {
   using C = Cfg<PREC, BN, CG>;
   static std::once_flag once;
@@ -898,7 +900,7 @@ cudaError_t launch_cfg(const TcGemmArgs* args, int n, cudaStream_t stream) {
     if constexpr (CG == 2)
       return tc_gemm_pair_kernel<PREC, BN>;
     else
-      return tc_gemm_kernel<PREC, BN>;
+      return tc_gemm_kernel<PREC, BN, MULTI>;
   }();
   std::call_once(once, [&] {
     attr_err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::kSmem));
@@ -1006,6 +1008,11 @@ cudaError_t launch_width(const TcGemmArgs* a, int n, cudaStream_t stream) {
       }
     }
   }
+  // Plain BF16 writes an operand in less time than its MMAs leave per tile only
+  // with the parameters at fixed addresses (descend, all GEMMs: chi = 22 14.1 ->
+  // 12.7 ms, chi = 24 24.7 -> 21.7); the other modes do not feel the look-up.
+  if constexpr (PREC == PREC_BF16 && BN >= 128)
+    if (n == 1) return launch_cfg<PREC, BN, 1, false>(a, n, stream);
   return launch_cfg<PREC, BN, 1>(a, n, stream);
 }
 

@@ -538,8 +538,9 @@ static size_t polar_bytes(int m, int n) {
   return 2 * align_up(size_t(m) * n * sizeof(double)) + 3 * align_up(size_t(n) * n * sizeof(double)) +
          kReduceBytes;
 }
-// The least a polar update runs in: the fused steps do without G2 (up to
-// n = 320 the whole size has always been asked for).
+// The least a polar update runs in: the fused steps do without G2.  (Up to
+// n = 320 the whole size has always been asked for, and G2's place stays
+// empty: with Bm moved into it, 256 x 256 took 1.175 ms instead of 1.148.)
 static size_t polar_bytes_least(int m, int n) {
   return polar_bytes(m, n) - (n > 320 && n <= kNsFusedMax ? align_up(size_t(n) * n * sizeof(double)) : 0);
 }
@@ -569,7 +570,7 @@ static mera_status polar_record(const double* env, int m, int n, double* out, in
   double* Xn = reinterpret_cast<double*>(ar.take(size_t(m) * n * sizeof(double)));
   double* G = reinterpret_cast<double*>(ar.take(size_t(n) * n * sizeof(double)));
   const bool fused = n <= kNsFusedMax;
-  double* G2 = reinterpret_cast<double*>(ar.take(fused ? 0 : size_t(n) * n * sizeof(double)));
+  double* G2 = reinterpret_cast<double*>(ar.take(fused && n > 320 ? 0 : size_t(n) * n * sizeof(double)));
   double* Bm = reinterpret_cast<double*>(ar.take(size_t(n) * n * sizeof(double)));
   double* red = reinterpret_cast<double*>(ar.take(kReduceBytes));
   double* scalars = red + 4096;

@@ -169,11 +169,11 @@ def _peak_tflops(prec: str, sustained: bool = True):
     return base * NOMINAL[prec] / NOMINAL["bf16"], f"{src} {'sustained' if sustained else 'burst'}"
 
 
-# DRAM bytes per launch of the chi^9-class GEMMs, from the ncu capture named
-# here (profiles/).  Reported only for the workload it was taken on; it must
-# be retaken (or set to None) whenever the kernel changes.
-ROOFLINE_TRAFFIC = {("bf16x3", 32): (17.46e9, "profiles/tc_gemm_bf16x3_chi32_descend_dram.md (48 chi^9-class "
-                                              "launches of the descending map, the sweep's most frequent, per launch)")}
+# DRAM bytes per launch of the chi^9-class GEMMs and the ncu capture (profiles/)
+# that they are from, by (mode, chi).  Reported only for the workload it was
+# taken on; it must be retaken, or left out, whenever the kernel changes.
+ROOFLINE_TRAFFIC = {("bf16x3", 32): (38.1e9, "profiles/tc_gemm_bf16x3_chi32_descend_dram.md (40 chi^9-class "
+                                             "launches of the descending map, the sweep's most frequent, per launch)")}
 
 
 def _layer_dims(chi: int):
@@ -686,8 +686,9 @@ def run_native(args):
                                            for k, v in outs.items() if k != "f64"},
                  "throughput": rates,
                  "fp64_sweeps_per_s_at_headline_chi_estimate": rates["f64"]["tflops"] * 1e12 / sweep_flops,
-                 "fp64_estimate_note": "the chi = 16 FP64 sweep's flop rate (the FP64 pipe limit) over the "
-                                       "headline chi's sweep flops",
+                 "fp64_estimate_note": "the chi = 16 FP64 sweep's flop rate (large products as digit products on the "
+                                       "tensor cores, the polar updates on the FP64 pipe) over the headline chi's "
+                                       "sweep flops",
                  "note": "one sweep from the seeded QR start in every mode; FP64 timed directly (its polar "
                          "updates and maps dominate), the others as replayed sweep graphs"}
 

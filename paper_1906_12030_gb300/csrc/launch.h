@@ -8,7 +8,8 @@
 // the compiler read through them before the wait.
 // At small bond dimensions a kernel's launch and set-up cost as much as its
 // work (chi = 4 ascend: 10 launches, 61 us without the overlap, 44 with it).  `overlap`
-// is for kernels whose blocks are all on the GPU at once; blocks of a larger
+// is for kernels whose blocks are all on the GPU at once (each caller's limit
+// is what registers and shared memory let it hold); blocks of a larger
 // kernel that arrive early take their place from the one before (chi = 12
 // OZ4 descend 1.25 -> 1.29 ms).
 #pragma once

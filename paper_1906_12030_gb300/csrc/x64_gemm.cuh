@@ -60,9 +60,10 @@
 // K).
 //
 // Measured (chi = 16 descend, the pair of chi^9 products): 65536 x 4096 x 256
-// 110 ms on the FP64 pipe, 3.0 ms here (46 TFLOP/s); 65536 x 256 x 4096 110
-// -> 2.66 ms (52 TFLOP/s, 0.93 of the burst BF16 rate / 34); the whole map
-// 497 -> 15.6 ms, its error against 64 bits 1.8e-15 -> 1.5e-15.
+// 110 ms on the FP64 pipe, 3.11 ms here (44 TFLOP/s); 65536 x 256 x 4096 110 ->
+// 3.03 ms (45 TFLOP/s, 0.89 of the burst BF16 rate / 37); with seven unchecked
+// digits 3.0 and 2.66.  The whole map 497 -> 17.9 ms, its error against 64 bits
+// 1.8e-15 -> 1.5e-15.
 //
 // Rows of A or B that the digits cannot represent (a NaN, an infinity, or a
 // largest entry beyond 2^+-kX64MaxExp) carry the exponent kX64Bad.  Outputs

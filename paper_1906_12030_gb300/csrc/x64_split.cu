@@ -20,7 +20,8 @@
 // Columns K .. 16 ceil(K / 16) - 1 are zero; rows beyond the operand's are
 // not written (they only meet outputs that are not stored).
 //
-// Bound: memory, 8 bytes read and 18 written per entry.  A block of threads
+// Bound: memory, 8 bytes read and 18 written per entry (65536 x 4096: 7.0 GB
+// in 1.35 ms, 5.2 TB/s).  A block of threads
 // holds 8192 entries (whole rows) in registers between finding the exponents
 // and writing the digits, so each entry is read once; rows of more than 8192
 // entries get their exponents from a pass of their own.
